@@ -113,10 +113,12 @@ struct ara_ctx {
   DevBuf bits, word_cnt, word_pairs, rankdir, mask, slot_cnt, pairs, pairs_hot, pairs_w, pairs_ev, scan_tmp;
   DevBuf ev_buf, tile_cnt;  // hit-event records of the layer kernels
   // event-major index of the YET (ara_build_yet_index) and the indexed passes' buffers
-  DevBuf yix_occ, yix_grid;
+  DevBuf yix_occ, yix_grid, yix_work;
   bool yix_ready = false;
+  bool yix_building = false;  // its buffers are being filled
   bool yix_sorted = false;  // built by the radix sort (a bucket was too large)
   float yix_build_ms = 0.0f;
+  int64_t yix_bytes = 0;
   DevBuf u_flags, u_scan, u_event, u_first, idx_acc;
   DevBuf def_acc;           // per-trial FP64 sums of deferred occurrence losses
   DevBuf elt_stage, elt_recs_stage, elt_tab_stage, elt_flags;  // ELT load staging (grow-only)
@@ -217,6 +219,16 @@ void release(ara_ctx* c, DevBuf& b) {
   b.bytes = 0;
 }
 
+// Frees the index buffers that no index is in (kept from an earlier YET for
+// the next build); false when there is nothing to free.
+bool release_idle_index(ara_ctx* c) {
+  if (c->yix_ready || c->yix_building || (!c->yix_occ.ptr && !c->yix_grid.ptr && !c->yix_work.ptr)) return false;
+  release(c, c->yix_occ);
+  release(c, c->yix_grid);
+  release(c, c->yix_work);
+  return true;
+}
+
 // Make b hold at least `bytes` (contents are not preserved).
 int reserve(ara_ctx* c, DevBuf& b, size_t bytes) {
   if (bytes == 0) bytes = 16;
@@ -228,6 +240,10 @@ int reserve(ara_ctx* c, DevBuf& b, size_t bytes) {
                 bytes, c->used, c->budget, old);
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    if (release_idle_index(c)) e = cudaMalloc(&p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(c, ARA_ENOMEM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
@@ -369,9 +385,10 @@ int yet_begin(ara_ctx* c, int64_t n_trials, const int64_t* offsets, const int32_
     ARA_CUDA(c, cudaEventSynchronize(c->yet_ready));
   }
   c->yet_loaded = false;
-  c->yix_ready = false;  // the index belongs to the YET being replaced
-  release(c, c->yix_occ);
-  release(c, c->yix_grid);
+  // the index belongs to the YET being replaced; without a budget its buffers stay for the next build
+  // (allocating and freeing 8 bytes an event costs milliseconds), until an allocation needs their room
+  c->yix_ready = false;
+  if (c->budget) release_idle_index(c);
   if (!c->copy_stream) {
     ARA_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
     ARA_CUDA(c, cudaEventCreateWithFlags(&c->yet_ready, cudaEventDisableTiming));
@@ -1247,48 +1264,76 @@ int ara_build_yet_index(ara_ctx* c) {
     return fail(c, ARA_EINVAL, "%s: the YET holds 2^32 or more events", who);
   const int64_t n = c->n_events;
   const int64_t cells = ara::yet_grid_cells(c->n_trials, kYetGridShift);
-  DevBuf scratch;
-  if ((rc = reserve(c, c->yix_occ, sizeof(unsigned long long) * (n + 1))) ||
-      (rc = reserve(c, c->yix_grid, sizeof(uint32_t) * (static_cast<size_t>(c->catalogue) * (cells + 1) + 1))) ||
-      (rc = reserve(c, scratch, ara::yet_bucket_scratch_bytes(c->catalogue, cells)))) {
-    release(c, scratch);
+  // while the build runs, an allocation that fails may not take the index's buffers
+  struct Building {
+    ara_ctx* c;
+    explicit Building(ara_ctx* x) : c(x) { c->yix_building = true; }
+    ~Building() { c->yix_building = false; }
+  } building(c);
+  auto drop = [&]() {
     release(c, c->yix_occ);
     release(c, c->yix_grid);
+    release(c, c->yix_work);
+  };
+  if ((rc = reserve(c, c->yix_occ, sizeof(unsigned long long) * (n + 1))) ||
+      (rc = reserve(c, c->yix_grid, sizeof(uint32_t) * (static_cast<size_t>(c->catalogue) * (cells + 1) + 1)))) {
+    drop();
+    return rc;
+  }
+  // The partition build where its fields fit and its 8 bytes an event of scratch do (the event buffer of
+  // the streaming passes serves as that scratch), else the bucket build with its 4 bytes per (event, cell).
+  bool parts = ara::yet_parts_fit(c->n_trials, n, c->catalogue, cells, c->num_sms);
+  const size_t ev_before = c->ev_buf.bytes;
+  if (parts) {
+    const bool room = c->ev_buf.bytes >= sizeof(uint2) * static_cast<size_t>(n + 1) || !c->budget ||
+                      c->used - c->ev_buf.bytes + sizeof(uint2) * static_cast<size_t>(n + 1) +
+                              ara::yet_parts_scratch_bytes(n, c->catalogue, cells, c->num_sms) <=
+                          c->budget;
+    parts = room && reserve(c, c->ev_buf, sizeof(uint2) * (n + 1)) == ARA_OK &&
+            reserve(c, c->yix_work, ara::yet_parts_scratch_bytes(n, c->catalogue, cells, c->num_sms)) == ARA_OK;
+  }
+  if (!parts && (rc = reserve(c, c->yix_work, ara::yet_bucket_scratch_bytes(c->catalogue, cells)))) {
+    drop();
     return rc;
   }
   const int64_t* off = static_cast<const int64_t*>(c->yet_off.ptr);
   const int32_t* ids = static_cast<const int32_t*>(c->yet_ids.ptr);
   unsigned long long* occ = static_cast<unsigned long long*>(c->yix_occ.ptr);
+  unsigned long long* first = static_cast<unsigned long long*>(c->ev_buf.ptr);
   uint32_t* grid = static_cast<uint32_t*>(c->yix_grid.ptr);
   cudaEvent_t a = nullptr, b = nullptr;
   cudaError_t e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
   if (e == cudaSuccess) e = cudaEventRecord(a, c->stream);
   int launched = 0;
-  // buckets per (event, grid cell) while the largest is small; else the radix sort
+  // partitions or buckets while the largest (event, grid cell) is small; else the radix sort
   uint32_t max_bucket = 0;
   if (e == cudaSuccess)
-    e = ara::yet_index_count(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, scratch.ptr, c->stream,
-                             &launched);
+    e = parts ? ara::yet_parts_count(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, c->num_sms, first, grid,
+                                     c->yix_work.ptr, c->stream, &launched)
+              : ara::yet_index_count(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, c->yix_work.ptr,
+                                     c->stream, &launched);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&max_bucket, ara::yet_index_max_bucket(scratch.ptr, c->catalogue, cells), sizeof max_bucket,
-                        cudaMemcpyDeviceToHost, c->stream);
+    e = cudaMemcpyAsync(&max_bucket,
+                        parts ? c->yix_work.ptr : ara::yet_index_max_bucket(c->yix_work.ptr, c->catalogue, cells),
+                        sizeof max_bucket, cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   const bool buckets = max_bucket <= kYetBucketSortMax;
   if (e == cudaSuccess && buckets)
-    e = ara::yet_index_fill(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, occ, scratch.ptr, c->stream,
-                            &launched);
+    e = parts ? ara::yet_parts_fill(c->n_trials, n, c->catalogue, kYetGridShift, c->num_sms, first, grid, occ,
+                                    c->yix_work.ptr, c->stream, &launched)
+              : ara::yet_index_fill(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, occ, c->yix_work.ptr,
+                                    c->stream, &launched);
   if (e == cudaSuccess && !buckets) {
-    release(c, scratch);
-    if ((rc = reserve(c, scratch, ara::yet_index_scratch_bytes(n, c->catalogue)))) {
+    if (c->budget && c->ev_buf.bytes > ev_before) release(c, c->ev_buf);
+    if ((rc = reserve(c, c->yix_work, ara::yet_index_scratch_bytes(n, c->catalogue)))) {
       if (a) cudaEventDestroy(a);
       if (b) cudaEventDestroy(b);
-      release(c, c->yix_occ);
-      release(c, c->yix_grid);
+      drop();
       return rc;
     }
-    e = ara::build_yet_index(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, occ, grid, scratch.ptr, c->stream,
-                             &launched);
+    e = ara::build_yet_index(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, occ, grid, c->yix_work.ptr,
+                             c->stream, &launched);
   }
   if (e == cudaSuccess) e = cudaEventRecord(b, c->stream);
   if (e == cudaSuccess) e = cudaEventSynchronize(b);
@@ -1296,17 +1341,20 @@ int ara_build_yet_index(ara_ctx* c) {
   if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
   if (a) cudaEventDestroy(a);
   if (b) cudaEventDestroy(b);
-  release(c, scratch);
+  // scratch that a budget counts, or the sort build's 24 bytes an event, is given back
+  if (c->budget || !buckets) release(c, c->yix_work);
+  if (c->budget && c->ev_buf.bytes > ev_before) release(c, c->ev_buf);
   c->launches += launched;
   if (e != cudaSuccess) {
     cudaGetLastError();
-    release(c, c->yix_occ);
-    release(c, c->yix_grid);
+    drop();
     return fail(c, ARA_ECUDA, "%s: %s", who, cudaGetErrorString(e));
   }
   c->yix_sorted = !buckets;
   c->yix_ready = true;
   c->yix_build_ms = ms;
+  c->yix_bytes = static_cast<int64_t>(sizeof(unsigned long long) * (n + 1) +
+                                      sizeof(uint32_t) * (static_cast<size_t>(c->catalogue) * (cells + 1) + 1));
   c->serve_ready = false;  // the serving arena is sized again around the index
   return ARA_OK;
 }
@@ -1315,7 +1363,7 @@ int ara_yet_index_info(const ara_ctx* c, int32_t* built, int64_t* bytes, float* 
   if (!c) return ARA_EINVAL;
   if (built) *built = c->yix_ready ? 1 : 0;
   if (method) *method = c->yix_ready ? (c->yix_sorted ? 1 : 0) : -1;
-  if (bytes) *bytes = c->yix_ready ? static_cast<int64_t>(c->yix_occ.bytes + c->yix_grid.bytes) : 0;
+  if (bytes) *bytes = c->yix_ready ? c->yix_bytes : 0;
   if (build_ms) *build_ms = c->yix_ready ? c->yix_build_ms : 0.0f;
   return ARA_OK;
 }
@@ -2115,7 +2163,7 @@ void ara_destroy(ara_ctx* c) {
                     &c->yet_ids,    &c->bits,           &c->word_cnt,      &c->word_pairs,     &c->rankdir,
                     &c->mask,       &c->slot_cnt,       &c->pairs,         &c->pairs_hot,     &c->pairs_w,          &c->pairs_ev,         &c->scan_tmp,       &c->flags,
                     &c->counters,   &c->ylt_tmp,        &c->diag_tmp,      &c->sel,            &c->in_tmp,
-                    &c->out_tmp,    &c->serve_arena,    &c->serve_out,      &c->yix_occ,        &c->yix_grid,       &c->u_flags,
+                    &c->out_tmp,    &c->serve_arena,    &c->serve_out,      &c->yix_occ,        &c->yix_grid,       &c->yix_work,       &c->u_flags,
                     &c->u_scan,        &c->u_event,        &c->u_first,        &c->idx_acc,      &c->serve_sel,      &c->ev_occ,        &c->row_base,
                     &c->evr_stage,  &c->yet_flags};
   for (DevBuf* b : bufs) release(c, *b);

@@ -146,6 +146,335 @@ __global__ void k_sort_cells(const uint32_t* __restrict__ ev_grid, int64_t n_buc
   }
 }
 
+// ---- the partition build: two stable partitions by event id, staged in shared memory
+//
+// The first partition places the occurrences by the id's high digit, packed as
+// (low digit << 53 | trial << 22 | event index), into a buffer of 8 bytes an
+// event; the second partitions each of those buckets by the low digit and
+// unpacks.  Both keep the (trial, event index) order, so no sort follows.
+// What bounds it is memory: 4 B an event for the first count, 4 + 8 for the
+// first partition, 8 for the second count, 8 + 8 for the second partition.
+// Stores go out in runs of one digit (about 8 occurrences, 64 bytes, of a tile
+// of 16,384 at 2,048 digits), where the bucket build's atomic slot claims store
+// 8 bytes at a time; tiles follow one another in a segment, so the next run of
+// a digit completes the line in L2.  Each partition of 400M occurrences takes
+// about 2.7 ms (its counts 0.26 and 0.46 ms at the copy's rate), bound by shared
+// memory and its latency at 16 warps an SM: issue 31%.  One CTA of 512 threads
+// an SM with the next tile's items loaded while a tile goes out; without that
+// 3.6 ms, and as two CTAs of 256 threads with tiles of 8,192 (runs half as long)
+// 3.5 ms.  The build: 6.5 ms at 400,000 trials x 1,000 events, against 14.8 ms
+// by buckets.
+
+constexpr int kPartThreads = 512;
+constexpr int kPartWarps = kPartThreads / 32;
+constexpr int kPartItems = 32;                          // occurrences a lane holds
+constexpr int kPartTile = kPartThreads * kPartItems;    // 16,384: 128 KB of staging
+constexpr int kPartDigits = 2048;                       // digits of a partition, at most
+constexpr int kPartKBits = 22, kPartTrialBits = 31;     // event index, trial (64 = 11 + 31 + 22)
+constexpr uint32_t kPartNone = 0xFFFFu;                 // no occurrence in this slot
+constexpr uint32_t kPartCntBits = 11;                   // a warp's count of a digit (at most 1,024), then a lane
+constexpr uint32_t kPartCntMask = (1u << kPartCntBits) - 1u;
+static_assert(32 * kPartItems <= 1024 && kPartDigits % (2 * kPartThreads) == 0, "counts fit, digits split evenly");
+
+struct PartShared {
+  unsigned long long stage[kPartTile];
+  union {
+    uint16_t wc[kPartWarps][kPartDigits];  // per warp: a digit's count, then the first place of its items
+    uint16_t dig[kPartTile];               // the staged items' digits
+  };
+  uint32_t run[kPartDigits];  // the segment's next output position of each digit
+  uint32_t gb[kPartDigits];   // output position - place in the tile
+  uint32_t wsum[kPartWarps];
+};
+
+// The trial of YET position pos for a whole warp: the last t with off[t] <= pos
+// < off[t + 1], from a t known to be at or below it.  32 probes a round, their
+// spacing growing until one is past pos, then closing in.
+__device__ __forceinline__ int64_t warp_trial_of(const int64_t* __restrict__ off, int64_t n_trials, int64_t t,
+                                                 int64_t pos, uint32_t lane) {
+  int64_t step = 1;
+  for (;;) {
+    const int64_t q = t + 1 + static_cast<int64_t>(lane) * step;
+    const bool past = q >= n_trials || __ldg(off + q) > pos;
+    const uint32_t b = __ballot_sync(0xffffffffu, past);
+    const int first = b ? __ffs(b) - 1 : 32;  // probes before it are at or below pos
+    if (first > 0) t += 1 + static_cast<int64_t>(first - 1) * step;
+    if (b == 0u) step *= 32;
+    else if (step == 1) return t;
+    else step = step > 32 ? step / 32 : 1;
+  }
+}
+
+// Partitions items [begin, end) in tiles of kPartTile by digit, each digit's
+// items in order from sm.run[digit] on.  kFirst: the items are YET positions
+// (ids, off), packed into out; else they are first-partition items (in),
+// unpacked into out.
+template <bool kFirst>
+__device__ __forceinline__ void partition_items(PartShared& sm, const int64_t* __restrict__ off,
+                                                const int32_t* __restrict__ ids, int64_t n_trials, int lo_bits,
+                                                const unsigned long long* __restrict__ in, int64_t begin, int64_t end,
+                                                int n_digits, unsigned long long* __restrict__ out) {
+  n_digits = (n_digits + 7) & ~7;  // whole 16-byte words; the digits past the last have no items
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint32_t lt = (1u << lane) - 1u;
+  const int w0 = static_cast<int>(warp) * 32 * kPartItems;  // the warp's items of a tile: w0 + 32 j + lane
+  int64_t tw = 0;  // kFirst: a trial at or below the warp's items
+  unsigned long long v[kFirst ? 1 : kPartItems];
+  uint32_t id[kFirst ? kPartItems : 1];
+  // a tile's items: the next tile's are in flight while this tile's go out
+  auto load = [&](int64_t base) {
+#pragma unroll
+    for (int j = 0; j < kPartItems; ++j) {
+      const int64_t i = base + w0 + 32 * j + lane;
+      if constexpr (kFirst) id[j] = i < end ? static_cast<uint32_t>(__ldcs(ids + i)) : 0u;
+      else v[j] = i < end ? __ldcs(in + i) : 0ull;
+    }
+  };
+  load(begin);
+  for (int64_t base = begin; base < end; base += kPartTile) {
+    const int n = static_cast<int>(end - base < kPartTile ? end - base : kPartTile);
+    for (int i = 8 * static_cast<int>(lane); i < n_digits; i += 256)
+      *reinterpret_cast<uint4*>(&sm.wc[warp][i]) = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    // the items' ranks within the warp and digit, in order
+    uint32_t at[kPartItems];
+#pragma unroll
+    for (int j = 0; j < kPartItems; ++j) {
+      const bool in_tile = w0 + 32 * j + static_cast<int>(lane) < n;
+      uint32_t d = kPartNone;
+      if (in_tile) {
+        if constexpr (kFirst) d = id[j] >> lo_bits;
+        else d = static_cast<uint32_t>(v[j] >> (kPartTrialBits + kPartKBits));
+      }
+      // Each lane puts its number in the digit's word and reads it back: the lanes whose number stands
+      // there are alone with their digit or the one that the others see.  Few of 32 items share a digit,
+      // so the shared ones are taken a digit at a time (with a warp match on every step instead, a
+      // partition of 400M items took 5.2 ms against 3.6 ms, half its cycles in the unit that matches).
+      uint32_t have = in_tile ? (sm.wc[warp][d] & kPartCntMask) : 0u;
+      __syncwarp();
+      if (in_tile) sm.wc[warp][d] = static_cast<uint16_t>((have + 1u) | (lane << kPartCntBits));
+      __syncwarp();
+      const uint32_t seen = in_tile ? (sm.wc[warp][d] >> kPartCntBits) : lane;
+      uint32_t shared = __ballot_sync(0xffffffffu, seen != lane);
+      uint32_t before = 0u;
+      while (shared) {
+        const uint32_t ds = __shfl_sync(0xffffffffu, d, __ffs(shared) - 1);
+        const uint32_t peers = __ballot_sync(0xffffffffu, d == ds);
+        if (d == ds) {
+          before = __popc(peers & lt);
+          if (before == 0u) sm.wc[warp][d] = static_cast<uint16_t>(have + __popc(peers));
+        }
+        shared &= ~peers;
+      }
+      __syncwarp();
+      at[j] = (d << 16) | (have + before);
+    }
+    __syncthreads();
+    // a thread's digits: counts over the warps to first places, over the digits too
+    // (two digits a word: a tile's counts fit 16 bits)
+    {
+      constexpr int kW = kPartDigits / kPartThreads / 2;  // words a thread
+      const uint32_t d0 = 2u * kW * tid;
+      const bool mine = static_cast<int>(d0) < n_digits;
+      uint32_t t[kW];
+#pragma unroll
+      for (int q = 0; q < kW; ++q) t[q] = 0u;
+      if (mine) {
+#pragma unroll
+        for (int w = 0; w < kPartWarps; ++w) {
+          uint32_t* p = reinterpret_cast<uint32_t*>(&sm.wc[w][d0]);
+#pragma unroll
+          for (int q = 0; q < kW; ++q) {
+            const uint32_t c = p[q];
+            p[q] = t[q];
+            t[q] += c & (kPartCntMask | (kPartCntMask << 16));
+          }
+        }
+      }
+      uint32_t total = 0u;
+#pragma unroll
+      for (int q = 0; q < kW; ++q) total += (t[q] & 0xFFFFu) + (t[q] >> 16);
+      uint32_t incl = total;
+#pragma unroll
+      for (int s = 1; s < 32; s <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xffffffffu, incl, s);
+        if (lane >= static_cast<uint32_t>(s)) incl += o;
+      }
+      if (lane == 31u) sm.wsum[warp] = incl;
+      __syncthreads();
+      uint32_t first = incl - total;
+      for (uint32_t w = 0; w < warp; ++w) first += sm.wsum[w];
+      if (mine) {
+        uint32_t add[kW];
+#pragma unroll
+        for (int q = 0; q < kW; ++q) {
+          const uint32_t c0 = t[q] & 0xFFFFu, c1 = t[q] >> 16, d = d0 + 2u * q;
+          const uint32_t r0 = sm.run[d], r1 = sm.run[d + 1];
+          sm.gb[d] = r0 - first;
+          sm.gb[d + 1] = r1 - (first + c0);
+          sm.run[d] = r0 + c0;
+          sm.run[d + 1] = r1 + c1;
+          add[q] = first | ((first + c0) << 16);
+          first += c0 + c1;
+        }
+#pragma unroll
+        for (int w = 0; w < kPartWarps; ++w) {
+          uint32_t* p = reinterpret_cast<uint32_t*>(&sm.wc[w][d0]);
+#pragma unroll
+          for (int q = 0; q < kW; ++q) p[q] += add[q];
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kPartItems; ++j) {
+      const uint32_t d = at[j] >> 16;
+      if (d != kPartNone) at[j] += sm.wc[warp][d];  // below 2^16: the place in the tile
+    }
+    __syncthreads();  // dig shares wc's memory
+    if constexpr (kFirst) {
+      if (w0 < n) {
+        tw = warp_trial_of(off, n_trials, tw, base + w0, lane);
+        int64_t t = tw, cur = __ldg(off + t), next = __ldg(off + t + 1);
+#pragma unroll
+        for (int j = 0; j < kPartItems; ++j) {
+          const uint32_t d = at[j] >> 16;
+          if (d == kPartNone) continue;
+          const int64_t pos = base + w0 + 32 * j + lane;
+          if (pos >= next) {
+            for (int c = 0; pos >= next && c < 16; ++c) next = __ldg(off + (++t) + 1);
+            if (pos >= next) {  // many short trials: the first b with off[b + 1] > pos
+              int64_t a = t + 1, b = n_trials - 1;
+              while (a < b) {
+                const int64_t m = a + (b - a) / 2;
+                if (__ldg(off + m + 1) > pos) b = m;
+                else a = m + 1;
+              }
+              t = a;
+              next = __ldg(off + t + 1);
+            }
+            cur = __ldg(off + t);
+          }
+          const uint32_t place = at[j] & 0xFFFFu;
+          sm.stage[place] =
+              (static_cast<unsigned long long>(id[j] & ((1u << lo_bits) - 1u)) << (kPartTrialBits + kPartKBits)) |
+              (static_cast<unsigned long long>(t) << kPartKBits) | static_cast<unsigned long long>(pos - cur);
+          sm.dig[place] = static_cast<uint16_t>(d);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < kPartItems; ++j) {
+        const uint32_t d = at[j] >> 16;
+        if (d == kPartNone) continue;
+        const uint32_t place = at[j] & 0xFFFFu;
+        sm.stage[place] = (((v[j] >> kPartKBits) & ((1ull << kPartTrialBits) - 1ull)) << 32) |
+                          (v[j] & ((1ull << kPartKBits) - 1ull));
+        sm.dig[place] = static_cast<uint16_t>(d);
+      }
+    }
+    load(base + kPartTile);
+    __syncthreads();
+#pragma unroll 8
+    for (int i = static_cast<int>(tid); i < n; i += kPartThreads)
+      out[sm.gb[sm.dig[i]] + static_cast<uint32_t>(i)] = sm.stage[i];
+    __syncthreads();
+  }
+}
+
+// segment s of n_seg: YET positions [s E / n_seg, (s + 1) E / n_seg)
+__device__ __forceinline__ int64_t part_bound(int64_t n_events, int n_seg, int64_t s) {
+  return n_events / n_seg * s + n_events % n_seg * s / n_seg;
+}
+
+// cnt[d * n_seg + s]: the segment's events of each high digit (a CTA per segment)
+__global__ void __launch_bounds__(1024) k_part_count(const int32_t* __restrict__ ids, int64_t n_events, int n_seg,
+                                                     int lo_bits, int n_digits, uint32_t* cnt) {
+  __shared__ uint32_t h[kPartDigits];
+  for (int d = threadIdx.x; d < n_digits; d += blockDim.x) h[d] = 0u;
+  __syncthreads();
+  const int64_t end = part_bound(n_events, n_seg, blockIdx.x + 1);
+  constexpr int kU = 8;  // loads in flight
+  for (int64_t i = part_bound(n_events, n_seg, blockIdx.x) + threadIdx.x; i < end; i += kU * 1024) {
+    int32_t e[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) e[u] = i + u * 1024 < end ? __ldcs(ids + i + u * 1024) : -1;
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (e[u] >= 0) atomicAdd(&h[e[u] >> lo_bits], 1u);
+  }
+  __syncthreads();
+  for (int d = threadIdx.x; d < n_digits; d += blockDim.x) cnt[static_cast<int64_t>(d) * n_seg + blockIdx.x] = h[d];
+}
+
+__global__ void __launch_bounds__(kPartThreads, 1)
+    k_part_first(const int64_t* __restrict__ off, const int32_t* __restrict__ ids, int64_t n_trials, int64_t n_events,
+                 int n_seg, int lo_bits, int n_digits, const uint32_t* __restrict__ start,
+                 unsigned long long* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char part_smem[];
+  PartShared& sm = *reinterpret_cast<PartShared*>(part_smem);
+  for (int d = threadIdx.x; d < n_digits; d += kPartThreads)
+    sm.run[d] = start[static_cast<int64_t>(d) * n_seg + blockIdx.x];
+  __syncthreads();
+  partition_items<true>(sm, off, ids, n_trials, lo_bits, nullptr, part_bound(n_events, n_seg, blockIdx.x),
+                        part_bound(n_events, n_seg, blockIdx.x + 1), n_digits, out);
+}
+
+// A bucket's occurrences counted per (event, grid cell) into cnt (with the
+// zero of each event's end column), and the largest count into *max_cnt
+__global__ void __launch_bounds__(1024) k_part_cells(const unsigned long long* __restrict__ in, int n_seg, int lo_bits,
+                                                     const uint32_t* __restrict__ start, int32_t catalogue,
+                                                     int64_t cells, int grid_shift, uint32_t* __restrict__ cnt,
+                                                     uint32_t* max_cnt) {
+  extern __shared__ __align__(16) uint32_t cell_cnt[];
+  const int nc = static_cast<int>(cells);
+  const int64_t e0 = static_cast<int64_t>(blockIdx.x) << lo_bits;
+  const int n_ev = static_cast<int>(min(static_cast<int64_t>(catalogue) - e0, int64_t{1} << lo_bits));
+  for (int i = threadIdx.x; i < n_ev * nc; i += blockDim.x) cell_cnt[i] = 0u;
+  __syncthreads();
+  const uint32_t a = start[static_cast<int64_t>(blockIdx.x) * n_seg];
+  const uint32_t b = start[static_cast<int64_t>(blockIdx.x + 1) * n_seg];
+  constexpr int kU = 4;
+  for (uint64_t i = a + threadIdx.x; i < b; i += kU * 1024) {
+    unsigned long long v[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) v[u] = i + u * 1024 < b ? __ldcs(in + i + u * 1024) : ~0ull;
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (i + u * 1024 < b) {
+        const uint32_t el = static_cast<uint32_t>(v[u] >> (kPartTrialBits + kPartKBits));
+        const uint32_t t = static_cast<uint32_t>(v[u] >> kPartKBits) & ((1u << kPartTrialBits) - 1u);
+        atomicAdd(&cell_cnt[el * nc + (t >> grid_shift)], 1u);
+      }
+  }
+  __syncthreads();
+  uint32_t m = 0u;
+  for (int i = threadIdx.x; i < n_ev * (nc + 1); i += blockDim.x) {
+    const int el = i / (nc + 1), c = i - el * (nc + 1);
+    const uint32_t x = c < nc ? cell_cnt[el * nc + c] : 0u;
+    m = max(m, x);
+    cnt[e0 * (nc + 1) + i] = x;
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31u) == 0u && m) atomicMax(max_cnt, m);
+}
+
+__global__ void __launch_bounds__(kPartThreads, 1)
+    k_part_second(const unsigned long long* __restrict__ in, int n_seg, int lo_bits, const uint32_t* __restrict__ start,
+                  int32_t catalogue, int64_t cells1, const uint32_t* __restrict__ ev_grid,
+                  unsigned long long* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char part_smem[];
+  PartShared& sm = *reinterpret_cast<PartShared*>(part_smem);
+  const int64_t e0 = static_cast<int64_t>(blockIdx.x) << lo_bits;
+  const int n_ev = static_cast<int>(min(static_cast<int64_t>(catalogue) - e0, int64_t{1} << lo_bits));
+  const int64_t begin = start[static_cast<int64_t>(blockIdx.x) * n_seg];
+  const int64_t end = start[static_cast<int64_t>(blockIdx.x + 1) * n_seg];
+  if (begin >= end) return;
+  for (int d = threadIdx.x; d < n_ev; d += kPartThreads) sm.run[d] = ev_grid[(e0 + d) * cells1];
+  __syncthreads();
+  partition_items<false>(sm, nullptr, nullptr, 0, lo_bits, in, begin, end, n_ev, out);
+}
+
 constexpr int64_t kScatterEvents = int64_t{1} << 18;  // events a scatter pass places
 
 int grid_of(int64_t n, int threads) {
@@ -205,6 +534,111 @@ cudaError_t yet_index_fill(const int64_t* off, const int32_t* ids, int64_t n_tri
   }
   k_sort_cells<<<grid_of(n, 256), 256, 0, s>>>(ev_grid, n, occ);
   if (n_launch) *n_launch += launched;
+  return cudaGetLastError();
+}
+
+namespace {
+
+// The partition build's shape.  The high digit takes the bits that leave
+// buckets of about one tile or more (at least 256 of them, so that every SM
+// has some), the low digit the rest; each at most 11 bits.
+struct PartShape {
+  int lo_bits, n_digits, n_seg;
+};
+
+PartShape part_shape(int64_t n_events, int32_t catalogue, int num_sms) {
+  int bits = 1;
+  while (bits < 31 && (int64_t{1} << bits) < static_cast<int64_t>(catalogue)) ++bits;
+  int hi = 8;
+  while (hi < 11 && (n_events >> hi) > kPartTile) ++hi;
+  PartShape sh;
+  sh.lo_bits = bits - hi < 1 ? 1 : bits - hi > 11 ? 11 : bits - hi;
+  sh.n_digits = static_cast<int>(((catalogue - 1) >> sh.lo_bits) + 1);
+  const int64_t tiles = (n_events + kPartTile - 1) / kPartTile;
+  const int64_t most = int64_t{4} * num_sms;  // four segments an SM even out the last ones
+  sh.n_seg = static_cast<int>(tiles < 1 ? 1 : tiles < most ? tiles : most);
+  return sh;
+}
+
+constexpr size_t kPartCellBytes = 200 * 1024;  // shared memory of k_part_cells, at most
+
+}  // namespace
+
+bool yet_parts_fit(int64_t n_trials, int64_t n_events, int32_t catalogue, int64_t cells, int num_sms) {
+  const PartShape sh = part_shape(n_events, catalogue, num_sms);
+  return n_events > 0 && n_events < (int64_t{1} << 32) - 1 && n_trials <= (int64_t{1} << kPartTrialBits) &&
+         sh.n_digits <= kPartDigits && sizeof(uint32_t) * (static_cast<size_t>(cells) << sh.lo_bits) <= kPartCellBytes;
+}
+
+size_t yet_parts_scratch_bytes(int64_t n_events, int32_t catalogue, int64_t cells, int num_sms) {
+  const PartShape sh = part_shape(n_events, catalogue, num_sms);
+  const int64_t np = static_cast<int64_t>(sh.n_digits) * sh.n_seg, n = static_cast<int64_t>(catalogue) * (cells + 1);
+  return sizeof(uint32_t) * (64 + 2 * static_cast<size_t>(np) + 1 + static_cast<size_t>(n) +
+                             (scan_tmp_words(np) > scan_tmp_words(n) ? scan_tmp_words(np) : scan_tmp_words(n)));
+}
+
+namespace {
+
+// scratch: the largest count (in 32 words), the segments' digit counts, their
+// scan, the (event, cell) counts, the scans' scratch
+struct PartScratch {
+  uint32_t *max_cnt, *seg_cnt, *start, *cnt, *tmp;
+};
+
+PartScratch part_scratch(void* scratch, const PartShape& sh, int32_t catalogue, int64_t cells) {
+  const int64_t np = static_cast<int64_t>(sh.n_digits) * sh.n_seg;
+  PartScratch p;
+  p.max_cnt = static_cast<uint32_t*>(scratch);
+  p.seg_cnt = p.max_cnt + 32;
+  p.start = p.seg_cnt + np;
+  p.cnt = p.start + np + 1;
+  p.tmp = p.cnt + static_cast<int64_t>(catalogue) * (cells + 1);
+  return p;
+}
+
+}  // namespace
+
+cudaError_t yet_parts_count(const int64_t* off, const int32_t* ids, int64_t n_trials, int64_t n_events,
+                            int32_t catalogue, int grid_shift, int num_sms, unsigned long long* parts,
+                            uint32_t* ev_grid, void* scratch, cudaStream_t s, int* n_launch) {
+  const int64_t cells = yet_grid_cells(n_trials, grid_shift);
+  const PartShape sh = part_shape(n_events, catalogue, num_sms);
+  const PartScratch p = part_scratch(scratch, sh, catalogue, cells);
+  const int smem = static_cast<int>(sizeof(PartShared));
+  const int cell_smem = static_cast<int>(sizeof(uint32_t) * (static_cast<size_t>(cells) << sh.lo_bits));
+  cudaError_t err;
+  if ((err = cudaFuncSetAttribute(k_part_first, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
+      (err = cudaFuncSetAttribute(k_part_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, cell_smem)) !=
+          cudaSuccess ||
+      (err = cudaMemsetAsync(p.max_cnt, 0, sizeof(uint32_t), s)) != cudaSuccess)
+    return err;
+  k_part_count<<<sh.n_seg, 1024, 0, s>>>(ids, n_events, sh.n_seg, sh.lo_bits, sh.n_digits, p.seg_cnt);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  if ((err = scan_exclusive_u32(p.seg_cnt, p.start, static_cast<int64_t>(sh.n_digits) * sh.n_seg, p.tmp, s,
+                                n_launch)) != cudaSuccess)
+    return err;
+  k_part_first<<<sh.n_seg, kPartThreads, smem, s>>>(off, ids, n_trials, n_events, sh.n_seg, sh.lo_bits, sh.n_digits,
+                                                   p.start, parts);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  k_part_cells<<<sh.n_digits, 1024, cell_smem, s>>>(parts, sh.n_seg, sh.lo_bits, p.start, catalogue, cells, grid_shift,
+                                                   p.cnt, p.max_cnt);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  if (n_launch) *n_launch += 3;
+  return scan_exclusive_u32(p.cnt, ev_grid, static_cast<int64_t>(catalogue) * (cells + 1), p.tmp, s, n_launch);
+}
+
+cudaError_t yet_parts_fill(int64_t n_trials, int64_t n_events, int32_t catalogue, int grid_shift, int num_sms,
+                           const unsigned long long* parts, const uint32_t* ev_grid, unsigned long long* occ,
+                           void* scratch, cudaStream_t s, int* n_launch) {
+  const int64_t cells = yet_grid_cells(n_trials, grid_shift);
+  const PartShape sh = part_shape(n_events, catalogue, num_sms);
+  const PartScratch p = part_scratch(scratch, sh, catalogue, cells);
+  const int smem = static_cast<int>(sizeof(PartShared));
+  const cudaError_t err = cudaFuncSetAttribute(k_part_second, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (err != cudaSuccess) return err;
+  k_part_second<<<sh.n_digits, kPartThreads, smem, s>>>(parts, sh.n_seg, sh.lo_bits, p.start, catalogue, cells + 1,
+                                                       ev_grid, occ);
+  if (n_launch) *n_launch += 1;
   return cudaGetLastError();
 }
 

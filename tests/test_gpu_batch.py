@@ -405,3 +405,38 @@ def test_yet_index_default_and_errors(eng, small_batch):
     assert np.array_equal(dense, indexed)
     eng.load_yet(yet.offsets, yet.event_ids, yet.catalogue_size)
     assert not eng.yet_index_info()["built"] and eng.yet_index_info()["method"] is None
+
+
+@pytest.mark.parametrize("shape", ["one-event", "tile", "tile-and-one", "short-trials", "long-trials", "two-digits",
+                                   "wide-digits", "beyond-the-fields"])
+def test_yet_index_partitions(eng, shape):
+    """The partition build of the index at the edges of its tiles (16,384
+    occurrences), of its digits (2,048 ids each) and of its trial lookup (many
+    empty trials, trials longer than a tile): whole passes and passes whose
+    bounds lie inside a grid cell (found by a search over the occurrences'
+    trials) give the dense item's bits.  A catalogue beyond the partitions'
+    fields (2^22 ids) takes the bucket build."""
+    rng = np.random.default_rng(len(shape))
+    lens, C = {
+        "one-event": ([0, 1, 0], 300),
+        "tile": ([16_384 // 64] * 64, 2_048),
+        "tile-and-one": ([16_384 // 64] * 64 + [1], 2_049),
+        "short-trials": (list(rng.integers(0, 3, 30_000)) + [0] * 5_000 + list(rng.integers(0, 2, 20_000)), 5_000),
+        "long-trials": ([3, 40_000, 0, 17_000, 20_011], 70_001),
+        "two-digits": (list(rng.integers(0, 90, 3_001)), 131_072),
+        "wide-digits": (list(rng.integers(0, 400, 2_003)), 1 << 22),
+        "beyond-the-fields": (list(rng.integers(0, 400, 503)), (1 << 22) + 1),
+    }[shape]
+    offsets = np.zeros(len(lens) + 1, np.int64)
+    offsets[1:] = np.cumsum(lens)
+    n = int(offsets[-1])
+    pool = synth.make_elt_pool(5, min(C, 4_000), C, 33)
+    ev = rng.integers(0, C, n).astype(np.int32)
+    held = rng.random(n) < 0.5  # half the occurrences are of events that ELTs hold
+    ev[held] = rng.choice(pool.event_ids, int(held.sum()))
+    yet = synth.YET(offsets, ev, C)
+    layers = [(np.array(ids, np.int32), (10.0, 5e5, 1e2, 5e7), None) for ids in ([0, 1, 2], [2, 3, 4], [4])]
+    N = len(lens)
+    for t0, t1 in {(0, N), (N // 3, N - N // 5), (N // 2, N // 2 + 1)}:
+        _assert_same_bits(_run_items(eng, yet, pool, layers, 2, t0, t1))
+    assert eng.yet_index_info()["method"] == "buckets"
