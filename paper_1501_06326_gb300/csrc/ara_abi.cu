@@ -404,13 +404,13 @@ int yet_begin(ara_ctx* c, int64_t n_trials, const int64_t* offsets, const int32_
   if (first != 0 || n_events < 0) return fail(c, ARA_EINVAL, "%s: offsets[0] must be 0 and offsets[n] >= 0", who);
   if (n_events > 0 && !event_ids) return fail(c, ARA_EINVAL, "%s: event_ids is NULL", who);
   if ((rc = reserve(c, c->yet_off, sizeof(int64_t) * (n_trials + 1)))) return rc;
-  // ids: padded by 4 entries so that 16-byte loads near the end stay inside the buffer
-  if ((rc = reserve(c, c->yet_ids, sizeof(int32_t) * (n_events + 4)))) return rc;
+  // ids: padded by 8 entries so that 32-byte loads near the end stay inside the buffer
+  if ((rc = reserve(c, c->yet_ids, sizeof(int32_t) * (n_events + 8)))) return rc;
   cudaStream_t cs = c->copy_stream;
   uint32_t* flags = static_cast<uint32_t*>(c->yet_flags.ptr);
   ARA_CUDA(c, cudaMemsetAsync(flags, 0, sizeof(uint32_t), cs));
   ARA_CUDA(c, cudaMemcpyAsync(c->yet_off.ptr, offsets, sizeof(int64_t) * (n_trials + 1), kind_to_device(offsets), cs));
-  ARA_CUDA(c, cudaMemsetAsync(static_cast<int32_t*>(c->yet_ids.ptr) + n_events, 0, sizeof(int32_t) * 4, cs));
+  ARA_CUDA(c, cudaMemsetAsync(static_cast<int32_t*>(c->yet_ids.ptr) + n_events, 0, sizeof(int32_t) * 8, cs));
   ARA_CUDA(c, ara::launch_check_offsets(static_cast<const int64_t*>(c->yet_off.ptr), n_trials, n_events, flags, cs));
   int32_t* d_ids = static_cast<int32_t*>(c->yet_ids.ptr);
   if (n_events > 0 && is_mapped_host_ptr(event_ids)) {
@@ -752,8 +752,8 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   ix.n_words = n_words;
   ix.n_recs = n_recs;
   // ---- gather
-  pl->filt_words = ara::gather_filter_words(n_words, c->max_smem);
-  pl->smem = ara::gather_smem_bytes(pl->filt_words);
+  pl->filt_words = ara::gather_filter_words(n_words, c->max_smem, c->catalogue);
+  pl->smem = ara::gather_smem_bytes(pl->filt_words, c->catalogue);
   if (pl->filt_words < 1 || pl->smem > static_cast<size_t>(c->max_smem))
     return fail(c, ARA_ECUDA, "%s: kernel needs %zu bytes of shared memory, device allows %d", who, pl->smem,
                 c->max_smem);
@@ -776,6 +776,7 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   g.n_words = n_words;
   g.slot_start = ix.slot_cnt;
   g.filt_words = pl->filt_words;
+  g.catalogue = c->catalogue;
   g.ev_buf = static_cast<uint2*>(c->ev_buf.ptr);
   g.tile_cnt = static_cast<uint32_t*>(c->tile_cnt.ptr);
   g.queue = static_cast<unsigned long long*>(c->counters.ptr) + 4;

@@ -147,6 +147,7 @@ struct GatherParams {
   int64_t n_words;
   const uint32_t* slot_start;
   int32_t filt_words;  // filter words: at least n_words / 2, else a power of two
+  int32_t catalogue;   // event ids lie below it
   uint2* ev_buf;
   uint32_t* tile_cnt;
   unsigned long long* queue;  // tile counter
@@ -226,8 +227,8 @@ cudaError_t launch_losses_batch(const BatchParams& p, int item, int grid, cudaSt
 // CTAs of the dense kernel that one SM holds for n_layers layers (0 on error).
 int losses_dense_blocks_per_sm(int n_layers);
 
-size_t gather_smem_bytes(int filt_words);
-int gather_filter_words(int64_t n_words, int max_smem);
+size_t gather_smem_bytes(int filt_words, int32_t catalogue);
+int gather_filter_words(int64_t n_words, int max_smem, int32_t catalogue);
 cudaError_t launch_gather(const GatherParams& p, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_losses(const LossParams& p, int grid, cudaStream_t s);
 

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "ara_internal.h"
 
@@ -32,11 +33,21 @@ __device__ __forceinline__ T warp_inclusive_scan(T v) {
 // catalogue bitmap into a shared-memory membership filter once (as many words
 // as shared memory holds; word w of the catalogue lands on w mod filt_words);
 // then each warp independently takes tiles of kWarpTrials consecutive trials
-// and streams the tile's YET ids, 256 per step (two int4 per lane, not L1-allocated,
-// two more steps in flight).  Each id is tested against the filter; each
-// positive is resolved against the rank directory (8 bytes: the word's bits
-// and its pair base) and, if it is a member, becomes an event record written
-// in YET order to the tile's region of the event buffer.
+// and streams the tile's YET ids, 256 per step (32 bytes per lane, not
+// L1-allocated, two more steps in flight).  Each id is tested against the
+// filter; the positives collect in a small ring, in YET order, and every 32 of
+// them are resolved together against the rank directory (8 bytes: the word's
+// bits and its pair base), a group's directory words in flight while the next
+// step is filtered.  A member becomes an event record written in YET order to
+// the tile's region of the event buffer.
+// What bounds it is the SM's shared-memory and L1 data pipe (paper-1m: 79% of
+// its wavefronts; about 80 a step, of which the filter's lookups with their
+// bank conflicts take 27, the directory words 22, the id stream 16).  So the
+// ring takes one packed word a positive, the lanes' places come from ballots
+// and not from shuffles (which use that pipe too), groups are always full, and
+// a trial is searched only where a group crosses into the next one: 99
+// wavefronts a step before that and 311 warp instructions against 252; at
+// paper-1m 1.37 ms before, 1.14 ms now.
 //
 // k_losses: each warp takes tiles and reads their records one per lane.  An
 // event with one (event, ELT) pair is finished by its lane: Philox uniform,
@@ -52,17 +63,32 @@ namespace {
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
 
+// Filter positives waiting to be resolved, per warp: up to 31 left from earlier
+// steps and the 256 of one step.  kPacked: one word each, the event id above
+// the low kPosBits bits of its position in the tile; else the id and the
+// position in the step.
+constexpr int kGatherRing = 288;
+constexpr uint32_t kPosBits = 11;
+constexpr int32_t kPackedCatalogue = 1 << (32 - kPosBits);
 
 struct GatherWarp {
-  int32_t off[16];      // trial offsets relative to the tile's first event; INT32_MAX past the tile's end
-  uint32_t pos_id[256];  // filter positives of one step: event id
-  uint8_t pos_q[256];    //   and position in the step
+  int32_t off[16];            // trial offsets in the tile's positions; INT32_MAX past the tile's end
+  uint32_t ring[kGatherRing];
 };
+struct GatherWarpWide {
+  int32_t off[16];
+  uint32_t ring[kGatherRing];
+  uint8_t ring_q[kGatherRing];
+};
+
+template <bool kPacked>
+using GatherShared = typename std::conditional<kPacked, GatherWarp, GatherWarpWide>::type;
 
 }  // namespace
 
-size_t gather_smem_bytes(int filt_words) {
-  return sizeof(uint32_t) * static_cast<size_t>(filt_words) + sizeof(GatherWarp) * (kGatherThreads / 32) + 16;
+size_t gather_smem_bytes(int filt_words, int32_t catalogue) {
+  return sizeof(uint32_t) * static_cast<size_t>(filt_words) +
+         (catalogue <= kPackedCatalogue ? sizeof(GatherWarp) : sizeof(GatherWarpWide)) * (kGatherThreads / 32) + 16;
 }
 
 // k_gather's shared memory stays within the 196 KB carveout (less the 1 KB
@@ -72,9 +98,9 @@ size_t gather_smem_bytes(int filt_words) {
 // filter saves.
 constexpr int kGatherSmemBudget = 196 * 1024 - 1024;
 
-int gather_filter_words(int64_t n_words, int max_smem) {
+int gather_filter_words(int64_t n_words, int max_smem, int32_t catalogue) {
   const int64_t budget = max_smem < kGatherSmemBudget ? max_smem : kGatherSmemBudget;
-  const int64_t room = (budget - static_cast<int64_t>(gather_smem_bytes(0))) / 4;
+  const int64_t room = (budget - static_cast<int64_t>(gather_smem_bytes(0, catalogue))) / 4;
   const int64_t fw_max = room & ~int64_t(31);
   if (fw_max < 32) return 0;
   if (n_words <= 2 * fw_max) return static_cast<int>(n_words <= fw_max ? (n_words > 0 ? n_words : 1) : fw_max);
@@ -85,170 +111,189 @@ int gather_filter_words(int64_t n_words, int max_smem) {
 
 namespace {
 
-// State of one warp's pass over one tile.
-struct GatherTile {
-  const int4* ids4;  // the tile's ids from the 16-byte boundary at or below its first event
-  int32_t lead;      // ids before the tile's first event in the first int4
-  int32_t nev;       // events of the tile
-  int32_t span;      // nev + lead
-  uint2* out;        // the tile's region of the event buffer
-  uint32_t nout;     // records written
+// Eight YET ids (32 bytes, read once): not allocated in L1, whose capacity
+// holds the loads in flight (measured 1% faster than evict-first loads).
+struct Ids8 {
+  uint32_t e[8];
 };
-
-// One int4 of YET ids, read once: not allocated in L1, whose capacity holds
-// the loads in flight (measured 1% faster than evict-first loads).
-__device__ __forceinline__ int4 ld_ids(const int4* a) {
-  int4 v;
-  asm("ld.global.nc.L1::no_allocate.v4.s32 {%0, %1, %2, %3}, [%4];"
-      : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+__device__ __forceinline__ Ids8 ld_ids(const int32_t* a) {
+  Ids8 v;
+  asm("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(v.e[0]), "=r"(v.e[1]), "=r"(v.e[2]), "=r"(v.e[3]), "=r"(v.e[4]), "=r"(v.e[5]), "=r"(v.e[6]), "=r"(v.e[7])
       : "l"(a));
   return v;
 }
 
-// Loads step c0 (256 ids: int4 lane and int4 32 + lane of the step).
-__device__ __forceinline__ void gather_load(const GatherTile& g, int32_t c0, uint32_t lane, int4& v0, int4& v1) {
-  v0 = make_int4(0, 0, 0, 0);
-  v1 = make_int4(0, 0, 0, 0);
-  const int32_t i0 = c0 + 4 * static_cast<int32_t>(lane);
-  if (i0 < g.span) v0 = ld_ids(g.ids4 + (i0 >> 2));
-  if (i0 + 128 < g.span) v1 = ld_ids(g.ids4 + ((i0 + 128) >> 2));
-}
-
-// Positives of one step whose rank-directory words are in flight: entries
-// lane and 32 + lane of the step's staging list.
-struct GatherPending {
-  uint2 q0, q1;    // (event id, position in the step)
-  uint2 rd0, rd1;  // rank-directory words {bits, base}
-  int32_t c0;      // the step's first position
-  uint32_t npos;   // entries (at most 64; 0 = nothing pending)
+// State of one warp's pass over one tile.  Positions count from the 32-byte
+// boundary at or below the tile's first event.
+struct GatherTile {
+  const int32_t* ids;  // position 0
+  int32_t lead;        // positions before the tile's first event
+  int32_t span;        // positions up to the tile's end
+  uint2* out;          // the tile's region of the event buffer
+  uint32_t nout;       // records written
+  // the trial of the last position resolved: its end, and trial << 28 minus its first position (the key of
+  // a one-pair record of the trial is this plus its position)
+  int32_t t_end;
+  uint32_t t_key;
+  // positives left in the ring (fewer than 32), the lane's one of them, and the step they began in
+  uint32_t left;
+  uint32_t keep, keep_q;
+  int32_t left_c0;
+  // the group of positives whose rank-directory words are in flight
+  uint32_t pd_n, pd_id;
+  int32_t pd_pos;
+  uint2 pd_rd;
 };
 
-// Resolves one staged positive per lane (warp-wide call): if the event is a
-// member, its record is appended to the tile's records in lane order.
-__device__ __forceinline__ void gather_resolve(const GatherParams& p, const GatherWarp& ws, GatherTile& g, int32_t c0,
-                                               uint2 q, uint2 rd, bool valid, uint32_t lane) {
-  uint32_t key = 0, ps = 0;
-  const uint32_t bit = 1u << (q.x & 31);
-  const bool hit = valid && (rd.x & bit) != 0u;
-  if (hit) {
-    const uint32_t below = __popc(rd.x & (bit - 1u));
-    uint32_t cnt = 1;
-    if (rd.y & 0x80000000u) {
-      const uint32_t sl = (rd.y & 0x7FFFFFFFu) + below;
-      ps = __ldg(&p.slot_start[sl]);
-      cnt = __ldg(&p.slot_start[sl + 1]) - ps;
-    } else {
-      ps = rd.y + below;
-    }
-    // trial: the last t with off[t] <= rel (off is padded with INT32_MAX)
-    const int32_t rel = c0 + static_cast<int32_t>(q.y) - g.lead;
-    int t = (ws.off[4] <= rel) ? 4 : 0;
-    t += (ws.off[t + 2] <= rel) ? 2 : 0;
-    t += (ws.off[t + 1] <= rel) ? 1 : 0;
-    key = ((cnt - 1u) << kRecCntShift) | (static_cast<uint32_t>(t) << kRecTrialShift) |
-          static_cast<uint32_t>(rel - ws.off[t]);
+// The ids of step c0: positions c0 + 8 lane .. c0 + 8 lane + 7.
+__device__ __forceinline__ Ids8 gather_load(const GatherTile& g, int32_t c0, uint32_t lane) {
+  Ids8 v;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) v.e[j] = 0u;
+  const int32_t i0 = c0 + 8 * static_cast<int32_t>(lane);
+  if (i0 < g.span) v = ld_ids(g.ids + i0);
+  return v;
+}
+
+// Finishes the group in flight (warp-wide): an event that is a member has its
+// record appended to the tile's records, in lane order.
+template <class Shared>
+__device__ __forceinline__ void gather_complete(const GatherParams& p, const Shared& ws, GatherTile& g,
+                                                uint32_t lane) {
+  if (g.pd_n == 0u) return;
+  const bool valid = lane < g.pd_n;
+  // the word's bits up to the event's, the event's in the sign
+  const uint32_t upto = __funnelshift_l(0u, g.pd_rd.x, ~g.pd_id);
+  const bool hit = valid && static_cast<int32_t>(upto) < 0;
+  uint32_t key = g.t_key + static_cast<uint32_t>(g.pd_pos);
+  if (__any_sync(0xffffffffu, valid && g.pd_pos >= g.t_end)) {
+    // a later trial: the last t with off[t] <= pos (off is padded with INT32_MAX)
+    int t = (ws.off[4] <= g.pd_pos) ? 4 : 0;
+    t += (ws.off[t + 2] <= g.pd_pos) ? 2 : 0;
+    t += (ws.off[t + 1] <= g.pd_pos) ? 1 : 0;
+    const uint32_t tk = (static_cast<uint32_t>(t) << kRecTrialShift) - static_cast<uint32_t>(ws.off[t]);
+    key = tk + static_cast<uint32_t>(g.pd_pos);
+    g.t_end = __shfl_sync(0xffffffffu, ws.off[t + 1], g.pd_n - 1u);
+    g.t_key = __shfl_sync(0xffffffffu, tk, g.pd_n - 1u);
+  }
+  uint32_t ps = (g.pd_rd.y & 0x7FFFFFFFu) + __popc(upto) - 1u;
+  if (hit && static_cast<int32_t>(g.pd_rd.y) < 0) {  // the word holds an event with several pairs
+    const uint32_t first = __ldg(&p.slot_start[ps]);
+    key += (__ldg(&p.slot_start[ps + 1]) - first - 1u) << kRecCntShift;
+    ps = first;
   }
   const uint32_t hm = __ballot_sync(0xffffffffu, hit);
   if (hit) g.out[g.nout + __popc(hm & ((1u << lane) - 1u))] = make_uint2(key, ps);
   g.nout += __popc(hm);
 }
 
-// Finishes the pending positives of the previous step.
-__device__ __forceinline__ void gather_complete(const GatherParams& p, const GatherWarp& ws, GatherTile& g,
-                                                const GatherPending& pd, uint32_t lane) {
-  if (pd.npos == 0) return;
-  gather_resolve(p, ws, g, pd.c0, pd.q0, pd.rd0, lane < pd.npos, lane);
-  if (pd.npos > 32) gather_resolve(p, ws, g, pd.c0, pd.q1, pd.rd1, 32 + lane < pd.npos, lane);
+// Puts a group of n positives in flight (lane < n: event id, position).
+__device__ __forceinline__ void gather_launch(const GatherParams& p, GatherTile& g, uint32_t n, uint32_t id,
+                                              int32_t pos, uint32_t lane) {
+  g.pd_n = n;
+  g.pd_id = id;
+  g.pd_pos = pos;
+  g.pd_rd = lane < n ? __ldg(&p.rankdir[id >> 5]) : make_uint2(0u, 0u);
 }
 
-// One step of 256 YET positions: filter, compact the positives in YET order,
-// finish the previous step's positives, then either put this step's in flight
-// (up to 64) or resolve them at once.
+// One step of 256 YET positions: filter, append the positives to the ring in
+// YET order, then for every 32 of the ring finish the group in flight and put
+// the next in flight; fewer than 32 stay for the next step.
 // kSub: the catalogue has at most twice filt_words words, and word w folds
 // onto min(w, w - filt_words) (unsigned); otherwise filt_words is a power of
 // two and w folds onto w & (filt_words - 1).  fsel is filt_words or the mask.
-template <bool kSub>
+template <bool kSub, bool kPacked>
 __device__ __forceinline__ void gather_step(const GatherParams& p, const uint32_t* __restrict__ filt, uint32_t fsel,
-                                            GatherWarp& ws, GatherTile& g, GatherPending& pd, int32_t c0,
-                                            uint32_t lane, int4 v0, int4 v1) {
-  const uint32_t e[8] = {static_cast<uint32_t>(v0.x), static_cast<uint32_t>(v0.y), static_cast<uint32_t>(v0.z),
-                         static_cast<uint32_t>(v0.w), static_cast<uint32_t>(v1.x), static_cast<uint32_t>(v1.y),
-                         static_cast<uint32_t>(v1.z), static_cast<uint32_t>(v1.w)};
-  // 1. filter (the shift count of a funnel shift is taken mod 32)
+                                            GatherShared<kPacked>& ws, GatherTile& g, int32_t c0, uint32_t lane,
+                                            const Ids8& ids) {
+  // 1. filter: bit j of m is position 8 lane + j's (the shift count of a funnel shift is taken mod 32)
   uint32_t m = 0;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const uint32_t wi = e[j] >> 5;
+    const uint32_t wi = ids.e[j] >> 5;
     const uint32_t w = filt[kSub ? min(wi, wi - fsel) : (wi & fsel)];
-    m |= (__funnelshift_r(w, w, e[j]) & 1u) << j;
+    m = __funnelshift_r(m, __funnelshift_r(w, w, ids.e[j]), 1);
   }
-  const uint32_t q0 = 4u * lane;  // step positions of the lane's ids: q0 + j, q0 + 128 + j
+  m >>= 24;
+  const int32_t first = c0 + 8 * static_cast<int32_t>(lane);
   if (c0 == 0 || c0 + 256 > g.span) {
-    uint32_t vm = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int32_t rel = c0 + static_cast<int32_t>(q0 + (j & 3) + (j >> 2) * 128) - g.lead;
-      vm |= (static_cast<uint32_t>(rel) < static_cast<uint32_t>(g.nev) ? 1u : 0u) << j;
-    }
-    m &= vm;
+    // positions before the tile's first event and from its end on
+    const int32_t lo = g.lead - first, hi = g.span - first;
+    const uint32_t below = lo > 0 ? (lo < 8 ? (1u << lo) - 1u : 0xFFu) : 0u;
+    const uint32_t upto = hi > 0 ? (hi < 8 ? (1u << hi) - 1u : 0xFFu) : 0u;
+    m &= upto & ~below;
   }
-  // 2. compaction: one scan over both halves (16-bit fields)
-  const uint32_t cl = __popc(m & 15u), ch = __popc(m >> 4);
-  const uint32_t incl = warp_inclusive_scan(cl | (ch << 16));
-  const uint32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-  const uint32_t nlo = tot & 0xFFFFu;
-  const uint32_t npos = nlo + (tot >> 16);
-  // 3. the previous step's positives (their loads had this step's filter to land)
-  gather_complete(p, ws, g, pd, lane);
-  pd.npos = 0;
-  if (npos == 0) return;
-  // 4. this step's positives: staged, then in flight, or resolved at once when there are many
-  if (m) {
-    uint32_t at = (incl & 0xFFFFu) - cl;
+  auto entry = [&](uint32_t i, uint32_t* v, uint32_t* q) {
+    *v = ws.ring[i];
+    if constexpr (!kPacked) *q = ws.ring_q[i];
+  };
+  auto send = [&](uint32_t v, uint32_t q, uint32_t k) {
+    gather_complete(p, ws, g, lane);
+    if constexpr (kPacked) {
+      const int32_t last = c0 + 255;
+      gather_launch(p, g, k, v >> kPosBits,
+                    last - static_cast<int32_t>((static_cast<uint32_t>(last) - v) & ((1u << kPosBits) - 1u)), lane);
+    } else {
+      gather_launch(p, g, k, v, c0 + static_cast<int32_t>(q), lane);
+    }
+  };
+  // 2. places in the ring: the lanes' counts summed from ballots of their bits (no shuffles, which share
+  // the shared-memory pipe that bounds the kernel)
+  const uint32_t cnt = __popc(m), lt = (1u << lane) - 1u;
+  const uint32_t b0 = __ballot_sync(0xffffffffu, cnt & 1u), b1 = __ballot_sync(0xffffffffu, cnt & 2u),
+                 b2 = __ballot_sync(0xffffffffu, cnt & 4u), b3 = __ballot_sync(0xffffffffu, cnt & 8u);
+  if ((b0 | b1 | b2 | b3) != 0u) {
+    uint32_t at = g.left + __popc(b0 & lt) + 2u * __popc(b1 & lt) + 4u * __popc(b2 & lt) + 8u * __popc(b3 & lt);
+    if (g.left == 0u) g.left_c0 = c0;
+    uint32_t n = g.left + __popc(b0) + 2u * __popc(b1) + 4u * __popc(b2) + 8u * __popc(b3);
+    const uint32_t field = static_cast<uint32_t>(first) & ((1u << kPosBits) - 1u);
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < 8; ++j)
       if (m & (1u << j)) {
-        ws.pos_id[at] = e[j];
-        ws.pos_q[at] = static_cast<uint8_t>(q0 + j);
+        if constexpr (kPacked) {
+          ws.ring[at] = (ids.e[j] << kPosBits) + (field + j);
+        } else {
+          ws.ring[at] = ids.e[j];
+          ws.ring_q[at] = static_cast<uint8_t>(8u * lane + j);
+        }
         ++at;
       }
-    at = nlo + (incl >> 16) - ch;
-#pragma unroll
-    for (int j = 4; j < 8; ++j)
-      if (m & (1u << j)) {
-        ws.pos_id[at] = e[j];
-        ws.pos_q[at] = static_cast<uint8_t>(q0 + 124 + j);
-        ++at;
-      }
-  }
-  __syncwarp();
-  if (npos <= 64) {
-    pd.npos = npos;
-    pd.c0 = c0;
-    pd.q0 = lane < npos ? make_uint2(ws.pos_id[lane], ws.pos_q[lane]) : make_uint2(0u, 0u);
-    pd.q1 = 32 + lane < npos ? make_uint2(ws.pos_id[32 + lane], ws.pos_q[32 + lane]) : make_uint2(0u, 0u);
-    pd.rd0 = lane < npos ? __ldg(&p.rankdir[pd.q0.x >> 5]) : make_uint2(0u, 0u);
-    pd.rd1 = 32 + lane < npos ? __ldg(&p.rankdir[pd.q1.x >> 5]) : make_uint2(0u, 0u);
-  } else {
-    for (uint32_t r0 = 0; r0 < npos; r0 += 32) {
-      const bool valid = r0 + lane < npos;
-      const uint2 q = valid ? make_uint2(ws.pos_id[r0 + lane], ws.pos_q[r0 + lane]) : make_uint2(0u, 0u);
-      const uint2 rd = valid ? __ldg(&p.rankdir[q.x >> 5]) : make_uint2(0u, 0u);
-      gather_resolve(p, ws, g, c0, q, rd, valid, lane);
+    __syncwarp();
+    // 3. whole groups
+    uint32_t r0 = 0u;
+    uint32_t v = g.keep, q = g.keep_q;
+    if (lane >= g.left) entry(lane, &v, &q);
+    while (n >= 32u) {
+      send(v, q, 32u);
+      r0 += 32u;
+      n -= 32u;
+      entry(r0 + lane, &v, &q);  // past the last entry: a stale word that no group takes
+      g.left_c0 = c0;
     }
+    g.left = n;
+    g.keep = v;
+    g.keep_q = q;
+    __syncwarp();
   }
-  __syncwarp();
+  // 4. a packed position is told from its low bits while it lies within 2^kPosBits of the step's end, a position
+  // in the step only in the step itself
+  if (g.left > 0u && (!kPacked || c0 - g.left_c0 >= (1 << kPosBits) - 768)) {
+    send(g.keep, g.keep_q, g.left);
+    g.left = 0u;
+  }
 }
 
 }  // namespace
 
-template <bool kSub>
+template <bool kSub, bool kPacked>
 __global__ void __launch_bounds__(kGatherThreads, 1) k_gather(const GatherParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  GatherWarp* gw = reinterpret_cast<GatherWarp*>(smem_raw);
+  using Shared = GatherShared<kPacked>;
+  Shared* gw = reinterpret_cast<Shared*>(smem_raw);
   uint32_t* filt = reinterpret_cast<uint32_t*>(gw + (kGatherThreads / 32));
   const uint32_t lane = lane_id();
-  GatherWarp& ws = gw[threadIdx.x >> 5];
+  Shared& ws = gw[threadIdx.x >> 5];
   const uint32_t fsel = kSub ? static_cast<uint32_t>(p.filt_words) : static_cast<uint32_t>(p.filt_words) - 1u;
 
   for (int w = threadIdx.x; w < p.filt_words; w += blockDim.x) {
@@ -267,35 +312,43 @@ __global__ void __launch_bounds__(kGatherThreads, 1) k_gather(const GatherParams
     const int64_t tb = (ta + kWarpTrials < p.t_end) ? ta + kWarpTrials : p.t_end;
     const int ntr = static_cast<int>(tb - ta);
     const int64_t ea = __ldg(&p.off[ta]);
-    if (lane < 16)
-      ws.off[lane] = (lane <= static_cast<uint32_t>(ntr)) ? static_cast<int32_t>(__ldg(&p.off[ta + lane]) - ea)
-                                                          : INT32_MAX;
-    __syncwarp();
     GatherTile g;
-    g.nev = ws.off[ntr];
-    g.ids4 = reinterpret_cast<const int4*>(p.ids + (ea & ~int64_t(3)));
-    g.lead = static_cast<int32_t>(ea & 3);
-    g.span = g.nev + g.lead;
+    g.lead = static_cast<int32_t>(ea & 7);
+    if (lane < 16)
+      ws.off[lane] = (lane <= static_cast<uint32_t>(ntr))
+                         ? static_cast<int32_t>(__ldg(&p.off[ta + lane]) - ea) + g.lead
+                         : INT32_MAX;
+    __syncwarp();
+    g.span = ws.off[ntr];
+    g.ids = p.ids + (ea & ~int64_t(7));
     g.out = p.ev_buf + (ea - p.e0);
     g.nout = 0;
+    g.t_end = g.lead;  // the first group finds its trial
+    g.t_key = 0u;
+    g.left = 0u;
+    g.keep = g.keep_q = 0u;
+    g.left_c0 = 0;
+    g.pd_n = 0u;
     // three steps of ids in registers, two of them in flight while one is filtered;
     // unrolled by three so that no register of a load in flight is ever moved
-    int4 a0, a1, b0, b1, c0v, c1v;
-    GatherPending pd;
-    pd.npos = 0;
-    gather_load(g, 0, lane, a0, a1);
-    gather_load(g, 256, lane, b0, b1);
+    Ids8 a = gather_load(g, 0, lane), b = gather_load(g, 256, lane), c;
     for (int32_t c0 = 0; c0 < g.span; c0 += 768) {
-      gather_load(g, c0 + 512, lane, c0v, c1v);
-      gather_step<kSub>(p, filt, fsel, ws, g, pd, c0, lane, a0, a1);
+      c = gather_load(g, c0 + 512, lane);
+      gather_step<kSub, kPacked>(p, filt, fsel, ws, g, c0, lane, a);
       if (c0 + 256 >= g.span) break;
-      gather_load(g, c0 + 768, lane, a0, a1);
-      gather_step<kSub>(p, filt, fsel, ws, g, pd, c0 + 256, lane, b0, b1);
+      a = gather_load(g, c0 + 768, lane);
+      gather_step<kSub, kPacked>(p, filt, fsel, ws, g, c0 + 256, lane, b);
       if (c0 + 512 >= g.span) break;
-      gather_load(g, c0 + 1024, lane, b0, b1);
-      gather_step<kSub>(p, filt, fsel, ws, g, pd, c0 + 512, lane, c0v, c1v);
+      b = gather_load(g, c0 + 1024, lane);
+      gather_step<kSub, kPacked>(p, filt, fsel, ws, g, c0 + 512, lane, c);
     }
-    gather_complete(p, ws, g, pd, lane);
+    gather_complete(p, ws, g, lane);
+    if (g.left > 0u) {  // the last positives: within 2^kPosBits of the last step's end
+      const int32_t last = ((g.span - 1) | 255);
+      gather_launch(p, g, g.left, g.keep >> kPosBits,
+                    last - static_cast<int32_t>((static_cast<uint32_t>(last) - g.keep) & ((1u << kPosBits) - 1u)), lane);
+      gather_complete(p, ws, g, lane);
+    }
     if (lane == 0) p.tile_cnt[tile] = g.nout;
     __syncwarp();
   }
@@ -303,14 +356,15 @@ __global__ void __launch_bounds__(kGatherThreads, 1) k_gather(const GatherParams
 
 cudaError_t launch_gather(const GatherParams& p, int grid, size_t smem, cudaStream_t s) {
   const bool sub = p.n_words <= 2 * static_cast<int64_t>(p.filt_words);
-  const void* fn = sub ? reinterpret_cast<const void*>(k_gather<true>) : reinterpret_cast<const void*>(k_gather<false>);
-  cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (err != cudaSuccess) return err;
-  if (sub)
-    k_gather<true><<<grid, kGatherThreads, smem, s>>>(p);
-  else
-    k_gather<false><<<grid, kGatherThreads, smem, s>>>(p);
-  return cudaGetLastError();
+  auto launch = [&](auto kernel) -> cudaError_t {
+    const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 static_cast<int>(smem));
+    if (err != cudaSuccess) return err;
+    kernel<<<grid, kGatherThreads, smem, s>>>(p);
+    return cudaGetLastError();
+  };
+  if (p.catalogue > kPackedCatalogue) return sub ? launch(k_gather<true, false>) : launch(k_gather<false, false>);
+  return sub ? launch(k_gather<true, true>) : launch(k_gather<false, true>);
 }
 
 namespace {

@@ -443,3 +443,29 @@ def test_stress_1m_layer_full_parity(eng):
     """The precision-stress layer: the paper-1m YET and 15 ELTs x 10,000 records
     with Beta shapes log-uniform over [0.2, 50]."""
     _full_size_parity(eng, "stress-1m")
+
+
+@pytest.mark.parametrize("catalogue", [1 << 21, (1 << 21) + 1, 3_000_017], ids=["packed", "wide", "wide-folded"])
+@pytest.mark.parametrize("density", ["rare", "group", "full"])
+def test_gather_groups(eng, catalogue, density):
+    """The gather's groups of 32 filter positives: positives so rare that a
+    group waits over many steps, about 32 a step, and every position; trials
+    of every length around a step's 256 positions, empty ones, and one longer
+    than a packed position's 2,048.  Catalogues at and beyond the packed form's
+    2^21 ids, and beyond twice the filter.  Hit lists bit-exact."""
+    rng = np.random.default_rng(catalogue)
+    lens = np.concatenate([rng.integers(0, 40, 50), [0, 0, 255, 256, 257, 0, 1, 9_000, 7, 8, 33, 511],
+                           rng.integers(200, 900, 61), np.zeros(9, np.int64), rng.integers(0, 5, 40)])
+    offsets = np.zeros(len(lens) + 1, np.int64)
+    offsets[1:] = np.cumsum(lens)
+    pool = synth.make_elt_pool(3, 400, catalogue, 55)
+    ev = rng.integers(0, catalogue, int(offsets[-1])).astype(np.int32)
+    held = rng.random(len(ev)) < {"rare": 0.002, "group": 0.12, "full": 1.0}[density]
+    ev[held] = rng.choice(pool.event_ids, int(held.sum()))
+    yet = synth.YET(offsets, ev, catalogue)
+    terms = (100.0, 1e6, 1e3, 1e9)
+    for t0, t1 in ((0, yet.n_trials), (3, yet.n_trials - 5)):
+        ref = oracle.run_layer(yet, pool, terms, seed=9, trials=np.arange(t0, t1))
+        ylt, hits, hh = run_gpu(eng, yet, pool, terms, seed=9, t0=t0, t1=t1)
+        assert np.array_equal(hits, ref["hits"]) and np.array_equal(hh, ref["hit_hash"])
+        check_ylt(ylt, ref)
