@@ -110,7 +110,7 @@ struct ara_ctx {
   // ELT pool
   std::map<int32_t, Elt> pool;
   // per-layer index (grown on demand)
-  DevBuf bits, word_cnt, word_pairs, rankdir, mask, slot_cnt, pairs, pairs_hot, pairs_w, pairs_ev, scan_tmp;
+  DevBuf marks, word_base, rankdir, slot_start, pairs, pairs_hot, pairs_w, pairs_ev, scan_tmp;
   DevBuf ev_buf, tile_cnt;  // hit-event records of the layer kernels
   // event-major index of the YET (ara_build_yet_index) and the indexed passes' buffers
   DevBuf yix_occ, yix_grid, yix_work;
@@ -119,7 +119,7 @@ struct ara_ctx {
   bool yix_sorted = false;  // built by the radix sort (a bucket was too large)
   float yix_build_ms = 0.0f;
   int64_t yix_bytes = 0;
-  DevBuf u_flags, u_scan, u_event, u_first, idx_acc;
+  DevBuf u_event, idx_acc;
   DevBuf def_acc;           // per-trial FP64 sums of deferred occurrence losses
   DevBuf elt_stage, elt_recs_stage, elt_tab_stage, elt_flags;  // ELT load staging (grow-only)
   DevBuf elt_tabf_stage, elt_work;
@@ -724,33 +724,30 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   if (n_recs >= (int64_t(1) << 31) - 1) return fail(c, ARA_EINVAL, "%s: the ELTs hold too many records", who);
   // ---- index
   const int64_t n_words = (static_cast<int64_t>(c->catalogue) + 31) / 32;
-  const size_t tmp_words = std::max(ara::scan_tmp_words(n_words), ara::scan_tmp_words(n_recs));
-  if ((rc = reserve(c, c->bits, sizeof(uint32_t) * n_words)) ||
-      (rc = reserve(c, c->word_cnt, sizeof(uint32_t) * (n_words + 1))) ||
-      (rc = reserve(c, c->word_pairs, sizeof(uint32_t) * (n_words + 1))) ||
+  if ((rc = reserve(c, c->marks, ara::index_marks_bytes(n_words, n_recs))) ||
+      (rc = reserve(c, c->word_base, 2 * sizeof(uint32_t) * (n_words + 1))) ||
       (rc = reserve(c, c->rankdir, sizeof(uint2) * n_words)) ||
-      (rc = reserve(c, c->mask, sizeof(unsigned long long) * (n_recs + 1))) ||
-      (rc = reserve(c, c->slot_cnt, sizeof(uint32_t) * (n_recs + 2))) ||
+      (rc = reserve(c, c->slot_start, sizeof(uint32_t) * (n_recs + 2))) ||
       (rc = reserve(c, c->pairs, sizeof(ara::Pair) * (n_recs + 1))) ||
       (rc = reserve(c, c->pairs_hot, sizeof(ara::PairHot) * (n_recs + 1))) ||
       (any_corr && (rc = reserve(c, c->pairs_w, sizeof(float2) * (n_recs + 1)))) ||
       (rc = reserve(c, c->pairs_ev, sizeof(int32_t) * (n_recs + 1))) ||
-      (rc = reserve(c, c->scan_tmp, sizeof(uint32_t) * (tmp_words + 8))))
+      (rc = reserve(c, c->scan_tmp, sizeof(uint32_t) * ara::index_scan_words(n_words))))
     return rc;
   ara::LayerIndex& ix = pl->ix;
-  ix.bits = static_cast<uint32_t*>(c->bits.ptr);
-  ix.word_cnt = static_cast<uint32_t*>(c->word_cnt.ptr);
-  ix.word_pairs = static_cast<uint32_t*>(c->word_pairs.ptr);
+  ix.n_words = n_words;
+  ix.n_recs = n_recs;
+  ara::index_place_marks(ix, c->marks.ptr);
+  ix.slot_base = static_cast<uint32_t*>(c->word_base.ptr);
+  ix.pair_base = ix.slot_base + n_words + 1;
   ix.rankdir = static_cast<uint2*>(c->rankdir.ptr);
-  ix.mask = static_cast<unsigned long long*>(c->mask.ptr);
-  ix.slot_cnt = static_cast<uint32_t*>(c->slot_cnt.ptr);
+  ix.slot_start = static_cast<uint32_t*>(c->slot_start.ptr);
+  ix.slot_event = nullptr;
   ix.pairs = static_cast<ara::Pair*>(c->pairs.ptr);
   ix.hot = static_cast<ara::PairHot*>(c->pairs_hot.ptr);
   ix.pw = any_corr ? static_cast<float2*>(c->pairs_w.ptr) : nullptr;
   ix.pev = static_cast<int32_t*>(c->pairs_ev.ptr);
   ix.scan_tmp = static_cast<uint32_t*>(c->scan_tmp.ptr);
-  ix.n_words = n_words;
-  ix.n_recs = n_recs;
   // ---- gather
   pl->filt_words = ara::gather_filter_words(n_words, c->max_smem, c->catalogue);
   pl->smem = ara::gather_smem_bytes(pl->filt_words, c->catalogue);
@@ -774,7 +771,7 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   g.e0 = pl->e0;
   g.rankdir = ix.rankdir;
   g.n_words = n_words;
-  g.slot_start = ix.slot_cnt;
+  g.slot_start = ix.slot_start;
   g.filt_words = pl->filt_words;
   g.catalogue = c->catalogue;
   g.ev_buf = static_cast<uint2*>(c->ev_buf.ptr);
@@ -1144,10 +1141,7 @@ static int run_layers_impl(ara_ctx* c, int32_t n_layers, const ara_layer* layers
   const bool use_index = item == ara::kItemIndexed || (tune && c->yix_ready);
   if (use_index) {
     const int64_t n_recs = pl.ix.n_recs;
-    if ((rc = reserve(c, c->u_flags, sizeof(uint32_t) * (n_recs + 1))) ||
-        (rc = reserve(c, c->u_scan, sizeof(uint32_t) * (n_recs + 1))) ||
-        (rc = reserve(c, c->u_event, sizeof(int32_t) * (n_recs + 1))) ||
-        (rc = reserve(c, c->u_first, sizeof(uint32_t) * (n_recs + 1))) ||
+    if ((rc = reserve(c, c->u_event, sizeof(int32_t) * (n_recs + 1))) ||
         (rc = reserve(c, c->idx_acc,
                       sizeof(unsigned long long) * (n_layers * n_out + idx_queue_words(t0, t1, n_layers)))))
       return rc;
@@ -1157,9 +1151,10 @@ static int run_layers_impl(ara_ctx* c, int32_t n_layers, const ara_layer* layers
     q.grid_cells = ara::yet_grid_cells(c->n_trials, kYetGridShift);
     q.grid_shift = kYetGridShift;
     q.slice_shift = idx_slice_shift(n_layers);
-    q.u_event = static_cast<const int32_t*>(c->u_event.ptr);
-    q.u_first = static_cast<const uint32_t*>(c->u_first.ptr);
-    q.n_u = static_cast<const uint32_t*>(c->u_scan.ptr) + n_recs;
+    pl.ix.slot_event = static_cast<int32_t*>(c->u_event.ptr);  // the union's distinct events are the index's slots
+    q.u_event = pl.ix.slot_event;
+    q.u_first = pl.ix.slot_start;
+    q.n_u = pl.ix.slot_base + pl.ix.n_words;
     q.acc = static_cast<unsigned long long*>(c->idx_acc.ptr);
     q.yet_trials = c->n_trials;
     q.slice_queue = reinterpret_cast<uint32_t*>(q.acc + n_layers * n_out);
@@ -1178,16 +1173,6 @@ static int run_layers_impl(ara_ctx* c, int32_t n_layers, const ara_layer* layers
     if ((rc = launch_index(c, pl, who, &launched))) return rc;
   } else if ((rc = launch_index_and_gather(c, pl, who, &launched))) {
     return rc;
-  }
-  if (use_index) {
-    cudaEvent_t ua, ub;  // the union's events stand where the gather stands in a pass's timing
-    if (!timed_pair(c, 0, &ua, &ub)) return fail(c, ARA_ECUDA, "%s: cannot create timing events", who);
-    ARA_CUDA(c, record_ev(ua, c->stream));
-    ARA_CUDA(c, ara::launch_union_events(pl.ix.pev, pl.ix.n_recs, static_cast<uint32_t*>(c->u_flags.ptr),
-                                         static_cast<uint32_t*>(c->u_scan.ptr), pl.ix.scan_tmp,
-                                         static_cast<int32_t*>(c->u_event.ptr), static_cast<uint32_t*>(c->u_first.ptr),
-                                         c->stream, &launched));
-    ARA_CUDA(c, record_ev(ub, c->stream));
   }
   if (tune) {
     // every candidate once on this pass's records, timed on the stream; the fastest is kept
@@ -1541,27 +1526,21 @@ std::vector<std::pair<DevBuf*, size_t>> serve_workspace(ara_ctx* c) {
   int64_t n_recs = 0;
   for (size_t i = 0; i < sizes.size() && i < static_cast<size_t>(ARA_MAX_BATCH_ELTS); ++i) n_recs += sizes[i];
   const int64_t n_words = (static_cast<int64_t>(c->catalogue) + 31) / 32;
-  const size_t tmp_words = std::max(ara::scan_tmp_words(n_words), ara::scan_tmp_words(n_recs));
   const size_t chunk_tiles = static_cast<size_t>(kServeChunk / ara::kWarpTrials + 2);
   std::vector<std::pair<DevBuf*, size_t>> w = {
       {&c->ev_buf, sizeof(uint2) * static_cast<size_t>(max_ev + 1)},
       {&c->tile_cnt, sizeof(uint32_t) * chunk_tiles},
       {&c->def_acc, sizeof(double) * static_cast<size_t>(kServeChunk + 1)},
-      {&c->bits, sizeof(uint32_t) * n_words},
-      {&c->word_cnt, sizeof(uint32_t) * (n_words + 1)},
-      {&c->word_pairs, sizeof(uint32_t) * (n_words + 1)},
+      {&c->marks, ara::index_marks_bytes(n_words, n_recs)},
+      {&c->word_base, 2 * sizeof(uint32_t) * (n_words + 1)},
       {&c->rankdir, sizeof(uint2) * n_words},
-      {&c->mask, sizeof(unsigned long long) * (n_recs + 1)},
-      {&c->slot_cnt, sizeof(uint32_t) * (n_recs + 2)},
+      {&c->slot_start, sizeof(uint32_t) * (n_recs + 2)},
       {&c->pairs, sizeof(ara::Pair) * (n_recs + 1)},
       {&c->pairs_hot, sizeof(ara::PairHot) * (n_recs + 1)},
       {&c->pairs_ev, sizeof(int32_t) * (n_recs + 1)},
-      {&c->scan_tmp, sizeof(uint32_t) * (tmp_words + 8)},
+      {&c->scan_tmp, sizeof(uint32_t) * ara::index_scan_words(n_words)},
       {&c->serve_sel, serve_select_pool_bytes(c->n_trials)},
-      {&c->u_flags, sizeof(uint32_t) * (n_recs + 1)},
-      {&c->u_scan, sizeof(uint32_t) * (n_recs + 1)},
       {&c->u_event, sizeof(int32_t) * (n_recs + 1)},
-      {&c->u_first, sizeof(uint32_t) * (n_recs + 1)},
       {&c->idx_acc, sizeof(unsigned long long) * (ARA_MAX_BATCH_LAYERS * static_cast<size_t>(kServeChunk) +
                                                   idx_queue_words(0, kServeChunk, ARA_MAX_BATCH_LAYERS))},
       {&c->serve_out, 2 * sizeof(double) * ARA_SERVE_MAX_RP * kServeSlots},
@@ -2161,12 +2140,12 @@ void ara_destroy(ara_ctx* c) {
   }
   DevBuf* bufs[] = {&c->elt_stage,  &c->elt_recs_stage, &c->elt_tab_stage, &c->elt_tabf_stage, &c->elt_work,
                     &c->elt_flags,  &c->ev_buf,         &c->tile_cnt,      &c->def_acc,        &c->yet_off,
-                    &c->yet_ids,    &c->bits,           &c->word_cnt,      &c->word_pairs,     &c->rankdir,
-                    &c->mask,       &c->slot_cnt,       &c->pairs,         &c->pairs_hot,     &c->pairs_w,          &c->pairs_ev,         &c->scan_tmp,       &c->flags,
-                    &c->counters,   &c->ylt_tmp,        &c->diag_tmp,      &c->sel,            &c->in_tmp,
-                    &c->out_tmp,    &c->serve_arena,    &c->serve_out,      &c->yix_occ,        &c->yix_grid,       &c->yix_work,       &c->u_flags,
-                    &c->u_scan,        &c->u_event,        &c->u_first,        &c->idx_acc,      &c->serve_sel,      &c->ev_occ,        &c->row_base,
-                    &c->evr_stage,  &c->yet_flags};
+                    &c->yet_ids,    &c->marks,          &c->word_base,     &c->rankdir,        &c->slot_start,
+                    &c->pairs,      &c->pairs_hot,      &c->pairs_w,       &c->pairs_ev,       &c->scan_tmp,
+                    &c->flags,      &c->counters,       &c->ylt_tmp,       &c->diag_tmp,       &c->sel,
+                    &c->in_tmp,     &c->out_tmp,        &c->serve_arena,   &c->serve_out,      &c->yix_occ,
+                    &c->yix_grid,   &c->yix_work,       &c->u_event,       &c->idx_acc,        &c->serve_sel,
+                    &c->ev_occ,     &c->row_base,       &c->evr_stage,     &c->yet_flags};
   for (DevBuf* b : bufs) release(c, *b);
   for (auto& e : c->ev)
     if (e) cudaEventDestroy(e);

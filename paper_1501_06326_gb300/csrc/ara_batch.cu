@@ -981,24 +981,6 @@ __device__ __forceinline__ float indexed_pair_loss(const BatchParams& p, const D
   return ds.share[pos] * clamp_terms_f(loss, ds.ret[pos], ds.lim[pos]);
 }
 
-__global__ void k_event_flags(const int32_t* __restrict__ pev, int64_t n, uint32_t* flags) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride)
-    flags[i] = (i == 0 || pev[i] != pev[i - 1]) ? 1u : 0u;
-}
-
-__global__ void k_union_events(const int32_t* __restrict__ pev, const uint32_t* __restrict__ flags,
-                               const uint32_t* __restrict__ scan, int64_t n, int32_t* u_event, uint32_t* u_first) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) {
-    if (flags[i]) {
-      u_event[scan[i]] = pev[i];
-      u_first[scan[i]] = static_cast<uint32_t>(i);
-    }
-    if (i == n - 1) u_first[scan[n]] = static_cast<uint32_t>(n);
-  }
-}
-
 }  // namespace
 
 __global__ void __launch_bounds__(kIdxThreads, kIdxBlocksPerSm)
@@ -1162,19 +1144,6 @@ int grid_for_n(int64_t n, int threads) {
 }
 
 }  // namespace
-
-cudaError_t launch_union_events(const int32_t* pev, int64_t n_recs, uint32_t* flags, uint32_t* scan,
-                                uint32_t* scan_tmp, int32_t* u_event, uint32_t* u_first, cudaStream_t s,
-                                int* n_launch) {
-  if (n_recs == 0) return cudaMemsetAsync(scan, 0, sizeof(uint32_t), s);
-  k_event_flags<<<grid_for_n(n_recs, 256), 256, 0, s>>>(pev, n_recs, flags);
-  cudaError_t err = cudaGetLastError();
-  if (err != cudaSuccess) return err;
-  if ((err = scan_exclusive_u32(flags, scan, n_recs, scan_tmp, s, n_launch)) != cudaSuccess) return err;
-  k_union_events<<<grid_for_n(n_recs, 256), 256, 0, s>>>(pev, flags, scan, n_recs, u_event, u_first);
-  if (n_launch) *n_launch += 2;
-  return cudaGetLastError();
-}
 
 int losses_indexed_blocks_per_sm() {
   int b = 0;

@@ -97,7 +97,7 @@ struct IndexedParams {
   int slice_shift;                // the pass runs in slices [j << slice_shift, (j + 1) << slice_shift) of the
                                   // trials (clipped to the pass), every event over one slice before the next;
                                   // slice_shift >= grid_shift, so inner slice bounds are grid bounds
-  const int32_t* u_event;         // [n_u] the union's distinct events, in pair order
+  const int32_t* u_event;         // [n_u] the union's distinct events (the index's slots), ascending
   const uint32_t* u_first;        // [n_u + 1] each one's first pair; u_first[n_u] = the pair count
   const uint32_t* n_u;            // device: the number of distinct events
   unsigned long long* acc;        // [n_layers][t_end - t_begin] fixed-point sums (zeroed before)
@@ -107,12 +107,6 @@ struct IndexedParams {
 __host__ __device__ inline int64_t indexed_slices(int64_t t_begin, int64_t t_end, int slice_shift) {
   return t_end > t_begin ? ((t_end - 1) >> slice_shift) - (t_begin >> slice_shift) + 1 : 0;
 }
-// The union's distinct events from the pairs' event ids (pev, in pair order):
-// flags and scan hold n_recs + 1 words, scan_tmp scan_tmp_words(n_recs); the
-// count is left at scan[n_recs].
-cudaError_t launch_union_events(const int32_t* pev, int64_t n_recs, uint32_t* flags, uint32_t* scan,
-                                uint32_t* scan_tmp, int32_t* u_event, uint32_t* u_first, cudaStream_t s,
-                                int* n_launch);
 cudaError_t launch_losses_indexed(const IndexedParams& q, int grid, cudaStream_t s);
 // The year losses from acc: each layer's trials [t_begin, layer_t_end).
 cudaError_t launch_indexed_years(const IndexedParams& q, cudaStream_t s);

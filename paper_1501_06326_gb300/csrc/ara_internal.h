@@ -101,22 +101,38 @@ struct LayerEltRefs {
 };
 
 struct LayerIndex {
+  // zeroed together before the build (marks_bytes from mask on)
+  unsigned long long* mask;  // [n_recs + 1] per slot: bitmask of layer positions (words with a several-ELT event)
   uint32_t* bits;        // [n_words] membership bitmap over the catalogue
-  uint32_t* word_cnt;    // [n_words + 1] scratch: popcounts, then exclusive scan
-  uint32_t* word_pairs;  // [n_words + 1] scratch: pairs per word, then exclusive scan
-  uint2* rankdir;        // [n_words] {bits, base}: base = pairs before the word, or (1 << 31) | slots
-                         // before the word when the word holds an event with several ELT records
-  unsigned long long* mask;  // [n_recs] per slot: bitmask of layer positions
-  uint32_t* slot_cnt;    // [n_recs + 1] scratch -> slot_start
+  uint32_t* word_cnt;    // [n_words] records per word
+  size_t marks_bytes;
+  uint32_t* slot_base;   // [n_words + 1] member events (slots) before the word; their number at the end
+  uint32_t* pair_base;   // [n_words + 1] pairs before the word
+  uint2* rankdir;        // [n_words] {bits, y}, see kRank*
+  uint32_t* slot_start;  // [n_recs + 2] each slot's first pair, then the number of pairs
+  int32_t* slot_event;   // [n_recs + 1] each slot's event id (or NULL)
   Pair* pairs;           // [n_recs]
   PairHot* hot;          // [n_recs] the table-path part of each pair
   float2* pw;            // [n_recs] (w_I, w_C) of each pair's record (pairs of kind kKindBetaC)
   int32_t* pev;          // [n_recs] each pair's event id (the per-event output reads it)
-  uint32_t* scan_tmp;
+  uint32_t* scan_tmp;    // index_scan_words(n_words) words
   int64_t n_words;
   int64_t n_recs;
 };
 
+// A rank-directory word's y: where its events' pairs are.
+//   bit 31 clear: each event has one pair, and the r-th event of the word has pair y + r;
+//   bits 31 and 30 set: the event at bit (y >> 25) & 31 has two pairs, the others one, and the word's pairs
+//     start at y & kRankBaseMask (below 2^25);
+//   bit 31 alone: the r-th event is slot (y & kRankSlotMask) + r, its pairs from slot_start.
+constexpr uint32_t kRankSlots = 0x80000000u, kRankTwo = 0xC0000000u;
+constexpr uint32_t kRankSlotMask = 0x3FFFFFFFu, kRankBaseMask = (1u << 25) - 1u;
+constexpr uint32_t kRankTwoShift = 25;
+
+// Bytes of mask, bits and word_cnt together, and the placing of the three in them.
+size_t index_marks_bytes(int64_t n_words, int64_t n_recs);
+void index_place_marks(LayerIndex& ix, void* marks);
+size_t index_scan_words(int64_t n_words);
 cudaError_t build_layer_index(const LayerEltRefs& refs, LayerIndex& ix, cudaStream_t s, int* n_launch);
 
 // --------------------------------------------------------------- main kernels

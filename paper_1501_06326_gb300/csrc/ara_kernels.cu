@@ -762,20 +762,59 @@ cudaError_t scan_exclusive_u32(const uint32_t* in, uint32_t* out, int64_t n, uin
 // =============================================================== layer index
 namespace {
 
-__device__ __forceinline__ int find_pos(const LayerEltRefs& r, int64_t i) {
-  int p = 0;
-  while (p + 1 < r.n_elts && r.rec_begin[p + 1] <= i) ++p;
-  return p;
-}
+// The layer index in four launches and one memset, each bound by its launch and
+// the latency of a few dependent loads (15 ELTs of 10,000 records over 2M ids:
+// 37 us a build; 14 launches, with a scan for each of the three sums and a
+// search for each record's ELT, took 94 us).  A slot's first pair follows from
+// its word's pairs and the slots of the word before it, so the slots need no
+// scan of their own, and the slots are an indexed pass's distinct events.
+// Grids below: blockIdx.y is the ELT position, blockIdx.x strides over its records.
 
-__global__ void k_mark_members(LayerEltRefs r, uint32_t* bits, uint32_t* word_pairs) {
-  const int64_t n = r.rec_begin[r.n_elts];
+__global__ void k_mark_members(const __grid_constant__ LayerEltRefs r, uint32_t* bits, uint32_t* word_cnt) {
+  const int p = blockIdx.y;
+  const int32_t* ev = r.events[p];
+  const int64_t n = r.rec_begin[p + 1] - r.rec_begin[p];
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) {
-    const int p = find_pos(r, i);
-    const int32_t e = r.events[p][i - r.rec_begin[p]];
+    const int32_t e = ev[i];
     atomicOr(&bits[e >> 5], 1u << (e & 31));
-    atomicAdd(&word_pairs[e >> 5], 1u);  // every record is one (event, ELT) pair
+    atomicAdd(&word_cnt[e >> 5], 1u);  // every record is one (event, ELT) pair
+  }
+}
+
+// slot_base and pair_base: exclusive sums over the words of the member events
+// and of the records.  Block b sums the words before its own 1,024 itself (at
+// most kBasesWords of them, from L2): one launch of 8 us for both sums at
+// 62,500 words, where two scans took six launches and 23 us.
+constexpr int kBasesThreads = 1024;
+constexpr int64_t kBasesWords = 1 << 17;
+
+__global__ void __launch_bounds__(kBasesThreads) k_word_bases(const uint32_t* __restrict__ bits,
+                                                              const uint32_t* __restrict__ word_cnt, int64_t n_words,
+                                                              uint32_t* slot_base, uint32_t* pair_base) {
+  __shared__ uint32_t s_warp[33];
+  uint32_t slots = 0u, pairs = 0u;
+  const int64_t b0 = static_cast<int64_t>(blockIdx.x) * kBasesThreads;
+#pragma unroll 4
+  for (int64_t i = 4 * static_cast<int64_t>(threadIdx.x); i < b0; i += 4 * kBasesThreads) {
+    const uint4 x = *reinterpret_cast<const uint4*>(bits + i), c = *reinterpret_cast<const uint4*>(word_cnt + i);
+    slots += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+    pairs += c.x + c.y + c.z + c.w;
+  }
+  const int64_t w = b0 + threadIdx.x;
+  const uint32_t my_slots = w < n_words ? __popc(bits[w]) : 0u, my_pairs = w < n_words ? word_cnt[w] : 0u;
+  uint32_t before_slots, before_pairs, total;
+  block_exclusive_scan(slots, s_warp, &before_slots);
+  block_exclusive_scan(pairs, s_warp, &before_pairs);
+  const uint32_t s = before_slots + block_exclusive_scan(my_slots, s_warp, &total);
+  const uint32_t q = before_pairs + block_exclusive_scan(my_pairs, s_warp, &total);
+  if (w < n_words) {
+    slot_base[w] = s;
+    pair_base[w] = q;
+    if (w == n_words - 1) {
+      slot_base[n_words] = s + my_slots;
+      pair_base[n_words] = q + my_pairs;
+    }
   }
 }
 
@@ -785,65 +824,98 @@ __global__ void k_word_popc(const uint32_t* bits, int64_t n_words, uint32_t* cnt
     cnt[w] = __popc(bits[w]);
 }
 
-// rankdir[w] = {bits, base}: base = pairs before the word when every event of
-// the word has one ELT record (its pair is then base + rank in the word), else
-// (1 << 31) | slots before the word (pair range from slot_start).
-__global__ void k_pack_rankdir(const uint32_t* bits, const uint32_t* base, const uint32_t* pbase, int64_t n_words,
-                               uint2* rankdir) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t w = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; w < n_words; w += stride) {
-    const uint32_t b = bits[w];
-    const bool multi = (pbase[w + 1] - pbase[w] != static_cast<uint32_t>(__popc(b)));
-    rankdir[w] = make_uint2(b, multi ? (0x80000000u | base[w]) : pbase[w]);
-  }
+// Where the pairs of a member event e are: its word, and its rank in the word.
+struct Place {
+  uint32_t slot0, pair0, below;  // the word's first slot and pair, the word's events below e
+  bool several;                  // the word holds an event with several pairs
+};
+__device__ __forceinline__ Place place_of(const uint32_t* __restrict__ bits, const uint32_t* __restrict__ slot_base,
+                                          const uint32_t* __restrict__ pair_base, int32_t e) {
+  const int32_t w = e >> 5;
+  const uint32_t b = bits[w];
+  Place pl;
+  pl.slot0 = slot_base[w];
+  pl.pair0 = pair_base[w];
+  pl.below = __popc(b & ((1u << (e & 31)) - 1u));
+  pl.several = pair_base[w + 1] - pl.pair0 != static_cast<uint32_t>(__popc(b));
+  return pl;
 }
 
-// Slot (rank among the layer's events) of a member event e.
-__device__ __forceinline__ uint32_t rank_of(const uint32_t* bits, const uint32_t* slot_base, int32_t e) {
-  const uint32_t bit = 1u << (e & 31);
-  return slot_base[e >> 5] + __popc(bits[e >> 5] & (bit - 1u));
-}
-
-__global__ void k_mark_positions(LayerEltRefs r, const uint32_t* bits, const uint32_t* slot_base,
+__global__ void k_mark_positions(const __grid_constant__ LayerEltRefs r, const uint32_t* __restrict__ bits,
+                                 const uint32_t* __restrict__ slot_base, const uint32_t* __restrict__ pair_base,
                                  unsigned long long* mask) {
-  const int64_t n = r.rec_begin[r.n_elts];
+  const int p = blockIdx.y;
+  const int32_t* ev = r.events[p];
+  const int64_t n = r.rec_begin[p + 1] - r.rec_begin[p];
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) {
-    const int p = find_pos(r, i);
-    const int32_t e = r.events[p][i - r.rec_begin[p]];
-    atomicOr(&mask[rank_of(bits, slot_base, e)], 1ull << p);
+    const Place pl = place_of(bits, slot_base, pair_base, ev[i]);
+    if (pl.several) atomicOr(&mask[pl.slot0 + pl.below], 1ull << p);
   }
 }
 
-__global__ void k_slot_counts(const unsigned long long* mask, int64_t n, uint32_t* cnt) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride)
-    cnt[i] = __popcll(mask[i]);
+// One word's rank-directory entry and its slots' first pairs and events.
+__device__ __forceinline__ void fill_word(const LayerIndex& ix, int64_t w) {
+  const uint32_t b = ix.bits[w], slot0 = ix.slot_base[w], pair0 = ix.pair_base[w];
+  const uint32_t n = __popc(b), n_pairs = ix.pair_base[w + 1] - pair0;
+  uint32_t y = pair0;
+  if (n_pairs == n) {
+    for (uint32_t i = 0; i < n; ++i) ix.slot_start[slot0 + i] = pair0 + i;
+  } else {
+    y = kRankSlots | slot0;
+    uint32_t at = pair0, left = b;
+    for (uint32_t i = 0; i < n; ++i) {
+      const uint32_t c = __popcll(ix.mask[slot0 + i]);
+      ix.slot_start[slot0 + i] = at;
+      at += c;
+      if (n_pairs == n + 1u && c == 2u && pair0 <= kRankBaseMask)
+        y = kRankTwo | (static_cast<uint32_t>(__ffs(left) - 1) << kRankTwoShift) | pair0;
+      left &= left - 1u;
+    }
+  }
+  ix.rankdir[w] = make_uint2(b, y);
+  if (ix.slot_event) {
+    uint32_t left = b;
+    for (uint32_t i = 0; i < n; ++i, left &= left - 1u)
+      ix.slot_event[slot0 + i] = static_cast<int32_t>(32 * w + __ffs(left) - 1);
+  }
+  if (w == ix.n_words - 1) ix.slot_start[slot0 + n] = pair0 + n_pairs;
 }
 
-__global__ void k_fill_pairs(LayerEltRefs r, const uint32_t* bits, const uint32_t* slot_base,
-                             const unsigned long long* mask,
-                             const uint32_t* slot_start, Pair* pairs, PairHot* hot, float2* pw, int32_t* pev) {
-  const int64_t n = r.rec_begin[r.n_elts];
+// The pairs in (event, position) order; the blocks of the last blockIdx.y fill
+// the words' directory entries and slots.
+__global__ void k_fill_pairs(const __grid_constant__ LayerEltRefs r, const __grid_constant__ LayerIndex ix) {
+  const int p = blockIdx.y;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) {
-    const int p = find_pos(r, i);
-    const int64_t j = i - r.rec_begin[p];
-    const int32_t e = r.events[p][j];
-    const uint32_t slot = rank_of(bits, slot_base, e);
-    const uint32_t within = __popcll(mask[slot] & ((1ull << p) - 1ull));
-    Pair q = r.recs[p][j];
+  const int64_t i0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (p == r.n_elts) {
+    for (int64_t w = i0; w < ix.n_words; w += stride) fill_word(ix, w);
+    return;
+  }
+  const int32_t* ev = r.events[p];
+  const Pair* recs = r.recs[p];
+  const float2* wts = r.wts[p];
+  const int64_t n = r.rec_begin[p + 1] - r.rec_begin[p];
+  for (int64_t j = i0; j < n; j += stride) {
+    const int32_t e = ev[j];
+    Pair q = recs[j];
+    const Place pl = place_of(ix.bits, ix.slot_base, ix.pair_base, e);
+    uint32_t at = pl.pair0 + pl.below;
+    if (pl.several) {
+      at = pl.pair0;
+      for (uint32_t k = 0; k < pl.below; ++k) at += __popcll(ix.mask[pl.slot0 + k]);
+      at += __popcll(ix.mask[pl.slot0 + pl.below] & ((1ull << p) - 1ull));
+    }
     q.meta = (q.meta & ~kMetaPosMask) | static_cast<uint32_t>(p);
-    const uint32_t at = slot_start[slot] + within;
-    pairs[at] = q;
+    ix.pairs[at] = q;
     PairHot hq;
     hq.max_l = q.max_l;
     hq.mu = q.mu;
     hq.meta = q.meta;
     hq.node = pair_rec(q.meta) * (pair_fine(q.meta) ? kTabFineStride : kTabNodes);
-    hot[at] = hq;
-    if (pw && r.wts[p]) pw[at] = r.wts[p][j];
-    if (pev) pev[at] = e;
+    ix.hot[at] = hq;
+    if (ix.pw && wts) ix.pw[at] = wts[j];
+    if (ix.pev) ix.pev[at] = e;
   }
 }
 
@@ -852,50 +924,63 @@ inline int grid_for(int64_t n, int threads, int cap = 4096) {
   return static_cast<int>(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
+inline int64_t round4(int64_t n) { return (n + 3) & ~int64_t(3); }
+
 }  // namespace
+
+size_t index_marks_bytes(int64_t n_words, int64_t n_recs) {
+  return sizeof(unsigned long long) * static_cast<size_t>((n_recs + 2) & ~int64_t(1)) +
+         2 * sizeof(uint32_t) * static_cast<size_t>(round4(n_words));
+}
+
+void index_place_marks(LayerIndex& ix, void* marks) {
+  ix.mask = static_cast<unsigned long long*>(marks);
+  ix.bits = reinterpret_cast<uint32_t*>(ix.mask + ((ix.n_recs + 2) & ~int64_t(1)));
+  ix.word_cnt = ix.bits + round4(ix.n_words);
+  ix.marks_bytes = index_marks_bytes(ix.n_words, ix.n_recs);
+}
+
+size_t index_scan_words(int64_t n_words) { return n_words > kBasesWords ? scan_tmp_words(n_words) : 1; }
 
 cudaError_t build_layer_index(const LayerEltRefs& refs, LayerIndex& ix, cudaStream_t s, int* n_launch) {
   const int64_t n_recs = refs.rec_begin[refs.n_elts];
   cudaError_t err;
-  if ((err = cudaMemsetAsync(ix.bits, 0, sizeof(uint32_t) * ix.n_words, s)) != cudaSuccess) return err;
-  if ((err = cudaMemsetAsync(ix.word_pairs, 0, sizeof(uint32_t) * (ix.n_words + 1), s)) != cudaSuccess) return err;
-  if ((err = cudaMemsetAsync(ix.mask, 0, sizeof(unsigned long long) * (n_recs > 0 ? n_recs : 1), s)) !=
-      cudaSuccess)
-    return err;
+  if ((err = cudaMemsetAsync(ix.mask, 0, ix.marks_bytes, s)) != cudaSuccess) return err;
   int launched = 0;
+  int64_t longest = 0;
+  for (int p = 0; p < refs.n_elts; ++p) {
+    const int64_t n = refs.rec_begin[p + 1] - refs.rec_begin[p];
+    longest = n > longest ? n : longest;
+  }
+  const dim3 by_elt(grid_for(longest, 256, 64), refs.n_elts);
   if (n_recs > 0) {
-    k_mark_members<<<grid_for(n_recs, 256), 256, 0, s>>>(refs, ix.bits, ix.word_pairs);
+    k_mark_members<<<by_elt, 256, 0, s>>>(refs, ix.bits, ix.word_cnt);
     ++launched;
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
-  k_word_popc<<<grid_for(ix.n_words, 256), 256, 0, s>>>(ix.bits, ix.n_words, ix.word_cnt);
-  ++launched;
-  if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  // exclusive scan in place (each tile reads its inputs before writing)
-  if ((err = scan_exclusive_u32(ix.word_cnt, ix.word_cnt, ix.n_words, ix.scan_tmp, s, &launched)) != cudaSuccess)
-    return err;
-  if ((err = scan_exclusive_u32(ix.word_pairs, ix.word_pairs, ix.n_words, ix.scan_tmp, s, &launched)) != cudaSuccess)
-    return err;
-  k_pack_rankdir<<<grid_for(ix.n_words, 256), 256, 0, s>>>(ix.bits, ix.word_cnt, ix.word_pairs, ix.n_words,
-                                                           ix.rankdir);
-  ++launched;
-  if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  if (n_recs > 0) {
-    k_mark_positions<<<grid_for(n_recs, 256), 256, 0, s>>>(refs, ix.bits, ix.word_cnt, ix.mask);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    k_slot_counts<<<grid_for(n_recs, 256), 256, 0, s>>>(ix.mask, n_recs, ix.slot_cnt);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    if ((err = scan_exclusive_u32(ix.slot_cnt, ix.slot_cnt, n_recs, ix.scan_tmp, s, &launched)) != cudaSuccess)
-      return err;
-    k_fill_pairs<<<grid_for(n_recs, 256), 256, 0, s>>>(refs, ix.bits, ix.word_cnt, ix.mask, ix.slot_cnt, ix.pairs, ix.hot,
-                                                        ix.pw, ix.pev);
-    launched += 3;
+  if (ix.n_words <= kBasesWords) {
+    k_word_bases<<<grid_for(ix.n_words, kBasesThreads), kBasesThreads, 0, s>>>(ix.bits, ix.word_cnt, ix.n_words,
+                                                                              ix.slot_base, ix.pair_base);
+    ++launched;
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   } else {
-    if ((err = cudaMemsetAsync(ix.slot_cnt, 0, sizeof(uint32_t), s)) != cudaSuccess) return err;
+    k_word_popc<<<grid_for(ix.n_words, 256), 256, 0, s>>>(ix.bits, ix.n_words, ix.slot_base);
+    ++launched;
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    // in place: each tile reads its inputs before writing
+    if ((err = scan_exclusive_u32(ix.slot_base, ix.slot_base, ix.n_words, ix.scan_tmp, s, &launched)) != cudaSuccess ||
+        (err = scan_exclusive_u32(ix.word_cnt, ix.pair_base, ix.n_words, ix.scan_tmp, s, &launched)) != cudaSuccess)
+      return err;
   }
+  if (n_recs > 0) {
+    k_mark_positions<<<by_elt, 256, 0, s>>>(refs, ix.bits, ix.slot_base, ix.pair_base, ix.mask);
+    ++launched;
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  }
+  k_fill_pairs<<<dim3(64, refs.n_elts + 1), 256, 0, s>>>(refs, ix);
+  ++launched;
   if (n_launch) *n_launch += launched;
-  return cudaSuccess;
+  return cudaGetLastError();
 }
 
 }  // namespace ara

@@ -177,11 +177,18 @@ __device__ __forceinline__ void gather_complete(const GatherParams& p, const Sha
     g.t_end = __shfl_sync(0xffffffffu, ws.off[t + 1], g.pd_n - 1u);
     g.t_key = __shfl_sync(0xffffffffu, tk, g.pd_n - 1u);
   }
-  uint32_t ps = (g.pd_rd.y & 0x7FFFFFFFu) + __popc(upto) - 1u;
-  if (hit && static_cast<int32_t>(g.pd_rd.y) < 0) {  // the word holds an event with several pairs
-    const uint32_t first = __ldg(&p.slot_start[ps]);
-    key += (__ldg(&p.slot_start[ps + 1]) - first - 1u) << kRecCntShift;
-    ps = first;
+  const uint32_t below = __popc(upto) - 1u, y = g.pd_rd.y;
+  uint32_t ps = y + below;
+  if (hit && (y & kRankSlots)) {  // the word holds an event with several pairs
+    if ((y & kRankTwo) == kRankTwo) {
+      const uint32_t two = (y >> kRankTwoShift) & 31u, bit = g.pd_id & 31u;
+      ps = (y & kRankBaseMask) + below + (bit > two ? 1u : 0u);
+      key += (bit == two ? 1u : 0u) << kRecCntShift;
+    } else {
+      const uint32_t slot = (y & kRankSlotMask) + below;
+      ps = __ldg(&p.slot_start[slot]);
+      key += (__ldg(&p.slot_start[slot + 1]) - ps - 1u) << kRecCntShift;
+    }
   }
   const uint32_t hm = __ballot_sync(0xffffffffu, hit);
   if (hit) g.out[g.nout + __popc(hm & ((1u << lane) - 1u))] = make_uint2(key, ps);
