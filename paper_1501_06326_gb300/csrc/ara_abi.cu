@@ -134,15 +134,24 @@ struct ara_ctx {
   DevBuf sel;       // select / sort scratch
   DevBuf in_tmp;    // staging of host inputs for pml/sort
   DevBuf out_tmp;   // small device outputs
-  cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // of a pass without timing (the serving loop's)
+  double* h_out = nullptr;  // pinned results of ara_pml_tvar
+  size_t h_out_n = 0;
   ara_stats stats{};
-  // timing accumulators: event pairs recorded around launch groups since the last reset
+  bool stats_read = true;
+  // device times since the last reset: the calls whose events are still held, and the sums of those folded
+  // in (completed calls, so that their events serve later ones)
   struct Timed {
-    int kind;  // 0 gather kernel, 1 index build, 2 pml/tvar, 3 losses kernel
-    cudaEvent_t a, b;
+    int kind = -1;  // 0 layer pass: e[0] index e[1] gather e[2] losses e[3]; 1 the same with an autotuner's
+                    // runs between the gather and e[4], where the losses begin; 2 pml/tvar: e[0] select e[1]
+    cudaEvent_t e[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    int n() const { return kind == 2 ? 2 : kind == 1 ? 5 : 4; }
+    cudaEvent_t last() const { return e[kind == 2 ? 1 : 3]; }
   };
-  std::vector<cudaEvent_t> ev_pool;
-  std::vector<Timed> timed;
+  std::vector<cudaEvent_t> ev_all, ev_free;
+  std::deque<Timed> timed;
+  ara_timing timing_sum{};
+  Timed stat_ev;  // the last layer pass, until its times are read (ara_get_stats)
   int64_t launches = 0;
   int num_sms = 0;
   int max_smem = 0;
@@ -163,7 +172,6 @@ struct ara_ctx {
   DevBuf serve_arena;                   // year losses of the admitted requests
   std::map<size_t, size_t> arena_free;  // free blocks of the arena: offset -> bytes
   DevBuf serve_out;                     // device result slots (PML, TVaR)
-  DevBuf serve_sel;                     // select scratch of the requests' PML/TVaR
   cudaStream_t serve_side = nullptr;    // the requests' PML/TVaR and result copies, beside the passes
   cudaEvent_t serve_join = nullptr;     // the passes' stream up to a point, for the side stream to wait on
   double* serve_host = nullptr;         // pinned host result slots
@@ -173,26 +181,87 @@ struct ara_ctx {
 
 namespace {
 
-// Two events for one timed launch group (reused after a reset).
-bool timed_pair(ara_ctx* c, int kind, cudaEvent_t* a, cudaEvent_t* b) {
-  if (c->no_timing) {
-    *a = *b = nullptr;
-    return true;
-  }
-  const size_t need = 2 * (c->timed.size() + 1);
-  while (c->ev_pool.size() < need) {
-    cudaEvent_t e;
-    if (cudaEventCreate(&e) != cudaSuccess) return false;
-    c->ev_pool.push_back(e);
-  }
-  *a = c->ev_pool[need - 2];
-  *b = c->ev_pool[need - 1];
-  c->timed.push_back({kind, *a, *b});
+// The index and kernel times of the last layer pass, from its events (which must have completed).
+bool read_stat_times(ara_ctx* c) {
+  ara_ctx::Timed& t = c->stat_ev;
+  if (t.kind < 0) return true;
+  float index_ms = 0.0f, kernel_ms = 0.0f;
+  if (cudaEventElapsedTime(&index_ms, t.e[0], t.e[1]) != cudaSuccess ||
+      cudaEventElapsedTime(&kernel_ms, t.e[1], t.e[3]) != cudaSuccess)
+    return false;
+  c->stats.index_ms = index_ms;
+  c->stats.kernel_ms = kernel_ms;
+  t.kind = -1;
   return true;
 }
 
-// Records a timing event (a null event, from a pass without timing, is skipped).
-cudaError_t record_ev(cudaEvent_t e, cudaStream_t s) { return e ? cudaEventRecord(e, s) : cudaSuccess; }
+// Adds the oldest timed call's times to the sums and takes its events back.
+bool fold_timed(ara_ctx* c) {
+  const ara_ctx::Timed t = c->timed.front();
+  ara_timing& o = c->timing_sum;
+  float first = 0.0f, gather = 0.0f, losses = 0.0f;
+  if (cudaEventElapsedTime(&first, t.e[0], t.e[1]) != cudaSuccess) return false;
+  if (t.kind == 2) {
+    o.pml_calls += 1;
+    o.pml_ms += first;
+  } else {
+    if (cudaEventElapsedTime(&gather, t.e[1], t.e[2]) != cudaSuccess ||
+        cudaEventElapsedTime(&losses, t.e[t.kind == 1 ? 4 : 2], t.e[3]) != cudaSuccess)
+      return false;
+    o.layer_calls += 1;
+    o.index_ms += first;
+    o.gather_ms += gather;
+    o.losses_ms += losses;
+    o.kernel_ms += static_cast<double>(gather) + losses;
+  }
+  if (c->stat_ev.kind >= 0 && c->stat_ev.e[0] == t.e[0] && !read_stat_times(c)) return false;
+  for (int i = 0; i < t.n(); ++i) c->ev_free.push_back(t.e[i]);
+  c->timed.pop_front();
+  return true;
+}
+
+constexpr size_t kTimedHeld = 64;  // timed calls held before completed ones are folded in
+
+// Events for a call's launch groups (a pass without timing takes the context's own).
+bool timed_begin(ara_ctx* c, int kind, ara_ctx::Timed* t) {
+  t->kind = kind;
+  if (c->no_timing) {
+    for (int i = 0; i < t->n(); ++i) t->e[i] = c->ev[i];
+    return true;
+  }
+  if (c->timed.size() >= kTimedHeld) {
+    // (an event query is not allowed while a stream is captured)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+      cudaGetLastError();
+      cap = cudaStreamCaptureStatusActive;
+    }
+    while (cap == cudaStreamCaptureStatusNone && c->timed.size() >= kTimedHeld) {
+      if (cudaEventQuery(c->timed.front().last()) != cudaSuccess) {
+        cudaGetLastError();
+        break;
+      }
+      if (!fold_timed(c)) return false;
+    }
+  }
+  for (int i = 0; i < t->n(); ++i) {
+    if (!c->ev_free.empty()) {
+      t->e[i] = c->ev_free.back();
+      c->ev_free.pop_back();
+    } else if (cudaEventCreate(&t->e[i]) == cudaSuccess) {
+      c->ev_all.push_back(t->e[i]);
+    } else {
+      return false;
+    }
+  }
+  return true;
+}
+
+// The call's events are all recorded.
+void timed_end(ara_ctx* c, const ara_ctx::Timed& t) {
+  if (!c->no_timing) c->timed.push_back(t);
+  if (t.kind != 2) c->stat_ev = t;
+}
 
 int fail(ara_ctx* c, int code, const char* fmt, ...) {
   char buf[512];
@@ -782,29 +851,20 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   return ARA_OK;
 }
 
-// Index build and gather on the context stream (with their timing events).
-static int launch_index(ara_ctx* c, const PassPlan& pl, const char* who, int* launched) {
-  cudaEvent_t ia, ib;
-  if (!timed_pair(c, 1, &ia, &ib)) return fail(c, ARA_ECUDA, "%s: cannot create timing events", who);
+// Index build, and the gather unless the pass goes through the YET's index, on the context stream; `t`
+// receives the pass's events, the first three of them recorded.
+static int launch_index(ara_ctx* c, const PassPlan& pl, const char* who, bool gather, ara_ctx::Timed* t,
+                        int* launched, bool tune = false) {
+  if (!timed_begin(c, tune ? 1 : 0, t)) return fail(c, ARA_ECUDA, "%s: cannot create timing events", who);
   ARA_CUDA(c, cudaMemsetAsync(c->counters.ptr, 0, 8 * sizeof(unsigned long long), c->stream));
-  ARA_CUDA(c, cudaEventRecord(c->ev[0], c->stream));
-  ARA_CUDA(c, record_ev(ia, c->stream));
+  ARA_CUDA(c, cudaEventRecord(t->e[0], c->stream));
   ARA_CUDA(c, ara::build_layer_index(pl.refs, const_cast<ara::LayerIndex&>(pl.ix), c->stream, launched));
-  ARA_CUDA(c, record_ev(ib, c->stream));
-  ARA_CUDA(c, cudaEventRecord(c->ev[1], c->stream));
-  ARA_CUDA(c, cudaEventRecord(c->ev[2], c->stream));
-  return ARA_OK;
-}
-
-static int launch_index_and_gather(ara_ctx* c, const PassPlan& pl, const char* who, int* launched) {
-  int rc = launch_index(c, pl, who, launched);
-  if (rc) return rc;
-  cudaEvent_t ka, kb;
-  if (!timed_pair(c, 0, &ka, &kb)) return fail(c, ARA_ECUDA, "%s: cannot create timing events", who);
-  ARA_CUDA(c, record_ev(ka, c->stream));
-  ARA_CUDA(c, ara::launch_gather(pl.g, pl.grid, pl.smem, c->stream));
-  ARA_CUDA(c, record_ev(kb, c->stream));
-  *launched += 1;
+  ARA_CUDA(c, cudaEventRecord(t->e[1], c->stream));
+  if (gather) {
+    ARA_CUDA(c, ara::launch_gather(pl.g, pl.grid, pl.smem, c->stream));
+    *launched += 1;
+  }
+  ARA_CUDA(c, cudaEventRecord(t->e[2], c->stream));
   return ARA_OK;
 }
 
@@ -824,7 +884,7 @@ static void record_pass_stats(ara_ctx* c, const PassPlan& pl, int64_t t0, int64_
   c->stats.block = ara::kGatherThreads;
   c->stats.smem_bytes = static_cast<int32_t>(pl.smem);
   c->stats.filter_bits = pl.filt_words * 32;
-  c->stats.kernel_ms = -1.0f;  // device times are read lazily by ara_get_stats
+  c->stats_read = false;  // device times and counters are read lazily by ara_get_stats
 }
 
 // The rows of ara_run_layer_events after the losses kernel wrote O_k beside
@@ -968,13 +1028,11 @@ static int run_layer_impl(ara_ctx* c, const ara_layer* L, uint64_t seed, int64_t
                                                            (pl.n_tiles + loss_warps - 1) / loss_warps));
   // ---- launch
   int launched = 0;
-  if ((rc = launch_index_and_gather(c, pl, who, &launched))) return rc;
-  cudaEvent_t la, lb;
-  if (!timed_pair(c, 3, &la, &lb)) return fail(c, ARA_ECUDA, "%s: cannot create timing events", who);
-  ARA_CUDA(c, record_ev(la, c->stream));
+  ara_ctx::Timed timed;
+  if ((rc = launch_index(c, pl, who, true, &timed, &launched))) return rc;
   ARA_CUDA(c, ara::launch_losses(p, loss_grid, c->stream));
-  ARA_CUDA(c, record_ev(lb, c->stream));
-  ARA_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
+  ARA_CUDA(c, cudaEventRecord(timed.e[3], c->stream));
+  timed_end(c, timed);
   launched += 1;
   if (evr && (rc = emit_event_rows(c, pl, p, evr, &launched))) return rc;
   c->launches += launched;
@@ -1169,11 +1227,8 @@ static int run_layers_impl(ara_ctx* c, int32_t n_layers, const ara_layer* layers
     return e;
   };
   int launched = 0;
-  if (item == ara::kItemIndexed && !tune) {
-    if ((rc = launch_index(c, pl, who, &launched))) return rc;
-  } else if ((rc = launch_index_and_gather(c, pl, who, &launched))) {
-    return rc;
-  }
+  ara_ctx::Timed timed;
+  if ((rc = launch_index(c, pl, who, item != ara::kItemIndexed || tune, &timed, &launched, tune))) return rc;
   if (tune) {
     // every candidate once on this pass's records, timed on the stream; the fastest is kept
     float best = 0.0f;
@@ -1199,12 +1254,10 @@ static int run_layers_impl(ara_ctx* c, int32_t n_layers, const ara_layer* layers
     c->tune_cache[tshape] = {item, blocks};
     ARA_CUDA(c, cudaMemsetAsync(c->counters.ptr, 0, 4 * sizeof(unsigned long long), c->stream));
   }
-  cudaEvent_t la, lb;
-  if (!timed_pair(c, 3, &la, &lb)) return fail(c, ARA_ECUDA, "%s: cannot create timing events", who);
-  ARA_CUDA(c, record_ev(la, c->stream));
+  if (tune) ARA_CUDA(c, cudaEventRecord(timed.e[4], c->stream));
   ARA_CUDA(c, launch_item(item, blocks));
-  ARA_CUDA(c, record_ev(lb, c->stream));
-  ARA_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
+  ARA_CUDA(c, cudaEventRecord(timed.e[3], c->stream));
+  timed_end(c, timed);
   launched += item == ara::kItemIndexed ? 2 : 1;
   c->last_item = item;
   c->last_blocks = blocks;
@@ -1387,18 +1440,17 @@ int ara_get_stats(const ara_ctx* cc, ara_stats* out) {
   int rc = bind(c);
   if (rc) return rc;
   if (!out) return fail(c, ARA_EINVAL, "ara_get_stats: out is NULL");
-  if (c->stats.kernel_ms < 0.0f) {
-    ARA_CUDA(c, cudaEventSynchronize(c->ev[3]));
-    float ms = 0.0f;
-    ARA_CUDA(c, cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]));
-    c->stats.index_ms = ms;
-    ARA_CUDA(c, cudaEventElapsedTime(&ms, c->ev[2], c->ev[3]));
-    c->stats.kernel_ms = ms;
+  if (!c->stats_read) {
+    if (c->stat_ev.kind >= 0) {
+      ARA_CUDA(c, cudaEventSynchronize(c->stat_ev.e[3]));
+      if (!read_stat_times(c)) return fail(c, ARA_ECUDA, "ara_get_stats: %s", cudaGetErrorString(cudaGetLastError()));
+    }
     unsigned long long h[4];
     ARA_CUDA(c, cudaMemcpy(h, c->counters.ptr, sizeof h, cudaMemcpyDeviceToHost));
     c->stats.n_pairs_hit = static_cast<int64_t>(h[1]);
     c->stats.n_nonconverged = static_cast<int64_t>(h[2]);
     c->stats.n_newton = static_cast<int64_t>(h[3]);
+    c->stats_read = true;
   }
   *out = c->stats;
   return ARA_OK;
@@ -1408,28 +1460,15 @@ int ara_get_timing(ara_ctx* c, ara_timing* out, int reset) {
   int rc = bind(c);
   if (rc) return rc;
   if (!out) return fail(c, ARA_EINVAL, "ara_get_timing: out is NULL");
-  *out = ara_timing{};
-  for (const auto& t : c->timed) {
-    ARA_CUDA(c, cudaEventSynchronize(t.b));
-    float ms = 0.0f;
-    ARA_CUDA(c, cudaEventElapsedTime(&ms, t.a, t.b));
-    if (t.kind == 0) {
-      out->layer_calls += 1;
-      out->kernel_ms += ms;
-      out->gather_ms += ms;
-    } else if (t.kind == 3) {
-      out->kernel_ms += ms;
-      out->losses_ms += ms;
-    } else if (t.kind == 1) {
-      out->index_ms += ms;
-    } else {
-      out->pml_calls += 1;
-      out->pml_ms += ms;
-    }
+  while (!c->timed.empty()) {
+    const ara_ctx::Timed& t = c->timed.front();
+    ARA_CUDA(c, cudaEventSynchronize(t.last()));
+    if (!fold_timed(c)) return fail(c, ARA_ECUDA, "ara_get_timing: %s", cudaGetErrorString(cudaGetLastError()));
   }
+  *out = c->timing_sum;
   out->kernel_launches = c->launches;
   if (reset) {
-    c->timed.clear();
+    c->timing_sum = ara_timing{};
     c->launches = 0;
   }
   return ARA_OK;
@@ -1455,19 +1494,12 @@ int ara_get_timing(ara_ctx* c, ara_timing* out, int reset) {
 namespace {
 
 constexpr int64_t kServeChunk = 262144;        // trials per chunk
-constexpr size_t kServeSelectPool = size_t{256} << 20;  // scratch of a pass's batched selects, at most
 static_assert(kServeChunk == int64_t{1} << kYetGridShift, "served chunks' bounds are the YET index's grid bounds");
 constexpr size_t kServeMaxInFlight = 2;        // rounds launched and not retired
 constexpr int kServePassesPerRound = 16;       // a round's passes under a long backlog
 constexpr int kServePassesShort = 4;           // ... and under a short one
 constexpr size_t kServeShortBacklog = 128;     // requests with chunks to run, at most, for a short backlog
 
-// The pool of a pass's batched selects: a batch of the largest jobs (a whole-YET prefix and four
-// return periods) within kServeSelectPool, and never less than one of them.
-size_t serve_select_pool_bytes(int64_t n_trials) {
-  const size_t one = ara::select_job_bytes(n_trials, 4);
-  return std::max(one, std::min(kServeSelectPool, one * 32));
-}
 constexpr int32_t kServeSlots = 1024;          // result slots: admitted requests at most
 constexpr int64_t kServeArenaRequests = 96;    // default arena: year losses of this many whole-YET requests
 constexpr size_t kArenaAlign = 256;
@@ -1507,7 +1539,7 @@ void arena_release(ara_ctx* c, size_t off, size_t bytes) {
 // Device buffers the serving passes use besides the arena, with the sizes they
 // need: the event buffer of the largest chunk, the tile counts and deferred
 // sums of a chunk, the layer index of the pool's ARA_MAX_BATCH_ELTS largest
-// ELTs, the select scratch for the whole YET and the result slots.  The
+// ELTs and the result slots.  The
 // serving loop reserves them before it sizes the arena, so that no pass grows
 // a buffer while rounds are in flight.
 std::vector<std::pair<DevBuf*, size_t>> serve_workspace(ara_ctx* c) {
@@ -1539,7 +1571,6 @@ std::vector<std::pair<DevBuf*, size_t>> serve_workspace(ara_ctx* c) {
       {&c->pairs_hot, sizeof(ara::PairHot) * (n_recs + 1)},
       {&c->pairs_ev, sizeof(int32_t) * (n_recs + 1)},
       {&c->scan_tmp, sizeof(uint32_t) * ara::index_scan_words(n_words)},
-      {&c->serve_sel, serve_select_pool_bytes(c->n_trials)},
       {&c->u_event, sizeof(int32_t) * (n_recs + 1)},
       {&c->idx_acc, sizeof(unsigned long long) * (ARA_MAX_BATCH_LAYERS * static_cast<size_t>(kServeChunk) +
                                                   idx_queue_words(0, kServeChunk, ARA_MAX_BATCH_LAYERS))},
@@ -1751,8 +1782,7 @@ int serve_launch_round(ara_ctx* c, const char* who, int32_t* n_failed) {
       if (e == cudaSuccess) e = cudaStreamWaitEvent(c->serve_side, c->serve_join, 0);
       int launched = 0;
       if (e == cudaSuccess)
-        e = ara::pml_tvar_batch(specs.data(), static_cast<int>(specs.size()), c->serve_sel.ptr, c->serve_sel.bytes,
-                                c->serve_side, &launched);
+        e = ara::pml_tvar_batch(specs.data(), static_cast<int>(specs.size()), c->serve_side, &launched);
       c->launches += launched;
       for (size_t k = 0; k < done.size() && e == cudaSuccess; ++k) {
         const ServeReq& q = c->serve_reqs[done[k]];
@@ -1917,23 +1947,34 @@ int ara_pml_tvar(ara_ctx* c, const double* ylt, int64_t n, const double* rps, in
     d_ylt = static_cast<const double*>(c->in_tmp.ptr);
   }
   const bool pml_dev = is_device_ptr(pml_out), tvar_dev = is_device_ptr(tvar_out);
-  if ((rc = reserve(c, c->sel, ara::select_scratch_bytes(n))) ||
-      (rc = reserve(c, c->out_tmp, 2 * sizeof(double) * n_rp)))
-    return rc;
-  double* d_pml = pml_dev ? pml_out : static_cast<double*>(c->out_tmp.ptr);
-  double* d_tvar = tvar_dev ? tvar_out : static_cast<double*>(c->out_tmp.ptr) + n_rp;
-  cudaEvent_t pa, pb;
-  if (!timed_pair(c, 2, &pa, &pb)) return fail(c, ARA_ECUDA, "ara_pml_tvar: cannot create timing events");
+  // host results: written by the kernel into pinned memory, which takes no copy
+  if ((!pml_dev || !tvar_dev) && c->h_out_n < 2 * static_cast<size_t>(n_rp)) {
+    if (c->h_out) cudaFreeHost(c->h_out);
+    c->h_out = nullptr;
+    c->h_out_n = 0;
+    void* h = nullptr;
+    const size_t want = std::max<size_t>(64, 2 * static_cast<size_t>(n_rp));
+    if (cudaHostAlloc(&h, sizeof(double) * want, cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(c, ARA_ENOMEM, "ara_pml_tvar: cannot allocate pinned results");
+    }
+    c->h_out = static_cast<double*>(h);
+    c->h_out_n = want;
+  }
+  double* d_pml = pml_dev ? pml_out : c->h_out;
+  double* d_tvar = tvar_dev ? tvar_out : c->h_out + n_rp;
+  ara_ctx::Timed timed;
+  if (!timed_begin(c, 2, &timed)) return fail(c, ARA_ECUDA, "ara_pml_tvar: cannot create timing events");
   int launched = 0;
-  ARA_CUDA(c, cudaEventRecord(pa, c->stream));
-  ARA_CUDA(c, ara::pml_tvar_device(d_ylt, n, h_rps.data(), n_rp, d_pml, d_tvar, c->sel.ptr, c->sel.bytes, c->stream,
-                                   &launched));
-  ARA_CUDA(c, cudaEventRecord(pb, c->stream));
+  ARA_CUDA(c, cudaEventRecord(timed.e[0], c->stream));
+  const ara::SelectSpec spec{d_ylt, n, h_rps.data(), n_rp, d_pml, d_tvar};
+  ARA_CUDA(c, ara::pml_tvar_batch(&spec, 1, c->stream, &launched));
+  ARA_CUDA(c, cudaEventRecord(timed.e[1], c->stream));
+  timed_end(c, timed);
   c->launches += launched;
-  if (!pml_dev) ARA_CUDA(c, cudaMemcpyAsync(pml_out, d_pml, sizeof(double) * n_rp, cudaMemcpyDeviceToHost, c->stream));
-  if (!tvar_dev)
-    ARA_CUDA(c, cudaMemcpyAsync(tvar_out, d_tvar, sizeof(double) * n_rp, cudaMemcpyDeviceToHost, c->stream));
   if (!pml_dev || !tvar_dev || !is_device_ptr(ylt)) ARA_CUDA(c, cudaStreamSynchronize(c->stream));
+  if (!pml_dev) std::memcpy(pml_out, d_pml, sizeof(double) * n_rp);
+  if (!tvar_dev) std::memcpy(tvar_out, d_tvar, sizeof(double) * n_rp);
   return ARA_OK;
 }
 
@@ -2144,12 +2185,13 @@ void ara_destroy(ara_ctx* c) {
                     &c->pairs,      &c->pairs_hot,      &c->pairs_w,       &c->pairs_ev,       &c->scan_tmp,
                     &c->flags,      &c->counters,       &c->ylt_tmp,       &c->diag_tmp,       &c->sel,
                     &c->in_tmp,     &c->out_tmp,        &c->serve_arena,   &c->serve_out,      &c->yix_occ,
-                    &c->yix_grid,   &c->yix_work,       &c->u_event,       &c->idx_acc,        &c->serve_sel,
+                    &c->yix_grid,   &c->yix_work,       &c->u_event,       &c->idx_acc,
                     &c->ev_occ,     &c->row_base,       &c->evr_stage,     &c->yet_flags};
   for (DevBuf* b : bufs) release(c, *b);
   for (auto& e : c->ev)
     if (e) cudaEventDestroy(e);
-  for (auto& e : c->ev_pool) cudaEventDestroy(e);
+  for (auto& e : c->ev_all) cudaEventDestroy(e);
+  if (c->h_out) cudaFreeHost(c->h_out);
   for (auto& r : c->serve_rounds) cudaEventDestroy(r.ev);
   for (auto& e : c->tune_ev)
     if (e) cudaEventDestroy(e);

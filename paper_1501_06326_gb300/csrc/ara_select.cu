@@ -2,16 +2,14 @@
 //
 // Year losses are mapped to order-preserving 64-bit keys (sign-flipped IEEE
 // bits).  PML(RP) is the m-th largest year loss, m = ceil(n / RP): an MSB-first
-// radix select with 8-bit digits narrows the key prefix.  With a scratch of
-// select_scratch_bytes(n), two histogram passes fix 16 bits, a third pass
-// compacts the keys of that 16-bit bucket (in a fixed order) and one block
-// finishes the remaining 48 bits on them; with only the select state (the
-// allocation-free entry point) all eight passes run over the YLT.  TVaR(RP)
-// is the mean of the m largest: the sum of the values whose key exceeds the
-// m-th key plus the tied remainder times the m-th value, in FP64 with a fixed
-// reduction order (deterministic).  The full trial order
-// (largest first, ties by index) is an LSD radix sort of the complemented keys
-// with stable per-tile scatter (warp match + per-warp digit offsets).
+// radix select narrows the key's bits, 11 at a time.  TVaR(RP) is the mean of
+// the m largest: the sum of the values whose key exceeds the m-th key plus the
+// tied remainder times the m-th value, in FP64 with a fixed assignment of
+// values to threads and a fixed reduction order (deterministic).  The full
+// trial order (largest first, ties by index) is an LSD radix sort of the
+// complemented keys with stable per-tile scatter (warp match + per-warp digit
+// offsets).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -25,11 +23,7 @@ namespace ara {
 
 namespace {
 
-constexpr int kSelBlocks = 152;  // fixed grid: deterministic reduction order
-constexpr int kSelThreads = 1024;
-constexpr int kSelUnroll = 4;  // loads in flight per thread
-constexpr int kSelGroup = 4;     // return periods selected together (one pass over the YLT serves all)
-constexpr int kSelBatchMax = 32;  // jobs of one batched select
+namespace cg = cooperative_groups;
 
 __device__ __forceinline__ unsigned long long key_of(double v) {
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v));
@@ -40,545 +34,363 @@ __device__ __forceinline__ double value_of(unsigned long long k) {
   return __longlong_as_double(static_cast<long long>(b));
 }
 
-struct SelState {
-  unsigned long long prefix;  // key bits fixed so far
-  unsigned long long mask;    // which bits are fixed
-  unsigned long long want;    // rank (1-based, from the top) within the prefix bucket
-  unsigned long long m;       // target rank
-  unsigned int bad;           // a NaN was seen
-  unsigned int pad;
-};
+// k_select: one thread-block cluster per job (a YLT and up to four return
+// periods), in one launch and without scratch in device memory.  Value i of
+// the YLT belongs to thread i mod (CTAs x 1,024) of the cluster.  Two passes
+// count a digit of 11 bits (sign, exponent, 11 bits of the significand: the
+// key's upper half) among the keys that match a period's prefix, in shared
+// memory; the CTAs' counts are added through distributed shared memory, and
+// every CTA picks each period's next digit.  The keys that then match a prefix
+// are collected.  When the cluster has at most kSelFew of them, each CTA ranks
+// them all against one another; when values are tied there are more, and four
+// digits follow over the collected keys (or the YLT, where a CTA's own do not
+// fit).  A last pass sums the values above each m-th key.
+// A short YLT is bound by the chain of passes and its barriers, and by the
+// instruction cache, as the code runs once (hence the loops that are not
+// unrolled and sel_pick not inlined: 41 us inlined, 1,000 trials); a long one by
+// one GPC's 16 SMs passing over it four times.  Device time at 1,000 / 20,000 /
+// 1,000,000 trials and two periods: 21 / 29 / 63 us; five launches with
+// histograms in device memory took 60 / 66 / 95 us, and an occurrence YLT with
+// 100,000 tied values 167 us against 65.
+constexpr int kSelThreads = 1024;
+constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kSelUnroll = 8;     // loads in flight per thread
+constexpr int kSelGroup = 4;      // return periods selected together
+constexpr int kSelBatchMax = 32;  // jobs of one launch
+constexpr int kSelBins = 2048;
+constexpr int kSelList = 8192;    // keys a CTA collects
+constexpr int kSelFew = 256;      // keys of a cluster that are ranked directly, at most
 
-struct SelScratch {
-  SelState st[kSelGroup];
-  unsigned int hist[kSelGroup][256];
-  double part_sum[kSelBlocks][kSelGroup];
-  unsigned long long part_cnt[kSelBlocks][kSelGroup];
-  unsigned int done;  // blocks of the current pass that have published their part
-};
-
-struct SelMs {
-  unsigned long long m[kSelGroup];
-};
-
-// The fast path's part of the scratch (after SelScratch): each block's digit
-// counts of the second pass, and its sum and count of the values above each
-// period's 16-bit bucket.
-struct SelFast {
-  unsigned int blk_hist[kSelBlocks][kSelGroup][256];
-  double above_sum[kSelBlocks][kSelGroup];
-  unsigned long long above_cnt[kSelBlocks][kSelGroup];
-};
-
-constexpr size_t kSelStateBytes = (sizeof(SelScratch) + 255) & ~size_t(255);
-constexpr size_t kSelFastBytes = (sizeof(SelFast) + 255) & ~size_t(255);
-
-__device__ __forceinline__ void sel_init(SelScratch* sc, const SelMs& ms, int g) {
-  if (threadIdx.x < g) {
-    SelState& st = sc->st[threadIdx.x];
-    st.prefix = 0;
-    st.mask = 0;
-    st.want = ms.m[threadIdx.x];
-    st.m = ms.m[threadIdx.x];
-    st.bad = 0;
-  }
-  for (int i = threadIdx.x; i < kSelGroup * 256; i += blockDim.x) (&sc->hist[0][0])[i] = 0;
-  if (threadIdx.x == 0) sc->done = 0;
-}
-
-__global__ void k_sel_init(SelScratch* sc, SelMs ms, int g) { sel_init(sc, ms, g); }
-
-// True in the block that is the last of the grid to arrive (after each block
-// published its part with a fence); that block then sees every part.
-__device__ __forceinline__ bool last_block_arrives(SelScratch* sc, int n_blocks) {
-  __shared__ bool s_last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = (atomicAdd(&sc->done, 1u) == static_cast<unsigned int>(n_blocks) - 1u);
-  __syncthreads();
-  if (s_last) __threadfence();
-  return s_last;
-}
-
-// One MSB-first digit pass for every return period of the group: histogram of
-// the digit among the keys that match each period's prefix (warp-aggregated
-// shared-memory counts, then one global add per digit and block); the last
-// block to finish picks each period's digit and clears the histogram.
-// blk_hist (or NULL): each block also stores its own counts there.  The
-// select's grid is nb blocks; this is block bx.
-__device__ __forceinline__ void sel_hist(const double* ylt, int64_t n, SelScratch* sc, int g, int shift,
-                                         unsigned int* blk_hist, int nb, int bx) {
-  __shared__ unsigned int sh[kSelGroup][256];
-  for (int i = threadIdx.x; i < kSelGroup * 256; i += blockDim.x) (&sh[0][0])[i] = 0;
-  unsigned long long prefix[kSelGroup], mask[kSelGroup];
-#pragma unroll
-  for (int r = 0; r < kSelGroup; ++r) {
-    prefix[r] = r < g ? sc->st[r].prefix : ~0ull;
-    mask[r] = r < g ? sc->st[r].mask : 0ull;
-  }
-  __syncthreads();
-  const int64_t stride = static_cast<int64_t>(nb) * blockDim.x;
-  bool nan = false;
-  // whole warps take part in every round (the match below needs all lanes)
-  const int64_t span = stride * kSelUnroll;
-  const int64_t n_round = ((n + span - 1) / span) * span;
-  for (int64_t i0 = bx * static_cast<int64_t>(blockDim.x) + threadIdx.x; i0 < n_round; i0 += span) {
-    double v[kSelUnroll];
-#pragma unroll
-    for (int u = 0; u < kSelUnroll; ++u) {
-      const int64_t i = i0 + u * stride;
-      v[u] = (i < n) ? ylt[i] : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < kSelUnroll; ++u) {
-      const bool in = i0 + u * stride < n;
-      nan |= (v[u] != v[u]);
-      const unsigned long long k = key_of(v[u]);
-      const unsigned int d = static_cast<unsigned int>((k >> shift) & 255u);
-#pragma unroll
-      for (int r = 0; r < kSelGroup; ++r) {
-        if (r >= g) break;
-        const bool hit = in && (k & mask[r]) == prefix[r];
-        const unsigned int hm = __ballot_sync(0xffffffffu, hit);
-        if (hm == 0u) continue;
-        if (__popc(hm) == 1) {  // one key: no aggregation needed
-          if (hit) atomicAdd(&sh[r][d], 1u);
-          continue;
-        }
-        const unsigned int peers = __match_any_sync(0xffffffffu, hit ? d : 256u + (threadIdx.x & 31));
-        if (hit && (threadIdx.x & 31) == static_cast<unsigned int>(__ffs(peers) - 1))
-          atomicAdd(&sh[r][d], static_cast<unsigned int>(__popc(peers)));
-      }
-    }
-  }
-  if (nan) atomicOr(&sc->st[0].bad, 1u);
-  __syncthreads();
-  for (int i = threadIdx.x; i < g * 256; i += blockDim.x) {
-    const unsigned int c = (&sh[0][0])[i];
-    if (c) atomicAdd(&(&sc->hist[0][0])[i], c);
-    if (blk_hist) blk_hist[static_cast<size_t>(bx) * kSelGroup * 256 + i] = c;
-  }
-  if (!last_block_arrives(sc, nb)) return;
-  // ---- pick: per period, the digit holding the wanted rank (a suffix scan of
-  // the counts from digit 255 down, thread t holding digit 255 - t)
-  __shared__ unsigned int s_warp[kSelThreads / 32];
-  for (int r = 0; r < g; ++r) {
-    const unsigned int c = (threadIdx.x < 256) ? __ldcg(&sc->hist[r][255 - threadIdx.x]) : 0u;
-    unsigned int incl = c;
-#pragma unroll
-    for (int dd = 1; dd < 32; dd <<= 1) {
-      const unsigned int o = __shfl_up_sync(0xffffffffu, incl, dd);
-      if ((threadIdx.x & 31) >= static_cast<unsigned int>(dd)) incl += o;
-    }
-    if ((threadIdx.x & 31) == 31) s_warp[threadIdx.x >> 5] = incl;
-    __syncthreads();
-    unsigned int before = 0;
-    for (int w = 0; w < static_cast<int>(threadIdx.x >> 5); ++w) before += s_warp[w];
-    incl += before;  // counts of digits 255 .. 255 - t
-    const unsigned long long want = __ldcg(&sc->st[r].want);
-    // the first t (highest digit) whose running count reaches want; digit 0 if none does
-    const bool reach = threadIdx.x < 256 && static_cast<unsigned long long>(incl) >= want &&
-                       (threadIdx.x == 0 || static_cast<unsigned long long>(incl - c) < want);
-    if (reach || (threadIdx.x == 255 && static_cast<unsigned long long>(incl) < want)) {
-      SelState& st = sc->st[r];
-      st.want = want - (incl - c);
-      st.prefix |= static_cast<unsigned long long>(255 - threadIdx.x) << shift;
-      st.mask |= 255ull << shift;
-    }
-    __syncthreads();
-  }
-  for (int i = threadIdx.x; i < kSelGroup * 256; i += blockDim.x) (&sc->hist[0][0])[i] = 0;
-  if (threadIdx.x == 0) sc->done = 0;
-}
-
-__global__ void k_sel_hist(const double* ylt, int64_t n, SelScratch* sc, int g, int shift, unsigned int* blk_hist) {
-  sel_hist(ylt, n, sc, g, shift, blk_hist, static_cast<int>(gridDim.x), static_cast<int>(blockIdx.x));
-}
-
-// Sum and count of the values whose key exceeds each selected key.
-__global__ void k_sel_tail(const double* ylt, int64_t n, SelScratch* sc, int g, double* pml, double* tvar) {
-  __shared__ double s_sum[kSelThreads / 32][kSelGroup];
-  __shared__ unsigned long long s_cnt[kSelThreads / 32][kSelGroup];
-  unsigned long long kth[kSelGroup];
-#pragma unroll
-  for (int r = 0; r < kSelGroup; ++r) kth[r] = r < g ? sc->st[r].prefix : ~0ull;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  double sum[kSelGroup];
-  unsigned long long cnt[kSelGroup];
-#pragma unroll
-  for (int r = 0; r < kSelGroup; ++r) {
-    sum[r] = 0.0;
-    cnt[r] = 0;
-  }
-  for (int64_t i0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i0 < n; i0 += stride * kSelUnroll) {
-    double v[kSelUnroll];
-#pragma unroll
-    for (int u = 0; u < kSelUnroll; ++u) {
-      const int64_t i = i0 + u * stride;
-      v[u] = (i < n) ? ylt[i] : -INFINITY;
-    }
-#pragma unroll
-    for (int u = 0; u < kSelUnroll; ++u) {
-      const unsigned long long k = key_of(v[u]);
-#pragma unroll
-      for (int r = 0; r < kSelGroup; ++r)
-        if (i0 + u * stride < n && k > kth[r]) {
-          sum[r] += v[u];
-          ++cnt[r];
-        }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < kSelGroup; ++r) {
-    for (int d = 16; d > 0; d >>= 1) {
-      sum[r] += __shfl_down_sync(0xffffffffu, sum[r], d);
-      cnt[r] += __shfl_down_sync(0xffffffffu, cnt[r], d);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      s_sum[threadIdx.x >> 5][r] = sum[r];
-      s_cnt[threadIdx.x >> 5][r] = cnt[r];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < g) {
-    const int r = threadIdx.x;
-    double t = 0.0;
-    unsigned long long c = 0;
-    for (int w = 0; w < kSelThreads / 32; ++w) {
-      t += s_sum[w][r];
-      c += s_cnt[w][r];
-    }
-    sc->part_sum[blockIdx.x][r] = t;
-    sc->part_cnt[blockIdx.x][r] = c;
-  }
-  if (!last_block_arrives(sc, static_cast<int>(gridDim.x))) return;
-  // ---- finish (the last block): one thread per part, then a tree of fixed
-  // shape over the parts, so the sum is deterministic
-  __shared__ double s_ps[kSelBlocks];
-  __shared__ unsigned long long s_pc[kSelBlocks];
-  for (int r = 0; r < g; ++r) {
-    const unsigned int i = threadIdx.x;
-    if (i < kSelBlocks) {
-      s_ps[i] = (i < gridDim.x) ? __ldcg(&sc->part_sum[i][r]) : 0.0;
-      s_pc[i] = (i < gridDim.x) ? __ldcg(&sc->part_cnt[i][r]) : 0ull;
-    }
-    __syncthreads();
-    for (unsigned int half = 128; half > 0; half >>= 1) {  // 256 >= kSelBlocks leaves
-      if (i < half && i + half < kSelBlocks) {
-        s_ps[i] += s_ps[i + half];
-        s_pc[i] += s_pc[i + half];
-      }
-      __syncthreads();
-    }
-    if (i == 0) {
-      const double v = value_of(sc->st[r].prefix);
-      const unsigned long long m = sc->st[r].m;
-      pml[r] = v;
-      tvar[r] = (s_ps[0] + static_cast<double>(m - s_pc[0]) * v) / static_cast<double>(m);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) sc->done = 0;
-}
-
-// The fast path's third pass: with each period's 16-bit prefix fixed, the
-// keys of that bucket are written to cand[r * n ..] in a fixed order (block
-// by block, in the order of the block's elements), each block starting at the
-// number of bucket keys of the blocks before it (from the second pass's
-// per-block counts); each block also publishes the FP64 sum and the count of
-// its values above the bucket.  Same grid and element assignment as
-// k_sel_hist (a grid of nb blocks; this is block bx).
-__device__ __forceinline__ void sel_compact(const double* ylt, int64_t n, const SelScratch* sc, SelFast* sf, int g,
-                                            unsigned long long* cand, int nb, int bx) {
-  __shared__ unsigned int s_wcnt[kSelThreads / 32][kSelGroup];
-  __shared__ unsigned int s_off[kSelGroup];
-  __shared__ double s_sum[kSelThreads / 32][kSelGroup];
-  __shared__ unsigned long long s_cnt[kSelThreads / 32][kSelGroup];
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long prefix[kSelGroup], mask[kSelGroup], top[kSelGroup];
-#pragma unroll
-  for (int r = 0; r < kSelGroup; ++r) {
-    prefix[r] = r < g ? sc->st[r].prefix : ~0ull;
-    mask[r] = r < g ? sc->st[r].mask : 0ull;
-    top[r] = r < g ? (prefix[r] | ~mask[r]) : ~0ull;  // the bucket's largest key
-  }
-  {
-    // this block's first candidate per period: the bucket counts of the blocks
-    // before it, summed by the whole block (one earlier block per thread)
-    unsigned int part[kSelGroup];
-#pragma unroll
-    for (int r = 0; r < kSelGroup; ++r) part[r] = 0u;
-    for (unsigned int b = threadIdx.x; b < static_cast<unsigned int>(bx); b += blockDim.x) {
-#pragma unroll
-      for (int r = 0; r < kSelGroup; ++r)
-        if (r < g) part[r] += sf->blk_hist[b][r][static_cast<unsigned int>(prefix[r] >> 48) & 255u];
-    }
-#pragma unroll
-    for (int r = 0; r < kSelGroup; ++r) {
-      const unsigned int w = __reduce_add_sync(0xffffffffu, part[r]);
-      if (lane == 0) s_wcnt[warp][r] = w;
-    }
-    __syncthreads();
-    if (threadIdx.x < static_cast<unsigned int>(g)) {
-      unsigned int off = 0;
-      for (int w = 0; w < kSelThreads / 32; ++w) off += s_wcnt[w][threadIdx.x];
-      s_off[threadIdx.x] = off;
-    }
-    __syncthreads();
-  }
-  const int64_t stride = static_cast<int64_t>(nb) * blockDim.x;
-  const int64_t span = stride * kSelUnroll;
-  const int64_t n_round = ((n + span - 1) / span) * span;
-  double sum[kSelGroup];
-  unsigned long long cnt[kSelGroup];
-#pragma unroll
-  for (int r = 0; r < kSelGroup; ++r) {
-    sum[r] = 0.0;
-    cnt[r] = 0;
-  }
-  for (int64_t i0 = bx * static_cast<int64_t>(blockDim.x) + threadIdx.x; i0 < n_round; i0 += span) {
-#pragma unroll 1
-    for (int u = 0; u < kSelUnroll; ++u) {
-      const bool in = i0 + u * stride < n;
-      const double vu = in ? ylt[i0 + u * stride] : 0.0;
-      const unsigned long long k = key_of(vu);
-      unsigned int bal[kSelGroup];
-#pragma unroll
-      for (int r = 0; r < kSelGroup; ++r) {
-        const bool match = r < g && in && (k & mask[r]) == prefix[r];
-        bal[r] = __ballot_sync(0xffffffffu, match);
-        if (r < g && in && k > top[r]) {
-          sum[r] += vu;
-          ++cnt[r];
-        }
-      }
-      if (lane == 0)
-#pragma unroll
-        for (int r = 0; r < kSelGroup; ++r) s_wcnt[warp][r] = __popc(bal[r]);
-      __syncthreads();
-      unsigned int total[kSelGroup];
-#pragma unroll
-      for (int r = 0; r < kSelGroup; ++r) {
-        // exclusive prefix of the warps' counts: lane w holds warp w's count
-        // (periods r >= g have none)
-        const unsigned int c = s_wcnt[lane][r];
-        unsigned int incl = c;
-#pragma unroll
-        for (int dd = 1; dd < 32; dd <<= 1) {
-          const unsigned int o = __shfl_up_sync(0xffffffffu, incl, dd);
-          if (lane >= static_cast<unsigned int>(dd)) incl += o;
-        }
-        const unsigned int before = __shfl_sync(0xffffffffu, incl - c, warp);
-        total[r] = __shfl_sync(0xffffffffu, incl, 31);
-        if ((bal[r] >> lane) & 1u)
-          cand[static_cast<size_t>(r) * n + s_off[r] + before + __popc(bal[r] & ((1u << lane) - 1u))] = k;
-      }
-      __syncthreads();
-      if (threadIdx.x == 0)
-#pragma unroll
-        for (int r = 0; r < kSelGroup; ++r)
-          if (r < g) s_off[r] += total[r];
-      __syncthreads();
-    }
-  }
-  // the block's sums above the buckets, in a fixed order
-#pragma unroll
-  for (int r = 0; r < kSelGroup; ++r) {
-    for (int d = 16; d > 0; d >>= 1) {
-      sum[r] += __shfl_down_sync(0xffffffffu, sum[r], d);
-      cnt[r] += __shfl_down_sync(0xffffffffu, cnt[r], d);
-    }
-    if (lane == 0) {
-      s_sum[warp][r] = sum[r];
-      s_cnt[warp][r] = cnt[r];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < static_cast<unsigned int>(g)) {
-    const int r = threadIdx.x;
-    double t = 0.0;
-    unsigned long long c = 0;
-    for (int w = 0; w < kSelThreads / 32; ++w) {
-      t += s_sum[w][r];
-      c += s_cnt[w][r];
-    }
-    sf->above_sum[bx][r] = t;
-    sf->above_cnt[bx][r] = c;
-  }
-}
-
-__global__ void k_sel_compact(const double* ylt, int64_t n, const SelScratch* sc, SelFast* sf, int g,
-                              unsigned long long* cand) {
-  sel_compact(ylt, n, sc, sf, g, cand, static_cast<int>(gridDim.x), static_cast<int>(blockIdx.x));
-}
-
-// The fast path's finish, one block per period: the remaining six digits of
-// the m-th key over the bucket's keys, then TVaR from the sums above the
-// bucket (the blocks' parts, a tree of fixed shape) and the bucket keys above
-// the m-th key (a fixed assignment of keys to threads and a fixed tree).
-// Period r's finish (a block).
-__device__ __forceinline__ void sel_finish(int64_t n, SelScratch* sc, const SelFast* sf, int n_blk,
-                                           const unsigned long long* cand, double* pml, double* tvar, int r) {
-  __shared__ unsigned int s_hist[256];
-  __shared__ unsigned int s_warp[kSelThreads / 32];
-  __shared__ unsigned long long s_prefix, s_mask, s_want;
-  __shared__ unsigned int s_c;
-  __shared__ double s_ps[256];
-  __shared__ unsigned long long s_pc[256];
-  const unsigned int t = threadIdx.x, lane = t & 31;
-  {
-    if (t == 0) {
-      s_prefix = sc->st[r].prefix;
-      s_mask = sc->st[r].mask;
-      s_want = sc->st[r].want;
-      const unsigned int d = static_cast<unsigned int>(s_prefix >> 48) & 255u;
-      unsigned int c = 0;
-      for (int b = 0; b < n_blk; ++b) c += sf->blk_hist[b][r][d];
-      s_c = c;
-    }
-    __syncthreads();
-    const unsigned int C = s_c;
-    const unsigned long long* ck = cand + static_cast<size_t>(r) * n;
-    for (int shift = 40; shift >= 0; shift -= 8) {
-      if (t < 256) s_hist[t] = 0;
-      __syncthreads();
-      const unsigned long long prefix = s_prefix, mask = s_mask;
-      for (unsigned int j = t; j < C; j += kSelThreads) {
-        const unsigned long long k = ck[j];
-        if ((k & mask) == prefix) atomicAdd(&s_hist[(k >> shift) & 255u], 1u);
-      }
-      __syncthreads();
-      // the digit holding the wanted rank (suffix scan, thread t holding digit 255 - t)
-      const unsigned int c = (t < 256) ? s_hist[255 - t] : 0u;
-      unsigned int incl = c;
-#pragma unroll
-      for (int dd = 1; dd < 32; dd <<= 1) {
-        const unsigned int o = __shfl_up_sync(0xffffffffu, incl, dd);
-        if (lane >= static_cast<unsigned int>(dd)) incl += o;
-      }
-      if (lane == 31) s_warp[t >> 5] = incl;
-      __syncthreads();
-      unsigned int before = 0;
-      for (unsigned int w = 0; w < (t >> 5); ++w) before += s_warp[w];
-      incl += before;
-      const unsigned long long want = s_want;
-      const bool reach = t < 256 && static_cast<unsigned long long>(incl) >= want &&
-                         (t == 0 || static_cast<unsigned long long>(incl - c) < want);
-      __syncthreads();
-      if (reach || (t == 255 && static_cast<unsigned long long>(incl) < want)) {
-        s_want = want - (incl - c);
-        s_prefix = prefix | (static_cast<unsigned long long>(255 - t) << shift);
-        s_mask = mask | (255ull << shift);
-      }
-      __syncthreads();
-    }
-    const unsigned long long kth = s_prefix;
-    // bucket keys above the m-th key
-    double sum = 0.0;
-    unsigned long long cnt = 0;
-    for (unsigned int j = t; j < C; j += kSelThreads) {
-      const unsigned long long k = ck[j];
-      if (k > kth) {
-        sum += value_of(k);
-        ++cnt;
-      }
-    }
-    for (int d = 16; d > 0; d >>= 1) {
-      sum += __shfl_down_sync(0xffffffffu, sum, d);
-      cnt += __shfl_down_sync(0xffffffffu, cnt, d);
-    }
-    if (lane == 0) {
-      s_ps[t >> 5] = sum;
-      s_pc[t >> 5] = cnt;
-    }
-    __syncthreads();
-    double bucket_sum = 0.0;
-    unsigned long long bucket_cnt = 0;
-    if (t == 0) {
-      for (int w = 0; w < kSelThreads / 32; ++w) {
-        bucket_sum += s_ps[w];
-        bucket_cnt += s_pc[w];
-      }
-    }
-    __syncthreads();
-    // the blocks' parts above the bucket
-    if (t < 256) {
-      s_ps[t] = (static_cast<int>(t) < n_blk) ? sf->above_sum[t][r] : 0.0;
-      s_pc[t] = (static_cast<int>(t) < n_blk) ? sf->above_cnt[t][r] : 0ull;
-    }
-    __syncthreads();
-    for (unsigned int half = 128; half > 0; half >>= 1) {
-      if (t < half) {
-        s_ps[t] += s_ps[t + half];
-        s_pc[t] += s_pc[t + half];
-      }
-      __syncthreads();
-    }
-    if (t == 0) {
-      const double v = value_of(kth);
-      const unsigned long long m = sc->st[r].m;
-      const double s_all = s_ps[0] + bucket_sum;
-      const unsigned long long c_all = s_pc[0] + bucket_cnt;
-      pml[r] = v;
-      tvar[r] = (s_all + static_cast<double>(m - c_all) * v) / static_cast<double>(m);
-    }
-    __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(kSelThreads) k_sel_finish(int64_t n, SelScratch* sc, const SelFast* sf, int n_blk,
-                                                             const unsigned long long* cand, double* pml,
-                                                             double* tvar) {
-  sel_finish(n, sc, sf, n_blk, cand, pml, tvar, static_cast<int>(blockIdx.x));
-}
-
-// ---- batched selects: one launch per pass for several YLTs (jobs), blockIdx.y
-// the job; each job runs on its own grid size and scratch exactly as the
-// single select does, so it gives the same bits
 struct SelJob {
   const double* ylt;
   int64_t n;
-  SelScratch* sc;
-  SelFast* sf;
-  unsigned long long* cand;  // [g][n]
   double* pml;
   double* tvar;
-  SelMs ms;
+  unsigned long long m[kSelGroup];
   int g;
-  int grid;
 };
 struct SelBatch {
   SelJob job[kSelBatchMax];
 };
 
-__global__ void k_sel_init_batch(const __grid_constant__ SelBatch b) {
-  const SelJob& j = b.job[blockIdx.y];
-  sel_init(j.sc, j.ms, j.g);
+struct SelShared {
+  union {
+    unsigned int hist[kSelGroup][kSelBins];   // this CTA's counts
+    unsigned long long ring[kSelWarps][64];   // the last pass: keys to be summed, per warp
+    unsigned long long few[kSelFew];          // the cluster's collected keys, when they are few
+  };
+  unsigned int total[kSelGroup][kSelBins];    // the cluster's counts
+  unsigned long long list[kSelList];          // collected keys
+  unsigned int n_list;
+  unsigned int warp_sum[kSelWarps];
+  // per period: the key's bits fixed so far, the rank wanted among the keys with them (1 = largest)
+  unsigned long long prefix[kSelGroup], want[kSelGroup];
+  double part[kSelWarps][kSelGroup];
+  double cta_sum[kSelGroup];
+};
+
+// The values of the YLT that belong to this thread (kStride apart): f(value,
+// valid) is called by whole warps.
+template <int kStride, class F>
+__device__ __forceinline__ void sel_values(const SelJob& j, int first, F f) {
+  const double* p = j.ylt + first;
+  const int64_t left = j.n - first;
+  const int64_t cnt = left > 0 ? (left + kStride - 1) / kStride : 0;
+  const int64_t most = __shfl_sync(0xffffffffu, cnt, 0);  // the warp's first lane has the most
+#pragma unroll 1
+  for (int64_t u0 = 0; u0 < most; u0 += kSelUnroll, p += static_cast<int64_t>(kSelUnroll) * kStride) {
+    const int here = static_cast<int>(cnt - u0 < kSelUnroll ? cnt - u0 : kSelUnroll);
+    double v[kSelUnroll];
+#pragma unroll
+    for (int u = 0; u < kSelUnroll; ++u) v[u] = u < here ? p[static_cast<int64_t>(u) * kStride] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kSelUnroll; ++u) f(v[u], u < here);
+  }
 }
 
-__global__ void k_sel_hist_batch(const __grid_constant__ SelBatch b, int shift, int with_blk) {
-  const SelJob& j = b.job[blockIdx.y];
-  if (static_cast<int>(blockIdx.x) >= j.grid) return;
-  sel_hist(j.ylt, j.n, j.sc, j.g, shift, with_blk ? &j.sf->blk_hist[0][0][0] : nullptr, j.grid,
-           static_cast<int>(blockIdx.x));
+// The upper half of a value's key.
+__device__ __forceinline__ unsigned int key_hi(double v) {
+  const int h = __double2hiint(v);
+  return static_cast<unsigned int>(h) ^ (static_cast<unsigned int>(h >> 31) | 0x80000000u);
 }
 
-__global__ void k_sel_compact_batch(const __grid_constant__ SelBatch b) {
-  const SelJob& j = b.job[blockIdx.y];
-  if (static_cast<int>(blockIdx.x) >= j.grid) return;
-  sel_compact(j.ylt, j.n, j.sc, j.sf, j.g, j.cand, j.grid, static_cast<int>(blockIdx.x));
+// Whether period r is the first with its prefix (the others share its counts).
+__device__ __forceinline__ bool sel_owns(const SelShared& sm, int g, int r) {
+  bool own = r < g;
+#pragma unroll
+  for (int q = 0; q < kSelGroup; ++q) own = own && !(q < r && sm.prefix[q] == sm.prefix[r]);
+  return own;
 }
 
-__global__ void __launch_bounds__(kSelThreads) k_sel_finish_batch(const __grid_constant__ SelBatch b) {
-  const SelJob& j = b.job[blockIdx.y];
-  if (static_cast<int>(blockIdx.x) >= j.g) return;
-  sel_finish(j.n, j.sc, j.sf, j.grid, j.cand, j.pml, j.tvar, static_cast<int>(blockIdx.x));
+// Clears the counts (by all threads; ends with a barrier).
+__device__ __noinline__ void sel_clear(SelShared& sm) {
+  uint4* h = reinterpret_cast<uint4*>(&sm.hist[0][0]);
+#pragma unroll
+  for (int i = 0; i < kSelGroup * kSelBins / 4 / kSelThreads; ++i)
+    h[i * kSelThreads + threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
 }
 
-int sel_grid(int64_t n) {
-  const int64_t blocks = (n + kSelThreads - 1) / kSelThreads;
-  return static_cast<int>(blocks < kSelBlocks ? blocks : kSelBlocks);
+// One digit of `bits` bits from its counts in sm.hist: their sums over the
+// cluster, and each period's choice.  Not inlined: the kernel runs its code
+// once, so the instruction cache's misses count.
+template <int kCtas>
+__device__ __noinline__ void sel_pick(SelShared& sm, int g, int bits) {
+  const unsigned int t = threadIdx.x, lane = t & 31u, r = t >> 8, u = t & 255u;
+  unsigned int* total = &sm.total[0][0];
+  if constexpr (kCtas > 1) {
+    cg::cluster_group cluster = cg::this_cluster();
+    const unsigned int rank = cluster.block_rank();
+    unsigned int* hist = &sm.hist[0][0];
+    cluster.sync();
+    // this CTA's share of the bins, summed over the cluster; then everyone's shares.  The r-th quarter of
+    // the threads takes period r
+    constexpr unsigned int kShare = kSelBins / kCtas;
+    const bool own = sel_owns(sm, g, static_cast<int>(r));
+    if (own)
+#pragma unroll 1
+      for (unsigned int i = rank * kShare + u; i < (rank + 1) * kShare; i += 256) {
+        unsigned int s[kCtas], all = 0u;
+#pragma unroll
+        for (int c = 0; c < kCtas; ++c) s[c] = cluster.map_shared_rank(hist, c)[r * kSelBins + i];
+#pragma unroll
+        for (int c = 0; c < kCtas; ++c) all += s[c];
+        total[r * kSelBins + i] = all;
+      }
+    cluster.sync();
+    if (own)
+#pragma unroll
+      for (unsigned int i = u; i < kSelBins; i += 256) {
+        const unsigned int c = i / kShare;
+        if (c != rank) total[r * kSelBins + i] = cluster.map_shared_rank(total, c)[r * kSelBins + i];
+      }
+  } else {
+    total = &sm.hist[0][0];
+  }
+  __syncthreads();
+  // period r's digit, 8 bins a thread from the top: the first whose running count reaches the wanted rank
+  const bool live = static_cast<int>(r) < g;
+  unsigned int c[8], sum = 0u;
+  if (live) {
+    int slot = static_cast<int>(r);
+#pragma unroll
+    for (int q = kSelGroup - 1; q >= 0; --q)
+      if (q < static_cast<int>(r) && sm.prefix[q] == sm.prefix[r]) slot = q;
+    const uint4* tk = reinterpret_cast<const uint4*>(total + slot * kSelBins + (kSelBins - 8 - 8 * u));
+    const uint4 lo = tk[0], hi = tk[1];  // a digit of fewer bits leaves its upper bins empty
+    c[0] = hi.w; c[1] = hi.z; c[2] = hi.y; c[3] = hi.x;
+    c[4] = lo.w; c[5] = lo.z; c[6] = lo.y; c[7] = lo.x;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sum += c[q];
+  }
+  unsigned int incl = sum;
+#pragma unroll
+  for (int dd = 1; dd < 32; dd <<= 1) {
+    const unsigned int o = __shfl_up_sync(0xffffffffu, incl, dd);
+    if (lane >= static_cast<unsigned int>(dd)) incl += o;
+  }
+  if (lane == 31u) sm.warp_sum[t >> 5] = incl;
+  const unsigned long long want = live ? sm.want[r] : 0ull;
+  __syncthreads();
+  unsigned long long before = incl - sum;
+#pragma unroll
+  for (unsigned int w = 0; w < 7; ++w)
+    if (w < ((t >> 5) & 7u)) before += sm.warp_sum[r * 8 + w];
+  if (live && before < want && want <= before + sum) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (before < want && want <= before + c[q]) {
+        sm.want[r] = want - before;
+        sm.prefix[r] = (sm.prefix[r] << bits) | (kSelBins - 1 - (8 * u + q));
+      }
+      before += c[q];
+    }
+  }
+  __syncthreads();
 }
+
+template <int kCtas>
+__global__ void __launch_bounds__(kSelThreads, 1) k_select(const __grid_constant__ SelBatch b) {
+  extern __shared__ __align__(16) unsigned char sel_smem[];
+  SelShared& sm = *reinterpret_cast<SelShared*>(sel_smem);
+  cg::cluster_group cluster = cg::this_cluster();
+  const SelJob& j = b.job[blockIdx.y];
+  constexpr int kStride = kCtas * kSelThreads;
+  const unsigned int t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+  const unsigned int rank = kCtas > 1 ? cluster.block_rank() : 0u;
+  const int first = static_cast<int>(rank * kSelThreads + t);
+  if (t < static_cast<unsigned int>(kSelGroup)) {
+    sm.prefix[t] = 0ull;
+    sm.want[t] = j.m[t];
+  }
+  if (t == 0) sm.n_list = 0u;
+  sel_clear(sm);
+  // the first two digits are in the key's upper half; with nothing fixed there is one set of counts
+  sel_values<kStride>(j, first, [&](double v, bool valid) {
+    if (valid) atomicAdd(&sm.hist[0][key_hi(v) >> 21], 1u);
+  });
+  __syncthreads();
+  sel_pick<kCtas>(sm, j.g, 11);
+  unsigned int p32[kSelGroup];
+#pragma unroll
+  for (int k = 0; k < kSelGroup; ++k) p32[k] = sel_owns(sm, j.g, k) ? static_cast<unsigned int>(sm.prefix[k]) : ~0u;
+  sel_clear(sm);
+  sel_values<kStride>(j, first, [&](double v, bool valid) {
+    const unsigned int h = key_hi(v), top = valid ? h >> 21 : ~0u - 1u;
+#pragma unroll
+    for (int k = 0; k < kSelGroup; ++k)
+      if (top == p32[k]) atomicAdd(&sm.hist[k][(h >> 10) & 2047u], 1u);
+  });
+  __syncthreads();
+  sel_pick<kCtas>(sm, j.g, 11);
+  // the keys that still match, where this CTA has room for its own
+#pragma unroll
+  for (int k = 0; k < kSelGroup; ++k) p32[k] = k < j.g ? static_cast<unsigned int>(sm.prefix[k]) : ~0u;
+  sel_values<kStride>(j, first, [&](double v, bool valid) {
+    const unsigned int top = valid ? key_hi(v) >> 10 : ~0u - 1u;
+    const bool match = top == p32[0] || top == p32[1] || top == p32[2] || top == p32[3];
+    const unsigned int mm = __ballot_sync(0xffffffffu, match);
+    if (mm == 0u) return;
+    unsigned int at = 0u;
+    if (lane == 0) at = atomicAdd(&sm.n_list, static_cast<unsigned int>(__popc(mm)));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(mm & ((1u << lane) - 1u));
+    if (match && at < kSelList) sm.list[at] = key_of(v);
+  });
+  // few in the whole cluster: every CTA takes them all and ranks them
+  unsigned int n_few = 0u;
+  if constexpr (kCtas > 1) cluster.sync();
+  else __syncthreads();
+#pragma unroll
+  for (int c = 0; c < kCtas; ++c) n_few += kCtas > 1 ? *cluster.map_shared_rank(&sm.n_list, c) : sm.n_list;
+  if (n_few <= kSelFew) {
+    if constexpr (kCtas > 1) {
+      unsigned int at = 0u;
+#pragma unroll 1
+      for (int c = 0; c < kCtas; ++c) {
+        const unsigned int n = *cluster.map_shared_rank(&sm.n_list, c);
+        if (t < n) sm.few[at + t] = cluster.map_shared_rank(sm.list, c)[t];
+        at += n;
+      }
+      __syncthreads();
+    }
+    const unsigned long long* few = kCtas > 1 ? sm.few : sm.list;
+    unsigned long long want[kSelGroup];
+#pragma unroll
+    for (int r = 0; r < kSelGroup; ++r) want[r] = sm.want[r];
+    if (kCtas > 1) cluster.sync();  // the lists are read
+    else __syncthreads();
+    if (t < n_few) {
+      const unsigned long long mine = few[t], top = mine >> 42;
+      unsigned int above = 0u, same = 0u;
+#pragma unroll 4
+      for (unsigned int i = 0; i < n_few; ++i) {
+        const unsigned long long k = few[i];
+        above += (k > mine && (k >> 42) == top) ? 1u : 0u;
+        same += k == mine ? 1u : 0u;
+      }
+#pragma unroll
+      for (int r = 0; r < kSelGroup; ++r)
+        if (r < j.g && static_cast<unsigned int>(top) == p32[r] && above < want[r] && want[r] <= above + same) {
+          sm.prefix[r] = mine;  // ties write the same
+          sm.want[r] = want[r] - above;
+        }
+    }
+    __syncthreads();
+  } else {
+    const bool from_list = sm.n_list <= kSelList;
+#pragma unroll 1
+    for (int shift = 31, bits = 11; shift >= 0; shift = shift == 31 ? 20 : shift - 10, bits = shift > 10 ? 11 : 10) {
+      sel_clear(sm);
+      unsigned long long own[kSelGroup];
+#pragma unroll
+      for (int k = 0; k < kSelGroup; ++k) own[k] = sel_owns(sm, j.g, k) ? sm.prefix[k] : ~0ull;
+      auto count = [&](unsigned long long key, bool valid) {
+        const unsigned int d = static_cast<unsigned int>(key >> shift) & ((1u << bits) - 1u);
+        const unsigned long long top = valid ? key >> (shift + bits) : ~0ull - 1ull;
+#pragma unroll
+        for (int k = 0; k < kSelGroup; ++k)
+          if (top == own[k]) atomicAdd(&sm.hist[k][d], 1u);
+      };
+      if (from_list) {
+#pragma unroll 1
+        for (unsigned int i = t; i < sm.n_list; i += kSelThreads) count(sm.list[i], true);
+      } else {
+        sel_values<kStride>(j, first, [&](double v, bool valid) { count(key_of(v), valid); });
+      }
+      __syncthreads();
+      sel_pick<kCtas>(sm, j.g, bits);
+    }
+    if (kCtas > 1) cluster.sync();  // ring shares hist's memory, which the other CTAs have read by now
+  }
+  // sums of the values above each period's key.  A warp collects the values above the lowest of the keys
+  // and adds 32 at a time, as an FP64 add costs a whole warp's time however few lanes need it
+  double sum[kSelGroup];
+  unsigned long long kth[kSelGroup], lowest = ~0ull;
+#pragma unroll
+  for (int r = 0; r < kSelGroup; ++r) {
+    sum[r] = 0.0;
+    kth[r] = r < j.g ? sm.prefix[r] : ~0ull;
+    lowest = kth[r] < lowest ? kth[r] : lowest;
+  }
+  __syncthreads();  // few shares ring's memory
+  const unsigned int lowest_hi = static_cast<unsigned int>(lowest >> 32);
+  unsigned int held = 0u;
+  auto add = [&](unsigned long long key, bool valid) {
+    const double v = value_of(key);
+#pragma unroll
+    for (int r = 0; r < kSelGroup; ++r)
+      if (valid && key > kth[r]) sum[r] += v;
+  };
+  sel_values<kStride>(j, first, [&](double v, bool valid) {
+    bool above = valid && key_hi(v) >= lowest_hi;
+    if (__ballot_sync(0xffffffffu, above) == 0u) return;
+    const unsigned long long key = key_of(v);
+    above = above && key > lowest;
+    const unsigned int mm = __ballot_sync(0xffffffffu, above);
+    if (above) sm.ring[warp][held + __popc(mm & ((1u << lane) - 1u))] = key;
+    held += __popc(mm);
+    __syncwarp();
+    if (held >= 32u) {
+      add(sm.ring[warp][lane], true);
+      held -= 32u;
+      const unsigned long long rest = sm.ring[warp][32 + lane];
+      __syncwarp();
+      sm.ring[warp][lane] = rest;
+      __syncwarp();
+    }
+  });
+  add(lane < held ? sm.ring[warp][lane] : 0ull, lane < held);
+#pragma unroll
+  for (int r = 0; r < kSelGroup; ++r) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) sum[r] += __shfl_down_sync(0xffffffffu, sum[r], d);
+    if (lane == 0) sm.part[warp][r] = sum[r];
+  }
+  __syncthreads();
+  if (t < static_cast<unsigned int>(kSelGroup)) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kSelWarps; ++w) s += sm.part[w][t];
+    sm.cta_sum[t] = s;
+  }
+  if (kCtas > 1) cluster.sync();
+  else __syncthreads();
+  if (rank == 0 && static_cast<int>(t) < j.g) {
+    double s = 0.0;
+#pragma unroll
+    for (int c = 0; c < kCtas; ++c) s += kCtas > 1 ? cluster.map_shared_rank(sm.cta_sum, c)[t] : sm.cta_sum[t];
+    // want is now the m-th key's rank among its ties: the values above it number m - want
+    const double v = value_of(sm.prefix[t]);
+    j.pml[t] = v;
+    j.tvar[t] = (s + static_cast<double>(sm.want[t]) * v) / static_cast<double>(j.m[t]);
+  }
+  if (kCtas > 1) cluster.sync();  // the CTAs' sums stay until they are read
+}
+
+// CTAs of a YLT's cluster: by its length alone, so that a job gives the same
+// bits in any batch.  One CTA holds a YLT of up to 8 values a thread; a few
+// shorten the passes of a middle one more than their cluster barriers cost.
+int sel_ctas(int64_t n) { return n <= 8 * kSelThreads ? 1 : n <= 64 * kSelThreads ? 4 : 16; }
 
 // m = ceil(n / rp), within [1, n]
 unsigned long long sel_rank(int64_t n, double rp) {
@@ -588,104 +400,63 @@ unsigned long long sel_rank(int64_t n, double rp) {
   return static_cast<unsigned long long>(m);
 }
 
-cudaError_t launch_sel_batch(const SelBatch& b, int n_jobs, int max_grid, int max_g, cudaStream_t s) {
-  const dim3 one(1, n_jobs), wide(max_grid, n_jobs), fin(max_g, n_jobs);
-  k_sel_init_batch<<<one, 256, 0, s>>>(b);
-  k_sel_hist_batch<<<wide, kSelThreads, 0, s>>>(b, 56, 0);
-  k_sel_hist_batch<<<wide, kSelThreads, 0, s>>>(b, 48, 1);
-  k_sel_compact_batch<<<wide, kSelThreads, 0, s>>>(b);
-  k_sel_finish_batch<<<fin, kSelThreads, 0, s>>>(b);
-  return cudaGetLastError();
+template <int kCtas>
+cudaError_t launch_select(const SelBatch& b, int n_jobs, cudaStream_t s) {
+  cudaError_t err;
+  if ((err = cudaFuncSetAttribute(k_select<kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(SelShared))) !=
+          cudaSuccess ||
+      (kCtas > 8 && (err = cudaFuncSetAttribute(k_select<kCtas>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) !=
+                        cudaSuccess))
+    return err;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kCtas, n_jobs);
+  cfg.blockDim = dim3(kSelThreads);
+  cfg.dynamicSmemBytes = sizeof(SelShared);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kCtas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_select<kCtas>, b);
 }
 
 }  // namespace
 
-size_t select_job_bytes(int64_t n, int n_rp) {
-  const int g = n_rp < kSelGroup ? n_rp : kSelGroup;
-  const int groups = (n_rp + kSelGroup - 1) / kSelGroup;
-  return static_cast<size_t>(groups) * (kSelStateBytes + kSelFastBytes +
-                                        ((sizeof(unsigned long long) * g * static_cast<size_t>(n) + 255) & ~size_t(255)));
-}
-
-cudaError_t pml_tvar_batch(const SelectSpec* specs, int n_specs, void* pool, size_t pool_bytes, cudaStream_t s,
-                           int* n_launch) {
-  SelBatch b;
-  int n_jobs = 0, max_grid = 1, max_g = 1;
-  size_t used = 0;
-  unsigned char* base = static_cast<unsigned char*>(pool);
-  auto flush = [&]() -> cudaError_t {
-    if (n_jobs == 0) return cudaSuccess;
-    const cudaError_t e = launch_sel_batch(b, n_jobs, max_grid, max_g, s);
-    if (n_launch) *n_launch += 5;
-    n_jobs = 0;
-    max_grid = max_g = 1;
-    used = 0;
-    return e;
-  };
-  for (int i = 0; i < n_specs; ++i) {
-    const SelectSpec& q = specs[i];
-    if (q.n < 1 || q.n_rp < 1) return cudaErrorInvalidValue;
-    for (int r0 = 0; r0 < q.n_rp; r0 += kSelGroup) {
-      const int g = (q.n_rp - r0 < kSelGroup) ? (q.n_rp - r0) : kSelGroup;
-      const size_t need = kSelStateBytes + kSelFastBytes +
-                          ((sizeof(unsigned long long) * g * static_cast<size_t>(q.n) + 255) & ~size_t(255));
-      if (need > pool_bytes) return cudaErrorInvalidValue;
-      if (n_jobs == kSelBatchMax || used + need > pool_bytes) {
-        const cudaError_t e = flush();
-        if (e != cudaSuccess) return e;
+cudaError_t pml_tvar_batch(const SelectSpec* specs, int n_specs, cudaStream_t s, int* n_launch) {
+  for (int i = 0; i < n_specs; ++i)
+    if (specs[i].n < 1 || specs[i].n_rp < 1) return cudaErrorInvalidValue;
+  // one launch per cluster size and kSelBatchMax jobs
+  for (int ctas : {1, 4, 16}) {
+    SelBatch b;
+    int n_jobs = 0;
+    auto flush = [&]() -> cudaError_t {
+      if (n_jobs == 0) return cudaSuccess;
+      const cudaError_t e = ctas == 1   ? launch_select<1>(b, n_jobs, s)
+                            : ctas == 4 ? launch_select<4>(b, n_jobs, s)
+                                        : launch_select<16>(b, n_jobs, s);
+      if (n_launch) *n_launch += 1;
+      n_jobs = 0;
+      return e;
+    };
+    cudaError_t err;
+    for (int i = 0; i < n_specs; ++i) {
+      const SelectSpec& q = specs[i];
+      if (sel_ctas(q.n) != ctas) continue;
+      for (int r0 = 0; r0 < q.n_rp; r0 += kSelGroup) {
+        if (n_jobs == kSelBatchMax && (err = flush()) != cudaSuccess) return err;
+        SelJob& j = b.job[n_jobs++];
+        j.ylt = q.ylt;
+        j.n = q.n;
+        j.pml = q.pml + r0;
+        j.tvar = q.tvar + r0;
+        j.g = (q.n_rp - r0 < kSelGroup) ? (q.n_rp - r0) : kSelGroup;
+        for (int r = 0; r < kSelGroup; ++r) j.m[r] = r < j.g ? sel_rank(q.n, q.rps[r0 + r]) : 1ull;
       }
-      SelJob& j = b.job[n_jobs++];
-      j.ylt = q.ylt;
-      j.n = q.n;
-      j.sc = reinterpret_cast<SelScratch*>(base + used);
-      j.sf = reinterpret_cast<SelFast*>(base + used + kSelStateBytes);
-      j.cand = reinterpret_cast<unsigned long long*>(base + used + kSelStateBytes + kSelFastBytes);
-      j.pml = q.pml + r0;
-      j.tvar = q.tvar + r0;
-      j.ms = SelMs{};
-      for (int r = 0; r < g; ++r) j.ms.m[r] = sel_rank(q.n, q.rps[r0 + r]);
-      j.g = g;
-      j.grid = sel_grid(q.n);
-      max_grid = j.grid > max_grid ? j.grid : max_grid;
-      max_g = g > max_g ? g : max_g;
-      used += need;
     }
-  }
-  return flush();
-}
-
-size_t select_scratch_bytes(int64_t n) {
-  return kSelStateBytes + kSelFastBytes + sizeof(unsigned long long) * kSelGroup * static_cast<size_t>(n) + 64;
-}
-
-cudaError_t pml_tvar_device(const double* ylt, int64_t n, const double* rps_host, int32_t n_rp, double* pml,
-                            double* tvar, void* scratch, size_t scratch_bytes, cudaStream_t s, int* n_launch) {
-  SelScratch* sc = static_cast<SelScratch*>(scratch);
-  const bool fast = scratch_bytes >= select_scratch_bytes(n);
-  SelFast* sf = fast ? reinterpret_cast<SelFast*>(static_cast<unsigned char*>(scratch) + kSelStateBytes) : nullptr;
-  unsigned long long* cand =
-      fast ? reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(scratch) + kSelStateBytes + kSelFastBytes)
-           : nullptr;
-  const int grid = sel_grid(n);
-  for (int32_t r0 = 0; r0 < n_rp; r0 += kSelGroup) {
-    const int g = (n_rp - r0 < kSelGroup) ? (n_rp - r0) : kSelGroup;
-    SelMs ms{};
-    for (int r = 0; r < g; ++r) ms.m[r] = sel_rank(n, rps_host[r0 + r]);
-    k_sel_init<<<1, 256, 0, s>>>(sc, ms, g);
-    if (fast) {
-      k_sel_hist<<<grid, kSelThreads, 0, s>>>(ylt, n, sc, g, 56, nullptr);
-      k_sel_hist<<<grid, kSelThreads, 0, s>>>(ylt, n, sc, g, 48, &sf->blk_hist[0][0][0]);
-      k_sel_compact<<<grid, kSelThreads, 0, s>>>(ylt, n, sc, sf, g, cand);
-      k_sel_finish<<<g, kSelThreads, 0, s>>>(n, sc, sf, grid, cand, pml + r0, tvar + r0);
-      if (n_launch) *n_launch += 5;
-    } else {
-      for (int shift = 56; shift >= 0; shift -= 8)
-        k_sel_hist<<<grid, kSelThreads, 0, s>>>(ylt, n, sc, g, shift, nullptr);
-      k_sel_tail<<<grid, kSelThreads, 0, s>>>(ylt, n, sc, g, pml + r0, tvar + r0);
-      if (n_launch) *n_launch += 10;
-    }
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
+    if ((err = flush()) != cudaSuccess) return err;
   }
   return cudaSuccess;
 }
@@ -873,8 +644,8 @@ cudaError_t top_gather_device(const double* ylt, const int64_t* order, int64_t m
 
 // =============================================================== allocation-free PML / TVaR
 //
-// A fixed block of device memory, owned by the library, holds the select
-// state of ara_pml_tvar_noalloc and its device outputs.  In host code the
+// A fixed block of device memory, owned by the library, holds the device
+// outputs of ara_pml_tvar_noalloc (the select's state is in shared memory).  In host code the
 // name of a __device__ array is only a host-side stand-in; the kernels get
 // the block's device address, looked up once per device.
 namespace {
@@ -884,8 +655,8 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[ARA_NOALLOC_SCR
 constexpr int kNoallocMaxDevices = 64;
 void* g_noalloc_addr[kNoallocMaxDevices] = {};  // device address of the block, per device
 
-static_assert(ARA_NOALLOC_SCRATCH_BYTES >= 2 * ARA_NOALLOC_MAX_RP * sizeof(double) + sizeof(ara::SelScratch) + 256,
-              "fixed block too small for the select state");
+static_assert(ARA_NOALLOC_SCRATCH_BYTES >= 2 * ARA_NOALLOC_MAX_RP * sizeof(double),
+              "fixed block too small for the outputs");
 
 }  // namespace
 
@@ -916,7 +687,6 @@ extern "C" ARA_API int ara_pml_tvar_noalloc(const double* ylt, int64_t n, const 
   }
   unsigned char* block = static_cast<unsigned char*>(g_noalloc_addr[dev]);
   double* d_out = reinterpret_cast<double*>(block);                      // 2 * ARA_NOALLOC_MAX_RP doubles
-  void* state = block + 2 * ARA_NOALLOC_MAX_RP * sizeof(double);          // select state (256-aligned)
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   // 0: host memory, 1: device (or managed) memory of this GPU, -1: another GPU's memory
   auto kind_of = [dev](const void* p) {
@@ -934,10 +704,8 @@ extern "C" ARA_API int ara_pml_tvar_noalloc(const double* ylt, int64_t n, const 
   const bool pml_dev = pml_kind == 1, tvar_dev = tvar_kind == 1;
   double* d_pml = pml_dev ? pml_out : d_out;
   double* d_tvar = tvar_dev ? tvar_out : d_out + ARA_NOALLOC_MAX_RP;
-  // the select kernels reset their own histogram and state on every call
-  if (ara::pml_tvar_device(ylt, n, return_periods, n_rp, d_pml, d_tvar, state, sizeof(ara::SelScratch), s, nullptr) !=
-      cudaSuccess)
-    return ARA_ECUDA;
+  const ara::SelectSpec spec{ylt, n, return_periods, n_rp, d_pml, d_tvar};
+  if (ara::pml_tvar_batch(&spec, 1, s, nullptr) != cudaSuccess) return ARA_ECUDA;
   if (!pml_dev && cudaMemcpyAsync(pml_out, d_pml, sizeof(double) * n_rp, cudaMemcpyDeviceToHost, s) != cudaSuccess)
     return ARA_ECUDA;
   if (!tvar_dev && cudaMemcpyAsync(tvar_out, d_tvar, sizeof(double) * n_rp, cudaMemcpyDeviceToHost, s) != cudaSuccess)
