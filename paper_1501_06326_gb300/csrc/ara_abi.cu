@@ -1993,9 +1993,14 @@ int ara_top_m(ara_ctx* c, const double* ylt, int64_t n, int64_t m, int64_t trial
     d_ylt = static_cast<const double*>(c->in_tmp.ptr);
   }
   const bool vals_dev = is_device_ptr(values_out), trials_dev = is_device_ptr(trials_out);
-  // scratch: the sort's, then the order of all n, then staged outputs for host arrays
-  const size_t sort_bytes = (ara::sort_scratch_bytes(n) + 255) & ~size_t(255);
-  const size_t order_bytes = (sizeof(int64_t) * static_cast<size_t>(n) + 255) & ~size_t(255);
+  // The m largest alone are collected and ordered where they are at most an eighth of a long YLT: a select,
+  // a collection and the sort of 20,000 take 163 us at 1M against 234 for the sort of all, but 143 against 123
+  // at 300,000.
+  const int64_t m_valid = std::min(m, n);
+  const bool collect = n >= (int64_t(1) << 19) && m_valid <= n / 8;
+  // scratch: the sort's, then the order, then staged outputs for host arrays
+  const size_t sort_bytes = ((collect ? ara::top_scratch_bytes(m_valid) : ara::sort_scratch_bytes(n)) + 255) & ~size_t(255);
+  const size_t order_bytes = (sizeof(int64_t) * static_cast<size_t>(collect ? m_valid : n) + 255) & ~size_t(255);
   const size_t stage_bytes = (vals_dev && trials_dev) ? 0 : 2 * sizeof(int64_t) * static_cast<size_t>(m);
   if ((rc = reserve(c, c->sel, sort_bytes + order_bytes + stage_bytes))) return rc;
   char* base = static_cast<char*>(c->sel.ptr);
@@ -2003,7 +2008,8 @@ int ara_top_m(ara_ctx* c, const double* ylt, int64_t n, int64_t m, int64_t trial
   double* d_vals = vals_dev ? values_out : reinterpret_cast<double*>(base + sort_bytes + order_bytes);
   int64_t* d_trials = trials_dev ? trials_out : reinterpret_cast<int64_t*>(base + sort_bytes + order_bytes) + m;
   int launched = 0;
-  ARA_CUDA(c, ara::sort_desc_device(d_ylt, n, d_order, c->sel.ptr, c->stream, &launched));
+  ARA_CUDA(c, collect ? ara::top_order_device(d_ylt, n, m_valid, d_order, c->sel.ptr, c->stream, &launched)
+                      : ara::sort_desc_device(d_ylt, n, d_order, c->sel.ptr, c->stream, &launched));
   ARA_CUDA(c, ara::top_gather_device(d_ylt, d_order, std::min(m, n), m, trial_offset, d_vals, d_trials, c->stream));
   c->launches += launched + 1;
   if (!vals_dev)

@@ -6,9 +6,8 @@
 // the m largest: the sum of the values whose key exceeds the m-th key plus the
 // tied remainder times the m-th value, in FP64 with a fixed assignment of
 // values to threads and a fixed reduction order (deterministic).  The full
-// trial order (largest first, ties by index) is an LSD radix sort of the
-// complemented keys with stable per-tile scatter (warp match + per-warp digit
-// offsets).
+// trial order (largest first, ties by index) is a stable LSD radix sort of the
+// complemented keys.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -65,7 +64,8 @@ struct SelJob {
   const double* ylt;
   int64_t n;
   double* pml;
-  double* tvar;
+  double* tvar;               // or NULL: no sums
+  unsigned long long* ties;   // or NULL: of the m-th value's ties, how many are among the m largest
   unsigned long long m[kSelGroup];
   int g;
 };
@@ -322,6 +322,11 @@ __global__ void __launch_bounds__(kSelThreads, 1) k_select(const __grid_constant
     }
     if (kCtas > 1) cluster.sync();  // ring shares hist's memory, which the other CTAs have read by now
   }
+  if (j.ties && rank == 0 && static_cast<int>(t) < j.g) j.ties[t] = sm.want[t];
+  if (!j.tvar) {
+    if (rank == 0 && static_cast<int>(t) < j.g) j.pml[t] = value_of(sm.prefix[t]);
+    return;  // (no CTA reads another's shared memory any more)
+  }
   // sums of the values above each period's key.  A warp collects the values above the lowest of the keys
   // and adds 32 at a time, as an FP64 add costs a whole warp's time however few lanes need it
   double sum[kSelGroup];
@@ -401,7 +406,7 @@ unsigned long long sel_rank(int64_t n, double rp) {
 }
 
 template <int kCtas>
-cudaError_t launch_select(const SelBatch& b, int n_jobs, cudaStream_t s) {
+cudaError_t launch_select_of(const SelBatch& b, int n_jobs, cudaStream_t s) {
   cudaError_t err;
   if ((err = cudaFuncSetAttribute(k_select<kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(SelShared))) !=
           cudaSuccess ||
@@ -422,6 +427,11 @@ cudaError_t launch_select(const SelBatch& b, int n_jobs, cudaStream_t s) {
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_select<kCtas>, b);
 }
+cudaError_t launch_select(const SelBatch& b, int n_jobs, int ctas, cudaStream_t s) {
+  return ctas == 1 ? launch_select_of<1>(b, n_jobs, s)
+         : ctas == 4 ? launch_select_of<4>(b, n_jobs, s)
+                     : launch_select_of<16>(b, n_jobs, s);
+}
 
 }  // namespace
 
@@ -434,9 +444,7 @@ cudaError_t pml_tvar_batch(const SelectSpec* specs, int n_specs, cudaStream_t s,
     int n_jobs = 0;
     auto flush = [&]() -> cudaError_t {
       if (n_jobs == 0) return cudaSuccess;
-      const cudaError_t e = ctas == 1   ? launch_select<1>(b, n_jobs, s)
-                            : ctas == 4 ? launch_select<4>(b, n_jobs, s)
-                                        : launch_select<16>(b, n_jobs, s);
+      const cudaError_t e = launch_select(b, n_jobs, ctas, s);
       if (n_launch) *n_launch += 1;
       n_jobs = 0;
       return e;
@@ -452,6 +460,7 @@ cudaError_t pml_tvar_batch(const SelectSpec* specs, int n_specs, cudaStream_t s,
         j.n = q.n;
         j.pml = q.pml + r0;
         j.tvar = q.tvar + r0;
+        j.ties = nullptr;
         j.g = (q.n_rp - r0 < kSelGroup) ? (q.n_rp - r0) : kSelGroup;
         for (int r = 0; r < kSelGroup; ++r) j.m[r] = r < j.g ? sel_rank(q.n, q.rps[r0 + r]) : 1ull;
       }
@@ -461,126 +470,343 @@ cudaError_t pml_tvar_batch(const SelectSpec* specs, int n_specs, cudaStream_t s,
   return cudaSuccess;
 }
 
-// =============================================================== LSD radix sort (descending)
+// =============================================================== LSD radix sort
+//
+// Eight bits a pass, stable.  The items are cut into at most kRxSegments
+// segments, one CTA each: k_radix_count counts a segment's digits, and
+// k_radix_scatter first sums the segments' counts to its own first places
+// (every CTA reads all of them: at most 152 KB, from L2, in place of a scan's
+// three launches a pass), then places its items a tile at a time.  An item's
+// rank among the tile's equal digits comes from eight ballots a warp (a warp
+// match is several times slower) and the warps' counts.  The 16 launches take
+// 96 us up to 100,000 year losses, about 6 us each by their latency, and 234 us
+// at 1M; with a scan over tiles of 1,024 they were 49 launches, 215 and 356 us.
+// Tiles of 2,048: with 4,096 a segment 115 us at 100,000 and no faster at 1M.
+// Up to kRxSmall year losses one CTA sorts in shared memory, in one launch: 21
+// us at 1,000 and 60 at 8,192, against 116.
 namespace {
 
-constexpr int kSortThreads = 1024;  // one key per thread per tile
+constexpr int kRxThreads = 512;
+constexpr int kRxWarps = kRxThreads / 32;
+constexpr int kRxItems = 4;
+constexpr int kRxTile = kRxThreads * kRxItems;
+constexpr int kRxSegments = 152;  // one CTA an SM
+constexpr int kRxSmallThreads = 1024;
+constexpr int kRxSmallItems = 8;
+constexpr int kRxSmall = kRxSmallThreads * kRxSmallItems;
 
-__global__ void k_sort_keys(const double* ylt, int64_t n, unsigned long long* keys, int64_t* idx) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) {
-    keys[i] = ~key_of(ylt[i]);  // ascending order of ~key = descending year loss
-    idx[i] = i;
-  }
+int radix_segments(int64_t n) {
+  const int64_t tiles = (n + kRxTile - 1) / kRxTile;
+  return static_cast<int>(tiles < 1 ? 1 : tiles < kRxSegments ? tiles : kRxSegments);
+}
+// segment s of n_seg: whole tiles
+__host__ __device__ __forceinline__ int64_t radix_bound(int64_t n, int n_seg, int s) {
+  const int64_t tiles = (n + kRxTile - 1) / kRxTile;
+  const int64_t at = tiles * s / n_seg * kRxTile;
+  return at < n ? at : n;
 }
 
-__global__ void k_sort_count(const unsigned long long* keys, int64_t n, int shift, unsigned int* counts,
-                             int n_tiles) {
+// The items of a pass: the keys and values of the pass before, or (kYlt) a
+// YLT's keys, complemented so that ascending keys are descending losses, and
+// their trial indices.
+template <bool kYlt>
+__device__ __forceinline__ unsigned long long radix_key(const double* ylt, const unsigned long long* keys, int64_t i) {
+  if constexpr (kYlt) return ~key_of(ylt[i]);
+  else return keys[i];
+}
+
+template <bool kYlt>
+__global__ void __launch_bounds__(kRxThreads) k_radix_count(const double* ylt, const unsigned long long* keys,
+                                                            int64_t n, int shift, unsigned int* counts) {
   __shared__ unsigned int sh[256];
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) sh[i] = 0;
+  for (int i = threadIdx.x; i < 256; i += kRxThreads) sh[i] = 0u;
   __syncthreads();
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * kSortThreads + threadIdx.x;
-  if (i < n) atomicAdd(&sh[(keys[i] >> shift) & 255u], 1u);
+  const int64_t end = radix_bound(n, gridDim.x, blockIdx.x + 1);
+#pragma unroll 4
+  for (int64_t i = radix_bound(n, gridDim.x, blockIdx.x) + threadIdx.x; i < end; i += kRxThreads)
+    atomicAdd(&sh[(radix_key<kYlt>(ylt, keys, i) >> shift) & 255u], 1u);
   __syncthreads();
-  for (int d = threadIdx.x; d < 256; d += blockDim.x) counts[static_cast<int64_t>(d) * n_tiles + blockIdx.x] = sh[d];
+  if (threadIdx.x < 256) counts[blockIdx.x * 256 + threadIdx.x] = sh[threadIdx.x];
 }
 
-__global__ void k_sort_scatter(const unsigned long long* keys_in, const int64_t* idx_in, int64_t n, int shift,
-                               const unsigned int* offsets, int n_tiles, unsigned long long* keys_out,
-                               int64_t* idx_out) {
-  __shared__ unsigned int s_wc[32][256];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < 32 * 256; i += blockDim.x) (&s_wc[0][0])[i] = 0;
-  __syncthreads();
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * kSortThreads + threadIdx.x;
-  const bool valid = i < n;
-  const unsigned long long key = valid ? keys_in[i] : 0ull;
-  const unsigned int d = valid ? static_cast<unsigned int>((key >> shift) & 255u) : 256u;
-  const unsigned int peers = __match_any_sync(0xffffffffu, d);
-  const unsigned int rank = __popc(peers & ((1u << lane) - 1u));
-  if (valid && rank == 0) s_wc[warp][d] = __popc(peers);
-  __syncthreads();
-  if (threadIdx.x < 256) {
-    const int dd = threadIdx.x;
-    unsigned int run = offsets[static_cast<int64_t>(dd) * n_tiles + blockIdx.x];
-    for (int w = 0; w < 32; ++w) {
-      const unsigned int c = s_wc[w][dd];
-      s_wc[w][dd] = run;
-      run += c;
+// The lanes whose digit is this lane's, among the valid ones.
+__device__ __forceinline__ unsigned int radix_peers(unsigned int d, bool valid) {
+  unsigned int peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const unsigned int b = __ballot_sync(0xffffffffu, (d >> k) & 1u);
+    peers &= ((d >> k) & 1u) ? b : ~b;
+  }
+  return peers;
+}
+
+template <bool kYlt, class V, class VOut>
+__global__ void __launch_bounds__(kRxThreads) k_radix_scatter(const double* ylt, const unsigned long long* keys,
+                                                              const V* vals, int64_t n, int shift,
+                                                              const unsigned int* counts,
+                                                              unsigned long long* keys_out, VOut* vals_out) {
+  __shared__ unsigned int wc[kRxWarps][256];  // per warp: a digit's count in the tile, then the place of its items
+  __shared__ unsigned int base[256];          // the segment's next place of each digit
+  __shared__ unsigned int part[2][kRxThreads];
+  __shared__ unsigned int warp_sum[8];
+  const unsigned int t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+  {
+    // the segments before this one and all segments, a digit a thread over a part of the segments
+    constexpr unsigned int kParts = kRxThreads / 256;
+    const unsigned int d = t & 255u;
+    unsigned int before = 0u, total = 0u;
+#pragma unroll 8
+    for (unsigned int s = t >> 8; s < gridDim.x; s += kParts) {
+      const unsigned int c = counts[s * 256 + d];
+      total += c;
+      before += s < blockIdx.x ? c : 0u;
+    }
+    part[0][t] = before;
+    part[1][t] = total;
+    __syncthreads();
+    unsigned int incl = 0u;
+    if (t < 256u) {
+#pragma unroll
+      for (unsigned int q = 1; q < kParts; ++q) {
+        before += part[0][q * 256 + t];
+        total += part[1][q * 256 + t];
+      }
+      incl = total;
+#pragma unroll
+      for (int dd = 1; dd < 32; dd <<= 1) {
+        const unsigned int o = __shfl_up_sync(0xffffffffu, incl, dd);
+        if (lane >= static_cast<unsigned int>(dd)) incl += o;
+      }
+      if (lane == 31u) warp_sum[warp] = incl;
+    }
+    __syncthreads();
+    if (t < 256u) {
+      unsigned int at = incl - total + before;
+      for (unsigned int w = 0; w < warp; ++w) at += warp_sum[w];
+      base[t] = at;
     }
   }
-  __syncthreads();
-  if (valid) {
-    const unsigned int dst = s_wc[warp][d] + rank;
-    keys_out[dst] = key;
-    idx_out[dst] = idx_in[i];
+  const int64_t end = radix_bound(n, gridDim.x, blockIdx.x + 1);
+  for (int64_t tile = radix_bound(n, gridDim.x, blockIdx.x); tile < end; tile += kRxTile) {
+    __syncthreads();  // the tile before is placed (and base is there)
+    for (int i = lane; i < 256; i += 32) wc[warp][i] = 0u;
+    __syncwarp();
+    unsigned long long key[kRxItems];
+    V val[kRxItems];
+    unsigned int at[kRxItems];
+#pragma unroll
+    for (int j = 0; j < kRxItems; ++j) {
+      const int64_t i = tile + warp * (32 * kRxItems) + 32 * j + lane;
+      key[j] = i < end ? radix_key<kYlt>(ylt, keys, i) : 0ull;
+      if constexpr (kYlt) val[j] = static_cast<V>(i);
+      else val[j] = i < end ? vals[i] : V{};
+    }
+#pragma unroll
+    for (int j = 0; j < kRxItems; ++j) {
+      const bool valid = tile + warp * (32 * kRxItems) + 32 * j + lane < end;
+      const unsigned int d = static_cast<unsigned int>(key[j] >> shift) & 255u;
+      const unsigned int peers = radix_peers(d, valid);
+      const unsigned int below = __popc(peers & ((1u << lane) - 1u));
+      const unsigned int have = wc[warp][d];
+      __syncwarp();
+      if (valid && below == 0u) wc[warp][d] = have + __popc(peers);
+      __syncwarp();
+      at[j] = have + below;
+    }
+    __syncthreads();
+    if (t < 256u) {
+      unsigned int run = base[t];
+#pragma unroll
+      for (int w = 0; w < kRxWarps; ++w) {
+        const unsigned int c = wc[w][t];
+        wc[w][t] = run;
+        run += c;
+      }
+      base[t] = run;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kRxItems; ++j)
+      if (tile + warp * (32 * kRxItems) + 32 * j + lane < end) {
+        const unsigned int dst = at[j] + wc[warp][(key[j] >> shift) & 255u];
+        if (keys_out) keys_out[dst] = key[j];
+        vals_out[dst] = static_cast<VOut>(val[j]);
+      }
   }
+}
+
+struct RxSmall {
+  unsigned long long key[kRxSmall];
+  uint32_t val[kRxSmall];
+  unsigned int wc[kRxSmallThreads / 32][256];
+  unsigned int first[256];
+  unsigned int warp_sum[8];
+};
+
+// The order of at most kRxSmall items, all passes in one CTA.
+template <bool kYlt>
+__global__ void __launch_bounds__(kRxSmallThreads, 1) k_radix_small(const double* ylt,
+                                                                        const unsigned long long* keys,
+                                                                        const uint32_t* vals, int n, int64_t* order) {
+  extern __shared__ __align__(16) unsigned char rx_smem[];
+  RxSmall& sm = *reinterpret_cast<RxSmall*>(rx_smem);
+  const unsigned int t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+  // the warps that hold items; a warp's items are contiguous
+  const int per_warp = 32 * kRxSmallItems, i0 = static_cast<int>(warp) * per_warp + static_cast<int>(lane);
+  const unsigned int n_warps = static_cast<unsigned int>((n + per_warp - 1) / per_warp);
+  unsigned long long key[kRxSmallItems];
+  uint32_t val[kRxSmallItems];
+#pragma unroll
+  for (int j = 0; j < kRxSmallItems; ++j) {
+    key[j] = i0 + 32 * j < n ? radix_key<kYlt>(ylt, keys, i0 + 32 * j) : 0ull;
+    val[j] = kYlt ? static_cast<uint32_t>(i0 + 32 * j) : i0 + 32 * j < n ? vals[i0 + 32 * j] : 0u;
+  }
+#pragma unroll 1
+  for (int shift = 0; shift < 64; shift += 8) {
+    unsigned int at[kRxSmallItems];
+    for (int i = lane; i < 256; i += 32) sm.wc[warp][i] = 0u;
+    __syncwarp();
+    if (warp < n_warps) {
+#pragma unroll
+      for (int j = 0; j < kRxSmallItems; ++j) {
+        const bool valid = i0 + 32 * j < n;
+        const unsigned int d = static_cast<unsigned int>(key[j] >> shift) & 255u;
+        const unsigned int peers = radix_peers(d, valid);
+        const unsigned int below = __popc(peers & ((1u << lane) - 1u));
+        const unsigned int have = sm.wc[warp][d];
+        __syncwarp();
+        if (valid && below == 0u) sm.wc[warp][d] = have + __popc(peers);
+        __syncwarp();
+        at[j] = have + below;
+      }
+    }
+    __syncthreads();
+    unsigned int total = 0u, incl = 0u;
+    if (t < 256u) {
+#pragma unroll 8
+      for (unsigned int w = 0; w < kRxSmallThreads / 32; ++w) {
+        const unsigned int c = sm.wc[w][t];
+        sm.wc[w][t] = total;
+        total += c;
+      }
+      incl = total;
+#pragma unroll
+      for (int dd = 1; dd < 32; dd <<= 1) {
+        const unsigned int o = __shfl_up_sync(0xffffffffu, incl, dd);
+        if (lane >= static_cast<unsigned int>(dd)) incl += o;
+      }
+      if (lane == 31u) sm.warp_sum[warp] = incl;
+    }
+    __syncthreads();
+    if (t < 256u) {
+      unsigned int first = incl - total;
+      for (unsigned int w = 0; w < warp; ++w) first += sm.warp_sum[w];
+      sm.first[t] = first;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kRxSmallItems; ++j)
+      if (i0 + 32 * j < n) {
+        const unsigned int d = static_cast<unsigned int>(key[j] >> shift) & 255u;
+        const unsigned int dst = at[j] + sm.wc[warp][d] + sm.first[d];
+        sm.key[dst] = key[j];
+        sm.val[dst] = val[j];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kRxSmallItems; ++j)
+      if (i0 + 32 * j < n) {
+        key[j] = sm.key[i0 + 32 * j];
+        val[j] = sm.val[i0 + 32 * j];
+      }
+  }
+#pragma unroll
+  for (int j = 0; j < kRxSmallItems; ++j)
+    if (i0 + 32 * j < n) order[i0 + 32 * j] = static_cast<int64_t>(val[j]);
 }
 
 }  // namespace
 
-size_t sort_scratch_bytes(int64_t n) {
-  const int64_t tiles = (n + kSortThreads - 1) / kSortThreads;
-  const int64_t cnt = 256 * tiles;
-  return static_cast<size_t>(n) * (2 * sizeof(unsigned long long) + sizeof(int64_t)) +
-         sizeof(unsigned int) * (2 * static_cast<size_t>(cnt) + 1 + scan_tmp_words(cnt)) + 256;
+namespace {
+
+// scratch of the passes: two key and two index arrays, then the segments' digit counts
+struct RxScratch {
+  unsigned long long* keys[2];
+  uint32_t* vals[2];
+  unsigned int* counts;
+};
+size_t radix_scratch_bytes(int64_t n) {
+  return static_cast<size_t>(n) * 2 * (sizeof(unsigned long long) + sizeof(uint32_t)) +
+         sizeof(unsigned int) * 256 * static_cast<size_t>(radix_segments(n)) + 256;
 }
+RxScratch radix_scratch(void* scratch, int64_t n) {
+  RxScratch x;
+  x.keys[0] = static_cast<unsigned long long*>(scratch);
+  x.keys[1] = x.keys[0] + n;
+  x.vals[0] = reinterpret_cast<uint32_t*>(x.keys[1] + n);
+  x.vals[1] = x.vals[0] + n;
+  x.counts = reinterpret_cast<unsigned int*>(x.vals[1] + n);
+  return x;
+}
+
+// The indices in ascending key order: of a YLT (kYlt), or of n (key, index)
+// pairs in x.keys[1] and x.vals[1].
+template <bool kYlt>
+cudaError_t radix_order(const double* ylt, const RxScratch& x, int64_t n, int64_t* order, cudaStream_t s,
+                        int* n_launch) {
+  cudaError_t err;
+  if (n <= kRxSmall) {
+    if ((err = cudaFuncSetAttribute(k_radix_small<kYlt>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    sizeof(RxSmall))) != cudaSuccess)
+      return err;
+    k_radix_small<kYlt><<<1, kRxSmallThreads, sizeof(RxSmall), s>>>(ylt, x.keys[1], x.vals[1], static_cast<int>(n),
+                                                                   order);
+    if (n_launch) *n_launch += 1;
+    return cudaGetLastError();
+  }
+  const int n_seg = radix_segments(n);
+  for (int pass = 0; pass < 8; ++pass) {
+    const int shift = 8 * pass, from = (pass + 1) & 1, to = pass & 1;
+    if (kYlt && pass == 0) {
+      k_radix_count<true><<<n_seg, kRxThreads, 0, s>>>(ylt, nullptr, n, shift, x.counts);
+      k_radix_scatter<true, uint32_t, uint32_t><<<n_seg, kRxThreads, 0, s>>>(ylt, nullptr, nullptr, n, shift, x.counts,
+                                                                            x.keys[to], x.vals[to]);
+    } else {
+      k_radix_count<false><<<n_seg, kRxThreads, 0, s>>>(nullptr, x.keys[from], n, shift, x.counts);
+      if (pass < 7)
+        k_radix_scatter<false, uint32_t, uint32_t><<<n_seg, kRxThreads, 0, s>>>(
+            nullptr, x.keys[from], x.vals[from], n, shift, x.counts, x.keys[to], x.vals[to]);
+      else
+        k_radix_scatter<false, uint32_t, int64_t><<<n_seg, kRxThreads, 0, s>>>(
+            nullptr, x.keys[from], x.vals[from], n, shift, x.counts, nullptr, order);
+    }
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  }
+  if (n_launch) *n_launch += 16;
+  return cudaSuccess;
+}
+
+}  // namespace
+
+size_t sort_scratch_bytes(int64_t n) { return radix_scratch_bytes(n); }
 
 cudaError_t sort_desc_device(const double* ylt, int64_t n, int64_t* order, void* scratch, cudaStream_t s,
                              int* n_launch) {
-  const int64_t tiles = (n + kSortThreads - 1) / kSortThreads;
-  const int64_t cnt = 256 * tiles;
-  unsigned char* base = static_cast<unsigned char*>(scratch);
-  unsigned long long* keys_a = reinterpret_cast<unsigned long long*>(base);
-  unsigned long long* keys_b = keys_a + n;
-  int64_t* idx_b = reinterpret_cast<int64_t*>(keys_b + n);
-  unsigned int* counts = reinterpret_cast<unsigned int*>(idx_b + n);
-  unsigned int* offsets = counts + cnt;
-  unsigned int* tmp = offsets + cnt + 1;
-  // the final pass must land in `order`; with 8 passes the ping-pong ends where it started
-  int64_t* idx_a = order;
-  const int grid = static_cast<int>((n + 255) / 256 < 65535 ? (n + 255) / 256 : 65535);
-  k_sort_keys<<<grid, 256, 0, s>>>(ylt, n, keys_a, idx_a);
-  if (n_launch) *n_launch += 1 + 8 * 2;
-  cudaError_t err = cudaGetLastError();
-  if (err != cudaSuccess) return err;
-  unsigned long long *ki = keys_a, *ko = keys_b;
-  int64_t *ii = idx_a, *io = idx_b;
-  for (int shift = 0; shift < 64; shift += 8) {
-    k_sort_count<<<static_cast<int>(tiles), kSortThreads, 0, s>>>(ki, n, shift, counts, static_cast<int>(tiles));
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    if ((err = scan_exclusive_u32(counts, offsets, cnt, tmp, s, n_launch)) != cudaSuccess) return err;
-    k_sort_scatter<<<static_cast<int>(tiles), kSortThreads, 0, s>>>(ki, ii, n, shift, offsets,
-                                                                   static_cast<int>(tiles), ko, io);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    unsigned long long* tk = ki;
-    ki = ko;
-    ko = tk;
-    int64_t* ti = ii;
-    ii = io;
-    io = ti;
-  }
-  return cudaSuccess;  // 8 swaps: the result is back in idx_a == order
+  return radix_order<true>(ylt, radix_scratch(scratch, n), n, order, s, n_launch);
 }
 
 size_t sort_pairs_scratch_bytes(int64_t n) {
-  const int64_t tiles = (n + kSortThreads - 1) / kSortThreads;
-  const int64_t cnt = 256 * tiles;
   return static_cast<size_t>(n) * (sizeof(unsigned long long) + sizeof(int64_t)) +
-         sizeof(unsigned int) * (2 * static_cast<size_t>(cnt) + 1 + scan_tmp_words(cnt)) + 256;
+         sizeof(unsigned int) * 256 * static_cast<size_t>(radix_segments(n)) + 256;
 }
 
 cudaError_t sort_pairs_ascending(unsigned long long* keys, int64_t* vals, int64_t n, int key_bits, void* scratch,
                                  cudaStream_t s, int* n_launch) {
-  const int64_t tiles = (n + kSortThreads - 1) / kSortThreads;
-  const int64_t cnt = 256 * tiles;
   const int passes = (key_bits + 7) / 8;
-  unsigned char* base = static_cast<unsigned char*>(scratch);
-  unsigned long long* keys_b = reinterpret_cast<unsigned long long*>(base);
+  const int n_seg = radix_segments(n);
+  unsigned long long* keys_b = static_cast<unsigned long long*>(scratch);
   int64_t* vals_b = reinterpret_cast<int64_t*>(keys_b + n);
   unsigned int* counts = reinterpret_cast<unsigned int*>(vals_b + n);
-  unsigned int* offsets = counts + cnt;
-  unsigned int* tmp = offsets + cnt + 1;
   cudaError_t err = cudaSuccess;
   // an odd number of passes ends in the scratch buffers: the data start there, so the result
   // lands in (keys, vals)
@@ -596,12 +822,9 @@ cudaError_t sort_pairs_ascending(unsigned long long* keys, int64_t* vals, int64_
     io = vals;
   }
   for (int pass = 0; pass < passes; ++pass) {
-    const int shift = 8 * pass;
-    k_sort_count<<<static_cast<int>(tiles), kSortThreads, 0, s>>>(ki, n, shift, counts, static_cast<int>(tiles));
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    if ((err = scan_exclusive_u32(counts, offsets, cnt, tmp, s, n_launch)) != cudaSuccess) return err;
-    k_sort_scatter<<<static_cast<int>(tiles), kSortThreads, 0, s>>>(ki, ii, n, shift, offsets,
-                                                                   static_cast<int>(tiles), ko, io);
+    k_radix_count<false><<<n_seg, kRxThreads, 0, s>>>(nullptr, ki, n, 8 * pass, counts);
+    k_radix_scatter<false, int64_t, int64_t><<<n_seg, kRxThreads, 0, s>>>(nullptr, ki, ii, n, 8 * pass, counts, ko,
+                                                                         io);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     std::swap(ki, ko);
     std::swap(ii, io);
@@ -630,6 +853,85 @@ __global__ void k_top_gather(const double* ylt, const int64_t* order, int64_t m_
   }
 }
 
+// The m largest without the whole order: the m-th key comes from k_select, and
+// these kernels collect, in trial order, the values above it and the first of
+// its ties (as many as the m largest hold).  Segment s of the YLT is a CTA's;
+// counts[2 s] and [2 s + 1]: its values above the m-th key and its ties.
+constexpr int kTopThreads = 1024;
+constexpr int kTopSegments = 152;
+
+struct TopKth {
+  double value;            // the m-th largest value
+  unsigned long long ties;  // of its ties, how many are among the m largest
+};
+
+__global__ void __launch_bounds__(kTopThreads) k_top_count(const double* ylt, int64_t n, const TopKth* kth,
+                                                           unsigned int* counts) {
+  __shared__ unsigned int s_above, s_ties;
+  if (threadIdx.x == 0) s_above = s_ties = 0u;
+  __syncthreads();
+  const unsigned long long k = key_of(kth->value);
+  const int64_t begin = n * blockIdx.x / gridDim.x, end = n * (blockIdx.x + 1) / gridDim.x;
+  unsigned int above = 0u, ties = 0u;
+#pragma unroll 4
+  for (int64_t i = begin + threadIdx.x; i < end; i += kTopThreads) {
+    const unsigned long long x = key_of(ylt[i]);
+    above += x > k;
+    ties += x == k;
+  }
+  above = __reduce_add_sync(0xffffffffu, above);
+  ties = __reduce_add_sync(0xffffffffu, ties);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&s_above, above);
+    atomicAdd(&s_ties, ties);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    counts[2 * blockIdx.x] = s_above;
+    counts[2 * blockIdx.x + 1] = s_ties;
+  }
+}
+
+__global__ void __launch_bounds__(kTopThreads) k_top_collect(const double* ylt, int64_t n, const TopKth* kth,
+                                                             const unsigned int* counts, unsigned long long* keys,
+                                                             uint32_t* idx) {
+  __shared__ unsigned int w_above[kTopThreads / 32], w_ties[kTopThreads / 32];
+  const unsigned int t = threadIdx.x, lane = t & 31u, warp = t >> 5, lt = (1u << lane) - 1u;
+  const unsigned long long k = key_of(kth->value), most = kth->ties;
+  // the items before this segment
+  unsigned long long above = 0ull, ties = 0ull;
+  for (unsigned int s = 0; s < blockIdx.x; ++s) {
+    above += counts[2 * s];
+    ties += counts[2 * s + 1];
+  }
+  const int64_t begin = n * blockIdx.x / gridDim.x, end = n * (blockIdx.x + 1) / gridDim.x;
+  for (int64_t i0 = begin; i0 < end; i0 += kTopThreads) {
+    const int64_t i = i0 + t;
+    const unsigned long long x = i < end ? key_of(ylt[i]) : 0ull;
+    const unsigned int a = __ballot_sync(0xffffffffu, i < end && x > k), e = __ballot_sync(0xffffffffu, i < end && x == k);
+    if (lane == 0) {
+      w_above[warp] = __popc(a);
+      w_ties[warp] = __popc(e);
+    }
+    __syncthreads();
+    unsigned int pa = lane < warp ? w_above[lane] : 0u, pe = lane < warp ? w_ties[lane] : 0u;
+    unsigned int ta = w_above[lane], te = w_ties[lane];
+    pa = __reduce_add_sync(0xffffffffu, pa);
+    pe = __reduce_add_sync(0xffffffffu, pe);
+    ta = __reduce_add_sync(0xffffffffu, ta);
+    te = __reduce_add_sync(0xffffffffu, te);
+    const unsigned long long my_ties = ties + pe + __popc(e & lt);  // ties before this item
+    const unsigned long long at = above + pa + __popc(a & lt) + (my_ties < most ? my_ties : most);
+    if (i < end && (x > k || (x == k && my_ties < most))) {
+      keys[at] = ~x;
+      idx[at] = static_cast<uint32_t>(i);
+    }
+    above += ta;
+    ties += te;
+    __syncthreads();
+  }
+}
+
 }  // namespace
 
 cudaError_t top_gather_device(const double* ylt, const int64_t* order, int64_t m_valid, int64_t m, int64_t trial_offset,
@@ -638,6 +940,32 @@ cudaError_t top_gather_device(const double* ylt, const int64_t* order, int64_t m
   k_top_gather<<<static_cast<int>(blocks < 1024 ? (blocks > 0 ? blocks : 1) : 1024), 256, 0, s>>>(
       ylt, order, m_valid, m, trial_offset, vals, trials);
   return cudaGetLastError();
+}
+
+size_t top_scratch_bytes(int64_t m) { return radix_scratch_bytes(m) + 2 * sizeof(unsigned int) * kTopSegments + 512; }
+
+cudaError_t top_order_device(const double* ylt, int64_t n, int64_t m, int64_t* order, void* scratch, cudaStream_t s,
+                             int* n_launch) {
+  unsigned char* base = static_cast<unsigned char*>(scratch);
+  TopKth* kth = reinterpret_cast<TopKth*>(base);
+  unsigned int* counts = reinterpret_cast<unsigned int*>(base + 256);
+  const RxScratch x = radix_scratch(base + 256 + ((2 * sizeof(unsigned int) * kTopSegments + 255) & ~size_t(255)), m);
+  SelBatch b;
+  SelJob& j = b.job[0];
+  j.ylt = ylt;
+  j.n = n;
+  j.pml = &kth->value;
+  j.tvar = nullptr;
+  j.ties = &kth->ties;
+  j.g = 1;
+  for (int r = 0; r < kSelGroup; ++r) j.m[r] = r == 0 ? static_cast<unsigned long long>(m) : 1ull;
+  cudaError_t err = launch_select(b, 1, sel_ctas(n), s);
+  if (err != cudaSuccess) return err;
+  k_top_count<<<kTopSegments, kTopThreads, 0, s>>>(ylt, n, kth, counts);
+  k_top_collect<<<kTopSegments, kTopThreads, 0, s>>>(ylt, n, kth, counts, x.keys[1], x.vals[1]);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  if (n_launch) *n_launch += 3;
+  return radix_order<false>(nullptr, x, m, order, s, n_launch);
 }
 
 }  // namespace ara

@@ -340,6 +340,31 @@ def test_pml_tvar_and_sort(eng, n):
     assert np.array_equal(order, np.lexsort((np.arange(n), -y)))
 
 
+@pytest.mark.parametrize("n", [2, 31, 4096, 8191, 8192, 8193, 65_536, 65_537, 1_245_185])
+@pytest.mark.parametrize("values", ["spread", "tied", "one"])
+def test_select_and_sort_edges(eng, n, values):
+    """The select's and the sort's edges: lengths around one thread-block
+    cluster's size classes, the shared-memory sort's capacity and the sort's
+    segments; year losses all distinct (negative ones among them), nearly all
+    tied at a limit (more ties than a CTA collects), and all equal; more return
+    periods than one group of four.  PML and the order exact, TVaR a sum of
+    the same values in another order."""
+    rng = np.random.default_rng(n)
+    y = rng.normal(0.0, 1e6, n) if values == "spread" else np.full(n, 7.5e7)
+    if values == "tied":
+        some = rng.random(n) < 0.1
+        y[some] = rng.lognormal(17.0, 1.0, int(some.sum())).clip(0.0, 7.5e7)
+    rps = np.array([1.0, 1.5, 7.0, 10.0, 100.0, 250.0, 1e3, 1e4, 1e9])
+    pml, tvar = eng.pml_tvar(y, rps)
+    rpml, rtvar = oracle.pml_tvar(y, rps)
+    assert np.array_equal(pml, rpml)
+    assert np.allclose(tvar, rtvar, rtol=1e-12, atol=1e-12 * float(np.abs(y).sum()))
+    order = np.lexsort((np.arange(n), -y))
+    assert np.array_equal(eng.sort_ylt(y), order)
+    vals, trials = eng.top_m(y, min(n, 5_000), 3)
+    assert np.array_equal(trials, order[: min(n, 5_000)] + 3) and np.array_equal(vals, y[order[: min(n, 5_000)]])
+
+
 @pytest.mark.parametrize("n,m", [(1, 3), (999, 10), (100_000, 1000), (100_000, 100_007)])
 def test_top_m_against_a_host_sort(eng, n, m):
     """ara_top_m: the m largest year losses, descending, ties by trial index, with
