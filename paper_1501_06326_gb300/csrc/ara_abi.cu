@@ -6,6 +6,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <deque>
@@ -17,6 +18,10 @@
 #include "ara_batch.h"
 
 namespace {
+
+// Records of an ELT load from which their tables are built in order of their shapes (the order takes about
+// 30 us; a load of fewer is one wave of blocks).
+constexpr int64_t kShapeOrderMin = 4096;
 
 // The YET index keeps each event's occurrence offsets at every 2^kYetGridShift trials (the serving
 // chunk: 262,144 trials measured better than 131,072 on the serving workload, p99 18.6 against 35.8 ms
@@ -124,7 +129,6 @@ struct ara_ctx {
   DevBuf elt_stage, elt_recs_stage, elt_tab_stage, elt_flags;  // ELT load staging (grow-only)
   DevBuf elt_tabf_stage, elt_work;
   // misc scratch
-  DevBuf flags;     // uint32 flags + int32 max event
   DevBuf counters;  // 4 x u64
   DevBuf ylt_tmp;   // device YLT when the caller's output is on the host
   DevBuf diag_tmp;  // device diagnostics when the caller's outputs are on the host
@@ -395,7 +399,7 @@ int ara_create(ara_ctx** out, int device, size_t hbm_budget_bytes, void* cuda_st
       return ARA_ECUDA;
     }
   }
-  if (reserve(c, c->flags, 64) != ARA_OK || reserve(c, c->counters, 64) != ARA_OK) {
+  if (reserve(c, c->counters, 64) != ARA_OK) {
     ara_destroy(c);
     return ARA_ENOMEM;
   }
@@ -568,11 +572,14 @@ static int load_elts_impl(ara_ctx* c, const char* who, int32_t n_elts, const int
   if (R > 0 && (!event_ids || !mean || !sigma || !exposure))
     return fail(c, ARA_EINVAL, "%s: record arrays are NULL", who);
   // ---- stage: inputs, prepared records and tables of all ELTs (grow-only context buffers)
-  std::vector<int64_t> fine_off(static_cast<size_t>(n_elts) + 1, 0), work_off(static_cast<size_t>(n_elts) + 1, 0);
+  std::vector<int64_t> fine_off(static_cast<size_t>(n_elts) + 1, 0);
+  std::vector<ara::FineJob> jobs;
+  int64_t longest = 0;
   for (int32_t i = 0; i < n_elts; ++i) {
     const int64_t n = offs[i + 1] - offs[i];
     fine_off[i + 1] = fine_off[i] + ara::fine_table_cap(n);
-    work_off[i + 1] = work_off[i] + static_cast<int64_t>(ara::build_tables_work_words(n));
+    longest = std::max(longest, n);
+    if (n > 0) jobs.push_back(ara::FineJob{offs[i], n, fine_off[i], ara::fine_table_cap(n), i});
   }
   const size_t in_bytes =
       static_cast<size_t>(R) * (sizeof(int32_t) + 4 * sizeof(float) + sizeof(ara::BetaShape) + sizeof(float2)) + 64;
@@ -580,9 +587,10 @@ static int load_elts_impl(ara_ctx* c, const char* who, int32_t n_elts, const int
       (rc = reserve(c, c->elt_recs_stage, sizeof(ara::Pair) * (R + 1))) ||
       (rc = reserve(c, c->elt_tab_stage, sizeof(float4) * ara::kTabNodes * (R + 1))) ||
       (rc = reserve(c, c->elt_tabf_stage, sizeof(float4) * ara::kTabFineStride * (fine_off[n_elts] + 1))) ||
-      (rc = reserve(c, c->elt_work, sizeof(uint32_t) * (work_off[n_elts] + R + 8) +
-                                        sizeof(ara::FineJob) * static_cast<size_t>(n_elts))) ||
-      (rc = reserve(c, c->elt_flags, sizeof(uint32_t) * 4 * n_elts)))
+      (rc = reserve(c, c->elt_work, sizeof(uint32_t) * ara::build_tables_work_words(R))) ||
+      (rc = reserve(c, c->elt_flags, sizeof(int64_t) * (static_cast<size_t>(n_elts) + 1) +
+                                         (sizeof(ara::FineJob) + sizeof(uint32_t) * ara::kEltWords) *
+                                             static_cast<size_t>(n_elts))))
     return rc;
   int32_t* d_ev = static_cast<int32_t*>(c->elt_stage.ptr);
   float* d_mu = reinterpret_cast<float*>(d_ev + R);
@@ -596,8 +604,19 @@ static int load_elts_impl(ara_ctx* c, const char* who, int32_t n_elts, const int
   float4* d_tab = static_cast<float4*>(c->elt_tab_stage.ptr);
   float4* d_tabf = static_cast<float4*>(c->elt_tabf_stage.ptr);
   uint32_t* d_work = static_cast<uint32_t*>(c->elt_work.ptr);
-  uint32_t* d_need = d_work + work_off[n_elts];  // [R] fine-table candidates, all ELTs
-  uint32_t* d_flags = static_cast<uint32_t*>(c->elt_flags.ptr);
+  // the load's parameters in one block: record offsets, fine-table jobs, the ELTs' words
+  std::vector<unsigned char> param(sizeof(int64_t) * offs.size() + sizeof(ara::FineJob) * jobs.size() +
+                                   sizeof(uint32_t) * ara::kEltWords * static_cast<size_t>(n_elts));
+  unsigned char* h_param = param.data();
+  std::memcpy(h_param, offs.data(), sizeof(int64_t) * offs.size());
+  const size_t jobs_at = sizeof(int64_t) * offs.size(), words_at = jobs_at + sizeof(ara::FineJob) * jobs.size();
+  if (!jobs.empty()) std::memcpy(h_param + jobs_at, jobs.data(), sizeof(ara::FineJob) * jobs.size());
+  for (int32_t i = 0; i < n_elts; ++i)
+    std::memcpy(h_param + words_at + sizeof ara::kEltInit * i, ara::kEltInit, sizeof ara::kEltInit);
+  unsigned char* d_param = static_cast<unsigned char*>(c->elt_flags.ptr);
+  const int64_t* d_offs = reinterpret_cast<const int64_t*>(d_param);
+  const ara::FineJob* d_jobs = reinterpret_cast<const ara::FineJob*>(d_param + jobs_at);
+  uint32_t* d_flags = reinterpret_cast<uint32_t*>(d_param + words_at);
   if (R > 0) {
     ARA_CUDA(c, cudaMemcpyAsync(d_ev, event_ids, sizeof(int32_t) * R, kind_to_device(event_ids), c->stream));
     ARA_CUDA(c, cudaMemcpyAsync(d_mu, mean, sizeof(float) * R, kind_to_device(mean), c->stream));
@@ -605,48 +624,18 @@ static int load_elts_impl(ara_ctx* c, const char* who, int32_t n_elts, const int
     ARA_CUDA(c, cudaMemcpyAsync(d_ex, exposure, sizeof(float) * R, kind_to_device(exposure), c->stream));
     if (sigma_c) ARA_CUDA(c, cudaMemcpyAsync(d_sc, sigma_c, sizeof(float) * R, kind_to_device(sigma_c), c->stream));
   }
-  // per ELT: flags word, the largest event id (0xFFFFFFFF = none), candidates for fine
-  // tables, the largest loss (FP32 bits)
-  std::vector<uint32_t> init(4 * static_cast<size_t>(n_elts));
-  for (int32_t i = 0; i < n_elts; ++i) {
-    init[4 * i] = 0u;
-    init[4 * i + 1] = 0xFFFFFFFFu;
-    init[4 * i + 2] = 0u;
-    init[4 * i + 3] = 0u;
-  }
-  ARA_CUDA(c, cudaMemcpyAsync(d_flags, init.data(), sizeof(uint32_t) * init.size(), cudaMemcpyHostToDevice, c->stream));
-  for (int32_t i = 0; i < n_elts; ++i) {
-    const int64_t o = offs[i], n = offs[i + 1] - offs[i];
-    uint32_t* f = d_flags + 4 * i;
-    ARA_CUDA(c, ara::launch_prepare_records(d_ev + o, d_mu + o, d_sg + o, d_ex + o, n, d_recs + o, d_shapes + o, f,
-                                            reinterpret_cast<int32_t*>(f + 1), f + 3, c->stream,
-                                            sigma_c ? d_sc + o : nullptr, sigma_c ? d_w + o : nullptr));
-    c->launches += 1;
-  }
-  // coarse tables of every record in one launch, then each ELT's fine tables
-  ARA_CUDA(c, ara::launch_build_coarse(d_recs, d_shapes, R, d_tab, d_need, c->stream));
-  c->launches += (R > 0) ? 1 : 0;
-  std::vector<ara::FineJob> jobs;
-  for (int32_t i = 0; i < n_elts; ++i) {
-    const int64_t o = offs[i], n = offs[i + 1] - offs[i];
-    if (n == 0) continue;
-    int launched = 0;
-    uint32_t* w = d_work + work_off[i];
-    ARA_CUDA(c, ara::scan_exclusive_u32(d_need + o, w, n, w + n + 1, c->stream, &launched));
-    ARA_CUDA(c, cudaMemcpyAsync(d_flags + 4 * i + 2, w + n, sizeof(uint32_t), cudaMemcpyDeviceToDevice, c->stream));
-    c->launches += launched;
-    jobs.push_back(ara::FineJob{o, n, w, fine_off[i], ara::fine_table_cap(n), 0});
-  }
-  if (!jobs.empty()) {
-    // fine tables of every ELT in one launch (the job list is staged after the need flags)
-    ara::FineJob* d_jobs = reinterpret_cast<ara::FineJob*>(
-        (reinterpret_cast<uintptr_t>(d_need + R) + 15) & ~uintptr_t(15));
-    ARA_CUDA(c, cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(ara::FineJob) * jobs.size(), cudaMemcpyHostToDevice,
-                                c->stream));
-    ARA_CUDA(c, ara::launch_build_fine_jobs(d_recs, d_shapes, d_jobs, static_cast<int>(jobs.size()),
-                                            fine_off[n_elts], d_tabf, c->stream));
-    c->launches += 1;
-  }
+  ARA_CUDA(c, cudaMemcpyAsync(d_param, h_param, param.size(), cudaMemcpyHostToDevice, c->stream));
+  int launched = 0;
+  ARA_CUDA(c, ara::launch_prepare_records(d_ev, d_mu, d_sg, d_ex, d_offs, n_elts, longest, d_recs, d_shapes, d_flags,
+                                          c->stream, sigma_c ? d_sc : nullptr, sigma_c ? d_w : nullptr, &launched));
+  // (the records in order of their shapes, where there are enough for it to pay and its scratch fits)
+  int64_t* order = nullptr;
+  if (R >= kShapeOrderMin && (!c->budget || c->used + ara::shape_order_bytes(R) <= c->budget) &&
+      reserve(c, c->sel, ara::shape_order_bytes(R)) == ARA_OK)
+    ARA_CUDA(c, ara::launch_shape_order(d_shapes, R, c->sel.ptr, &order, c->stream, &launched));
+  ARA_CUDA(c, ara::launch_build_tables(d_recs, d_shapes, R, order, d_jobs, static_cast<int>(jobs.size()),
+                                       fine_off[n_elts], d_tab, d_tabf, d_work, d_flags, c->stream, &launched));
+  c->launches += launched;
   std::vector<uint32_t> hf(4 * static_cast<size_t>(n_elts));
   ARA_CUDA(c, cudaMemcpyAsync(hf.data(), d_flags, sizeof(uint32_t) * hf.size(), cudaMemcpyDeviceToHost, c->stream));
   ARA_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -2122,7 +2111,7 @@ int ara_debug_record_losses(ara_ctx* c, int64_t n, const float* mean, const floa
   const size_t bytes = static_cast<size_t>(n) * (sizeof(ara::Pair) + 6 * sizeof(float) + sizeof(int32_t) +
                                                  sizeof(ara::BetaShape) + sizeof(float4) * ara::kTabNodes) +
                        sizeof(float4) * ara::kTabFineStride * (ara::fine_table_cap(n) + 1) +
-                       sizeof(uint32_t) * ara::build_tables_work_words(n) + 256;
+                       sizeof(uint32_t) * ara::build_tables_work_words(n) + 512;
   if ((rc = reserve(c, tmp, bytes))) return rc;
   ara::Pair* d_p = static_cast<ara::Pair*>(tmp.ptr);
   float* d_mu = reinterpret_cast<float*>(d_p + n);
@@ -2137,8 +2126,16 @@ int ara_debug_record_losses(ara_ctx* c, int64_t n, const float* mean, const floa
   float4* d_tab = reinterpret_cast<float4*>(d_sh + n);
   float4* d_tabf = d_tab + n * ara::kTabNodes;
   uint32_t* d_work = reinterpret_cast<uint32_t*>(d_tabf + ara::kTabFineStride * (ara::fine_table_cap(n) + 1));
-  uint32_t* flags = static_cast<uint32_t*>(c->flags.ptr);
-  int32_t* max_ev = reinterpret_cast<int32_t*>(flags + 1);
+  // the records as one ELT: its offsets, its fine-table job, its words
+  struct {
+    int64_t offs[2];
+    ara::FineJob job;
+    uint32_t words[ara::kEltWords];
+  } one = {{0, n}, {0, n, 0, ara::fine_table_cap(n), 0}, {}};
+  std::memcpy(one.words, ara::kEltInit, sizeof one.words);
+  unsigned char* d_one = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(d_work + ara::build_tables_work_words(n)) + 15) & ~uintptr_t(15));
+  uint32_t* flags = reinterpret_cast<uint32_t*>(d_one + offsetof(decltype(one), words));
   cudaError_t e = cudaMemcpyAsync(d_mu, mean, sizeof(float) * n, cudaMemcpyDefault, c->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_sg, sigma, sizeof(float) * n, cudaMemcpyDefault, c->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_ex, exposure, sizeof(float) * n, cudaMemcpyDefault, c->stream);
@@ -2147,11 +2144,16 @@ int ara_debug_record_losses(ara_ctx* c, int64_t n, const float* mean, const floa
   std::vector<int32_t> ev(static_cast<size_t>(n));
   for (int64_t i = 0; i < n; ++i) ev[i] = static_cast<int32_t>(i);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_ev, ev.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 2 * sizeof(uint32_t), c->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d_one, &one, sizeof one, cudaMemcpyHostToDevice, c->stream);
+  int launched = 1;  // the losses
   if (e == cudaSuccess)
-    e = ara::launch_prepare_records(d_ev, d_mu, d_sg, d_ex, n, d_p, d_sh, flags, max_ev, nullptr, c->stream);
-  int launched = 2;
-  if (e == cudaSuccess) e = ara::launch_build_tables(d_p, d_sh, n, d_tab, d_tabf, d_work, c->stream, &launched);
+    e = ara::launch_prepare_records(d_ev, d_mu, d_sg, d_ex,
+                                    reinterpret_cast<const int64_t*>(d_one + offsetof(decltype(one), offs)), 1, n, d_p,
+                                    d_sh, flags, c->stream, nullptr, nullptr, &launched);
+  if (e == cudaSuccess)
+    e = ara::launch_build_tables(d_p, d_sh, n, nullptr,
+                                 reinterpret_cast<const ara::FineJob*>(d_one + offsetof(decltype(one), job)), 1,
+                                 ara::fine_table_cap(n), d_tab, d_tabf, d_work, flags, c->stream, &launched);
   if (e == cudaSuccess) e = ara::launch_debug_losses(d_p, d_tab, d_tabf, d_z, n, newton_only, d_o, d_it, c->stream);
   c->launches += launched;
   uint32_t hf = 0;
@@ -2189,7 +2191,7 @@ void ara_destroy(ara_ctx* c) {
                     &c->elt_flags,  &c->ev_buf,         &c->tile_cnt,      &c->def_acc,        &c->yet_off,
                     &c->yet_ids,    &c->marks,          &c->word_base,     &c->rankdir,        &c->slot_start,
                     &c->pairs,      &c->pairs_hot,      &c->pairs_w,       &c->pairs_ev,       &c->scan_tmp,
-                    &c->flags,      &c->counters,       &c->ylt_tmp,       &c->diag_tmp,       &c->sel,
+                    &c->counters,       &c->ylt_tmp,       &c->diag_tmp,       &c->sel,
                     &c->in_tmp,     &c->out_tmp,        &c->serve_arena,   &c->serve_out,      &c->yix_occ,
                     &c->yix_grid,   &c->yix_work,       &c->u_event,       &c->idx_acc,
                     &c->ev_occ,     &c->row_base,       &c->evr_stage,     &c->yet_flags};

@@ -358,18 +358,28 @@ __device__ __forceinline__ float pair_quantile_newton_zc(const Pair& p, float z,
   return 1.0f - beta_solve_oriented(p.b, p.a, y0, x0, p.c, ln1mz, lnz, y_start, st);
 }
 
-// InvCDF_beta(z; a, b) of a Beta record by the FP32 Halley iteration; x_start
-// in (0, 1) seeds it (otherwise the analytic start point is used).
-__device__ __forceinline__ float pair_quantile_newton(const Pair& p, float z, float x_start, BetaSolveStats* st) {
+// The root of a Beta record by the FP32 Halley iteration on its own side: x =
+// InvCDF_beta(z; a, b) itself (*is_x), or 1 - x where x is above about 1/2.
+// x_start in (0, 1) seeds it (otherwise the analytic start point is used).
+__device__ __forceinline__ float pair_root_newton(const Pair& p, float z, float x_start, BetaSolveStats* st,
+                                                  bool* is_x) {
   const bool m0x = signbit(p.m0);
   const float m0 = fabsf(p.m0);
   const float x0 = m0x ? m0 : 1.0f - m0;
   const float y0 = m0x ? 1.0f - m0 : m0;
   const float lnz = logf(z), ln1mz = log1pf(-z);
+  *is_x = z <= p.p_half;
   if (z <= p.p_half) return beta_solve_oriented(p.a, p.b, x0, y0, p.c, lnz, ln1mz, x_start, st);
   // root above 1/2: 1 - x solves I_{1-x}(b, a) = 1 - z
   const float y_start = (x_start > 0.0f && x_start < 1.0f) ? 1.0f - x_start : -1.0f;
-  return 1.0f - beta_solve_oriented(p.b, p.a, y0, x0, p.c, ln1mz, lnz, y_start, st);
+  return beta_solve_oriented(p.b, p.a, y0, x0, p.c, ln1mz, lnz, y_start, st);
+}
+
+// InvCDF_beta(z; a, b) of a Beta record by the FP32 Halley iteration.
+__device__ __forceinline__ float pair_quantile_newton(const Pair& p, float z, float x_start, BetaSolveStats* st) {
+  bool is_x;
+  const float r = pair_root_newton(p, z, x_start, st, &is_x);
+  return is_x ? r : 1.0f - r;
 }
 
 // Loss of one pair: max_l * InvCDF(z; a, b) for Beta records, the mean for

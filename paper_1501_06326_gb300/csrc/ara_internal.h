@@ -36,45 +36,46 @@ cudaError_t launch_check_ids(const int32_t* ids, int64_t n, int32_t catalogue, u
 cudaError_t launch_upload_ids(const int32_t* src, int32_t* dst, int64_t n, int32_t catalogue, uint32_t* flags,
                               cudaStream_t s);
 
-// Prepare the Pair records of one ELT from (mean, sigma, exposure) in FP64:
-// Beta shapes, x0/y0, C, I_{1/2}(a, b), kind.  Also checks order and values
-// and reduces the largest event id into *max_event and the largest loss a
-// record can produce (max(exposure, mean) over records with a loss, as FP32
-// bits) into *max_loss (both atomicMax; max_loss may be null).
-cudaError_t launch_prepare_records(const int32_t* events, const float* mean, const float* sigma,
-                                   const float* exposure, int64_t n, Pair* out, BetaShape* shapes, uint32_t* flags,
-                                   int32_t* max_event, uint32_t* max_loss, cudaStream_t s,
-                                   const float* sigma_c = nullptr, float2* weights = nullptr);
+// Per ELT of a load, kEltWords words (device): its validation flags, the
+// largest event id (0xFFFFFFFF: none), the candidates for fine tables, and the
+// largest loss a record can produce (max(exposure, mean) over records with a
+// loss, as FP32 bits).  The caller sets them to kEltInit first.
+constexpr int kEltWords = 4, kEltMaxEvent = 1, kEltFine = 2, kEltMaxLoss = 3;
+constexpr uint32_t kEltInit[kEltWords] = {0u, 0xFFFFFFFFu, 0u, 0u};
 
-// Quantile tables of prepared records, built in FP64: kTabNodes float4 per
-// record in `tab`; then, for the first fine_table_cap(n) records (in record
-// order) whose coarse table fails its check, kTabFineStride float4 per slot in
-// `tabf`.  Sets each record's table-exact and fine bits.  `work` holds
-// build_tables_work_words(n) words; on return work[n] is the number of
-// candidates for fine tables (min(work[n], cap) slots are used).
-size_t build_tables_work_words(int64_t n);
-uint32_t fine_table_cap(int64_t n);
-cudaError_t launch_build_tables(Pair* recs, const BetaShape* shapes, int64_t n, float4* tab, float4* tabf,
-                                uint32_t* work, cudaStream_t s, int* n_launch);
-// The two halves of launch_build_tables: coarse tables of n records (need[rec]
-// = 1 marks a candidate for a fine table; one launch may span several ELTs),
-// then the fine tables of one ELT (`work`: build_tables_work_words(n) words).
-cudaError_t launch_build_coarse(Pair* recs, const BetaShape* shapes, int64_t n, float4* tab, uint32_t* need,
-                                cudaStream_t s);
-cudaError_t launch_build_fine(Pair* recs, const BetaShape* shapes, int64_t n, const uint32_t* need, float4* tabf,
-                              uint32_t* work, cudaStream_t s, int* n_launch);
-// Fine tables of several ELTs in one launch: job i covers records
-// [rec_begin, rec_begin + n) whose candidates were scanned into `slot` (n + 1
-// words), and owns fine slots [slot_begin, slot_begin + cap) of `tabf`.  `jobs`
-// is a device array, ordered by slot_begin.
+// Prepare the Pair records of n_elts ELTs from (mean, sigma, exposure) in FP64:
+// Beta shapes, x0/y0, C, I_{1/2}(a, b), kind.  ELT i owns records rec_off[i] ..
+// rec_off[i + 1] (device array), at most `longest`.  Also checks order and
+// values and fills the ELTs' words.
+cudaError_t launch_prepare_records(const int32_t* events, const float* mean, const float* sigma,
+                                   const float* exposure, const int64_t* rec_off, int n_elts, int64_t longest,
+                                   Pair* out, BetaShape* shapes, uint32_t* elts, cudaStream_t s, const float* sigma_c,
+                                   float2* weights, int* n_launch);
+
+// Quantile tables of n prepared records, built in FP64: kTabNodes float4 per
+// record in `tab`; then fine tables, kTabFineStride float4 per slot in `tabf`:
+// job i covers the records [rec_begin, rec_begin + n) of ELT `elt` (an entry of
+// `elts`), and the first fine_table_cap(n) of them, in record order, whose
+// coarse table fails its check take its slots [slot_begin, slot_begin + cap).
+// Sets each record's table-exact and fine bits and each ELT's kEltFine word.
+// `jobs` is a device array, ordered by slot_begin; `work` holds
+// build_tables_work_words(n) words.  `order` (or NULL): the records in an
+// order that puts like shapes together, as launch_shape_order makes it in
+// scratch of shape_order_bytes(n).
 struct FineJob {
   int64_t rec_begin, n;
-  const uint32_t* slot;
   int64_t slot_begin;
-  uint32_t cap, pad;
+  uint32_t cap;
+  int32_t elt;
 };
-cudaError_t launch_build_fine_jobs(Pair* recs, const BetaShape* shapes, const FineJob* jobs, int n_jobs,
-                                   int64_t total_slots, float4* tabf, cudaStream_t s);
+size_t build_tables_work_words(int64_t n);
+uint32_t fine_table_cap(int64_t n);
+cudaError_t launch_build_tables(Pair* recs, const BetaShape* shapes, int64_t n, const int64_t* order,
+                                const FineJob* jobs, int n_jobs, int64_t total_slots, float4* tab, float4* tabf,
+                                uint32_t* work, uint32_t* elts, cudaStream_t s, int* n_launch);
+size_t shape_order_bytes(int64_t n);
+cudaError_t launch_shape_order(const BetaShape* shapes, int64_t n, void* scratch, int64_t** order, cudaStream_t s,
+                               int* n_launch);
 
 // Check kernels (device functions of the hot path on given inputs).
 cudaError_t launch_debug_uniforms(uint32_t seed_lo, uint32_t seed_hi, int64_t n, const int64_t* trials,

@@ -7,7 +7,7 @@
 #include <cstdint>
 
 #include "ara_df.cuh"
-#include "ara_internal.h"
+#include "ara_batch.h"
 
 namespace ara {
 
@@ -195,9 +195,9 @@ __device__ double beta_cf_f64_ref(double a, double b, double x) {
 // the 1e-13 relative tolerance used here (the table nodes are FP32; their
 // polish and check need the CDF to about 1e-10).  FP32's exponent range is
 // kept by rescaling the four convergents by a power of two each iteration
-// (exact; the ratio is unchanged).  Returns NaN when a value leaves the FP32
-// range or the iteration does not converge, for the FP64 fallback.
-__device__ double beta_cf_df(double a, double b, double x) {
+// (exact; the ratio is unchanged).  False when a value leaves the FP32 range or
+// the iteration does not converge, for the FP64 fallback.
+__device__ bool beta_cf_df(double a, double b, double x, double* num, double* den) {
   const DF X = df_of(x);
   DF v = df_of(a);          // a + m
   DF w = df_of(a + b);      // a + b + m
@@ -205,7 +205,7 @@ __device__ double beta_cf_df(double a, double b, double x) {
   DF u = df_of(a);          // a + 2m
   DF A2{1.0f, 0.0f}, B2{0.0f, 0.0f}, A1{1.0f, 0.0f}, B1{1.0f, 0.0f};
   DF q_prev{1.0f, 0.0f};
-  double f_prev = 1.0;
+  DF Ap{1.0f, 0.0f}, Bp{1.0f, 0.0f};  // the convergent of the last test
   for (int m = 0; m < 20000; ++m) {
     const DF u1 = df_add_f(u, 1.0f), u2 = df_add_f(u, 2.0f);
     // odd term n = 2m + 1: p = -(a + m)(a + b + m) x, q = (a + 2m)(a + 2m + 1)
@@ -228,25 +228,34 @@ __device__ double beta_cf_df(double a, double b, double x) {
     y = df_add_f(y, -1.0f);
     u = u2;
     const float big = fmaxf(fabsf(A1.hi), fabsf(B1.hi));
-    if (!(big < 3.0e38f) || !(big > 0.0f)) return __longlong_as_double(0x7ff8000000000000ll);
+    if (!(big < 3.0e38f) || !(big > 0.0f)) return false;
     const int k = -f_exponent(big);
     A1 = df_scale(A1, k);
     A2 = df_scale(A2, k);
     B1 = df_scale(B1, k);
     B2 = df_scale(B2, k);
     if ((m & 3) == 3) {
-      const double f = df_val(A1) / df_val(B1);
-      if (fabs(f - f_prev) <= 1e-13 * fabs(f)) return df_val(B1) / df_val(A1);
-      f_prev = f;
+      // |A1/B1 - Ap/Bp| <= 1e-13 |A1/B1|, cross-multiplied (48 bits tell 1e-13; an FP64 division a test,
+      // with its conversions, took a third of the table build)
+      const DF f = df_mul(A1, Bp);
+      const DF d = df_add(f, df_neg(df_mul(Ap, B1)));
+      if (fabsf(d.hi) <= 1e-13f * fabsf(f.hi)) {
+        *num = df_val(B1);
+        *den = df_val(A1);
+        return true;
+      }
+      Ap = A1;
+      Bp = B1;
     }
   }
-  return __longlong_as_double(0x7ff8000000000000ll);
+  return false;
 }
 
-// The continued fraction of I_x(a, b): double-float, else FP64.
-__device__ double beta_cf_f64(double a, double b, double x) {
-  const double r = beta_cf_df(a, b, x);
-  return isfinite(r) ? r : beta_cf_f64_ref(a, b, x);
+// The continued fraction of I_x(a, b), num / den: double-float, else FP64.
+__device__ void beta_cf_f64(double a, double b, double x, double* num, double* den) {
+  if (beta_cf_df(a, b, x, num, den) && isfinite(*num) && isfinite(*den) && *den != 0.0) return;
+  *num = beta_cf_f64_ref(a, b, x);
+  *den = 1.0;
 }
 
 }  // namespace
@@ -258,18 +267,24 @@ __device__ double beta_cf_f64(double a, double b, double x) {
 // (Section 3.2 step i) and a record with sigma_C > 0 is of kind kKindBetaC,
 // with weights (sigma_I, sigma_C) / sqrt(sigma_I^2 + sigma_C^2) for the
 // combination of its two normal variables.
+// blockIdx.y is the ELT, of records [rec_off[y], rec_off[y + 1]), with its
+// results at elts + kEltWords y.
 __global__ void k_prepare_records(const int32_t* events, const float* mean, const float* sigma,
-                                  const float* exposure, int64_t n, Pair* out, BetaShape* shapes, uint32_t* flags,
-                                  int32_t* max_event, uint32_t* max_loss, const float* sigma_c, float2* weights) {
+                                  const float* exposure, const int64_t* rec_off, Pair* out, BetaShape* shapes,
+                                  uint32_t* elts, const float* sigma_c, float2* weights) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const int64_t begin = rec_off[blockIdx.y], end = rec_off[blockIdx.y + 1];
+  uint32_t* flags = elts + static_cast<int64_t>(blockIdx.y) * kEltWords;
+  int32_t* max_event = reinterpret_cast<int32_t*>(flags + kEltMaxEvent);
+  uint32_t* max_loss = flags + kEltMaxLoss;
   uint32_t f = 0;
   int32_t emax = -1;
   float lmax = 0.0f;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) {
+  for (int64_t i = begin + blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < end; i += stride) {
     const int32_t e = events[i];
     emax = max(emax, e);
     if (e < 0) f |= kBadEventId;
-    if (i > 0 && events[i - 1] >= e) f |= kBadOrder;
+    if (i > begin && events[i - 1] >= e) f |= kBadOrder;
     const double mu = mean[i], si = sigma[i], ex = exposure[i];
     const double sc = sigma_c ? static_cast<double>(sigma_c[i]) : 0.0;
     const double sg = si + sc;
@@ -301,11 +316,13 @@ __global__ void k_prepare_records(const int32_t* events, const float* mean, cons
       const double c = a * log(x0) + b * log(y0) - lnB;
       // I_{1/2}(a, b), only used to pick the side of the root
       const double lfront = -(a + b) * 0.69314718055994530942 - lnB;
-      double ph;
+      double ph, num, den;
       if (0.5 < (a + 1.0) / (a + b + 2.0)) {
-        ph = exp(lfront) * beta_cf_f64(a, b, 0.5) / a;
+        beta_cf_f64(a, b, 0.5, &num, &den);
+        ph = exp(lfront) * num / (den * a);
       } else {
-        ph = 1.0 - exp(lfront) * beta_cf_f64(b, a, 0.5) / b;
+        beta_cf_f64(b, a, 0.5, &num, &den);
+        ph = 1.0 - exp(lfront) * num / (den * b);
       }
       p.a = static_cast<float>(a);
       p.b = static_cast<float>(b);
@@ -322,10 +339,10 @@ __global__ void k_prepare_records(const int32_t* events, const float* mean, cons
         w = make_float2(static_cast<float>(si / nrm), static_cast<float>(sc / nrm));
       }
     }
-    p.meta = (kind << kMetaKindShift) | (static_cast<uint32_t>(i) << kMetaRecShift);
+    p.meta = (kind << kMetaKindShift) | (static_cast<uint32_t>(i - begin) << kMetaRecShift);
     if (kind != kKindZero) lmax = fmaxf(lmax, fmaxf(p.max_l, p.mu));
     out[i] = p;
-    if (shapes) shapes[i] = BetaShape{sa, sb_, slnb, 0.0};
+    shapes[i] = BetaShape{sa, sb_, slnb, 0.0};
     if (weights) weights[i] = w;
   }
   if (f) atomicOr(flags, f);
@@ -336,17 +353,21 @@ __global__ void k_prepare_records(const int32_t* events, const float* mean, cons
   }
   if ((threadIdx.x & 31) == 0 && emax >= 0) atomicMax(max_event, emax);
   // non-negative floats order as their bit patterns
-  if ((threadIdx.x & 31) == 0 && max_loss && lmax > 0.0f) atomicMax(max_loss, __float_as_uint(lmax));
+  if ((threadIdx.x & 31) == 0 && lmax > 0.0f) atomicMax(max_loss, __float_as_uint(lmax));
 }
 
 cudaError_t launch_prepare_records(const int32_t* events, const float* mean, const float* sigma,
-                                   const float* exposure, int64_t n, Pair* out, BetaShape* shapes, uint32_t* flags,
-                                   int32_t* max_event, uint32_t* max_loss, cudaStream_t s, const float* sigma_c,
-                                   float2* weights) {
-  if (n == 0) return cudaSuccess;
-  const int64_t blocks = (n + 127) / 128;
-  k_prepare_records<<<static_cast<int>(blocks < 65535 ? blocks : 65535), 128, 0, s>>>(
-      events, mean, sigma, exposure, n, out, shapes, flags, max_event, max_loss, sigma_c, weights);
+                                   const float* exposure, const int64_t* rec_off, int n_elts, int64_t longest,
+                                   Pair* out, BetaShape* shapes, uint32_t* elts, cudaStream_t s, const float* sigma_c,
+                                   float2* weights, int* n_launch) {
+  if (longest == 0) return cudaSuccess;
+  const int64_t blocks = (longest + 127) / 128;
+  for (int y = 0; y < n_elts; y += 65535) {  // the grid's y limit
+    const dim3 grid(static_cast<int>(blocks < 65535 ? blocks : 65535), n_elts - y < 65535 ? n_elts - y : 65535);
+    k_prepare_records<<<grid, 128, 0, s>>>(events, mean, sigma, exposure, rec_off + y, out, shapes,
+                                           elts + static_cast<int64_t>(y) * kEltWords, sigma_c, weights);
+    if (n_launch) *n_launch += 1;
+  }
   return cudaGetLastError();
 }
 
@@ -357,7 +378,7 @@ namespace {
 // symmetry).  *front_out (optional) receives x^a (1-x)^b / B(a, b), which is
 // x (1 - x) f(x) for the Beta density f.
 __device__ void beta_inc_pair_f64(double x, double a, double b, double lnB, double* I, double* Ic,
-                                  double* front_out = nullptr) {
+                                  double* front_out = nullptr, double* lx_out = nullptr, double* l1mx_out = nullptr) {
   if (!(x > 0.0)) {
     *I = 0.0;
     *Ic = 1.0;
@@ -370,14 +391,19 @@ __device__ void beta_inc_pair_f64(double x, double a, double b, double lnB, doub
     if (front_out) *front_out = 0.0;
     return;
   }
-  const double front = exp(a * log(x) + b * log1p(-x) - lnB);
+  const double lx = log(x), l1mx = log1p(-x);
+  const double front = exp(a * lx + b * l1mx - lnB);
   if (front_out) *front_out = front;
+  if (lx_out) *lx_out = lx;
+  if (l1mx_out) *l1mx_out = l1mx;
   // the fraction on the side where it converges fast: the side is chosen per
   // lane and the fraction called once, so that the lanes of a warp do not
   // run it twice
-  const bool lower = x < (a + 1.0) / (a + b + 2.0);
+  const bool lower = x * (a + b + 2.0) < a + 1.0;
   const double p = lower ? a : b, q = lower ? b : a, y = lower ? x : 1.0 - x;
-  const double v = front * beta_cf_f64(p, q, y) / p;
+  double num, den;
+  beta_cf_f64(p, q, y, &num, &den);
+  const double v = front * num / (den * p);
   *I = lower ? v : 1.0 - v;
   *Ic = lower ? 1.0 - v : v;
 }
@@ -410,27 +436,99 @@ __device__ double beta_root_f64(double p, double A, double B, double lnB, double
   return r;
 }
 
-// Polish of an FP32 root r of I_r(A, B) = p (p <= 1/2): Newton on u = ln r in
-// FP64, where I ~ r^A near 0 makes the step almost exact.  The seed is good to
+// ln(1 + e), e^q - 1: a short series near 0 (to 1e-16 relative below 1e-3),
+// where the polish below nearly always is; the library's functions elsewhere.
+__device__ __forceinline__ double log1p_near(double e) {
+  if (!(fabs(e) < 1e-3)) return log1p(e);
+  return e * fma(e, fma(e, fma(e, fma(e, 0.2, -0.25), 1.0 / 3.0), -0.5), 1.0);
+}
+__device__ __forceinline__ double expm1_near(double q) {
+  if (!(fabs(q) < 1e-3)) return expm1(q);
+  return q * fma(q, fma(q, fma(q, fma(q, 1.0 / 120.0, 1.0 / 24.0), 1.0 / 6.0), 0.5), 1.0);
+}
+
+// A root r of I_r(A, B) = p, with ln r, ln(1 - r) and B(A, B) / (r^A (1 - r)^B).
+struct BetaRoot {
+  double r, lr, l1mr, inv_front;
+};
+
+__device__ __noinline__ BetaRoot beta_root_of(double p, double A, double B, double lnB, double guess) {
+  BetaRoot x;
+  x.r = beta_root_f64(p, A, B, lnB, guess);
+  x.lr = log(x.r);
+  x.l1mr = log1p(-x.r);
+  x.inv_front = exp(lnB - A * x.lr - B * x.l1mr);
+  return x;
+}
+
+// Newton on u = ln r in FP64 from r towards the root of I_r(A, B) = p (p <=
+// 1/2), where I ~ r^A near 0 makes the step almost exact: up to `steps` steps,
+// ended by one of |du| < tol.  The last step's logarithms and front factor are
+// moved along by du, a short series, in place of new ones, and one division
+// serves a step.  False when it does not converge; r is then where it stood.
+__device__ bool beta_newton_f64(double p, double A, double B, double lnB, int steps, double tol, double* r_io,
+                                BetaRoot* out) {
+  double r = *r_io;
+  for (int it = 0; it < steps; ++it) {
+    if (!(r > 0.0 && r < 1.0)) return false;
+    double I, Ic, front, lr, l1mr;
+    beta_inc_pair_f64(r, A, B, lnB, &I, &Ic, &front, &lr, &l1mr);
+    if (!(I > 0.0) || !(front > 0.0)) return false;
+    const double y = 1.0 - r;
+    const double inv = 1.0 / (y * front * p);
+    const double e = (I - p) * (inv * y * front);              // (I - p) / p
+    const double du = -log1p_near(e) * (y * y * I * p * inv);  // d ln I / d ln r = front / ((1 - r) I)
+    if (!(fabs(du) < 0.5)) return false;
+    const double rn = fma(r, expm1_near(du), r);
+    if (!(rn > 0.0 && rn < 1.0)) return false;
+    if (fabs(du) < tol) {
+      const double dl = log1p_near((r - rn) * (inv * front * p));  // ln((1 - rn) / (1 - r))
+      const double inv_front = inv * y * p * (1.0 + expm1_near(-(A * du + B * dl)));
+      if (!(inv_front > 0.0) || !isfinite(inv_front)) return false;
+      *out = BetaRoot{rn, lr + du, l1mr + dl, inv_front};
+      return true;
+    }
+    r = rn;
+    *r_io = rn;
+  }
+  return false;
+}
+
+// The root where the polish of the plain seed failed (a root near 1 whose
+// complement the seed has lost, one below the FP32 range): the same steps from
+// the seed of the root's own side, or from the power law I ~ r^A / (A B(A, B))
+// where that is the root to FP64 precision.  They end at |du| < 1e-7, so that
+// what is left (du^2) is below the bracketed solver's 2e-10, which takes what
+// does not converge here (dozens of FP64 fractions a root: with it alone the
+// stress recipe's tables took five times as long as the plain recipe's).
+__device__ __noinline__ BetaRoot beta_root_again(double p, double A, double B, double lnB, double own_seed,
+                                                 double guess) {
+  const double lpow = (log(p) + log(A) + lnB) / A;
+  double r = lpow < -46.0 ? exp(lpow) : own_seed;  // below 1e-20
+  BetaRoot x;
+  if (r > 1e-290 && beta_newton_f64(p, A, B, lnB, 6, 1e-7, &r, &x)) return x;
+  return beta_root_of(p, A, B, lnB, guess);
+}
+
+// Polish of an FP32 root r of I_r(A, B) = p (p <= 1/2).  The seed is good to
 // ~1e-6, so a step |du| < 1e-5 leaves an error of order du^2 (~1e-10, below
 // the FP32 resolution of the stored node) and ends the iteration; at most 3
-// steps.  A seed that does not converge goes to the bracketed solver.
-__device__ double beta_polish_f64(double p, double A, double B, double lnB, double seed) {
+// steps.
+__device__ BetaRoot beta_polish_f64(double p, double A, double B, double lnB, double seed, double own_seed) {
+  BetaRoot x;
   double r = seed;
-  if (!(r > 0.0 && r < 1.0)) return beta_root_f64(p, A, B, lnB, -1.0);
-  for (int it = 0; it < 3; ++it) {
-    double I, Ic, front;
-    beta_inc_pair_f64(r, A, B, lnB, &I, &Ic, &front);
-    if (!(I > 0.0) || !(front > 0.0)) return beta_root_f64(p, A, B, lnB, seed);
-    const double g = front / ((1.0 - r) * I);  // d ln I / d ln r = r f(r) / I
-    const double du = -log1p((I - p) / p) / g;
-    if (!(fabs(du) < 0.5)) return beta_root_f64(p, A, B, lnB, seed);
-    const double rn = fma(r, expm1(du), r);
-    if (!(rn > 0.0 && rn < 1.0)) return beta_root_f64(p, A, B, lnB, seed);
-    r = rn;
-    if (fabs(du) < 1e-5) return r;
-  }
-  return beta_root_f64(p, A, B, lnB, r);
+  // (a seed more than a factor of two off its own side's fails at the first step)
+  if (seed < 2.1 * own_seed && own_seed < 2.1 * seed && beta_newton_f64(p, A, B, lnB, 3, 1e-5, &r, &x)) return x;
+  return beta_root_again(p, A, B, lnB, own_seed, seed > 0.0 && seed < 1.0 ? r : -1.0);
+}
+
+// What a table's nodes need of t alone: the smaller tail Phi(-|t|) and the
+// normal density.
+struct TabPoint {
+  double t, zl, phi;
+};
+__device__ TabPoint tab_point(double t) {
+  return TabPoint{t, normcdf(-fabs(t)), exp(-0.5 * t * t - 0.91893853320467274178)};
 }
 
 }  // namespace
@@ -439,43 +537,43 @@ __device__ double beta_polish_f64(double p, double A, double B, double lnB, doub
 // FP32 Halley solver), w = ln x, and the derivatives in t, w' = phi(t) / (x f(x))
 // and w'' = w' (-t - w' (a - (b-1) x/(1-x))).  Returns {x, 0, h w', h^2 w''}
 // (the caller fills in w_{j+1} - w_j) and w.
-__device__ float4 table_node(const Pair& pr, double a, double b, double lnB, double t, double h, double* w_out) {
-  const double zl = normcdf(-fabs(t));  // the smaller tail probability
+__device__ float4 table_node(const Pair& pr, double a, double b, double lnB, const TabPoint& q, double h,
+                             double* w_out) {
+  const double t = q.t, zl = q.zl;
   // FP32 seed, then FP64 polish on the side where the root keeps relative precision
   BetaSolveStats st;
   const float zf = (t <= 0.0) ? static_cast<float>(zl) : static_cast<float>(1.0 - zl);
-  const float seed = pair_quantile_newton(pr, fminf(fmaxf(zf, 5.9604645e-08f), 0.99999994f), -1.0f, &st);
+  const float z = fminf(fmaxf(zf, 5.9604645e-08f), 0.99999994f);
+  bool is_x;
+  const float root = pair_root_newton(pr, z, -1.0f, &st, &is_x);
+  const float seed = is_x ? root : 1.0f - root;
   // the root x (t <= 0) or y = 1 - x (t > 0): the shapes are swapped per lane
   // and the polish called once (ln B is symmetric), so that the two halves of
   // the warp do not run it in turn
   const bool lo = t <= 0.0;
-  const double r = beta_polish_f64(zl, lo ? a : b, lo ? b : a, lnB,
-                                   lo ? static_cast<double>(seed) : 1.0 - static_cast<double>(seed));
-  const double l_r = log(r), l_1mr = log1p(-r);
-  const double w = lo ? l_r : l_1mr;
-  const double lny = lo ? l_1mr : l_r;
-  const double lpdf = (a - 1.0) * w + (b - 1.0) * lny - lnB;
-  const double lphi = -0.5 * t * t - 0.91893853320467274178;
-  const double D = exp(lphi - w - lpdf);
-  const double E = D * (-t - D * (a - (b - 1.0) * exp(w - lny)));
-  *w_out = w;
-  return make_float4(static_cast<float>(exp(w)), 0.0f, static_cast<float>(h * D), static_cast<float>(h * h * E));
+  const BetaRoot v = beta_polish_f64(zl, lo ? a : b, lo ? b : a, lnB,
+                                     lo ? static_cast<double>(seed) : 1.0 - static_cast<double>(seed),
+                                     lo == is_x ? static_cast<double>(root) : 1.0 - static_cast<double>(root));
+  const double x = lo ? v.r : 1.0 - v.r, y = lo ? 1.0 - v.r : v.r;
+  const double D = q.phi * y * v.inv_front;  // phi / (x f(x)), as x (1 - x) f(x) is the front factor
+  const double E = D * (-t - D * (a - (b - 1.0) * (x / y)));
+  *w_out = lo ? v.lr : v.l1mr;
+  return make_float4(static_cast<float>(x), 0.0f, static_cast<float>(h * D), static_cast<float>(h * h * E));
 }
 
 // Accuracy of the segment [t, t + h] of a table (node nd = {x, dw, h w', h^2 w''}
-// at t; d1, e1 the derivative terms of the next node), checked at the midpoint,
+// at t; d1, e1 the derivative terms of the next node), checked at the midpoint
+// tq = t + h / 2, zq = Phi(-|tq|),
 // where the error kernel s^3 (1-s)^3 of quintic Hermite interpolation peaks:
 // the FP32 interpolant (as the hot path evaluates it) against the FP64 CDF.
 // True when the implied relative error of x there is within kTabTol (a bound
 // set by the FP32 evaluation of the interpolant, ~2e-7, more than by the
 // interpolation error, which elsewhere in the segment is below its midpoint
 // value), or x < 1e-30 (negligible losses).
-__device__ bool table_segment_ok(float4 nd, float d1, float e1, double t, double h, double a, double b, double lnB) {
+__device__ bool table_segment_ok(float4 nd, float d1, float e1, double tq, double zq, double a, double b, double lnB) {
   if (!(isfinite(nd.x) && isfinite(nd.y) && isfinite(nd.z) && isfinite(nd.w))) return false;
   const float xq = (nd.x > 0.0f) ? nd.x * expf(tab_increment(0.5f, nd.y, nd.z, nd.w, d1, e1)) : 0.0f;
   if (!(xq >= 1e-30f)) return true;
-  const double tq = t + 0.5 * h;
-  const double zq = normcdf(-fabs(tq));
   double I, Ic, front, rel;
   if (xq >= 1.0f) {
     // the FP32 ceiling: fine iff the quantile itself is within 2^-24 of 1
@@ -490,153 +588,224 @@ __device__ bool table_segment_ok(float4 nd, float d1, float e1, double t, double
   return (rel <= kTabTol) && isfinite(rel);
 }
 
-// Coarse tables, one warp per record, lane j = node j at t_j = -T1 + j h.  The
+// Coarse tables: a block builds those of 32 records, lane l of every warp the
+// record order[32 block + l] (or that record itself without an order), warp w
+// the nodes j = w, w + 8, .. at t_j = -T1 + j h, then the segments' checks.  The
 // stored float4 is {x_j, w_{j+1} - w_j, h w'_j, h^2 w''_j}.  need[rec] = 1 for
 // a Beta record whose coarse table is not exact (a candidate for a fine table).
-__global__ void __launch_bounds__(256, 2) k_build_tables(Pair* recs, const BetaShape* shapes, int64_t n, float4* tab,
-                                                        uint32_t* need) {
-  const int lane = threadIdx.x & 31;
-  const int64_t rec = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  if (rec >= n) return;
-  const Pair pr = recs[rec];
-  float4* out = tab + rec * kTabNodes;
-  if (!kind_is_beta(pair_kind(pr.meta))) {
-    out[lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (lane == 0) need[rec] = 0u;
-    return;
-  }
-  const double a = shapes[rec].a, b = shapes[rec].b, lnB = shapes[rec].lnB;
+// The iteration and fraction lengths follow the shapes and t: with the records
+// in order of a + b a warp's lanes, at the same t, run about equally long,
+// where a warp per record with a lane per node ran 13 of its 32 lanes (30 now).
+// Bound by the FP64 pipe (76% active: logs, exps and divisions around the
+// double-float fraction).  150,000 records of the plain recipe: 3.6 ms, a warp
+// per record 10.7, and 15.1 with an FP64 division for each test of the
+// fraction and new logarithms and exponentials after the last Newton step; of
+// the stress recipe 4.2 ms, 19.8 with the bracketed solver for the roots near
+// 1.  In order of a + b alone 4.0 and 10.2 ms.
+constexpr int kTabRecs = 32;     // records of a block
+constexpr int kTabWarps = 8;
+
+__global__ void __launch_bounds__(32 * kTabWarps, 2) k_build_tables(Pair* recs, const BetaShape* shapes, int64_t n,
+                                                                   const int64_t* order, float4* tab,
+                                                                   uint32_t* need) {
+  // the nodes' and midpoints' normal values, the same for every record
+  __shared__ TabPoint pt[kTabNodes];
+  __shared__ double mid_t[kTabNodes], mid_z[kTabNodes];
+  __shared__ double s_w[kTabRecs][kTabNodes + 1];
+  __shared__ float4 s_node[kTabRecs][kTabNodes + 1];
+  __shared__ int64_t s_rec[kTabRecs];
+  __shared__ uint32_t s_bad;  // records with a segment that fails its check
   const double h = 2.0 * kTabT1 / (kTabNodes - 1);
-  const double t = -kTabT1 + h * lane;
-  double w;
-  float4 node = table_node(pr, a, b, lnB, t, h, &w);
-  const double w_next = __shfl_down_sync(0xffffffffu, w, 1);
-  if (lane < kTabNodes - 1) node.y = static_cast<float>(w_next - w);
-  out[lane] = node;
-  const float d1 = __shfl_down_sync(0xffffffffu, node.z, 1);
-  const float e1 = __shfl_down_sync(0xffffffffu, node.w, 1);
-  const bool ok = (lane < kTabNodes - 1) ? table_segment_ok(node, d1, e1, t, h, a, b, lnB)
-                                         : (isfinite(node.x) && isfinite(node.z) && isfinite(node.w));
-  const bool all_ok = __all_sync(0xffffffffu, ok);
-  if (lane == 0) {
-    if (all_ok) recs[rec].meta = pr.meta | (1u << kMetaExactBit);
-    need[rec] = all_ok ? 0u : 1u;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * kTabRecs + lane;
+  const int64_t rec = i < n ? (order ? order[i] : i) : -1;
+  if (warp == 0) {
+    const double t = -kTabT1 + h * lane;
+    pt[lane] = tab_point(t);
+    s_rec[lane] = rec;
+    if (lane == 0) s_bad = 0u;
+  } else if (warp == 1) {
+    const double t = -kTabT1 + h * lane + 0.5 * h;
+    mid_t[lane] = t;
+    mid_z[lane] = normcdf(-fabs(t));
+  }
+  __syncthreads();
+  Pair pr{};
+  double a = 0.0, b = 0.0, lnB = 0.0;
+  bool beta = false;
+  if (rec >= 0) {
+    pr = recs[rec];
+    beta = kind_is_beta(pair_kind(pr.meta));
+    a = shapes[rec].a;
+    b = shapes[rec].b;
+    lnB = shapes[rec].lnB;
+  }
+#pragma unroll 1
+  for (int j = warp; j < kTabNodes; j += kTabWarps) {
+    double w = 0.0;
+    float4 node = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (beta) node = table_node(pr, a, b, lnB, pt[j], h, &w);
+    s_w[lane][j] = w;
+    s_node[lane][j] = node;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int j = warp; j < kTabNodes; j += kTabWarps) {
+    float4 node = s_node[lane][j];
+    bool ok = true;
+    if (j < kTabNodes - 1) {
+      node.y = static_cast<float>(s_w[lane][j + 1] - s_w[lane][j]);
+      s_node[lane][j].y = node.y;
+      const float4* next = &s_node[lane][j + 1];
+      if (beta) ok = table_segment_ok(node, next->z, next->w, mid_t[j], mid_z[j], a, b, lnB);
+    } else {
+      ok = isfinite(node.x) && isfinite(node.z) && isfinite(node.w);
+    }
+    const uint32_t bad = __ballot_sync(0xffffffffu, !ok);
+    if (lane == 0 && bad) atomicOr(&s_bad, bad);
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int r = warp; r < kTabRecs; r += kTabWarps)
+    if (s_rec[r] >= 0) tab[s_rec[r] * kTabNodes + lane] = s_node[r][lane];
+  if (warp == 0 && rec >= 0) {
+    const bool all_ok = ((s_bad >> lane) & 1u) == 0u;
+    if (beta && all_ok) recs[rec].meta = pr.meta | (1u << kMetaExactBit);
+    need[rec] = beta && !all_ok ? 1u : 0u;
+  }
+}
+
+// Keys that put records with like shapes together: a + b in steps of a quarter
+// of its power of two, then the mean a / (a + b) in 64 steps (0 for records
+// without a Beta).
+__global__ void k_shape_keys(const BetaShape* shapes, int64_t n, unsigned long long* keys, int64_t* order) {
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += stride) {
+    const float sum = static_cast<float>(shapes[i].a + shapes[i].b), mean = static_cast<float>(shapes[i].a) / sum;
+    keys[i] = sum > 0.0f ? (((__float_as_uint(sum) >> 21) & 0x3FFu) << 6) | static_cast<uint32_t>(63.0f * mean) : 0u;
+    order[i] = i;
   }
 }
 
 // Fine tables: global block b is slot b - slot_begin of the job (ELT) whose
 // slot range holds b, for that job's (b - slot_begin)-th candidate in record
-// order (slot = exclusive prefix of its need flags); thread j = node j at
+// order (slots = exclusive prefix of all records' need flags); thread j = node j at
 // t_j = -T1 + j h / kTabRefine.  The record's meta then addresses its fine
 // table (by the ELT-local slot); it is table-exact if the fine table passes
 // the check.
-__global__ void __launch_bounds__(kTabFineStride) k_build_fine(Pair* recs, const BetaShape* shapes,
-                                                              const FineJob* jobs, int n_jobs, float4* tabf) {
+// A block takes slots blockIdx.x, blockIdx.x + gridDim.x, .., so that the nodes'
+// and midpoints' normal values are computed once a block.
+__global__ void __launch_bounds__(kTabFineStride, 2) k_build_fine(Pair* recs, const BetaShape* shapes,
+                                                                 const FineJob* jobs, int n_jobs, const uint32_t* slots,
+                                                                 int64_t total_slots, float4* tabf) {
   __shared__ double s_w[kTabFineStride];
   __shared__ float4 s_node[kTabFineStride];
   __shared__ int64_t s_rec;
   __shared__ uint32_t s_ls;
-  const int64_t gb = blockIdx.x;
-  if (threadIdx.x == 0) {
-    int lo = 0, hi = n_jobs - 1;  // the last job with slot_begin <= gb
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (jobs[mid].slot_begin <= gb) lo = mid; else hi = mid - 1;
-    }
-    const FineJob jb = jobs[lo];
-    const uint32_t ls = static_cast<uint32_t>(gb - jb.slot_begin);
-    int64_t rec = -1;
-    if (jb.n > 0 && ls < jb.cap && ls < jb.slot[jb.n]) {
-      int64_t l = 0, h = jb.n - 1;  // the first r with slot[r + 1] > ls
-      while (l < h) {
-        const int64_t mid = (l + h) >> 1;
-        if (jb.slot[mid + 1] > ls) h = mid; else l = mid + 1;
-      }
-      rec = jb.rec_begin + l;
-    }
-    s_rec = rec;
-    s_ls = ls;
-  }
-  __syncthreads();
-  const int64_t rec = s_rec;
-  if (rec < 0) return;
-  const uint32_t ls = s_ls;
-  const Pair pr = recs[rec];
-  const double a = shapes[rec].a, b = shapes[rec].b, lnB = shapes[rec].lnB;
   const double h = 2.0 * kTabT1 / (kTabFineNodes - 1);
   const int j = threadIdx.x;
   const double t = -kTabT1 + h * (j < kTabFineNodes ? j : kTabFineNodes - 1);
-  double w = 0.0;
-  float4 node = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  if (j < kTabFineNodes) node = table_node(pr, a, b, lnB, t, h, &w);
-  s_w[j] = w;
-  s_node[j] = node;
-  __syncthreads();
-  bool ok = true;
-  if (j < kTabFineNodes - 1) {
-    node.y = static_cast<float>(s_w[j + 1] - w);
-    ok = table_segment_ok(node, s_node[j + 1].z, s_node[j + 1].w, t, h, a, b, lnB);
-  } else if (j == kTabFineNodes - 1) {
-    ok = isfinite(node.x) && isfinite(node.z) && isfinite(node.w);
+  const TabPoint pt = tab_point(t);
+  const double mid_z = normcdf(-fabs(t + 0.5 * h));
+  for (int64_t gb = blockIdx.x; gb < total_slots; gb += gridDim.x) {
+    if (threadIdx.x == 0) {
+      int lo = 0, hi = n_jobs - 1;  // the last job with slot_begin <= gb
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (jobs[mid].slot_begin <= gb) lo = mid; else hi = mid - 1;
+      }
+      const FineJob jb = jobs[lo];
+      const uint32_t ls = static_cast<uint32_t>(gb - jb.slot_begin);
+      int64_t rec = -1;
+      const uint32_t* slot = slots + jb.rec_begin;
+      if (jb.n > 0 && ls < jb.cap && ls < slot[jb.n] - slot[0]) {
+        int64_t l = 0, hh = jb.n - 1;  // the first r with slot[r + 1] > ls
+        while (l < hh) {
+          const int64_t mid = (l + hh) >> 1;
+          if (slot[mid + 1] - slot[0] > ls) hh = mid; else l = mid + 1;
+        }
+        rec = jb.rec_begin + l;
+      }
+      s_rec = rec;
+      s_ls = ls;
+    }
+    __syncthreads();
+    const int64_t rec = s_rec;
+    const uint32_t ls = s_ls;
+    if (rec < 0) {
+      __syncthreads();  // the next slot rewrites s_rec
+      continue;
+    }
+    const Pair pr = recs[rec];
+    const double a = shapes[rec].a, b = shapes[rec].b, lnB = shapes[rec].lnB;
+    double w = 0.0;
+    float4 node = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (j < kTabFineNodes) node = table_node(pr, a, b, lnB, pt, h, &w);
+    s_w[j] = w;
+    s_node[j] = node;
+    __syncthreads();
+    bool ok = true;
+    if (j < kTabFineNodes - 1) {
+      node.y = static_cast<float>(s_w[j + 1] - w);
+      ok = table_segment_ok(node, s_node[j + 1].z, s_node[j + 1].w, t + 0.5 * h, mid_z, a, b, lnB);
+    } else if (j == kTabFineNodes - 1) {
+      ok = isfinite(node.x) && isfinite(node.z) && isfinite(node.w);
+    }
+    if (j < kTabFineNodes) tabf[gb * kTabFineStride + j] = node;
+    const bool all_ok = __syncthreads_and(ok) != 0;
+    if (j == 0)
+      recs[rec].meta = (pr.meta & ((1u << kMetaFineBit) - 1u)) | (1u << kMetaFineBit) |
+                       (all_ok ? (1u << kMetaExactBit) : 0u) | (ls << kMetaRecShift);
   }
-  if (j < kTabFineNodes) tabf[gb * kTabFineStride + j] = node;
-  const bool all_ok = __syncthreads_and(ok) != 0;
-  if (j == 0)
-    recs[rec].meta = (pr.meta & ((1u << kMetaFineBit) - 1u)) | (1u << kMetaFineBit) |
-                     (all_ok ? (1u << kMetaExactBit) : 0u) | (ls << kMetaRecShift);
 }
 
-size_t build_tables_work_words(int64_t n) {
-  // need/slot (n + 1), scan scratch, then room for one 16-byte aligned FineJob
-  return static_cast<size_t>(n) + 1 + scan_tmp_words(n + 1) + (sizeof(FineJob) + 16) / sizeof(uint32_t);
-}
+size_t build_tables_work_words(int64_t n) { return 2 * static_cast<size_t>(n) + 1 + scan_tmp_words(n); }
 
 uint32_t fine_table_cap(int64_t n) {
   const int64_t cap = n / 16 + 16;
   return static_cast<uint32_t>(cap < n ? cap : n);
 }
 
-cudaError_t launch_build_coarse(Pair* recs, const BetaShape* shapes, int64_t n, float4* tab, uint32_t* need,
-                                cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  const int64_t blocks = (n + 7) / 8;  // 8 warps (records) per block
-  k_build_tables<<<static_cast<int>(blocks < 2147483647 ? blocks : 2147483647), 256, 0, s>>>(recs, shapes, n, tab,
-                                                                                          need);
-  return cudaGetLastError();
+size_t shape_order_bytes(int64_t n) {
+  return static_cast<size_t>(n) * (sizeof(unsigned long long) + sizeof(int64_t)) + sort_pairs_scratch_bytes(n) + 256;
 }
 
-cudaError_t launch_build_fine_jobs(Pair* recs, const BetaShape* shapes, const FineJob* jobs, int n_jobs,
-                                   int64_t total_slots, float4* tabf, cudaStream_t s) {
-  if (n_jobs == 0 || total_slots == 0) return cudaSuccess;
-  k_build_fine<<<static_cast<int>(total_slots), kTabFineStride, 0, s>>>(recs, shapes, jobs, n_jobs, tabf);
-  return cudaGetLastError();
-}
-
-// One ELT: its scan, then its fine tables (a one-job launch; the job record
-// sits after the scan's scratch in `work`).
-cudaError_t launch_build_fine(Pair* recs, const BetaShape* shapes, int64_t n, const uint32_t* need, float4* tabf,
-                              uint32_t* work, cudaStream_t s, int* n_launch) {
-  if (n == 0) return cudaSuccess;
-  int launched = 0;
-  cudaError_t err = scan_exclusive_u32(need, work, n, work + n + 1, s, &launched);
-  if (err != cudaSuccess) return err;
-  FineJob jb{0, n, work, 0, fine_table_cap(n), 0};
-  FineJob* d_job = reinterpret_cast<FineJob*>(
-      (reinterpret_cast<uintptr_t>(work + n + 1 + scan_tmp_words(n + 1)) + 15) & ~uintptr_t(15));
-  if ((err = cudaMemcpyAsync(d_job, &jb, sizeof(FineJob), cudaMemcpyHostToDevice, s)) != cudaSuccess) return err;
-  if ((err = cudaStreamSynchronize(s)) != cudaSuccess) return err;  // jb lives on this stack frame
-  if ((err = launch_build_fine_jobs(recs, shapes, d_job, 1, jb.cap, tabf, s)) != cudaSuccess) return err;
-  if (n_launch) *n_launch += launched + 1;
-  return cudaSuccess;
-}
-
-cudaError_t launch_build_tables(Pair* recs, const BetaShape* shapes, int64_t n, float4* tab, float4* tabf,
-                                uint32_t* work, cudaStream_t s, int* n_launch) {
-  if (n == 0) return cudaSuccess;
-  cudaError_t err = launch_build_coarse(recs, shapes, n, tab, work, s);
-  if (err != cudaSuccess) return err;
+cudaError_t launch_shape_order(const BetaShape* shapes, int64_t n, void* scratch, int64_t** order, cudaStream_t s,
+                               int* n_launch) {
+  unsigned long long* keys = static_cast<unsigned long long*>(scratch);
+  *order = reinterpret_cast<int64_t*>(keys + n);
+  const int64_t blocks = (n + 255) / 256;
+  k_shape_keys<<<static_cast<int>(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(shapes, n, keys, *order);
   if (n_launch) *n_launch += 1;
-  return launch_build_fine(recs, shapes, n, work, tabf, work, s, n_launch);
+  const cudaError_t err = cudaGetLastError();
+  return err != cudaSuccess ? err : sort_pairs_ascending(keys, *order, n, 16, *order + n, s, n_launch);
+}
+
+// Each job's candidates for fine tables, from the scan of the need flags.
+__global__ void k_fine_counts(const FineJob* jobs, int n_jobs, const uint32_t* slots, uint32_t* elts) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_jobs; i += gridDim.x * blockDim.x)
+    elts[static_cast<int64_t>(jobs[i].elt) * kEltWords + kEltFine] =
+        slots[jobs[i].rec_begin + jobs[i].n] - slots[jobs[i].rec_begin];
+}
+
+cudaError_t launch_build_tables(Pair* recs, const BetaShape* shapes, int64_t n, const int64_t* order,
+                                const FineJob* jobs, int n_jobs, int64_t total_slots, float4* tab, float4* tabf,
+                                uint32_t* work, uint32_t* elts, cudaStream_t s, int* n_launch) {
+  if (n == 0) return cudaSuccess;
+  uint32_t *need = work, *slots = work + n, *tmp = slots + n + 1;
+  const int64_t blocks = (n + kTabRecs - 1) / kTabRecs;
+  k_build_tables<<<static_cast<int>(blocks < 2147483647 ? blocks : 2147483647), 32 * kTabWarps, 0, s>>>(
+      recs, shapes, n, order, tab, need);
+  cudaError_t err = cudaGetLastError();
+  if (err != cudaSuccess) return err;
+  if ((err = scan_exclusive_u32(need, slots, n, tmp, s, n_launch)) != cudaSuccess) return err;
+  k_fine_counts<<<(n_jobs + 255) / 256, 256, 0, s>>>(jobs, n_jobs, slots, elts);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  const int64_t most = 4096;
+  k_build_fine<<<static_cast<int>(total_slots < most ? total_slots : most), kTabFineStride, 0, s>>>(
+      recs, shapes, jobs, n_jobs, slots, total_slots, tabf);
+  if (n_launch) *n_launch += 3;
+  return cudaGetLastError();
 }
 
 // =============================================================== check kernels

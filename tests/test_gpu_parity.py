@@ -494,3 +494,27 @@ def test_gather_groups(eng, catalogue, density):
         ylt, hits, hh = run_gpu(eng, yet, pool, terms, seed=9, t0=t0, t1=t1)
         assert np.array_equal(hits, ref["hits"]) and np.array_equal(hh, ref["hit_hash"])
         check_ylt(ylt, ref)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 4_095, 4_096, 4_129])
+def test_table_blocks(eng, n):
+    """Quantile tables at the edges of the builder's blocks (32 records) and of
+    the load from which records are taken in order of their shapes (4,096), with
+    records of every kind among them and two ELTs of unlike length in the load:
+    every record's losses against the oracle, through a layer over both."""
+    rng = np.random.default_rng(n)
+    C = 5_000
+    pool = synth.make_elt_pool(2, C, C, 77, recipe="stress")
+    keep = [np.sort(rng.choice(C, k, replace=False)) for k in (n, 7)]
+    pick = np.concatenate([keep[0], C + keep[1]])
+    cut = {f: getattr(pool, f)[pick] for f in ("event_ids", "mean", "sigma", "exposure")}
+    cut["sigma"][rng.random(len(pick)) < 0.1] = 0.0  # the mean
+    cut["mean"][rng.random(len(pick)) < 0.1] = 0.0  # no loss
+    sub = synth.ELTPool(elt_ids=pool.elt_ids, rec_offsets=np.array([0, n, n + 7], np.int64), terms=pool.terms, **cut)
+    held = np.unique(sub.event_ids)
+    yet = synth.YET(np.arange(0, 40_001, 40, dtype=np.int64), rng.choice(held, 40_000).astype(np.int32), C)
+    terms = (0.0, 1e12, 0.0, 1e15)
+    ref = oracle.run_layer(yet, sub, terms, seed=6)
+    ylt, hits, hh = run_gpu(eng, yet, sub, terms, seed=6)
+    assert np.array_equal(hits, ref["hits"]) and np.array_equal(hh, ref["hit_hash"])
+    check_ylt(ylt, ref)
