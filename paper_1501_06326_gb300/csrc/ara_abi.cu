@@ -719,6 +719,7 @@ struct PassPlan {
   ara::LayerIndex ix{};
   ara::GatherParams g{};
   int64_t n_out = 0, n_tiles = 0, e0 = 0;
+  int32_t tile_trials = ara::kWarpTrials;
   int grid = 0;
   size_t smem = 0;
   int filt_words = 0;
@@ -813,7 +814,24 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
     return fail(c, ARA_ECUDA, "%s: kernel needs %zu bytes of shared memory, device allows %d", who, pl->smem,
                 c->max_smem);
   pl->n_out = t1 - t0;
-  pl->n_tiles = (pl->n_out + ara::kWarpTrials - 1) / ara::kWarpTrials;
+  // Trials per tile.  Eight share a tile's set-up and the lanes left over at its end, which counts where a
+  // trial has few records (75 a trial, 1M trials: eight 1,029 us in the losses, four 1,117, two 1,378).  Fewer
+  // where a tile of half the trials still has 512 records, so that no warp is left a long last tile (750 a
+  // trial: 33,333 trials 948 us with eight, 620 with one; 100,003 trials 1,875 and 1,737), where the losses'
+  // 24 warps an SM would get under three tiles each and half a tile still has 128 records (75 a trial, 20,011
+  // trials, gather and losses: 117 us with eight, 102 with two, 116 with one), and where they would not get
+  // one each (30 a trial, 1,000 trials: 33 us with eight, 22 with one).  Neither sums nor rows depend on it.
+  const int64_t warps = int64_t(24) * c->num_sms;
+  const double recs_trial = static_cast<double>(n_recs) * static_cast<double>(c->h_off[t1] - c->h_off[t0]) /
+                            (static_cast<double>(pl->n_out) * c->catalogue);
+  pl->tile_trials = ara::kWarpTrials;
+  while (pl->tile_trials > 1) {
+    const int64_t tiles = (pl->n_out + pl->tile_trials - 1) / pl->tile_trials;
+    const double half = recs_trial * (pl->tile_trials / 2);
+    if (!(half >= 512.0 || tiles < warps || (tiles < 3 * warps && half >= 128.0))) break;
+    pl->tile_trials /= 2;
+  }
+  pl->n_tiles = (pl->n_out + pl->tile_trials - 1) / pl->tile_trials;
   pl->e0 = c->h_off[t0];
   const int64_t e1 = c->h_off[t1];
   if ((rc = reserve(c, c->ev_buf, sizeof(uint2) * (e1 - pl->e0 + 1))) ||
@@ -826,6 +844,7 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   g.t_begin = t0;
   g.t_end = t1;
   g.n_tiles = pl->n_tiles;
+  g.tile_trials = pl->tile_trials;
   g.e0 = pl->e0;
   g.rankdir = ix.rankdir;
   g.n_words = n_words;
@@ -835,8 +854,8 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   g.ev_buf = static_cast<uint2*>(c->ev_buf.ptr);
   g.tile_cnt = static_cast<uint32_t*>(c->tile_cnt.ptr);
   g.queue = static_cast<unsigned long long*>(c->counters.ptr) + 4;
-  const int64_t warps_per_sm = ara::kGatherThreads / 32;
-  pl->grid = static_cast<int>(std::min<int64_t>(c->num_sms, (pl->n_tiles + warps_per_sm - 1) / warps_per_sm));
+  // a CTA of 32 warps on each SM, or at least 8 tiles a CTA
+  pl->grid = static_cast<int>(std::min<int64_t>(c->num_sms, (pl->n_tiles + 7) / 8));
   return ARA_OK;
 }
 
@@ -915,6 +934,7 @@ static int emit_event_rows(ara_ctx* c, const PassPlan& pl, const ara::LossParams
   q.t_begin = p.t_begin;
   q.t_end = p.t_end;
   q.n_tiles = n_tiles;
+  q.tile_trials = pl.tile_trials;
   q.e0 = p.e0;
   q.ev_buf = p.ev_buf;
   q.occ = p.occ;
@@ -983,6 +1003,7 @@ static int run_layer_impl(ara_ctx* c, const ara_layer* L, uint64_t seed, int64_t
   p.t_begin = t0;
   p.t_end = t1;
   p.n_tiles = pl.n_tiles;
+  p.tile_trials = pl.tile_trials;
   p.e0 = pl.e0;
   p.ev_buf = pl.g.ev_buf;
   p.tile_cnt = pl.g.tile_cnt;
@@ -1124,6 +1145,7 @@ static int run_layers_impl(ara_ctx* c, int32_t n_layers, const ara_layer* layers
   p.t_begin = t0;
   p.t_end = t1;
   p.n_tiles = pl.n_tiles;
+  p.tile_trials = pl.tile_trials;
   p.e0 = pl.e0;
   p.ev_buf = pl.g.ev_buf;
   p.tile_cnt = pl.g.tile_cnt;
@@ -1177,7 +1199,7 @@ static int run_layers_impl(ara_ctx* c, int32_t n_layers, const ara_layer* layers
   }
   const int64_t warps = ara::kBatchThreads / 32;
   auto grid_of = [&](int it, int b) {
-    const int64_t items = it == ara::kItemTrial     ? pl.n_tiles * ara::kWarpTrials
+    const int64_t items = it == ara::kItemTrial     ? pl.n_tiles * pl.tile_trials
                           : it == ara::kItemIndexed ? pl.ix.n_recs
                                                     : pl.n_tiles;
     return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(static_cast<int64_t>(c->num_sms) * b,
@@ -1547,7 +1569,7 @@ std::vector<std::pair<DevBuf*, size_t>> serve_workspace(ara_ctx* c) {
   int64_t n_recs = 0;
   for (size_t i = 0; i < sizes.size() && i < static_cast<size_t>(ARA_MAX_BATCH_ELTS); ++i) n_recs += sizes[i];
   const int64_t n_words = (static_cast<int64_t>(c->catalogue) + 31) / 32;
-  const size_t chunk_tiles = static_cast<size_t>(kServeChunk / ara::kWarpTrials + 2);
+  const size_t chunk_tiles = static_cast<size_t>(kServeChunk + 2);  // of one trial each at most
   std::vector<std::pair<DevBuf*, size_t>> w = {
       {&c->ev_buf, sizeof(uint2) * static_cast<size_t>(max_ev + 1)},
       {&c->tile_cnt, sizeof(uint32_t) * chunk_tiles},

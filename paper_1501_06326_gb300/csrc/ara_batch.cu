@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kBatchThreads, kBatchBlocksPerSm) k_losses_bat
   unsigned long long nc = 0ull;
   uint32_t n_pairs = 0;
   for (int l = 0; l < nl; ++l) ws.acc[l][lane] = 0ull;
-  const int64_t n_items = kPerTrial ? p.n_tiles * kWarpTrials : p.n_tiles;
+  const int64_t n_items = kPerTrial ? p.n_tiles * p.tile_trials : p.n_tiles;
 
   // items are claimed one ahead, so that the claim's latency overlaps an item's work
   unsigned long long next = 0ull;
@@ -325,10 +325,10 @@ __global__ void __launch_bounds__(kBatchThreads, kBatchBlocksPerSm) k_losses_bat
     const int64_t item = static_cast<int64_t>(__shfl_sync(0xffffffffu, next, 0));
     if (item >= n_items) break;
     if (lane == 0) next = atomicAdd(&p.counters[0], 1ull);
-    const int64_t tile = kPerTrial ? item / kWarpTrials : item;
-    const uint32_t tl0 = kPerTrial ? static_cast<uint32_t>(item % kWarpTrials) : 0u;  // the item's first trial
-    const int64_t ta = p.t_begin + tile * kWarpTrials;
-    const int ntr = static_cast<int>((ta + kWarpTrials < p.t_end) ? kWarpTrials : p.t_end - ta);
+    const int64_t tile = kPerTrial ? item / p.tile_trials : item;
+    const uint32_t tl0 = kPerTrial ? static_cast<uint32_t>(item % p.tile_trials) : 0u;  // the item's first trial
+    const int64_t ta = p.t_begin + tile * p.tile_trials;
+    const int ntr = static_cast<int>((ta + p.tile_trials < p.t_end) ? p.tile_trials : p.t_end - ta);
     if (kPerTrial && static_cast<int>(tl0) >= ntr) continue;
     const int t_lo = static_cast<int>(tl0);  // the item's (first) trial in the tile
     // per trial of the item, the layers whose trials reach it (all of them unless a layer ends early)
@@ -664,8 +664,8 @@ __global__ void __launch_bounds__(kBatchThreads, kDenseBlocksPerSm)
     const int64_t tile = static_cast<int64_t>(__shfl_sync(0xffffffffu, next, 0));
     if (tile >= p.n_tiles) break;
     if (lane == 0) next = atomicAdd(&p.counters[0], 1ull);
-    const int64_t ta = p.t_begin + tile * kWarpTrials;
-    const int ntr = static_cast<int>((ta + kWarpTrials < p.t_end) ? kWarpTrials : p.t_end - ta);
+    const int64_t ta = p.t_begin + tile * p.tile_trials;
+    const int ntr = static_cast<int>((ta + p.tile_trials < p.t_end) ? p.tile_trials : p.t_end - ta);
     uint32_t any = 0u;
 #pragma unroll
     for (int t = 0; t < kWarpTrials; ++t) {

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kEventRowsThreads) k_event_rows(const EventRow
   terms.rd = q.agg_r;
   terms.ld = q.agg_l;
   for (int64_t tile = warp; tile < q.n_tiles; tile += n_warps) {
-    const int64_t ta = q.t_begin + tile * kWarpTrials;
+    const int64_t ta = q.t_begin + tile * q.tile_trials;
     const int64_t rb = __ldg(&q.off[ta]) - q.e0;
     const uint32_t n = __ldg(&q.tile_cnt[tile]);
     const int64_t row0 = __ldg(&q.row_base[tile]);

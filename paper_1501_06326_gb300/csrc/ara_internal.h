@@ -137,7 +137,7 @@ size_t index_scan_words(int64_t n_words);
 cudaError_t build_layer_index(const LayerEltRefs& refs, LayerIndex& ix, cudaStream_t s, int* n_launch);
 
 // --------------------------------------------------------------- main kernels
-// The layer runs as two kernels over tiles of kWarpTrials consecutive trials:
+// The layer runs as two kernels over tiles of up to kWarpTrials consecutive trials:
 //   k_gather  streams the YET, filters the events, resolves the hits and writes
 //             one 8-byte record per hit event into the tile's region of an
 //             event buffer (the region of a tile starts at its first event);
@@ -152,13 +152,14 @@ constexpr uint32_t kRecTrialShift = 28;
 constexpr uint32_t kRecCntShift = 22;
 constexpr uint32_t kRecCntMask = 63u;
 constexpr uint32_t kRecKMask = (1u << 22) - 1u;
-constexpr int kWarpTrials = 8;        // trials per tile (< 32)
+constexpr int kWarpTrials = 8;        // trials per tile, at most (a record's trial field and the kernels' sums)
 constexpr int kMaxTrialEvents = 1 << 22;
 
 struct GatherParams {
   const int64_t* off;
   const int32_t* ids;
   int64_t t_begin, t_end, n_tiles;
+  int32_t tile_trials;  // trials per tile, 1 .. kWarpTrials
   int64_t e0;  // off[t_begin]: the event buffer is indexed from here
   const uint2* rankdir;
   int64_t n_words;
@@ -173,6 +174,7 @@ struct GatherParams {
 struct LossParams {
   const int64_t* off;
   int64_t t_begin, t_end, n_tiles;
+  int32_t tile_trials;  // trials per tile, 1 .. kWarpTrials
   int64_t e0;
   const uint2* ev_buf;
   const uint32_t* tile_cnt;
@@ -207,6 +209,7 @@ constexpr int kBatchBlocksPerSm = 4;
 struct BatchParams {
   const int64_t* off;
   int64_t t_begin, t_end, n_tiles;
+  int32_t tile_trials;  // trials per tile, 1 .. kWarpTrials
   int64_t e0;
   const uint2* ev_buf;
   const uint32_t* tile_cnt;
@@ -258,6 +261,7 @@ cudaError_t launch_losses(const LossParams& p, int grid, cudaStream_t s);
 struct EventRowsParams {
   const int64_t* off;
   int64_t t_begin, t_end, n_tiles, e0;
+  int32_t tile_trials;
   const uint2* ev_buf;
   const float* occ;
   const uint32_t* tile_cnt;

@@ -315,8 +315,8 @@ __global__ void __launch_bounds__(kGatherThreads, 1) k_gather(const GatherParams
     if (lane == 0) tile = static_cast<int64_t>(atomicAdd(p.queue, 1ull));
     tile = __shfl_sync(0xffffffffu, tile, 0);
     if (tile >= p.n_tiles) break;
-    const int64_t ta = p.t_begin + tile * kWarpTrials;
-    const int64_t tb = (ta + kWarpTrials < p.t_end) ? ta + kWarpTrials : p.t_end;
+    const int64_t ta = p.t_begin + tile * p.tile_trials;
+    const int64_t tb = (ta + p.tile_trials < p.t_end) ? ta + p.tile_trials : p.t_end;
     const int ntr = static_cast<int>(tb - ta);
     const int64_t ea = __ldg(&p.off[ta]);
     GatherTile g;
@@ -713,8 +713,8 @@ __global__ void __launch_bounds__(kLossThreads, kLossBlocksPerSm) k_losses(const
     if (lane == 0) tile = static_cast<int64_t>(atomicAdd(&p.counters[0], 1ull));
     tile = __shfl_sync(0xffffffffu, tile, 0);
     if (tile >= p.n_tiles) break;
-    const int64_t ta = p.t_begin + tile * kWarpTrials;
-    const int64_t tb = (ta + kWarpTrials < p.t_end) ? ta + kWarpTrials : p.t_end;
+    const int64_t ta = p.t_begin + tile * p.tile_trials;
+    const int64_t tb = (ta + p.tile_trials < p.t_end) ? ta + p.tile_trials : p.t_end;
     const int ntr = static_cast<int>(tb - ta);
     const int64_t rb = __ldg(&p.off[ta]) - p.e0;  // the tile's first event buffer entry
     const uint2* recs = p.ev_buf + rb;

@@ -496,6 +496,35 @@ def test_gather_groups(eng, catalogue, density):
         check_ylt(ylt, ref)
 
 
+@pytest.mark.parametrize("n,lo,hi", [(1, 0, 60), (9, 500, 2_000), (401, 300, 900), (3_649, 0, 12), (21_901, 0, 80),
+                                     (30_003, 20, 50)])
+def test_tile_sizes(eng, n, lo, hi):
+    """Tiles of one to eight trials (few trials, many records a trial): a trial's
+    hits and loss do not depend on the tile that it falls in, so a whole run and
+    runs over pieces of it (other tile sizes, other first trials) give the same
+    bits, alone and in a batched pass; the ends against the oracle."""
+    rng = np.random.default_rng(n)
+    offsets = np.zeros(n + 1, np.int64)
+    offsets[1:] = np.cumsum(rng.integers(lo, hi, n))
+    pool = synth.make_elt_pool(3, 700, 1_000, 12)
+    yet = synth.YET(offsets, rng.integers(0, 1_000, int(offsets[-1])).astype(np.int32), 1_000)
+    terms = (100.0, 1e6, 1e3, 1e9)
+    ylt, hits, hh = run_gpu(eng, yet, pool, terms, seed=4, t0=0, t1=n)
+    many = np.empty((2, n))
+    ids = [int(i) for i in pool.elt_ids]
+    eng.run_layers([(ids, terms), (ids[:1], terms)], 4, 0, n, many)
+    assert np.array_equal(hits[:5], oracle.run_layer(yet, pool, terms, seed=4, trials=np.arange(0, min(n, 5)))["hits"])
+    for t0, t1 in ((0, min(n, 5)), (n // 3, n), (max(0, n - 40), n)):
+        part, h, hash_ = run_gpu(eng, yet, pool, terms, seed=4, t0=t0, t1=t1)
+        assert np.array_equal(part, ylt[t0:t1]) and np.array_equal(h, hits[t0:t1])
+        assert np.array_equal(hash_, hh[t0:t1])
+        if t1 - t0 <= 40:
+            check_ylt(part, oracle.run_layer(yet, pool, terms, seed=4, trials=np.arange(t0, t1)))
+        sub = np.empty((2, t1 - t0))
+        eng.run_layers([(ids, terms), (ids[:1], terms)], 4, t0, t1, sub)
+        assert np.array_equal(sub, many[:, t0:t1])
+
+
 @pytest.mark.parametrize("n", [1, 31, 33, 4_095, 4_096, 4_129])
 def test_table_blocks(eng, n):
     """Quantile tables at the edges of the builder's blocks (32 records) and of
