@@ -1176,7 +1176,7 @@ static int run_layers_impl(ara_ctx* c, int32_t n_layers, const ara_layer* layers
                                       static_cast<int64_t>(std::lround(4.0 * std::log2(recs_per_trial + 1.0)))};
   const int dense_max = ara::losses_dense_blocks_per_sm(n_layers);
   if (dense_max < 1) return fail(c, ARA_ECUDA, "%s: the dense losses kernel fits no SM", who);
-  const int idx_max = c->yix_ready ? ara::losses_indexed_blocks_per_sm() : 0;
+  const int idx_max = c->yix_ready ? ara::losses_indexed_blocks_per_sm(n_layers) : 0;
   if (c->yix_ready && idx_max < 1) return fail(c, ARA_ECUDA, "%s: the indexed losses kernel fits no SM", who);
   auto max_blocks = [&](int it) {
     return it == ara::kItemDense ? dense_max : it == ara::kItemIndexed ? idx_max : ara::kBatchBlocksPerSm;

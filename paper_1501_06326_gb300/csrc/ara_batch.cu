@@ -927,15 +927,31 @@ cudaError_t launch_losses_batch(const BatchParams& p, int item, int grid, cudaSt
 // fixed-point sum with a 64-bit atomic add: the same numbers as the other
 // work items, so the same bits.  A second kernel turns the sums into year
 // losses.
+//
+// Cost: issue (70% of the slots; Philox, Phi^-1 and the table are most of the
+// ~350 instructions a window of 32 occurrences) and, before, the adds: L2 takes
+// 8-byte adds to scattered sectors at 210 G/s at most, two in a sector at 360,
+// four at 450.  So a trial's sums stand side by side, and the adds of a window
+// go by lanes of four with three or more layers (a lane a layer).  Events of
+// one pair with an exact table, nearly all, keep the pair's fields in registers
+// over their windows, and the next window is loaded ahead.  16 layers over 64
+// ELTs, 1M trials of 1,000 events: 4,200 us, 5,195 with an add per layer from
+// each occurrence's lane, sums by layer and the fields loaded per window.
+// 32 warps an SM (64 registers, a few spilled outside the window) against 28:
+// 4,200 and 4,330 us; 36: 4,315.
 namespace {
 
 constexpr int kIdxThreads = 128;
-constexpr int kIdxBlocksPerSm = 7;
+constexpr int kIdxBlocksPerSm = 8;
 constexpr int kIdxClaim = 8;  // events a warp claims at a time
 
 struct IdxWarp {
-  float gacc[kBatchLayers][32];      // per layer and lane: the running sum of an occurrence's pair losses
   uint32_t pmask[kMaxIndexElts];     // the event's pairs: layers holding their ELTs
+  float4 held[32];                   // the layers that the event serves, ascending: occurrence terms, scale, byte offset
+                                     // in a trial's sums
+  uint32_t last[32];                 // ... their last trials
+  uint32_t trial[32];                // a window's trials
+  uint32_t lay[32];                  // ... and their numbers
   uint4 meta[2 * kIdxClaim];         // the claimed events: [j] (first pair, pair end, range of the slice's first
                                      // occurrence), [kIdxClaim + j] (range of its end, -, -)
   int64_t span[2];                   // the trials of the claim's slice
@@ -990,21 +1006,32 @@ __global__ void __launch_bounds__(kIdxThreads, kIdxBlocksPerSm)
   __shared__ DenseShared ds;
   const uint32_t lane = lane_id();
   IdxWarp& ws = iwarp[threadIdx.x >> 5];
+  // per warp, layer and lane: the running sum of an occurrence's pair losses (of events of several pairs)
+  extern __shared__ float4 idx_gacc[];
+  float (*gacc)[32] = reinterpret_cast<float (*)[32]>(idx_gacc) + (threadIdx.x >> 5) * p.n_layers;
   load_dense_shared(p, ds);
   __syncthreads();
   const int nl = p.n_layers;
-  const int64_t t0 = p.t_begin, stride = p.t_end - p.t_begin;
+  const int64_t t0 = p.t_begin;
   int64_t t_full = p.t_end;  // below it every layer reaches the trial
   for (int l = 0; l < nl; ++l) t_full = min(t_full, ds.t_end[l]);
   const uint32_t all = nl >= 32 ? 0xffffffffu : (1u << nl) - 1u;
-  for (int l = 0; l < nl; ++l) ws.gacc[l][lane] = 0.0f;
+  for (int l = 0; l < nl; ++l) gacc[l][lane] = 0.0f;
   const uint32_t n_u = *q.n_u;
+  const uint32_t row_bytes = 8u * static_cast<uint32_t>(nl);
+  char* const acc0 = reinterpret_cast<char*>(q.acc - t0 * nl);
   unsigned long long nc = 0ull;
   uint32_t n_pairs = 0;
   // the occurrences (read once) are the first to leave L2, so that the trials' sums, which the atomic
   // adds revisit, stay (batched-16: 5.98 against 6.07 ms a pass)
   uint64_t occ_pol;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(occ_pol));
+
+  auto load_occ = [&](const unsigned long long* at) {
+    unsigned long long o;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u64 %0, [%1], %2;" : "=l"(o) : "l"(at), "l"(occ_pol));
+    return o;
+  };
 
   // the queue's groups: kIdxClaim events over one trial slice, every event of a slice before the next
   // slice, so that the sums being added to stay within a slice's trials; a warp moves to the next slice
@@ -1055,60 +1082,129 @@ __global__ void __launch_bounds__(kIdxThreads, kIdxBlocksPerSm)
       const uint32_t lo = first_occ_at(q.occ, m4.z, m4.w, ws.span[0], lane);
       const uint32_t hi = first_occ_at(q.occ, max(lo, h4.x), h4.y, ws.span[1], lane);
       if (lo >= hi) continue;
-      for (uint32_t j = lane; j < cnt; j += 32) ws.pmask[j] = ds.layers_of[pair_pos(p.hot[ps + j].meta)];
+      uint32_t touched = 0u;  // the event's layers
+      for (uint32_t j = lane; j < cnt; j += 32) {
+        const uint32_t m = ds.layers_of[pair_pos(p.hot[ps + j].meta)];
+        ws.pmask[j] = m;
+        touched |= m;
+      }
+      touched = __reduce_or_sync(0xffffffffu, touched);
+      const int n_held = __popc(touched);
+      if ((touched >> lane) & 1u) {
+        const int at = __popc(touched & ((1u << lane) - 1u));
+        const float4 oc = ds.occ[lane];
+        ws.held[at] = make_float4(oc.x, oc.y, oc.z, __uint_as_float(8u * lane));
+        ws.lay[at] = lane;
+        ws.last[at] = static_cast<uint32_t>(ds.t_end[lane] - 1);
+      }
       __syncwarp();
-      for (uint32_t r = lo; r < hi; r += 32) {
-        const uint32_t i = r + lane;
-        const bool valid = i < hi;
-        unsigned long long o = 0ull;
-        if (valid)
-          asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u64 %0, [%1], %2;"
-                       : "=l"(o)
-                       : "l"(q.occ + i), "l"(occ_pol));
-        const int64_t trial = static_cast<int64_t>(o >> 32);
-        const uint32_t k = static_cast<uint32_t>(o);
-        uint32_t act = 0u;  // the layers whose trials reach this one
-        if (valid) {
-          act = all;
-          if (trial >= t_full) {
-            act = 0u;
-            for (int l = 0; l < nl; ++l)
-              if (trial < ds.t_end[l]) act |= 1u << l;
-          }
+      unsigned long long o_next = 0ull;
+      if (lo + lane < hi) o_next = load_occ(q.occ + lo + lane);
+      auto layers_at = [&](uint32_t trial) {  // the layers whose trials reach this one
+        uint32_t act = all;
+        if (trial >= t_full) {
+          act = 0u;
+          for (int l = 0; l < nl; ++l)
+            if (trial < ds.t_end[l]) act |= 1u << l;
         }
-        unsigned long long* acc = q.acc + (trial - t0);
-        if (cnt == 1u) {
-          const uint32_t m = ws.pmask[0] & act;
-          if (m) {
-            const float L = indexed_pair_loss(p, ds, ps, trial, k, &nc);
-            ++n_pairs;
-            for (uint32_t mm = m; mm; mm &= mm - 1u) {
-              const int l = __ffs(mm) - 1;
-              const float4 c = ds.occ[l];
-              const float O = clamp_terms_f(L, c.x, c.y);
-              if (O > 0.0f) atomicAdd(acc + static_cast<int64_t>(l) * stride, fixed_units(O, c.z));
+        return act;
+      };
+      auto add = [&](uint32_t tj, float G, const float4& h, uint32_t last, bool on) {
+        const float O = clamp_terms_f(G, h.x, h.y);
+        if (on && tj <= last && O > 0.0f)
+          atomicAdd(reinterpret_cast<unsigned long long*>(acc0 + (static_cast<uint64_t>(tj) * row_bytes +
+                                                                  __float_as_uint(h.w))),
+                    fixed_units(O, h.z));
+      };
+      const PairHot h0 = p.hot[ps];
+      const uint32_t kind = pair_kind(h0.meta), pos = pair_pos(h0.meta);
+      if (cnt == 1u && kind_is_beta(kind) && pair_tab_exact(h0.meta) && !p.primary_only && !p.newton_only) {
+        // most events: one pair, its loss from a table; the pair's fields stay in registers over the event
+        const bool fine = pair_fine(h0.meta);
+        const float4* const tab = (fine ? ds.tabf[pos] : ds.tab[pos]) + h0.node;
+        const uint32_t elt = ds.elt_id[pos];
+        const float ret = ds.ret[pos], lim = ds.lim[pos], share = ds.share[pos];
+        for (uint32_t r = lo; r < hi; r += 32) {
+          const uint32_t i = r + lane;
+          const unsigned long long o = o_next;
+          if (i + 32u < hi) o_next = load_occ(q.occ + i + 32u);
+          uint32_t trial = 0xffffffffu;  // above every layer's last trial
+          float L = 0.0f;
+          if (i < hi) {
+            trial = static_cast<uint32_t>(o >> 32);
+            if (touched & layers_at(trial)) {
+              ++n_pairs;
+              float t;
+              if (batch_pair_normal(p, kind, elt, ps, trial, static_cast<uint32_t>(o), &t))
+                L = share * clamp_terms_f(h0.max_l * tab_quantile_t(tab, t, fine), ret, lim);
+              else
+                L = pair_loss_slow(p, p.pairs[ps], ps, trial, static_cast<uint32_t>(o), &nc);
             }
           }
-        } else {
+          // the adds: three or four layers at a time go by lanes of four (lane c of four adds the c-th layer of the
+          // four's occurrences in turn, so that a trial's adds to one sector leave together), two by lanes of two,
+          // one by each occurrence's own lane
+          int at = 0;
+          if (n_held >= 3) {
+            uint32_t tq[4];
+            float Lq[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              tq[c] = __shfl_sync(0xffffffffu, trial, (lane & 28u) + c);
+              Lq[c] = __shfl_sync(0xffffffffu, L, (lane & 28u) + c);
+            }
+            for (; n_held - at >= 3; at += 4) {
+              const int slot = at + static_cast<int>(lane & 3u);  // at most 31
+              const float4 h = ws.held[slot];
+              const uint32_t last = ws.last[slot];
+#pragma unroll
+              for (int c = 0; c < 4; ++c) add(tq[c], Lq[c], h, last, slot < n_held);
+            }
+          }
+          if (n_held - at == 2) {
+            const float4 h = ws.held[at + (lane & 1u)];
+            const uint32_t last = ws.last[at + (lane & 1u)];
+            for (uint32_t c = 0; c < 2; ++c) {
+              const uint32_t src = (lane & 30u) + c;
+              const uint32_t tj = __shfl_sync(0xffffffffu, trial, src);
+              add(tj, __shfl_sync(0xffffffffu, L, src), h, last, true);
+            }
+          } else if (n_held - at == 1) {
+            add(trial, L, ws.held[at], ws.last[at], true);
+          }
+        }
+      } else {
+        for (uint32_t r = lo; r < hi; r += 32) {
+          const uint32_t i = r + lane;
+          const unsigned long long o = o_next;
+          if (i + 32u < hi) o_next = load_occ(q.occ + i + 32u);
+          const uint32_t trial = static_cast<uint32_t>(o >> 32);
+          const uint32_t act = i < hi ? layers_at(trial) : 0u;
           // the pairs in order: each layer's running sum is the left-to-right sum of its pairs' losses
-          uint32_t touched = 0u;
           for (uint32_t j = 0; j < cnt; ++j) {
             const uint32_t m = ws.pmask[j] & act;
             if (m) {
-              const float L = indexed_pair_loss(p, ds, ps + j, trial, k, &nc);
+              const float L = indexed_pair_loss(p, ds, ps + j, trial, static_cast<uint32_t>(o), &nc);
               ++n_pairs;
-              touched |= m;
-              for (uint32_t mm = m; mm; mm &= mm - 1u) ws.gacc[__ffs(mm) - 1][lane] += L;
+              for (uint32_t mm = m; mm; mm &= mm - 1u) gacc[__ffs(mm) - 1][lane] += L;
             }
           }
-          for (uint32_t mm = touched; mm; mm &= mm - 1u) {
-            const int l = __ffs(mm) - 1;
-            const float G = ws.gacc[l][lane];
-            ws.gacc[l][lane] = 0.0f;
-            const float4 c = ds.occ[l];
-            const float O = clamp_terms_f(G, c.x, c.y);
-            if (O > 0.0f) atomicAdd(acc + static_cast<int64_t>(l) * stride, fixed_units(O, c.z));
+          ws.trial[lane] = i < hi ? trial : 0xffffffffu;
+          __syncwarp();
+          // the adds, by lanes of four as above
+          for (int at = 0; at < n_held; at += 4) {
+            const int slot = at + static_cast<int>(lane & 3u);
+            if (slot >= n_held) continue;
+            const float4 h = ws.held[slot];
+            const uint32_t last = ws.last[slot];
+            const float4 G = *reinterpret_cast<const float4*>(&gacc[ws.lay[slot]][lane & 28u]);
+            const float Gq[4] = {G.x, G.y, G.z, G.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              add(ws.trial[(lane & 28u) + c], Gq[c], h, last, true);
           }
+          __syncwarp();
+          for (uint32_t mm = touched; mm; mm &= mm - 1u) gacc[__ffs(mm) - 1][lane] = 0.0f;
         }
       }
       __syncwarp();  // pmask is rewritten for the next event
@@ -1127,16 +1223,16 @@ namespace {
 
 __global__ void k_indexed_years(const __grid_constant__ IndexedParams q) {
   const BatchParams& p = q.b;
-  const int64_t stride = p.t_end - p.t_begin;
-  const int64_t n = stride * p.n_layers;
+  const int64_t n = p.t_end - p.t_begin;
   const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n; i += step) {
-    const int l = static_cast<int>(i / stride);
-    const int64_t tt = i - static_cast<int64_t>(l) * stride;
-    if (p.t_begin + tt < p.layer_t_end[l])
-      p.ylt_l[l][tt] = clamp_terms_d(__ull2double_rn(q.acc[i]) * p.inv_scale[l], p.agg_r[l], p.agg_l[l]);
-  }
+  for (int64_t tt = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; tt < n; tt += step)
+    for (int l = 0; l < p.n_layers; ++l)
+      if (p.t_begin + tt < p.layer_t_end[l])
+        p.ylt_l[l][tt] = clamp_terms_d(__ull2double_rn(q.acc[tt * p.n_layers + l]) * p.inv_scale[l], p.agg_r[l],
+                                       p.agg_l[l]);
 }
+
+size_t idx_smem_bytes(int n_layers) { return sizeof(float) * kIdxThreads * n_layers; }
 
 int grid_for_n(int64_t n, int threads) {
   const int64_t b = (n + threads - 1) / threads;
@@ -1145,19 +1241,19 @@ int grid_for_n(int64_t n, int threads) {
 
 }  // namespace
 
-int losses_indexed_blocks_per_sm() {
+int losses_indexed_blocks_per_sm(int n_layers) {
   int b = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_losses_indexed, kIdxThreads, 0) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_losses_indexed, kIdxThreads, idx_smem_bytes(n_layers)) != cudaSuccess) return 0;
   return b;
 }
 
 cudaError_t launch_losses_indexed(const IndexedParams& q, int grid, cudaStream_t s) {
-  k_losses_indexed<<<grid, kIdxThreads, 0, s>>>(q);
+  k_losses_indexed<<<grid, kIdxThreads, idx_smem_bytes(q.b.n_layers), s>>>(q);
   return cudaGetLastError();
 }
 
 cudaError_t launch_indexed_years(const IndexedParams& q, cudaStream_t s) {
-  k_indexed_years<<<grid_for_n((q.b.t_end - q.b.t_begin) * q.b.n_layers, 256), 256, 0, s>>>(q);
+  k_indexed_years<<<grid_for_n(q.b.t_end - q.b.t_begin, 256), 256, 0, s>>>(q);
   return cudaGetLastError();
 }
 

@@ -96,7 +96,7 @@ struct IndexedParams {
   const int32_t* u_event;         // [n_u] the union's distinct events (the index's slots), ascending
   const uint32_t* u_first;        // [n_u + 1] each one's first pair; u_first[n_u] = the pair count
   const uint32_t* n_u;            // device: the number of distinct events
-  unsigned long long* acc;        // [n_layers][t_end - t_begin] fixed-point sums (zeroed before)
+  unsigned long long* acc;        // [t_end - t_begin][n_layers] fixed-point sums (zeroed before)
   int64_t yet_trials;             // the YET's trials
   uint32_t* slice_queue;          // [indexed_slices(t_begin, t_end, slice_shift)] each slice's queue (zeroed before)
 };
@@ -106,6 +106,6 @@ __host__ __device__ inline int64_t indexed_slices(int64_t t_begin, int64_t t_end
 cudaError_t launch_losses_indexed(const IndexedParams& q, int grid, cudaStream_t s);
 // The year losses from acc: each layer's trials [t_begin, layer_t_end).
 cudaError_t launch_indexed_years(const IndexedParams& q, cudaStream_t s);
-int losses_indexed_blocks_per_sm();
+int losses_indexed_blocks_per_sm(int n_layers);
 
 }  // namespace ara

@@ -344,6 +344,34 @@ def test_indexed_pass_across_slices_and_grid_cells(eng):
         check_ylt(out[l], oracle.run_layer(yet, sub, terms, seed=8, trials=np.arange(t0, t1)))
 
 
+@pytest.mark.parametrize("n_layers", [1, 2, 3, 4, 6, 32])
+def test_indexed_layers_of_an_event(eng, n_layers):
+    """The indexed item's adds by lanes of four, two and one: ELT i serves the
+    first i + 1 layers, so events serve 1 to n_layers of them, events of one
+    pair and of several, of every kind of record, with 0 to 70 occurrences
+    (windows of 32 and what is left over); the dense item's bits."""
+    rng = np.random.default_rng(n_layers)
+    C = 1_500
+    base = synth.make_elt_pool(n_layers, 220, C, 70, recipe="stress")
+    sigma = np.where(rng.random(len(base.sigma)) < 0.1, 0.0, base.sigma).astype(base.sigma.dtype)
+    mean = np.where(rng.random(len(base.mean)) < 0.1, 0.0, base.mean).astype(base.mean.dtype)
+    pool = synth.ELTPool(elt_ids=base.elt_ids, rec_offsets=base.rec_offsets, event_ids=base.event_ids, mean=mean,
+                         sigma=sigma, exposure=base.exposure, terms=base.terms)
+    ev = np.repeat(np.arange(C), rng.integers(0, 71, C)).astype(np.int32)
+    rng.shuffle(ev)
+    n = 5_003
+    offsets = np.zeros(n + 1, np.int64)
+    offsets[1:] = np.sort(rng.integers(0, len(ev) + 1, n))
+    offsets[-1] = len(ev)
+    yet = synth.YET(offsets, ev, C)
+    ids = pool.elt_ids
+    layers = [(ids[l:], (50.0 * l, 4e5, 1e2, 5e7), None) for l in range(n_layers)]
+    for kw in ({}, {"primary_only": True}):
+        out = _assert_same_bits(_run_items(eng, yet, pool, layers, 3, **kw))
+        assert np.count_nonzero(out[0]) > 0
+    _assert_same_bits(_run_items(eng, yet, pool, layers, 3, 17, 4_001))
+
+
 def test_yet_index_by_radix_sort_where_an_event_is_frequent(eng):
     """An event in every trial of a 3,000-trial YET (a bucket of 3,000
     occurrences, above the bucket build's 2,048) has the index built by the
