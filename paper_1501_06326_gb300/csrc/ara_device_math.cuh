@@ -236,17 +236,31 @@ __device__ __forceinline__ float tab_increment(float s, float dw, float d0, floa
 // x = InvCDF_beta(Phi(t)) from a record's table (nodes are float4 {x_i,
 // w_{i+1} - w_i, h w'_i, h^2 w''_i} on a grid in t); `fine` selects the 8x
 // refined grid.  t outside the grid's range [-T1, T1] is clamped to it.
-__device__ __forceinline__ float tab_quantile_t(const float4* __restrict__ tab, float t, bool fine) {
+// The interval of a table that holds t, and the place in it.
+struct TabPlace {
+  int i;
+  float s;
+};
+__device__ __forceinline__ TabPlace tab_place(float t, bool fine) {
   const int nseg = fine ? kTabFineNodes - 1 : kTabNodes - 1;
   float u = (t + kTabT1f) * (fine ? kTabInvH * kTabRefine : kTabInvH);
   u = fminf(fmaxf(u, 0.0f), static_cast<float>(nseg));
   int i = static_cast<int>(u);
   if (i > nseg - 1) i = nseg - 1;
-  const float s = u - static_cast<float>(i);
-  const float4 n0 = __ldg(tab + i);
+  return {i, u - static_cast<float>(i)};
+}
+
+// The value there: n0 the interval's node, n1 the second half of the next one.
+__device__ __forceinline__ float tab_value(float s, float4 n0, float2 n1) {
   if (!(n0.x > 0.0f)) return 0.0f;  // below the FP32 range
-  const float2 n1 = __ldg(reinterpret_cast<const float2*>(tab + i + 1) + 1);
   return n0.x * expf(tab_increment(s, n0.y, n0.z, n0.w, n1.x, n1.y));
+}
+
+__device__ __forceinline__ float tab_quantile_t(const float4* __restrict__ tab, float t, bool fine) {
+  const TabPlace at = tab_place(t, fine);
+  const float4 n0 = __ldg(tab + at.i);
+  if (!(n0.x > 0.0f)) return 0.0f;
+  return tab_value(at.s, n0, __ldg(reinterpret_cast<const float2*>(tab + at.i + 1) + 1));
 }
 
 // x = InvCDF_beta(z) from a record's table.

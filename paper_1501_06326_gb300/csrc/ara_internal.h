@@ -175,6 +175,7 @@ struct LossParams {
   const int64_t* off;
   int64_t t_begin, t_end, n_tiles;
   int32_t tile_trials;  // trials per tile, 1 .. kWarpTrials
+  int32_t windows;      // take all events in windows of 32 pairs
   int64_t e0;
   const uint2* ev_buf;
   const uint32_t* tile_cnt;

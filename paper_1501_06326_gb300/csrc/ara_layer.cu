@@ -54,8 +54,8 @@ __device__ __forceinline__ T warp_inclusive_scan(T v) {
 // inverse Beta through the record's quantile table, ELT and occurrence terms,
 // and a double-float add into the lane's sum for the event's trial.  Events
 // with several pairs are queued and processed in windows of 32 pairs with a
-// segmented sum.  Events with a pair whose record's table is not exact are
-// deferred and resolved, 32 at a time, by the FP32 Halley iteration.  At the
+// segmented sum; layers of many pairs an event take all events so.  Events
+// with a pair whose record's table is not exact are deferred and resolved, 32 at a time, by the FP32 Halley iteration.  At the
 // end of a tile a reduce-scatter over the lanes gives the trials' sums, and
 // the aggregate terms turn each into the trial's year loss.
 
@@ -566,88 +566,135 @@ struct EltShared {
   float ret[32], lim[32], share[32];
 };
 
-// Loss after ELT terms of one pair from its hot record, for the table path;
-// returns false when the pair needs the Halley iteration.
-__device__ __forceinline__ bool pair_fast_hot(const LossParams& p, const EltShared& es, const PairHot& h, uint32_t pi,
-                                              int64_t trial, uint32_t k, float* out) {
-  const uint32_t kind = pair_kind(h.meta);
-  const uint32_t pos = pair_pos(h.meta);
-  float loss = h.mu;
-  if (kind == kKindZero) {
-    loss = 0.0f;
-  } else if (!p.primary_only && kind_is_beta(kind)) {
-    if (p.newton_only || !pair_tab_exact(h.meta)) return false;
-    float t;
-    if (!pair_normal(p, kind, es.elt_id[pos], pi, trial, k, &t)) return false;
-    const bool fine = pair_fine(h.meta);
-    const float4* tb = (fine ? es.tabf[pos] : es.tab[pos]) + h.node;
-    loss = h.max_l * tab_quantile_t(tb, t, fine);
-  }
-  *out = es.share[pos] * clamp_terms_f(loss, es.ret[pos], es.lim[pos]);
-  return true;
+// A window: up to 32 pairs of whole events, one per lane.  Of lane q < np: its
+// event's record (x, y), the event's first lane and its place among the
+// window's events.
+struct PairWindow {
+  uint32_t ex, ey, epre, ev, np;
+  int n_take;  // events
+};
+
+// The window of the first events of lanes' records (cnt: lane's event's pairs, 0 beyond the last).
+__device__ __forceinline__ PairWindow make_window(uint2 r, uint32_t cnt) {
+  const uint32_t q = lane_id();
+  PairWindow w;
+  const uint32_t incl = warp_inclusive_scan(cnt);
+  const uint32_t pre = incl - cnt;
+  const bool take = cnt != 0 && incl <= 32u;
+  w.n_take = __popc(__ballot_sync(0xffffffffu, take));
+  w.np = w.n_take > 0 ? __shfl_sync(0xffffffffu, incl, w.n_take - 1) : 0u;
+  const uint32_t starts = __reduce_or_sync(0xffffffffu, take ? (1u << pre) : 0u);
+  // lane q's event: the last start at or below q
+  w.ev = static_cast<uint32_t>(__popc(starts & (0xffffffffu >> (31u - q)))) - 1u;
+  w.ex = __shfl_sync(0xffffffffu, r.x, w.ev);
+  w.ey = __shfl_sync(0xffffffffu, r.y, w.ev);
+  w.epre = __shfl_sync(0xffffffffu, pre, w.ev);
+  return w;
 }
 
-// The queued multi-ELT events, in windows of at most 32 pairs (one per lane):
-// losses of the pairs, a segmented sum per event (pairs in layer order), the
-// occurrence terms at each event's last lane.  Returns (deferred list length,
+// A pair's loss between its two halves: known (kLossKnown: a), or from a table
+// interval (kLossTable: a = max_l, s the place in the interval n0, n1), or by
+// the Halley iteration (kLossSlow).
+enum : uint32_t { kLossKnown = 0, kLossTable = 1, kLossSlow = 2 };
+struct PairEval {
+  uint32_t mode, pos;  // pos: the pair's ELT position
+  float a, s;
+  float4 n0;
+  float2 n1;
+};
+
+// The first half, for lanes with `in`: the pair's normal and the loads of its
+// table interval.  Callers put what they have to do for the next pairs between
+// the halves, so that the loads are not waited for.
+__device__ __forceinline__ PairEval pair_begin(const LossParams& p, const EltShared& es, LossWarp& ws, bool in,
+                                               const PairHot& h, uint32_t pi, int64_t ta, uint32_t key, bool diag) {
+  PairEval e{kLossKnown, pair_pos(h.meta), 0.0f, 0.0f, make_float4(0.0f, 0.0f, 0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+  if (in) {
+    const uint32_t tl = key >> kRecTrialShift, k = key & kRecKMask;
+    const uint32_t kind = pair_kind(h.meta);
+    e.a = kind == kKindZero ? 0.0f : h.mu;
+    if (!p.primary_only && kind_is_beta(kind)) {
+      float t;
+      if (p.newton_only || !pair_tab_exact(h.meta) || !pair_normal(p, kind, es.elt_id[e.pos], pi, ta + tl, k, &t)) {
+        e.mode = kLossSlow;
+      } else {
+        const bool fine = pair_fine(h.meta);
+        const TabPlace at = tab_place(t, fine);
+        const float4* node = (fine ? es.tabf[e.pos] : es.tab[e.pos]) + h.node + at.i;
+        e.mode = kLossTable;
+        e.a = h.max_l;
+        e.s = at.s;
+        e.n0 = __ldg(node);
+        e.n1 = __ldg(reinterpret_cast<const float2*>(node + 1) + 1);
+      }
+    }
+    if (diag) {
+      const uint32_t elt = es.elt_id[e.pos];
+      atomicAdd(&ws.hits[tl], 1ull);
+      atomicAdd(&ws.hash[tl], static_cast<unsigned long long>(fmix64((static_cast<uint64_t>(k) << 32) | elt)));
+    }
+  }
+  return e;
+}
+
+// The second half: the pair's loss after ELT terms (meaningless for kLossSlow).
+__device__ __forceinline__ float pair_end(const EltShared& es, const PairEval& e) {
+  float loss = e.a;
+  if (e.mode == kLossTable) loss = e.a * tab_value(e.s, e.n0, e.n1);
+  return es.share[e.pos] * clamp_terms_f(loss, es.ret[e.pos], es.lim[e.pos]);
+}
+
+// A window's second half: the pairs' losses, a segmented sum per event (pairs
+// in layer order), the occurrence terms at each event's last lane.  rec
+// (kEmit): the lane's event's record's place in the tile.  Returns the deferred
+// list's length.
+template <bool kEmit>
+__device__ __forceinline__ int window_end(const LossParams& p, const EltShared& es, LossWarp& ws, int nd,
+                                          const PairWindow& w, const PairEval& e, int64_t ta, int64_t rb,
+                                          uint32_t rec) {
+  const uint32_t q = lane_id();
+  const uint32_t ecnt = ((w.ex >> kRecCntShift) & kRecCntMask) + 1u;
+  const uint32_t etl = w.ex >> kRecTrialShift;
+  float L = pair_end(es, e);
+  // segmented inclusive sum within each event's lanes
+#pragma unroll
+  for (uint32_t d = 1; d < 32; d <<= 1) {
+    const float o = __shfl_up_sync(0xffffffffu, L, d);
+    if (q >= w.epre + d) L += o;
+  }
+  const uint32_t smask = __ballot_sync(0xffffffffu, e.mode == kLossSlow);
+  const bool end = q < w.np && q == w.epre + ecnt - 1u;
+  const bool seg_slow = ((smask >> w.epre) & (0xffffffffu >> (31u - (q - w.epre)))) != 0u;
+  if (end && !seg_slow) {
+    const float O = clamp_terms_f(L, p.occ_r, p.occ_l);
+    acc_add(ws, etl, O);
+    if constexpr (kEmit) p.occ[rb + rec] = O;
+  }
+  return defer_events<kEmit>(p, ws, nd, end && seg_slow, make_uint2(w.ex, w.ey), ta + etl - p.t_begin, rb + rec);
+}
+
+// The queued multi-ELT events, in windows.  Returns (deferred list length,
 // pairs processed).  kEmit: the occurrence losses also go beside the records
 // (the tile's records start at event buffer entry rb).
 template <bool kEmit>
 __device__ __forceinline__ int2 process_multi(const LossParams& p, const EltShared& es, LossWarp& ws, int nd, int nq,
                                               int64_t ta, bool diag, int64_t rb) {
   const uint32_t q = lane_id();
-  const uint32_t upto = 0xffffffffu >> (31u - q);  // lanes 0..q
   int n_pairs = 0;
 #pragma unroll 1
   for (int i0 = 0; i0 < nq;) {
     const int ie = i0 + static_cast<int>(q);
     const uint2 r = (ie < nq) ? ws.mq[ie] : make_uint2(0u, 0u);
-    const uint32_t cnt = (ie < nq) ? ((r.x >> kRecCntShift) & kRecCntMask) + 1u : 0u;
-    const uint32_t incl = warp_inclusive_scan(cnt);
-    const uint32_t pre = incl - cnt;
-    const bool take = cnt != 0 && incl <= 32u;
-    const int n_take = __popc(__ballot_sync(0xffffffffu, take));
-    const uint32_t np = __shfl_sync(0xffffffffu, incl, n_take - 1);
-    const uint32_t starts = __reduce_or_sync(0xffffffffu, take ? (1u << pre) : 0u);
-    // lane q's event: the last start at or below q
-    const uint32_t ev = static_cast<uint32_t>(__popc(starts & upto)) - 1u;
-    const uint32_t ex = __shfl_sync(0xffffffffu, r.x, ev);
-    const uint32_t ey = __shfl_sync(0xffffffffu, r.y, ev);
-    const uint32_t epre = __shfl_sync(0xffffffffu, pre, ev);
-    const uint32_t ecnt = __shfl_sync(0xffffffffu, cnt, ev);
-    const uint32_t etl = ex >> kRecTrialShift, ek = ex & kRecKMask;
-    float L = 0.0f;
-    bool slow = false;
-    if (q < np) {
-      const uint32_t pi = ey + (q - epre);
-      const PairHot h = p.hot[pi];
-      slow = !pair_fast_hot(p, es, h, pi, ta + etl, ek, &L);
-      if (diag) {
-        const uint32_t elt = es.elt_id[pair_pos(h.meta)];
-        atomicAdd(&ws.hits[etl], 1ull);
-        atomicAdd(&ws.hash[etl], static_cast<unsigned long long>(fmix64((static_cast<uint64_t>(ek) << 32) | elt)));
-      }
-    }
-    n_pairs += static_cast<int>(np);
-    // segmented inclusive sum within each event's lanes
-#pragma unroll
-    for (uint32_t d = 1; d < 32; d <<= 1) {
-      const float o = __shfl_up_sync(0xffffffffu, L, d);
-      if (q >= epre + d) L += o;
-    }
-    const uint32_t smask = __ballot_sync(0xffffffffu, slow);
-    const bool end = q < np && q == epre + ecnt - 1u;
-    const bool seg_slow = ((smask >> epre) & (0xffffffffu >> (31u - (q - epre)))) != 0u;
-    if (end && !seg_slow) {
-      const float O = clamp_terms_f(L, p.occ_r, p.occ_l);
-      acc_add(ws, etl, O);
-      if constexpr (kEmit) p.occ[rb + ws.mqi[i0 + ev]] = O;
-    }
-    int64_t idx = 0;  // lane q < np holds a pair of queue entry i0 + ev; only event ends read it
+    const PairWindow w = make_window(r, (ie < nq) ? ((r.x >> kRecCntShift) & kRecCntMask) + 1u : 0u);
+    PairHot h{0.0f, 0.0f, kKindZero << kMetaKindShift, 0u};
+    if (q < w.np) h = p.hot[w.ey + (q - w.epre)];
+    n_pairs += static_cast<int>(w.np);
+    const PairEval e = pair_begin(p, es, ws, q < w.np, h, w.ey + (q - w.epre), ta, w.ex, diag);
+    uint32_t rec = 0u;
     if constexpr (kEmit)
-      if (end) idx = rb + ws.mqi[i0 + ev];
-    nd = defer_events<kEmit>(p, ws, nd, end && seg_slow, make_uint2(ex, ey), ta + etl - p.t_begin, idx);
-    i0 += n_take;
+      if (q < w.np) rec = ws.mqi[i0 + w.ev];
+    nd = window_end<kEmit>(p, es, ws, nd, w, e, ta, rb, rec);
+    i0 += w.n_take;
   }
   __syncwarp();
   return make_int2(nd, n_pairs);
@@ -672,17 +719,29 @@ __device__ __forceinline__ void reduce_scatter_stage(float (&h)[kWarpTrials], fl
 
 }  // namespace
 
-// k_losses: each warp takes tiles and reads their event records one per lane
-// (the records two rounds ahead and the hot pair records one round ahead are
-// in flight).  An event with one (event, ELT) pair -- nearly all of them -- is
-// finished by its lane: Philox uniform, inverse Beta through the record's
-// quantile table, ELT terms, occurrence terms, and a double-float add into the
-// lane's sum for the event's trial.  Events with several pairs are queued and
-// processed in windows of 32 pairs with a segmented sum.  At the end of the
-// tile one reduce-scatter over the lanes turns the per-lane sums into the
-// trials' sums.  kEmit (per-event output) also stores each hit event's
-// occurrence loss beside its record.
-template <bool kEmit>
+// k_losses: each warp takes tiles and sums their events' occurrence losses: per
+// pair the Philox uniform, the inverse Beta through the record's quantile table
+// and the ELT terms, per event the occurrence terms and a double-float add into
+// the lane's sum for the event's trial.  At the end of the tile one
+// reduce-scatter over the lanes turns the per-lane sums into the trials' sums.
+// kEmit (per-event output) also stores each hit event's occurrence loss beside
+// its record.
+//
+// !kWindows: a lane per event record (the records two rounds ahead and the hot
+// pair records one round ahead are in flight); events with several pairs are
+// queued and processed in windows of 32 pairs with a segmented sum.  For layers
+// where nearly all hit events have one pair.
+// kWindows: every event in windows of up to 32 pairs of whole events, a lane
+// per pair, laid out from the records as they come.
+//
+// Bound by the latency of the table intervals (random 24-byte reads, past L1)
+// with 24 warps an SM, then by L1's rate of misses: so each pair is computed in
+// two halves, its interval's loads and its loss, and the next round or window
+// is prepared between them.  1M trials of 75 pairs, a lane per event: 1,005 us
+// (1,030 with the loads waited for); 100,003 trials of 750 pairs over 30 ELTs of
+// 100,000 events, in windows: 1,140 us (1,740 with a lane per event and the
+// events of several pairs, most of them there, queued).
+template <bool kEmit, bool kWindows>
 __global__ void __launch_bounds__(kLossThreads, kLossBlocksPerSm) k_losses(const LossParams p) {
   __shared__ LossWarp lw[kLossThreads / 32];
   __shared__ EltShared es;
@@ -727,58 +786,76 @@ __global__ void __launch_bounds__(kLossThreads, kLossBlocksPerSm) k_losses(const
       ws.hash[lane] = 0ull;
     }
     __syncwarp();
-    int nq = 0;
-    // pipeline: r1 = records of the next round, r0/h0 = this round's record and hot pair
-    uint2 r0 = (lane < n) ? __ldcs(recs + lane) : make_uint2(0u, 0u);
-    uint2 r1 = (32 + lane < n) ? __ldcs(recs + 32 + lane) : make_uint2(0u, 0u);
-    PairHot h0{0.0f, 0.0f, kKindZero << kMetaKindShift, 0u};
-    if (lane < n && ((r0.x >> kRecCntShift) & kRecCntMask) == 0u) h0 = p.hot[r0.y];
-    for (uint32_t base = 0;;) {
+    if constexpr (!kWindows) {
+      int nq = 0;
+      // pipeline: r1 = records of the next round, r0/h0 = this round's record and hot pair
+      uint2 r0 = (lane < n) ? __ldcs(recs + lane) : make_uint2(0u, 0u);
+      uint2 r1 = (32 + lane < n) ? __ldcs(recs + 32 + lane) : make_uint2(0u, 0u);
+      PairHot h0{0.0f, 0.0f, kKindZero << kMetaKindShift, 0u};
+      if (lane < n && ((r0.x >> kRecCntShift) & kRecCntMask) == 0u) h0 = p.hot[r0.y];
+      for (uint32_t base = 0;;) {
 #pragma unroll 1
-      for (; base < n && nq <= kQueue - 32; base += 32) {
-        const uint2 r = r0;
-        const PairHot h = h0;
-        const bool valid = base + lane < n;
-        r0 = r1;
-        if (base + 64 + lane < n) r1 = __ldcs(recs + base + 64 + lane);
-        if (base + 32 + lane < n && ((r0.x >> kRecCntShift) & kRecCntMask) == 0u) h0 = p.hot[r0.y];
-        const uint32_t cnt = ((r.x >> kRecCntShift) & kRecCntMask) + 1u;
-        const uint32_t tl = r.x >> kRecTrialShift, k = r.x & kRecKMask;
-        const bool single = valid && cnt == 1u;
-        bool slow = false;
-        if (single) {
-          float L;
-          slow = !pair_fast_hot(p, es, h, r.y, ta + tl, k, &L);
-          if (!slow) {
-            const float O = clamp_terms_f(L, p.occ_r, p.occ_l);
-            acc_add(ws, tl, O);
+        for (; base < n && nq <= kQueue - 32; base += 32) {
+          const uint2 r = r0;
+          const bool valid = base + lane < n;
+          const uint32_t cnt = ((r.x >> kRecCntShift) & kRecCntMask) + 1u;
+          const bool single = valid && cnt == 1u;
+          const PairEval e = pair_begin(p, es, ws, single, h0, r.y, ta, r.x, diag);
+          // the next round's loads and the queue, while the table interval comes
+          r0 = r1;
+          if (base + 64 + lane < n) r1 = __ldcs(recs + base + 64 + lane);
+          if (base + 32 + lane < n && ((r0.x >> kRecCntShift) & kRecCntMask) == 0u) h0 = p.hot[r0.y];
+          const uint32_t mmask = __ballot_sync(0xffffffffu, valid && cnt > 1u);
+          if (mmask) {
+            if (valid && cnt > 1u) {
+              ws.mq[nq + __popc(mmask & lt_mask)] = r;
+              if constexpr (kEmit) ws.mqi[nq + __popc(mmask & lt_mask)] = base + lane;
+            }
+            nq += __popc(mmask);
+          }
+          const bool slow = single && e.mode == kLossSlow;
+          if (single && !slow) {
+            const float O = clamp_terms_f(pair_end(es, e), p.occ_r, p.occ_l);
+            acc_add(ws, r.x >> kRecTrialShift, O);
             if constexpr (kEmit) p.occ[rb + base + lane] = O;
           }
-          if (diag) {
-            const uint32_t elt = es.elt_id[pair_pos(h.meta)];
-            atomicAdd(&ws.hits[tl], 1ull);
-            atomicAdd(&ws.hash[tl], static_cast<unsigned long long>(fmix64((static_cast<uint64_t>(k) << 32) | elt)));
-          }
+          n_pairs += __popc(__ballot_sync(0xffffffffu, single));
+          nd = defer_events<kEmit>(p, ws, nd, slow, r, ta + (r.x >> kRecTrialShift) - p.t_begin, rb + base + lane);
         }
-        n_pairs += __popc(__ballot_sync(0xffffffffu, single));
-        nd = defer_events<kEmit>(p, ws, nd, slow, r, ta + tl - p.t_begin, rb + base + lane);
-        const uint32_t mmask = __ballot_sync(0xffffffffu, valid && cnt > 1u);
-        if (mmask) {
-          if (valid && cnt > 1u) {
-            ws.mq[nq + __popc(mmask & lt_mask)] = r;
-            if constexpr (kEmit) ws.mqi[nq + __popc(mmask & lt_mask)] = base + lane;
-          }
-          nq += __popc(mmask);
+        __syncwarp();
+        if (nq > 0) {
+          const int2 rv = process_multi<kEmit>(p, es, ws, nd, nq, ta, diag, rb);
+          nd = rv.x;
+          n_pairs += static_cast<uint32_t>(rv.y);
+          nq = 0;
         }
+        if (base >= n) break;
       }
-      __syncwarp();
-      if (nq > 0) {
-        const int2 rv = process_multi<kEmit>(p, es, ws, nd, nq, ta, diag, rb);
-        nd = rv.x;
-        n_pairs += static_cast<uint32_t>(rv.y);
-        nq = 0;
+    } else {
+      // a window's table intervals are in flight while the next window is laid out, that one's hot records
+      // while this one's sums are made, and the records after it meanwhile
+      auto count_of = [](uint2 r, bool in) { return in ? ((r.x >> kRecCntShift) & kRecCntMask) + 1u : 0u; };
+      uint2 r = (lane < n) ? __ldg(recs + lane) : make_uint2(0u, 0u);
+      uint32_t next = 0u;  // the first record after the window
+      PairWindow w;
+      PairHot h;
+      auto next_window = [&]() {
+        w = make_window(r, count_of(r, next + lane < n));
+        h = PairHot{0.0f, 0.0f, kKindZero << kMetaKindShift, 0u};
+        if (lane < w.np) h = p.hot[w.ey + (lane - w.epre)];
+        next += static_cast<uint32_t>(w.n_take);
+        if (next + lane < n) r = __ldg(recs + next + lane);
+      };
+      next_window();
+#pragma unroll 1
+      while (w.np != 0u) {
+        const PairEval e = pair_begin(p, es, ws, lane < w.np, h, w.ey + (lane - w.epre), ta, w.ex, diag);
+        const PairWindow v = w;
+        const uint32_t rec = next - static_cast<uint32_t>(w.n_take) + w.ev;
+        n_pairs += w.np;
+        next_window();
+        nd = window_end<kEmit>(p, es, ws, nd, v, e, ta, rb, rec);
       }
-      if (base >= n) break;
     }
     __syncwarp();
     // ---- trials' sums: reduce-scatter of the per-lane double-float sums; lane
@@ -841,10 +918,16 @@ __global__ void __launch_bounds__(kLossThreads, kLossBlocksPerSm) k_losses(const
 }
 
 cudaError_t launch_losses(const LossParams& p, int grid, cudaStream_t s) {
-  if (p.occ)
-    k_losses<true><<<grid, kLossThreads, 0, s>>>(p);
-  else
-    k_losses<false><<<grid, kLossThreads, 0, s>>>(p);
+  if (p.windows) {
+    if (p.occ)
+      k_losses<true, true><<<grid, kLossThreads, 0, s>>>(p);
+    else
+      k_losses<false, true><<<grid, kLossThreads, 0, s>>>(p);
+  } else if (p.occ) {
+    k_losses<true, false><<<grid, kLossThreads, 0, s>>>(p);
+  } else {
+    k_losses<false, false><<<grid, kLossThreads, 0, s>>>(p);
+  }
   return cudaGetLastError();
 }
 

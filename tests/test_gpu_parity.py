@@ -525,6 +525,37 @@ def test_tile_sizes(eng, n, lo, hi):
         assert np.array_equal(sub, many[:, t0:t1])
 
 
+@pytest.mark.parametrize("n_elts,entries", [(4, 199), (4, 200), (5, 1_000), (32, 2_000)])
+def test_pair_windows(eng, n_elts, entries):
+    """The losses by windows of 32 pairs (from 0.4 records a catalogue event on):
+    both sides of the line, events of one pair, and events whose pairs fill a
+    window each; records of every kind, tables and the Halley iteration, the
+    YLT alone and with per-event output."""
+    C = 2_000
+    rng = np.random.default_rng(n_elts + entries)
+    pool = synth.make_elt_pool(n_elts, entries, C, 31, recipe="stress")
+    sigma, mean = pool.sigma.copy(), pool.mean.copy()
+    sigma[rng.random(len(sigma)) < 0.1] = 0.0
+    mean[rng.random(len(mean)) < 0.1] = 0.0
+    pool = synth.ELTPool(elt_ids=pool.elt_ids, rec_offsets=pool.rec_offsets, event_ids=pool.event_ids, mean=mean,
+                         sigma=sigma, exposure=pool.exposure, terms=pool.terms)
+    lens = np.concatenate([[0, 1, 31, 32, 33, 0, 64, 300], rng.integers(0, 60, 40)])
+    offsets = np.zeros(len(lens) + 1, np.int64)
+    offsets[1:] = np.cumsum(lens)
+    yet = synth.YET(offsets, rng.integers(0, C, int(offsets[-1])).astype(np.int32), C)
+    terms = (100.0, 1e7, 1e3, 1e9)
+    for kw in ({}, {"newton_only": True}, {"primary_only": True}):
+        ref = oracle.run_layer(yet, pool, terms, seed=8, **{k: v for k, v in kw.items() if k == "primary_only"})
+        ylt, hits, hh = run_gpu(eng, yet, pool, terms, seed=8, **kw)
+        assert np.array_equal(hits, ref["hits"]) and np.array_equal(hh, ref["hit_hash"])
+        check_ylt(ylt, ref)
+        out, cap = np.zeros(yet.n_trials), int(offsets[-1])
+        trial, inc = np.zeros(cap, np.int64), np.zeros(cap)
+        rows = eng.run_layer_events(pool.elt_ids, terms, 8, 0, yet.n_trials, out, trial=trial, agg_inc=inc, **kw)
+        assert np.array_equal(out, ylt)
+        np.testing.assert_allclose(np.bincount(trial[:rows], inc[:rows], yet.n_trials), ylt, rtol=1e-9, atol=1e-6)
+
+
 @pytest.mark.parametrize("n", [1, 31, 33, 4_095, 4_096, 4_129])
 def test_table_blocks(eng, n):
     """Quantile tables at the edges of the builder's blocks (32 records) and of
