@@ -18,6 +18,7 @@
 #include <cstdint>
 
 #include "ara_batch.h"
+#include "ara_window.cuh"
 
 namespace ara {
 
@@ -517,38 +518,32 @@ namespace {
 
 // ------------------------------------------------------------------ dense kernel
 // One warp per tile, one lane per (event occurrence, ELT) pair.  The tile's
-// records stream through a per-warp record ring; each record's pairs take
-// consecutive slots of a pair ring.  A compute round takes the next 64 pending
-// pairs (two per lane, whatever their records), computes each pair's loss
-// after ELT terms once, and stores it with the layers it serves.  Records
-// whose pairs are all computed are combined up to 64 at a time, with the lanes
-// turned into layers: lane (s, l) holds layer l's fixed-point sum for the
-// current trial in registers and takes the group's records i = s mod S (S
-// record slots: 32 over the layers rounded up to a power of two) that serve
-// layer l, found by bit-matrix transposes of the records' layer masks.  For
-// each (single-ELT records first, then the others), it sums the record's pair
+// records go by windows of up to 32 pairs of whole events.  Each pair's loss
+// after ELT terms is computed once and stored with the layers it serves; then
+// the lanes turn into layers: lane (s, l) holds layer l's fixed-point sum for
+// the current trial in registers and takes the window's events i = s mod S (S
+// event slots: 32 over the layers rounded up to a power of two) that serve
+// layer l, found by a bit-matrix transpose of the events' layer masks.  For
+// each (single-ELT events first, then the others), it sums the event's pair
 // losses over the layer's ELTs from left to right (the pairs' order), applies
-// the occurrence terms and adds the result.
-// When a trial's records are all combined, the slots' sums give its year
-// losses.  The fill keeps a round's 64 pairs pending; a record has at most 64
-// pairs, so after a combine at most 63 computed pairs and 63 pending ones are
-// live, and the next record always fits the rings.
-constexpr int kDenseRecs = 128;   // record ring (slots: sequence number mod kDenseRecs)
-constexpr int kDensePairs = 256;  // pair ring (slots: pair sequence number mod kDensePairs)
-constexpr int kDenseBlocksPerSm = 7;  // 72 registers: 28 warps per SM (measured: 6 and 8 were slower)
-static_assert(kDensePairs >= 63 + 64 + 64 && kDenseRecs >= 64 + 32, "ring sizes");
-static_assert(kDenseRecs <= 256, "record slots are stored in bytes");
+// the occurrence terms and adds the result.  When a trial's events are all
+// taken, the slots' sums give its year losses.  An event of more than 32 pairs
+// goes alone.
+//
+// Bound by issue (62% of the slots, ~730 instructions a window: the pairs'
+// losses 200, the adds by layer 250, where a warp waits for its lane with the
+// most events) and the conversions to fixed point.  16 layers over 64 ELTs,
+// 150,001 trials of 320 pairs: 1,445 us (1,700 with records and pairs in rings,
+// 64 pairs a round); 30,000 trials over a 100,000-event catalogue 1,480 (3,070).
+// Two adds a step, or the conversion in integer arithmetic: the same or slower.
+constexpr int kDenseBlocksPerSm = 7;  // 72 registers, 28 warps per SM (6: 1,520 us, 8: 1,550)
 
 struct DenseWarp {
-  uint2 rec[kDenseRecs];        // the ring's records
-  uint32_t pre[kDenseRecs];     // each record's first pair (sequence number in the tile)
-  float loss[kDensePairs];      // each pair's loss after ELT terms
-  uint32_t lmask[kDensePairs];  // each pair's layers: those holding its ELT that reach its trial
-  uint8_t owner[kDensePairs];   // each pair's record slot
-  uint32_t act[kWarpTrials];    // per trial of the tile: the layers whose trials reach it
-  float g_l0[64];               // a combine group's records: first pair's loss,
-  uint32_t g_pre[64];           //   first pair (sequence number),
-  uint32_t g_cnt[64];           //   pair count
+  float loss[kMaxIndexElts];      // a window's pair losses after ELT terms
+  uint32_t lmask[kMaxIndexElts];  // and the pairs' layers: those holding its ELT that reach its trial
+  float first[32];                // the window's events: the first pair's loss,
+  uint32_t place[32];             //   the first pair and the pair count << 8
+  uint32_t act[kWarpTrials];      // per trial of the tile: the layers whose trials reach it
 };
 
 struct DenseShared {
@@ -562,19 +557,6 @@ struct DenseShared {
   double* ylt[kBatchLayers];
   int64_t t_end[kBatchLayers];
 };
-
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, uint32_t lane) {
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const uint32_t o = __shfl_up_sync(0xffffffffu, v, d);
-    if (lane >= static_cast<uint32_t>(d)) v += o;
-  }
-  return v;
-}
-
-__device__ __forceinline__ uint2 shfl_u2(uint2 v, uint32_t src) {
-  return make_uint2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
 
 // Loss after ELT terms by the Halley iteration, with its non-convergence as
 // the second value (0 or 1).
@@ -635,6 +617,90 @@ __device__ __forceinline__ void dense_finish_trial(const DenseShared& ds, unsign
 
 }  // namespace
 
+namespace {
+
+// A pair between its two halves: its loss known (a), from a table interval (a =
+// max_l, s the place in the interval n0, n1), or by the Halley iteration.
+struct DensePair {
+  uint32_t layers;  // the pair's layers that reach its trial
+  uint32_t mode, pos;
+  float a, s;
+  float4 n0;
+  float2 n1;
+};
+enum : uint32_t { kDenseKnown = 0, kDenseTable = 1, kDenseSlow = 2 };
+
+// The first half, for lanes with `in`: key is the record's first word, act the
+// layers that reach its trial.
+__device__ __forceinline__ DensePair dense_begin(const BatchParams& p, const DenseShared& ds, const DenseWarp& ws,
+                                                 bool in, const PairHot& h, uint32_t pi, int64_t ta, uint32_t key) {
+  DensePair e{0u, kDenseKnown, pair_pos(h.meta), 0.0f, 0.0f, make_float4(0.0f, 0.0f, 0.0f, 0.0f),
+              make_float2(0.0f, 0.0f)};
+  if (in) {
+    const uint32_t tl = key >> kRecTrialShift;
+    e.layers = ds.layers_of[e.pos] & ws.act[tl];
+    if (e.layers) {
+      const uint32_t kind = pair_kind(h.meta);
+      e.a = kind == kKindZero ? 0.0f : h.mu;
+      if (!p.primary_only && kind_is_beta(kind)) {
+        float t;
+        if (p.newton_only || !pair_tab_exact(h.meta) ||
+            !batch_pair_normal(p, kind, ds.elt_id[e.pos], pi, ta + tl, key & kRecKMask, &t)) {
+          e.mode = kDenseSlow;
+        } else {
+          const bool fine = pair_fine(h.meta);
+          const TabPlace at = tab_place(t, fine);
+          const float4* node = (fine ? ds.tabf[e.pos] : ds.tab[e.pos]) + h.node + at.i;
+          e.mode = kDenseTable;
+          e.a = h.max_l;
+          e.s = at.s;
+          e.n0 = __ldg(node);
+          e.n1 = __ldg(reinterpret_cast<const float2*>(node + 1) + 1);
+        }
+      }
+    }
+  }
+  return e;
+}
+
+// The second half: the pair's loss after ELT terms.
+__device__ __forceinline__ float dense_end(const BatchParams& p, const DenseShared& ds, const DensePair& e,
+                                           uint32_t pi, int64_t ta, uint32_t key, unsigned long long* nc) {
+  if (e.mode == kDenseSlow) {
+    const float2 r = dense_pair_slow(p, pi, ta + (key >> kRecTrialShift), key & kRecKMask);
+    *nc += static_cast<unsigned long long>(r.y);
+    return r.x;
+  }
+  float loss = e.a;
+  if (e.mode == kDenseTable) loss = e.a * tab_value(e.s, e.n0, e.n1);
+  return ds.share[e.pos] * clamp_terms_f(loss, ds.ret[e.pos], ds.lim[e.pos]);
+}
+
+// The sum, left to right, of the losses of pairs [first, first + n) that layer l holds.
+__device__ __forceinline__ float dense_event_sum(const DenseWarp& ws, uint32_t first, uint32_t n, uint32_t l) {
+  float G = 0.0f;
+  for (uint32_t j = first; j < first + n; ++j)
+    if ((ws.lmask[j] >> l) & 1u) G += ws.loss[j];
+  return G;
+}
+
+// An event of more than 32 pairs, by the whole warp: its pairs' losses and layers into ws.
+__device__ __noinline__ uint32_t dense_long_event(const BatchParams& p, const DenseShared& ds, DenseWarp& ws, uint2 r,
+                                                  uint32_t cnt, int64_t ta, unsigned long long* nc) {
+  uint32_t n_pairs = 0;
+  for (uint32_t j = lane_id(); j < cnt; j += 32) {
+    const uint32_t pi = r.y + j;
+    const DensePair e = dense_begin(p, ds, ws, true, p.hot[pi], pi, ta, r.x);
+    ws.loss[j] = dense_end(p, ds, e, pi, ta, r.x, nc);
+    ws.lmask[j] = e.layers;
+    n_pairs += e.layers != 0u;
+  }
+  __syncwarp();
+  return n_pairs;
+}
+
+}  // namespace
+
 __global__ void __launch_bounds__(kBatchThreads, kDenseBlocksPerSm)
     k_losses_dense(const __grid_constant__ BatchParams p) {
   __shared__ DenseWarp dwarp[kBatchThreads / 32];
@@ -645,7 +711,7 @@ __global__ void __launch_bounds__(kBatchThreads, kDenseBlocksPerSm)
   load_dense_shared(p, ds);
   __syncthreads();
   static_assert(kBatchLayers <= 32, "one lane per layer; 32-bit layer masks");
-  // the lane's layer l and record slot s; its records in a group: i = s mod S
+  // the lane's layer l and event slot s; its events in a window: i = s mod S
   int nlp = 1;
   while (nlp < nl) nlp <<= 1;
   const uint32_t my_l = lane & static_cast<uint32_t>(nlp - 1);
@@ -653,17 +719,16 @@ __global__ void __launch_bounds__(kBatchThreads, kDenseBlocksPerSm)
   uint32_t my_pattern = 0u;
   for (uint32_t i = lane / static_cast<uint32_t>(nlp); i < 32u; i += n_slots) my_pattern |= 1u << i;
   if (my_l >= static_cast<uint32_t>(nl)) my_pattern = 0u;
-  unsigned long long acc = 0ull;       // the layer's sum over the slot's records of the current trial
-  const uint2 zero2 = make_uint2(0u, 0u);
+  unsigned long long acc = 0ull;  // the layer's sum over the slot's events of the current trial
   unsigned long long nc = 0ull;
   uint32_t n_pairs = 0;
 
-  unsigned long long next = 0ull;  // tiles are claimed one ahead
-  if (lane == 0) next = atomicAdd(&p.counters[0], 1ull);
+  unsigned long long next_tile = 0ull;  // tiles are claimed one ahead
+  if (lane == 0) next_tile = atomicAdd(&p.counters[0], 1ull);
   for (;;) {
-    const int64_t tile = static_cast<int64_t>(__shfl_sync(0xffffffffu, next, 0));
+    const int64_t tile = static_cast<int64_t>(__shfl_sync(0xffffffffu, next_tile, 0));
     if (tile >= p.n_tiles) break;
-    if (lane == 0) next = atomicAdd(&p.counters[0], 1ull);
+    if (lane == 0) next_tile = atomicAdd(&p.counters[0], 1ull);
     const int64_t ta = p.t_begin + tile * p.tile_trials;
     const int ntr = static_cast<int>((ta + p.tile_trials < p.t_end) ? p.tile_trials : p.t_end - ta);
     uint32_t any = 0u;
@@ -676,207 +741,89 @@ __global__ void __launch_bounds__(kBatchThreads, kDenseBlocksPerSm)
     }
     __syncwarp();
     const uint2* recs = p.ev_buf + (__ldg(&p.off[ta]) - p.e0);
-    const int32_t n = any ? static_cast<int32_t>(__ldg(&p.tile_cnt[tile])) : 0;
-    // lane i holds records rec_next + i (rc) and rec_next + 32 + i (rx)
-    int32_t rec_next = 0;
-    uint2 rc = (static_cast<int32_t>(lane) < n) ? __ldcs(recs + lane) : zero2;
-    uint2 rx = (32 + static_cast<int32_t>(lane) < n) ? __ldcs(recs + 32 + lane) : zero2;
-    uint32_t p_fill = 0u, p_done = 0u;  // pairs appended, pairs computed
-    uint32_t r_fill = 0u, r_done = 0u;  // records appended, records combined
-    int cur = 0;  // the trial whose records are being combined
+    const uint32_t n = any ? __ldg(&p.tile_cnt[tile]) : 0u;
+    // a window's table intervals are in flight while the next window is laid out, that one's hot records
+    // while this one's sums are made, and the records after it meanwhile
+    auto count_of = [](uint2 x) { return ((x.x >> kRecCntShift) & kRecCntMask) + 1u; };
+    uint2 r = lane < n ? __ldg(recs + lane) : make_uint2(0u, 0u);
+    uint32_t next = 0u;  // the first record after the window
+    PairWindow w;
+    PairHot h;
+    uint32_t evx;  // of lane i < n_take: the window's event i's record's first word
+    auto next_window = [&]() {
+      w = make_window(r, next + lane < n ? count_of(r) : 0u);
+      evx = r.x;
+      h = PairHot{0.0f, 0.0f, kKindZero << kMetaKindShift, 0u};
+      if (lane < w.np) h = p.hot[w.ey + (lane - w.epre)];
+      if (w.n_take > 0) {
+        next += static_cast<uint32_t>(w.n_take);
+        if (next + lane < n) r = __ldg(recs + next + lane);
+      }
+    };
+    next_window();
+    int cur = 0;  // the trial whose events are being taken
     for (;;) {
-      // ---- fill: whole records, 32 at a time, until a round's 64 pairs are pending
-      while (p_fill - p_done < 64u && rec_next < n) {
-        const bool valid = rec_next + static_cast<int32_t>(lane) < n;
-        const uint32_t cnt = valid ? ((rc.x >> kRecCntShift) & kRecCntMask) + 1u : 0u;
-        const uint32_t incl = warp_incl_scan(cnt, lane);
-        const uint32_t live = (r_done < r_fill) ? ws.pre[r_done % kDenseRecs] : p_fill;  // oldest live pair
-        const bool fits = valid && r_fill - r_done + lane < static_cast<uint32_t>(kDenseRecs) &&
-                          p_fill + incl - live <= static_cast<uint32_t>(kDensePairs);
-        const uint32_t n_take = __popc(__ballot_sync(0xffffffffu, fits));  // a prefix of the lanes
-        if (n_take == 0u) {  // cannot happen (see above); drop the tile's remaining records rather than spin
-          if (lane == 0) atomicOr(&p.counters[3], 1ull);
-          rec_next = n;
-          break;
-        }
-        if (fits) {
-          const uint32_t slot = (r_fill + lane) % kDenseRecs;
-          const uint32_t pre = p_fill + incl - cnt;
-          ws.rec[slot] = rc;
-          ws.pre[slot] = pre;
-          for (uint32_t j = 0; j < cnt; ++j) ws.owner[(pre + j) % kDensePairs] = static_cast<uint8_t>(slot);
-        }
-        p_fill += __shfl_sync(0xffffffffu, incl, n_take - 1u);
-        r_fill += n_take;
-        rec_next += static_cast<int32_t>(n_take);
-        // slide the window of records by n_take
-        const uint32_t src = lane + n_take;
-        const uint2 a = shfl_u2(rc, src & 31u), b = shfl_u2(rx, src & 31u);
-        rc = src < 32u ? a : b;
-        const int32_t at = rec_next + 32 + static_cast<int32_t>(lane);
-        rx = src < 32u ? b : (at < n ? __ldcs(recs + at) : zero2);
-        __syncwarp();
-      }
-      // ---- compute: up to 64 pending pairs, two per lane
-      if (p_done < p_fill) {
-        const uint32_t np = min(64u, p_fill - p_done);
-        uint32_t q[2], pi[2], kk[2], tl[2], mk[2];
-        PairHot h[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const uint32_t i = 32u * j + lane;
-          q[j] = (p_done + i) % kDensePairs;
-          pi[j] = 0u;
-          kk[j] = 0u;
-          tl[j] = 0u;
-          h[j] = PairHot{0.0f, 0.0f, kKindZero << kMetaKindShift, 0u};
-          if (i < np) {
-            const uint32_t o = ws.owner[q[j]];
-            const uint2 r = ws.rec[o];
-            pi[j] = r.y + (p_done + i - ws.pre[o]);
-            tl[j] = r.x >> kRecTrialShift;
-            kk[j] = r.x & kRecKMask;
-            h[j] = p.hot[pi[j]];
-          }
-        }
-        int mode[2];  // 0: no layer, 1: loss known (no loss / mean), 2: table, 3: Halley
-        float val[2], sfrac[2];
-        const float4* node[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const uint32_t pos = pair_pos(h[j].meta);
-          mk[j] = (32u * j + lane < np) ? ds.layers_of[pos] & ws.act[tl[j]] : 0u;
-          mode[j] = 0;
-          val[j] = 0.0f;
-          sfrac[j] = 0.0f;
-          node[j] = nullptr;
-          if (mk[j]) {
-            const uint32_t kind = pair_kind(h[j].meta);
-            mode[j] = 1;
-            val[j] = h[j].mu;
-            if (kind == kKindZero) {
-              val[j] = 0.0f;
-            } else if (!p.primary_only && kind_is_beta(kind)) {
-              float t = 0.0f;
-              if (p.newton_only || !pair_tab_exact(h[j].meta) ||
-                  !batch_pair_normal(p, kind, ds.elt_id[pos], pi[j], ta + tl[j], kk[j], &t)) {
-                mode[j] = 3;
-              } else {
-                mode[j] = 2;
-                const bool fine = pair_fine(h[j].meta);
-                const int nseg = fine ? kTabFineNodes - 1 : kTabNodes - 1;
-                float u = (t + kTabT1f) * (fine ? kTabInvH * kTabRefine : kTabInvH);
-                u = fminf(fmaxf(u, 0.0f), static_cast<float>(nseg));
-                int ix = static_cast<int>(u);
-                if (ix > nseg - 1) ix = nseg - 1;
-                sfrac[j] = u - static_cast<float>(ix);
-                node[j] = (fine ? ds.tabf[pos] : ds.tab[pos]) + h[j].node + ix;
-              }
-            }
-          }
-        }
-        float4 n0[2];
-        float2 n1[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          if (mode[j] == 2) {
-            n0[j] = __ldg(node[j]);
-            n1[j] = __ldg(reinterpret_cast<const float2*>(node[j] + 1) + 1);
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          float L = 0.0f;
-          if (mode[j] == 3) {
-            const float2 r = dense_pair_slow(p, pi[j], ta + tl[j], kk[j]);
-            L = r.x;
-            nc += static_cast<unsigned long long>(r.y);
-          } else if (mode[j] != 0) {
-            const uint32_t pos = pair_pos(h[j].meta);
-            float loss = val[j];
-            if (mode[j] == 2)
-              loss = (n0[j].x > 0.0f)
-                         ? h[j].max_l * (n0[j].x * expf(tab_increment(sfrac[j], n0[j].y, n0[j].z, n0[j].w, n1[j].x,
-                                                                       n1[j].y)))
-                         : 0.0f;
-            L = ds.share[pos] * clamp_terms_f(loss, ds.ret[pos], ds.lim[pos]);
-          }
-          if (32u * j + lane < np) {
-            ws.loss[q[j]] = L;
-            ws.lmask[q[j]] = mk[j];
-          }
-          n_pairs += mk[j] != 0u;
-        }
-        p_done += np;
-        __syncwarp();
-      }
-      // ---- combine: complete records of the current trial, up to 64 at a time (two per lane)
-      for (;;) {
-        uint32_t cnt[2], m[2], multi[2], col[2];
-        int rt[2];
-        bool have[2];
-        uint32_t n_ok = 0u;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const uint32_t gi = 32u * h + lane;  // the record's place in the group
-          const uint32_t R = r_done + gi;
-          have[h] = R < r_fill;
-          const uint32_t slot = R % kDenseRecs;
-          const uint2 r = have[h] ? ws.rec[slot] : zero2;
-          const uint32_t pre = have[h] ? ws.pre[slot] : 0u;
-          cnt[h] = ((r.x >> kRecCntShift) & kRecCntMask) + 1u;
-          rt[h] = static_cast<int>(r.x >> kRecTrialShift);
-          // a prefix of the group (records are in trial order; <= rather than == keeps the
-          // loop finite whatever the order)
-          const bool ok = have[h] && pre + cnt[h] <= p_done && rt[h] <= cur;
-          n_ok += __popc(__ballot_sync(0xffffffffu, ok));
-          multi[h] = __ballot_sync(0xffffffffu, ok && cnt[h] > 1u);
-          m[h] = 0u;  // the layers the record serves
-          if (ok) {
-            const uint32_t q0 = pre % kDensePairs;
-            m[h] = ws.lmask[q0];
-            for (uint32_t j = 1; j < cnt[h]; ++j) m[h] |= ws.lmask[(pre + j) % kDensePairs];
-            ws.g_l0[gi] = ws.loss[q0];
-            ws.g_pre[gi] = pre;
-            ws.g_cnt[gi] = cnt[h];
-          }
-          col[h] = __shfl_sync(0xffffffffu, bit_transpose32(m[h], lane), my_l) & my_pattern;
+      if (w.np == 0u) {
+        if (next >= n) break;
+        // the next event has more than 32 pairs
+        const uint2 x = make_uint2(__shfl_sync(0xffffffffu, r.x, 0), __shfl_sync(0xffffffffu, r.y, 0));
+        for (; cur < static_cast<int>(x.x >> kRecTrialShift); ++cur)
+          dense_finish_trial(ds, acc, lane, nlp, nl, ta + cur, p.t_begin);
+        const uint32_t cnt = count_of(x);
+        n_pairs += dense_long_event(p, ds, ws, x, cnt, ta, &nc);
+        if (lane < static_cast<uint32_t>(nl)) {
+          const float4 oc = ds.occ[lane];
+          acc += fixed_units(clamp_terms_f(dense_event_sum(ws, 0u, cnt, lane), oc.x, oc.y), oc.z);
         }
         __syncwarp();
-        // lane (s, l): the group's records of slot s that serve layer l
-        unsigned long long one = static_cast<unsigned long long>(col[0] & ~multi[0]) |
-                                 (static_cast<unsigned long long>(col[1] & ~multi[1]) << 32);
-        unsigned long long many = static_cast<unsigned long long>(col[0] & multi[0]) |
-                                  (static_cast<unsigned long long>(col[1] & multi[1]) << 32);
-        const float4 oc = ds.occ[my_l];  // the layer's occurrence terms and fixed-point scale
-        for (; one; one &= one - 1ull) {  // single-ELT records: the loss of their one pair
-          const float O = clamp_terms_f(ws.g_l0[__ffsll(one) - 1], oc.x, oc.y);
-          acc += fixed_units(O, oc.z);
-        }
-        for (; many; many &= many - 1ull) {  // the others: their pairs over the layer's ELTs, left to right
-          const int i = __ffsll(many) - 1;
-          const uint32_t c = ws.g_cnt[i], pr = ws.g_pre[i];
-          float G = 0.0f;
-          for (uint32_t j = 0; j < c; ++j) {
-            const uint32_t qq = (pr + j) % kDensePairs;
-            if ((ws.lmask[qq] >> my_l) & 1u) G += ws.loss[qq];
-          }
-          acc += fixed_units(clamp_terms_f(G, oc.x, oc.y), oc.z);
-        }
-        __syncwarp();  // the group's staging is rewritten by the next group
-        r_done += n_ok;
-        if (n_ok == 64u) continue;
-        // the first record not combined: of a later trial (the current one is done), or not complete
-        const bool hi = n_ok >= 32u;
-        const bool stop_have = __shfl_sync(0xffffffffu, (hi ? have[1] : have[0]) ? 1 : 0, n_ok & 31u) != 0;
-        const int stop_t = __shfl_sync(0xffffffffu, hi ? rt[1] : rt[0], n_ok & 31u);
-        if (stop_have && stop_t > cur) {
-          for (; cur < stop_t; ++cur) dense_finish_trial(ds, acc, lane, nlp, nl, ta + cur, p.t_begin);
-          continue;
-        }
-        break;
+        ++next;
+        if (next + lane < n) r = __ldg(recs + next + lane);
+        next_window();
+        continue;
       }
-      if (rec_next >= n && r_done == r_fill) break;
+      const uint32_t pi = w.ey + (lane - w.epre), key = w.ex, np = w.np;
+      const DensePair e = dense_begin(p, ds, ws, lane < np, h, pi, ta, key);
+      const uint32_t n_take = static_cast<uint32_t>(w.n_take), ev_first = w.pre, ev_key = evx;
+      next_window();
+      ws.loss[lane] = dense_end(p, ds, e, pi, ta, key, &nc);
+      ws.lmask[lane] = e.layers;
+      n_pairs += e.layers != 0u;
+      __syncwarp();
+      // lane i as event i: the layers it serves
+      uint32_t m = 0u, cnt = 0u;
+      int t = -1;
+      if (lane < n_take) {
+        cnt = ((ev_key >> kRecCntShift) & kRecCntMask) + 1u;
+        t = static_cast<int>(ev_key >> kRecTrialShift);
+        m = ws.lmask[ev_first];
+        for (uint32_t j = 1; j < cnt; ++j) m |= ws.lmask[ev_first + j];
+        ws.first[lane] = ws.loss[ev_first];
+        ws.place[lane] = ev_first | cnt << 8;
+      }
+      const uint32_t multi = __ballot_sync(0xffffffffu, cnt > 1u);
+      // lane (s, l): the slot's events that serve layer l
+      const uint32_t col = __shfl_sync(0xffffffffu, bit_transpose32(m, lane), my_l) & my_pattern;
+      __syncwarp();
+      const float4 oc = ds.occ[my_l];  // the layer's occurrence terms and fixed-point scale
+      for (uint32_t done = 0; done < n_take;) {  // by trial
+        const int tr = __shfl_sync(0xffffffffu, t, done);
+        for (; cur < tr; ++cur) dense_finish_trial(ds, acc, lane, nlp, nl, ta + cur, p.t_begin);
+        // (records are in trial order; <= keeps the loop finite whatever the order)
+        const uint32_t seg = __ballot_sync(0xffffffffu, lane >= done && lane < n_take && t <= tr);
+        for (uint32_t one = col & seg & ~multi; one;) {  // events of one pair
+          const int i = 31 - __clz(one);
+          one ^= 1u << i;
+          acc += fixed_units(clamp_terms_f(ws.first[i], oc.x, oc.y), oc.z);
+        }
+        for (uint32_t many = col & seg & multi; many;) {
+          const int i = 31 - __clz(many);
+          many ^= 1u << i;
+          const uint32_t pl = ws.place[i];
+          acc += fixed_units(clamp_terms_f(dense_event_sum(ws, pl & 0xffu, pl >> 8, my_l), oc.x, oc.y), oc.z);
+        }
+        done += __popc(seg);
+      }
+      __syncwarp();  // the window's losses are rewritten
     }
     for (; cur < ntr; ++cur) dense_finish_trial(ds, acc, lane, nlp, nl, ta + cur, p.t_begin);
     __syncwarp();

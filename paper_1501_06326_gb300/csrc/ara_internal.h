@@ -233,7 +233,7 @@ struct BatchParams {
   int32_t primary_only;
   int32_t newton_only;
   double* ylt_l[kBatchLayers];         // layer l's year losses of trials [t_begin, layer_t_end[l]) (indexed from t_begin)
-  unsigned long long* counters;        // [0] tile queue, [1] pairs, [2] non-converged, [3] ring overflow (0)
+  unsigned long long* counters;        // [0] tile queue, [1] pairs, [2] non-converged, [3] unused
   int64_t layer_t_end[kBatchLayers];   // layer l's trials end here (<= t_end): later trials get no losses, no output
 };
 
@@ -242,7 +242,7 @@ struct BatchParams {
 enum BatchItem : int {
   kItemTile = 0,   // one warp per tile of kWarpTrials trials, a lane per record
   kItemTrial = 1,  // one warp per trial of a tile, a lane per record
-  kItemDense = 2,  // one warp per tile, a lane per pair (records streamed through per-warp rings)
+  kItemDense = 2,  // one warp per tile, a lane per pair (windows of 32 pairs)
 };
 cudaError_t launch_losses_batch(const BatchParams& p, int item, int grid, cudaStream_t s);
 // CTAs of the dense kernel that one SM holds for n_layers layers (0 on error).

@@ -9,23 +9,9 @@
 #include <type_traits>
 
 #include "ara_internal.h"
+#include "ara_window.cuh"
 
 namespace ara {
-
-namespace {
-
-template <typename T>
-__device__ __forceinline__ T warp_inclusive_scan(T v) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const T o = __shfl_up_sync(0xffffffffu, v, d);
-    if (lane >= d) v += o;
-  }
-  return v;
-}
-
-}  // namespace
 
 // =============================================================== layer kernels
 //
@@ -55,9 +41,10 @@ __device__ __forceinline__ T warp_inclusive_scan(T v) {
 // and a double-float add into the lane's sum for the event's trial.  Events
 // with several pairs are queued and processed in windows of 32 pairs with a
 // segmented sum; layers of many pairs an event take all events so.  Events
-// with a pair whose record's table is not exact are deferred and resolved, 32 at a time, by the FP32 Halley iteration.  At the
-// end of a tile a reduce-scatter over the lanes gives the trials' sums, and
-// the aggregate terms turn each into the trial's year loss.
+// with a pair whose record's table is not exact are deferred and resolved, 32
+// at a time, by the FP32 Halley iteration.  At the end of a tile a
+// reduce-scatter over the lanes gives the trials' sums, and the aggregate terms
+// turn each into the trial's year loss.
 
 namespace {
 
@@ -565,32 +552,6 @@ struct EltShared {
   uint32_t elt_id[32];
   float ret[32], lim[32], share[32];
 };
-
-// A window: up to 32 pairs of whole events, one per lane.  Of lane q < np: its
-// event's record (x, y), the event's first lane and its place among the
-// window's events.
-struct PairWindow {
-  uint32_t ex, ey, epre, ev, np;
-  int n_take;  // events
-};
-
-// The window of the first events of lanes' records (cnt: lane's event's pairs, 0 beyond the last).
-__device__ __forceinline__ PairWindow make_window(uint2 r, uint32_t cnt) {
-  const uint32_t q = lane_id();
-  PairWindow w;
-  const uint32_t incl = warp_inclusive_scan(cnt);
-  const uint32_t pre = incl - cnt;
-  const bool take = cnt != 0 && incl <= 32u;
-  w.n_take = __popc(__ballot_sync(0xffffffffu, take));
-  w.np = w.n_take > 0 ? __shfl_sync(0xffffffffu, incl, w.n_take - 1) : 0u;
-  const uint32_t starts = __reduce_or_sync(0xffffffffu, take ? (1u << pre) : 0u);
-  // lane q's event: the last start at or below q
-  w.ev = static_cast<uint32_t>(__popc(starts & (0xffffffffu >> (31u - q)))) - 1u;
-  w.ex = __shfl_sync(0xffffffffu, r.x, w.ev);
-  w.ey = __shfl_sync(0xffffffffu, r.y, w.ev);
-  w.epre = __shfl_sync(0xffffffffu, pre, w.ev);
-  return w;
-}
 
 // A pair's loss between its two halves: known (kLossKnown: a), or from a table
 // interval (kLossTable: a = max_l, s the place in the interval n0, n1), or by

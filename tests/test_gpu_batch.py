@@ -305,6 +305,29 @@ def test_work_items_on_events_with_64_pairs(eng):
         check_ylt(out[l], oracle.run_layer(yet, layers[l][2], layers[l][1], seed=6))
 
 
+@pytest.mark.parametrize("n_elts,n_layers", [(31, 16), (32, 17), (33, 5), (40, 32)])
+def test_work_items_around_a_window(eng, n_elts, n_layers):
+    """Events whose pairs just fill the dense kernel's window of 32, or are one
+    more (taken alone), among events of one pair, in trials of 0 to 70 events,
+    and a subrange of them: all work items agree."""
+    C = 500
+    rng = np.random.default_rng(n_elts)
+    base = synth.make_elt_pool(n_elts, 250, C, 55)
+    wide = rng.choice(C, 150, replace=False)  # held by every ELT
+    ids = np.concatenate([np.sort(np.concatenate([wide, rng.choice(np.setdiff1d(np.arange(C), wide), 100, replace=False)]))
+                          for _ in range(n_elts)]).astype(np.int32)
+    pool = synth.ELTPool(elt_ids=base.elt_ids, rec_offsets=base.rec_offsets, event_ids=ids, mean=base.mean,
+                         sigma=base.sigma, exposure=base.exposure, terms=base.terms)
+    offsets = np.zeros(302, np.int64)
+    offsets[1:] = np.cumsum(rng.integers(0, 71, 301))
+    yet = synth.YET(offsets, rng.integers(0, C, int(offsets[-1])).astype(np.int32), C)
+    layers = [(np.sort(rng.choice(pool.elt_ids, rng.integers(1, min(n_elts, 32) + 1), replace=False)),
+               (10.0 * l, 1e6, 1e2, 1e8), None) for l in range(n_layers - 1)] + [(pool.elt_ids[-32:], (0.0, 1e9, 0.0, 1e12), None)]
+    layers[0] = (pool.elt_ids[:32], layers[0][1], None)
+    _assert_same_bits(_run_items(eng, yet, pool, layers, 9))
+    _assert_same_bits(_run_items(eng, yet, pool, layers, 9, 5, 290))
+
+
 def test_work_items_on_empty_and_long_trials(eng):
     """Empty trials (at tile starts and ends), a 4,097-event trial, a partial last
     tile, and a subrange: all work items agree."""
