@@ -301,9 +301,9 @@ ARA_API int ara_run_layers(ara_ctx *ctx, int32_t n_layers, const ara_layer *laye
 /* The losses kernel of ara_run_layers (and of the serving loop's passes) has
  * three work items, which add the same fixed-point numbers and so give the
  * same bits:
- *   ARA_BATCH_ITEM_TILE   one warp per tile of 8 trials, a lane per hit record;
+ *   ARA_BATCH_ITEM_TILE   one warp per tile of up to 8 trials, a lane per hit record;
  *   ARA_BATCH_ITEM_TRIAL  one warp per trial, a lane per hit record;
- *   ARA_BATCH_ITEM_DENSE  one warp per tile of 8 trials, a lane per (event, ELT)
+ *   ARA_BATCH_ITEM_DENSE  one warp per tile of up to 8 trials, a lane per (event, ELT)
  *                         pair: each pair's loss once, then each record's
  *                         per-layer occurrence losses;
  *   ARA_BATCH_ITEM_INDEXED  (once ara_build_yet_index has run) a warp per

@@ -815,12 +815,12 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
                 c->max_smem);
   pl->n_out = t1 - t0;
   // Trials per tile.  Eight share a tile's set-up and the lanes left over at its end, which counts where a
-  // trial has few records (75 a trial, 1M trials: eight 1,029 us in the losses, four 1,117, two 1,378).  Fewer
+  // trial has few records (75 a trial, 1M trials: eight 1,005 us in the losses, four 1,083, two 1,316).  Fewer
   // where a tile of half the trials still has 512 records, so that no warp is left a long last tile (750 a
-  // trial: 33,333 trials 948 us with eight, 620 with one; 100,003 trials 1,875 and 1,737), where the losses'
+  // trial: 33,333 trials 546 us with eight, 408 with one; 100,003 trials 1,168 and 1,137), where the losses'
   // 24 warps an SM would get under three tiles each and half a tile still has 128 records (75 a trial, 20,011
-  // trials, gather and losses: 117 us with eight, 102 with two, 116 with one), and where they would not get
-  // one each (30 a trial, 1,000 trials: 33 us with eight, 22 with one).  Neither sums nor rows depend on it.
+  // trials, gather and losses: 108 us with eight, 98 with two, 110 with one), and where they would not get
+  // one each (30 a trial, 1,000 trials: 30 us with eight, 20 with one).  Neither sums nor rows depend on it.
   const int64_t warps = int64_t(24) * c->num_sms;
   const double recs_trial = static_cast<double>(n_recs) * static_cast<double>(c->h_off[t1] - c->h_off[t0]) /
                             (static_cast<double>(pl->n_out) * c->catalogue);

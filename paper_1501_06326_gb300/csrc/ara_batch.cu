@@ -273,7 +273,7 @@ __device__ __forceinline__ int32_t first_record_of(const uint2* recs, int32_t n,
 // One warp per item, the item's hit-event records two per lane per round
 // (records two rounds ahead and single-ELT hot pairs one round ahead in
 // flight); every lane keeps its own fixed-point sum per layer.
-// kPerTrial = false: an item is a tile of kWarpTrials trials.  A lane's
+// kPerTrial = false: an item is a tile of up to kWarpTrials trials.  A lane's
 //   records come in trial order, so its sums are for its current trial and
 //   move into the tile's per-trial sums (shared-memory atomics) when the
 //   trial changes.  Few records per trial fill the lanes this way.
