@@ -630,6 +630,7 @@ static int load_elts_impl(ara_ctx* c, const char* who, int32_t n_elts, const int
                                           c->stream, sigma_c ? d_sc : nullptr, sigma_c ? d_w : nullptr, &launched));
   // (the records in order of their shapes, where there are enough for it to pay and its scratch fits)
   int64_t* order = nullptr;
+  const size_t sel_before = c->sel.bytes;
   if (R >= kShapeOrderMin && (!c->budget || c->used + ara::shape_order_bytes(R) <= c->budget) &&
       reserve(c, c->sel, ara::shape_order_bytes(R)) == ARA_OK)
     ARA_CUDA(c, ara::launch_shape_order(d_shapes, R, c->sel.ptr, &order, c->stream, &launched));
@@ -639,6 +640,7 @@ static int load_elts_impl(ara_ctx* c, const char* who, int32_t n_elts, const int
   std::vector<uint32_t> hf(4 * static_cast<size_t>(n_elts));
   ARA_CUDA(c, cudaMemcpyAsync(hf.data(), d_flags, sizeof(uint32_t) * hf.size(), cudaMemcpyDeviceToHost, c->stream));
   ARA_CUDA(c, cudaStreamSynchronize(c->stream));
+  if (c->budget && c->sel.bytes > sel_before) release(c, c->sel);  // the ELTs' own buffers may need its room
   for (int32_t i = 0; i < n_elts; ++i) {
     const uint32_t f = hf[4 * i];
     const char* why = nullptr;
@@ -783,8 +785,14 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   if (n_recs >= (int64_t(1) << 31) - 1) return fail(c, ARA_EINVAL, "%s: the ELTs hold too many records", who);
   // ---- index
   const int64_t n_words = (static_cast<int64_t>(c->catalogue) + 31) / 32;
+  pl->e0 = c->h_off[t0];
+  const int64_t e1 = c->h_off[t1];
+  // the words' pair counts, which only the index build reads, lie in the event buffer where it is large enough
+  const size_t ev_bytes = sizeof(uint2) * static_cast<size_t>(e1 - pl->e0 + 1);
+  const size_t base_bytes = sizeof(uint32_t) * static_cast<size_t>(n_words + 1);
   if ((rc = reserve(c, c->marks, ara::index_marks_bytes(n_words, n_recs))) ||
-      (rc = reserve(c, c->word_base, 2 * sizeof(uint32_t) * (n_words + 1))) ||
+      (rc = reserve(c, c->word_base, (ev_bytes >= base_bytes ? 1 : 2) * base_bytes)) ||
+      (rc = reserve(c, c->ev_buf, ev_bytes)) ||
       (rc = reserve(c, c->rankdir, sizeof(uint2) * n_words)) ||
       (rc = reserve(c, c->slot_start, sizeof(uint32_t) * (n_recs + 2))) ||
       (rc = reserve(c, c->pairs, sizeof(ara::Pair) * (n_recs + 1))) ||
@@ -798,7 +806,7 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   ix.n_recs = n_recs;
   ara::index_place_marks(ix, c->marks.ptr);
   ix.slot_base = static_cast<uint32_t*>(c->word_base.ptr);
-  ix.pair_base = ix.slot_base + n_words + 1;
+  ix.pair_base = ev_bytes >= base_bytes ? static_cast<uint32_t*>(c->ev_buf.ptr) : ix.slot_base + n_words + 1;
   ix.rankdir = static_cast<uint2*>(c->rankdir.ptr);
   ix.slot_start = static_cast<uint32_t*>(c->slot_start.ptr);
   ix.slot_event = nullptr;
@@ -821,21 +829,19 @@ static int plan_pass(ara_ctx* c, const std::vector<int32_t>& ids, int64_t t0, in
   // 24 warps an SM would get under three tiles each and half a tile still has 128 records (75 a trial, 20,011
   // trials, gather and losses: 108 us with eight, 98 with two, 110 with one), and where they would not get
   // one each (30 a trial, 1,000 trials: 30 us with eight, 20 with one).  Neither sums nor rows depend on it.
+  // Eight under a budget: a tile's count and first row are buffers that it covers.
   const int64_t warps = int64_t(24) * c->num_sms;
   const double recs_trial = static_cast<double>(n_recs) * static_cast<double>(c->h_off[t1] - c->h_off[t0]) /
                             (static_cast<double>(pl->n_out) * c->catalogue);
   pl->tile_trials = ara::kWarpTrials;
-  while (pl->tile_trials > 1) {
+  while (!c->budget && pl->tile_trials > 1) {
     const int64_t tiles = (pl->n_out + pl->tile_trials - 1) / pl->tile_trials;
     const double half = recs_trial * (pl->tile_trials / 2);
     if (!(half >= 512.0 || tiles < warps || (tiles < 3 * warps && half >= 128.0))) break;
     pl->tile_trials /= 2;
   }
   pl->n_tiles = (pl->n_out + pl->tile_trials - 1) / pl->tile_trials;
-  pl->e0 = c->h_off[t0];
-  const int64_t e1 = c->h_off[t1];
-  if ((rc = reserve(c, c->ev_buf, sizeof(uint2) * (e1 - pl->e0 + 1))) ||
-      (rc = reserve(c, c->tile_cnt, sizeof(uint32_t) * (pl->n_tiles + 1))) ||
+  if ((rc = reserve(c, c->tile_cnt, sizeof(uint32_t) * (pl->n_tiles + 1))) ||
       (rc = reserve(c, c->def_acc, sizeof(double) * (pl->n_out + 1))))
     return rc;
   ara::GatherParams& g = pl->g;
@@ -1574,7 +1580,7 @@ std::vector<std::pair<DevBuf*, size_t>> serve_workspace(ara_ctx* c) {
   int64_t n_recs = 0;
   for (size_t i = 0; i < sizes.size() && i < static_cast<size_t>(ARA_MAX_BATCH_ELTS); ++i) n_recs += sizes[i];
   const int64_t n_words = (static_cast<int64_t>(c->catalogue) + 31) / 32;
-  const size_t chunk_tiles = static_cast<size_t>(kServeChunk + 2);  // of one trial each at most
+  const size_t chunk_tiles = static_cast<size_t>(kServeChunk / (c->budget ? ara::kWarpTrials : 1) + 2);
   std::vector<std::pair<DevBuf*, size_t>> w = {
       {&c->ev_buf, sizeof(uint2) * static_cast<size_t>(max_ev + 1)},
       {&c->tile_cnt, sizeof(uint32_t) * chunk_tiles},

@@ -525,6 +525,32 @@ def test_tile_sizes(eng, n, lo, hi):
         assert np.array_equal(sub, many[:, t0:t1])
 
 
+@pytest.mark.parametrize("n_trials,catalogue", [(900, 2_000), (3, 400_000)])
+def test_budget_keeps_the_bits(eng, n_trials, catalogue):
+    """Under a budget tiles stay at eight trials and the ELT load's scratch is
+    given back; the index's pair counts lie in the event buffer or, for a YET
+    too small for them, in their own: the bits of a context without a budget."""
+    from paper_1501_06326_gb300 import ara
+
+    yet = synth.make_yet(n_trials, 60.0, catalogue, 5)
+    pool = synth.make_elt_pool(5, 1_200, catalogue, 6)
+    terms = (100.0, 1e6, 1e3, 1e9)
+    ylt, hits, hh = run_gpu(eng, yet, pool, terms, seed=2)
+    many = np.empty((2, n_trials))
+    ids = [int(i) for i in pool.elt_ids]
+    eng.run_layers([(ids, terms), (ids[:2], terms)], 2, 0, n_trials, many)
+    small = ara.Ara(0, 64 << 20)
+    try:
+        got = run_gpu(small, yet, pool, terms, seed=2)
+        assert np.array_equal(got[0], ylt) and np.array_equal(got[1], hits) and np.array_equal(got[2], hh)
+        sub = np.empty((2, n_trials))
+        small.run_layers([(ids, terms), (ids[:2], terms)], 2, 0, n_trials, sub)
+        assert np.array_equal(sub, many)
+    finally:
+        small.close()
+    check_ylt(ylt, oracle.run_layer(yet, pool, terms, seed=2))
+
+
 @pytest.mark.parametrize("n_elts,entries", [(4, 199), (4, 200), (5, 1_000), (32, 2_000)])
 def test_pair_windows(eng, n_elts, entries):
     """The losses by windows of 32 pairs (from 0.4 records a catalogue event on):
