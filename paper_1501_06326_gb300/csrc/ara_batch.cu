@@ -906,15 +906,16 @@ struct IdxWarp {
 
 // First entry in [lo, hi) of the event's occurrences whose trial is >= key
 // (hi if none), by the whole warp: each round probes 32 evenly spaced entries.
+// (An index holds up to 2^32 - 2 occurrences: probes past hi are in 64 bits.)
 __device__ __forceinline__ uint32_t first_occ_at(const unsigned long long* occ, uint32_t lo, uint32_t hi,
                                                  int64_t key, uint32_t lane) {
   while (lo < hi) {
-    const uint32_t step = (hi - lo + 31u) / 32u;
-    const uint32_t pos = lo + lane * step;
+    const uint32_t step = (hi - lo - 1u) / 32u + 1u;
+    const uint64_t pos = static_cast<uint64_t>(lo) + lane * step;
     const bool ge = pos < hi && static_cast<int64_t>(__ldg(occ + pos) >> 32) >= key;
     const uint32_t b = __ballot_sync(0xffffffffu, ge);
     if (b == 0u) {
-      const uint32_t probes = (hi - lo + step - 1u) / step;
+      const uint32_t probes = (hi - lo - 1u) / step + 1u;
       lo += (probes - 1u) * step + 1u;
     } else {
       const uint32_t f = static_cast<uint32_t>(__ffs(b) - 1);
@@ -1046,7 +1047,7 @@ __global__ void __launch_bounds__(kIdxThreads, kIdxBlocksPerSm)
       }
       __syncwarp();
       unsigned long long o_next = 0ull;
-      if (lo + lane < hi) o_next = load_occ(q.occ + lo + lane);
+      if (lane < hi - lo) o_next = load_occ(q.occ + lo + lane);
       auto layers_at = [&](uint32_t trial) {  // the layers whose trials reach this one
         uint32_t act = all;
         if (trial >= t_full) {
@@ -1071,13 +1072,13 @@ __global__ void __launch_bounds__(kIdxThreads, kIdxBlocksPerSm)
         const float4* const tab = (fine ? ds.tabf[pos] : ds.tab[pos]) + h0.node;
         const uint32_t elt = ds.elt_id[pos];
         const float ret = ds.ret[pos], lim = ds.lim[pos], share = ds.share[pos];
-        for (uint32_t r = lo; r < hi; r += 32) {
-          const uint32_t i = r + lane;
+        for (uint32_t r = lo;; r += 32) {  // (windows by what is left: r + 32 may lie beyond 32 bits)
+          const uint32_t left = hi - r;
           const unsigned long long o = o_next;
-          if (i + 32u < hi) o_next = load_occ(q.occ + i + 32u);
+          if (lane + 32u < left) o_next = load_occ(q.occ + (r + lane + 32u));
           uint32_t trial = 0xffffffffu;  // above every layer's last trial
           float L = 0.0f;
-          if (i < hi) {
+          if (lane < left) {
             trial = static_cast<uint32_t>(o >> 32);
             if (touched & layers_at(trial)) {
               ++n_pairs;
@@ -1119,14 +1120,15 @@ __global__ void __launch_bounds__(kIdxThreads, kIdxBlocksPerSm)
           } else if (n_held - at == 1) {
             add(trial, L, ws.held[at], ws.last[at], true);
           }
+          if (left <= 32u) break;
         }
       } else {
-        for (uint32_t r = lo; r < hi; r += 32) {
-          const uint32_t i = r + lane;
+        for (uint32_t r = lo;; r += 32) {  // (windows by what is left: r + 32 may lie beyond 32 bits)
+          const uint32_t left = hi - r;
           const unsigned long long o = o_next;
-          if (i + 32u < hi) o_next = load_occ(q.occ + i + 32u);
+          if (lane + 32u < left) o_next = load_occ(q.occ + (r + lane + 32u));
           const uint32_t trial = static_cast<uint32_t>(o >> 32);
-          const uint32_t act = i < hi ? layers_at(trial) : 0u;
+          const uint32_t act = lane < left ? layers_at(trial) : 0u;
           // the pairs in order: each layer's running sum is the left-to-right sum of its pairs' losses
           for (uint32_t j = 0; j < cnt; ++j) {
             const uint32_t m = ws.pmask[j] & act;
@@ -1136,7 +1138,7 @@ __global__ void __launch_bounds__(kIdxThreads, kIdxBlocksPerSm)
               for (uint32_t mm = m; mm; mm &= mm - 1u) gacc[__ffs(mm) - 1][lane] += L;
             }
           }
-          ws.trial[lane] = i < hi ? trial : 0xffffffffu;
+          ws.trial[lane] = lane < left ? trial : 0xffffffffu;
           __syncwarp();
           // the adds, by lanes of four as above
           for (int at = 0; at < n_held; at += 4) {
@@ -1152,6 +1154,7 @@ __global__ void __launch_bounds__(kIdxThreads, kIdxBlocksPerSm)
           }
           __syncwarp();
           for (uint32_t mm = touched; mm; mm &= mm - 1u) gacc[__ffs(mm) - 1][lane] = 0.0f;
+          if (left <= 32u) break;
         }
       }
       __syncwarp();  // pmask is rewritten for the next event

@@ -435,7 +435,8 @@ __global__ void __launch_bounds__(1024) k_part_cells(const unsigned long long* _
   const uint32_t a = start[static_cast<int64_t>(blockIdx.x) * n_seg];
   const uint32_t b = start[static_cast<int64_t>(blockIdx.x + 1) * n_seg];
   constexpr int kU = 4;
-  for (uint64_t i = a + threadIdx.x; i < b; i += kU * 1024) {
+  // (64-bit positions: a may lie within a block of 2^32)
+  for (uint64_t i = static_cast<uint64_t>(a) + threadIdx.x; i < b; i += kU * 1024) {
     unsigned long long v[kU];
 #pragma unroll
     for (int u = 0; u < kU; ++u) v[u] = i + u * 1024 < b ? __ldcs(in + i + u * 1024) : ~0ull;

@@ -491,3 +491,46 @@ def test_yet_index_partitions(eng, shape):
     for t0, t1 in {(0, N), (N // 3, N - N // 5), (N // 2, N // 2 + 1)}:
         _assert_same_bits(_run_items(eng, yet, pool, layers, 2, t0, t1))
     assert eng.yet_index_info()["method"] == "buckets"
+
+
+def test_yet_index_at_its_event_limit(eng):
+    """A YET of 2^32 - 2 events, the most an index takes: the last digit's
+    bucket and the last events' occurrences end within a block and a window of
+    2^32, where a 32-bit position would wrap.  The indexed passes over the
+    first and last trials give the dense item's bits."""
+    import torch
+
+    from paper_1501_06326_gb300 import ara
+
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info()[0] < 140 << 30:
+        pytest.skip("needs 140 GB of device memory")
+    C, N, n = 1 << 22, 2048, (1 << 32) - 2
+    offsets = np.minimum(np.arange(N + 1, dtype=np.int64) << 21, n)
+    # the last 2,048 ids have 500 occurrences, in the last two trials
+    ids = torch.randint(0, C - 2048, (n,), dtype=torch.int32, device="cuda")
+    late = torch.arange(C - 2048, C, dtype=torch.int32, device="cuda")[-50:].repeat(10)
+    ids[n - (1 << 21):][torch.randperm(1 << 21, device="cuda")[:250]] = late[:250]
+    ids[n - (1 << 22): n - (1 << 21)][:250] = late[250:]
+    torch.cuda.synchronize()
+    pool = synth.make_elt_pool(3, 2_000, C, 8)
+    held = np.sort(np.random.default_rng(8).choice(C - 2048, 1_950, replace=False))
+    pool.event_ids[:2_000] = np.concatenate([held, late[:50].cpu().numpy()])
+    big = ara.Ara(0)
+    try:
+        big.load_yet(offsets, ids, C)
+        del ids, late
+        torch.cuda.empty_cache()
+        big.load_pool(pool)
+        big.build_yet_index()
+        layers = [([0, 1], (10.0, 5e5, 1e2, 5e9)), ([0], (0.0, 1e9, 0.0, 1e12))]
+        for t0, t1 in ((0, 2), (N - 3, N), (N - 1, N)):
+            got = {}
+            for item in (ara.ARA_BATCH_ITEM_DENSE, ara.ARA_BATCH_ITEM_INDEXED):
+                big.set_batch_config(item)
+                got[item] = np.zeros((2, t1 - t0))
+                big.run_layers(layers, 5, t0, t1, got[item])
+            assert np.array_equal(got[ara.ARA_BATCH_ITEM_DENSE], got[ara.ARA_BATCH_ITEM_INDEXED])
+            assert np.all(got[ara.ARA_BATCH_ITEM_DENSE][1] > 0.0)
+    finally:
+        big.close()
