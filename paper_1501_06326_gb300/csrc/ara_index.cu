@@ -609,7 +609,9 @@ cudaError_t yet_parts_count(const int64_t* off, const int32_t* ids, int64_t n_tr
   const int cell_smem = static_cast<int>(sizeof(uint32_t) * (static_cast<size_t>(cells) << sh.lo_bits));
   cudaError_t err;
   if ((err = cudaFuncSetAttribute(k_part_first, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
-      (err = cudaFuncSetAttribute(k_part_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, cell_smem)) !=
+      // (the limit belongs to the function: the most that any build asks for, as contexts on other threads
+      // launch it too)
+      (err = cudaFuncSetAttribute(k_part_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, kPartCellBytes)) !=
           cudaSuccess ||
       (err = cudaMemsetAsync(p.max_cnt, 0, sizeof(uint32_t), s)) != cudaSuccess)
     return err;

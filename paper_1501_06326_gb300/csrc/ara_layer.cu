@@ -351,8 +351,10 @@ __global__ void __launch_bounds__(kGatherThreads, 1) k_gather(const GatherParams
 cudaError_t launch_gather(const GatherParams& p, int grid, size_t smem, cudaStream_t s) {
   const bool sub = p.n_words <= 2 * static_cast<int64_t>(p.filt_words);
   auto launch = [&](auto kernel) -> cudaError_t {
+    // (the limit belongs to the function: the most that any call asks for, as contexts on other threads
+    // launch it too)
     const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 static_cast<int>(smem));
+                                                 kGatherSmemBudget);
     if (err != cudaSuccess) return err;
     kernel<<<grid, kGatherThreads, smem, s>>>(p);
     return cudaGetLastError();

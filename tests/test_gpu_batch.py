@@ -534,3 +534,61 @@ def test_yet_index_at_its_event_limit(eng):
             assert np.all(got[ara.ARA_BATCH_ITEM_DENSE][1] > 0.0)
     finally:
         big.close()
+
+
+def _on_two_threads(work, arguments):
+    """work(engine, argument) on two host threads, each with its own context."""
+    import threading
+
+    from paper_1501_06326_gb300 import ara
+
+    errors = []
+
+    def go(argument):
+        own = ara.Ara(0)
+        try:
+            work(own, argument)
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+        finally:
+            own.close()
+
+    threads = [threading.Thread(target=go, args=(a,)) for a in arguments]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+
+
+def test_contexts_on_threads_with_unlike_catalogues(eng):
+    """Two contexts on two threads whose gathers need 40 and 195 KB of shared
+    memory: a call on one does not lower the other's limit."""
+
+    def layers(own, catalogue):
+        yet, pool = synth.make_yet(200, 20.0, catalogue, 3), synth.make_elt_pool(2, 300, catalogue, 4)
+        own.load_yet(yet.offsets, yet.event_ids, catalogue)
+        own.load_pool(pool)
+        first, out = np.zeros(yet.n_trials), np.zeros(yet.n_trials)
+        own.run_layer(pool.elt_ids, (10.0, 1e6, 1e2, 1e8), 1, 0, yet.n_trials, first)
+        for _ in range(2_000):
+            own.run_layer(pool.elt_ids, (10.0, 1e6, 1e2, 1e8), 1, 0, yet.n_trials, out)
+            assert np.array_equal(out, first)
+
+    _on_two_threads(layers, (1_000, 2_000_000))
+
+
+def test_contexts_on_threads_index_unlike_yets(eng):
+    """Two contexts on two threads that index YETs of one and of eight grid
+    cells (8 and 64 KB of shared memory for the cells' counts)."""
+
+    def build(own, shape):
+        trials, per_trial = shape
+        offsets = np.arange(trials + 1, dtype=np.int64) * per_trial
+        ids = np.random.default_rng(1).integers(0, 1 << 22, int(offsets[-1])).astype(np.int32)
+        for _ in range(60):
+            own.load_yet(offsets, ids, 1 << 22)
+            own.build_yet_index()
+            assert own.yet_index_info()["method"] == "buckets"
+
+    _on_two_threads(build, ((2_000, 1_050), (2_097_152, 1)))
