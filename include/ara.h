@@ -328,8 +328,7 @@ ARA_API int ara_set_batch_config(ara_ctx *ctx, int32_t item, int32_t blocks_per_
  * ELT side): for each catalogue event, its occurrences (trial, event index) in
  * trial order, built on the device: by two stable partitions of the YET's
  * events by id (catalogues of up to 2^22 ids, with 8 bytes per event of
- * scratch, kept with the passes' event buffer unless the context has a
- * budget); where those do not fit, each occurrence is counted into and placed
+ * scratch); where those do not fit, each occurrence is counted into and placed
  * in a bucket per (event, 262,144-trial cell), and each bucket sorted; and
  * where a bucket would hold more than 2,048 occurrences, by a stable radix sort
  * of the YET's events by id (the same index each way).  Once built, batched passes (ara_run_layers and the serving loop)
@@ -341,9 +340,11 @@ ARA_API int ara_set_batch_config(ara_ctx *ctx, int32_t item, int32_t blocks_per_
  * 262,144 trials (the serving chunk), so that a pass's slices of trials find
  * their occurrences without a search.  It takes 8 bytes per YET event and
  * 4 * (ceil(n_trials / 262144) + 1) per catalogue id, and lasts until the next
- * YET load (without a budget its buffers stay allocated for the next build);
- * the partition and bucket builds need 4 bytes per (catalogue id, cell) of
- * scratch besides, the radix sort about 24 bytes per event.  Errors: ARA_ENOTLOADED; ARA_EINVAL (served requests queued or
+ * YET load.  That load frees its buffers, or, without a budget and where a
+ * quarter of the device's memory is free, leaves them for the new YET's build,
+ * and the next call on the context other than the build, an ELT load or
+ * ara_finish_yet frees them.  The partition and bucket builds need 4 bytes per
+ * (catalogue id, cell) of scratch besides, the radix sort about 24 bytes per event.  Errors: ARA_ENOTLOADED; ARA_EINVAL (served requests queued or
  * running, or 2^32 or more events); ARA_ENOMEM; ARA_ECUDA.
  * ara_yet_index_info reports whether the index is built, its bytes, the
  * device time of its build and how it was built (0 partitions or buckets, 1 radix sort, -1

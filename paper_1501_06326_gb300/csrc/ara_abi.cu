@@ -118,9 +118,9 @@ struct ara_ctx {
   DevBuf marks, word_base, rankdir, slot_start, pairs, pairs_hot, pairs_w, pairs_ev, scan_tmp;
   DevBuf ev_buf, tile_cnt;  // hit-event records of the layer kernels
   // event-major index of the YET (ara_build_yet_index) and the indexed passes' buffers
-  DevBuf yix_occ, yix_grid, yix_work;
+  DevBuf yix_occ, yix_grid;
   bool yix_ready = false;
-  bool yix_building = false;  // its buffers are being filled
+  bool yix_idle = false;   // its buffers are held without an index
   bool yix_sorted = false;  // built by the radix sort (a bucket was too large)
   float yix_build_ms = 0.0f;
   int64_t yix_bytes = 0;
@@ -292,14 +292,37 @@ void release(ara_ctx* c, DevBuf& b) {
   b.bytes = 0;
 }
 
-// Frees the index buffers that no index is in (kept from an earlier YET for
-// the next build); false when there is nothing to free.
+// Frees the index buffers that no index is in (those of a YET that was
+// replaced, held for the next one's build: see yet_begin); false when there is
+// nothing to free.
 bool release_idle_index(ara_ctx* c) {
-  if (c->yix_ready || c->yix_building || (!c->yix_occ.ptr && !c->yix_grid.ptr && !c->yix_work.ptr)) return false;
+  if (!c->yix_idle) return false;
+  c->yix_idle = false;
   release(c, c->yix_occ);
   release(c, c->yix_grid);
-  release(c, c->yix_work);
   return true;
+}
+
+// Makes the context's device current.  A call that shows that the YET is used
+// without an index, any but a load and the build, gives held index buffers back.
+int bind(ara_ctx* c, bool keep_index = false) {
+  if (!c) return ARA_EINVAL;
+  ARA_CUDA(c, cudaSetDevice(c->device));
+  if (!keep_index && c->yix_idle) {
+    // (memory cannot be freed while the stream is captured; a capture elsewhere is none of this call's)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess) {
+      cudaGetLastError();
+      capture = cudaStreamCaptureStatusActive;
+    }
+    if (capture == cudaStreamCaptureStatusNone) {
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      ARA_CUDA(c, cudaThreadExchangeStreamCaptureMode(&mode));
+      release_idle_index(c);
+      ARA_CUDA(c, cudaThreadExchangeStreamCaptureMode(&mode));
+    }
+  }
+  return ARA_OK;
 }
 
 // Make b hold at least `bytes` (contents are not preserved).
@@ -362,11 +385,6 @@ cudaMemcpyKind kind_to_device(const void* src) {
   return is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
 }
 
-int bind(ara_ctx* c) {
-  if (!c) return ARA_EINVAL;
-  ARA_CUDA(c, cudaSetDevice(c->device));
-  return ARA_OK;
-}
 
 }  // namespace
 
@@ -443,7 +461,7 @@ int yet_finish(ara_ctx* c) {
 // runs beside later work on the context's stream until yet_finish.
 int yet_begin(ara_ctx* c, int64_t n_trials, const int64_t* offsets, const int32_t* event_ids,
               int32_t catalogue_size, const char* who) {
-  int rc = bind(c);
+  int rc = bind(c, true);
   if (rc) return rc;
   if (n_trials < 1 || !offsets || catalogue_size < 1)
     return fail(c, ARA_EINVAL, "%s: need n_trials >= 1, offsets and catalogue_size >= 1", who);
@@ -458,8 +476,12 @@ int yet_begin(ara_ctx* c, int64_t n_trials, const int64_t* offsets, const int32_
     ARA_CUDA(c, cudaEventSynchronize(c->yet_ready));
   }
   c->yet_loaded = false;
-  // the index belongs to the YET being replaced; without a budget its buffers stay for the next build
-  // (allocating and freeing 8 bytes an event costs milliseconds), until an allocation needs their room
+  // The index belongs to the YET being replaced.  Its buffers are held for the next build (to free and
+  // allocate 8 bytes an event costs 2.7 ms at 400M events, in a renewal of 9.4) until the next call shows
+  // whether there is one; not under a budget, nor where the device then has less than a quarter free, nor
+  // from before the replaced YET.
+  release_idle_index(c);
+  c->yix_idle = c->yix_occ.ptr || c->yix_grid.ptr;
   c->yix_ready = false;
   if (c->budget) release_idle_index(c);
   if (!c->copy_stream) {
@@ -479,6 +501,11 @@ int yet_begin(ara_ctx* c, int64_t n_trials, const int64_t* offsets, const int32_
   if ((rc = reserve(c, c->yet_off, sizeof(int64_t) * (n_trials + 1)))) return rc;
   // ids: padded by 8 entries so that 32-byte loads near the end stay inside the buffer
   if ((rc = reserve(c, c->yet_ids, sizeof(int32_t) * (n_events + 8)))) return rc;
+  if (c->yix_idle) {
+    size_t room = 0, total = 0;
+    ARA_CUDA(c, cudaMemGetInfo(&room, &total));
+    if (room < total / 4) release_idle_index(c);
+  }
   cudaStream_t cs = c->copy_stream;
   uint32_t* flags = static_cast<uint32_t*>(c->yet_flags.ptr);
   ARA_CUDA(c, cudaMemsetAsync(flags, 0, sizeof(uint32_t), cs));
@@ -532,7 +559,7 @@ int ara_load_yet_async(ara_ctx* c, int64_t n_trials, const int64_t* offsets, con
 }
 
 int ara_finish_yet(ara_ctx* c) {
-  const int rc = bind(c);
+  const int rc = bind(c, true);
   return rc ? rc : yet_finish(c);
 }
 
@@ -540,7 +567,7 @@ int ara_finish_yet(ara_ctx* c) {
 static int load_elts_impl(ara_ctx* c, const char* who, int32_t n_elts, const int32_t* elt_ids,
                           const int64_t* rec_offsets, const int32_t* event_ids, const float* mean, const float* sigma,
                           const float* sigma_c, const float* exposure, const ara_elt_terms* terms) {
-  int rc = bind(c);
+  int rc = bind(c, true);
   if (rc) return rc;
   if (n_elts < 1 || !elt_ids || !rec_offsets) return fail(c, ARA_EINVAL, "%s: bad arguments", who);
   std::vector<int32_t> ids(n_elts);
@@ -702,7 +729,7 @@ int ara_load_elts(ara_ctx* c, int32_t n_elts, const int32_t* elt_ids, const int6
 int ara_load_xelts(ara_ctx* c, int32_t n_elts, const int32_t* elt_ids, const int64_t* rec_offsets,
                    const int32_t* event_ids, const float* mean, const float* sigma_i, const float* sigma_c,
                    const float* exposure, const ara_elt_terms* terms) {
-  int rc = bind(c);
+  int rc = bind(c, true);
   if (rc) return rc;
   if (!sigma_c && n_elts >= 1 && rec_offsets) {
     int64_t R = 0;
@@ -1314,7 +1341,7 @@ static_assert(ARA_BATCH_ITEM_TILE == ara::kItemTile && ARA_BATCH_ITEM_TRIAL == a
 
 int ara_build_yet_index(ara_ctx* c) {
   static const char* who = "ara_build_yet_index";
-  int rc = bind(c);
+  int rc = bind(c, true);
   if (rc) return rc;
   if ((rc = yet_finish(c))) return rc;
   if (!c->yet_loaded) return fail(c, ARA_ENOTLOADED, "%s: no YET loaded", who);
@@ -1325,42 +1352,44 @@ int ara_build_yet_index(ara_ctx* c) {
     return fail(c, ARA_EINVAL, "%s: the YET holds 2^32 or more events", who);
   const int64_t n = c->n_events;
   const int64_t cells = ara::yet_grid_cells(c->n_trials, kYetGridShift);
-  // while the build runs, an allocation that fails may not take the index's buffers
-  struct Building {
-    ara_ctx* c;
-    explicit Building(ara_ctx* x) : c(x) { c->yix_building = true; }
-    ~Building() { c->yix_building = false; }
-  } building(c);
+  DevBuf work, parts_buf;  // scratch
+  auto drop_scratch = [&]() {
+    release(c, work);
+    release(c, parts_buf);
+  };
   auto drop = [&]() {
+    drop_scratch();
     release(c, c->yix_occ);
     release(c, c->yix_grid);
-    release(c, c->yix_work);
   };
+  // held buffers are the index's again, unless they are more than twice what it needs
+  if (c->yix_occ.bytes > 2 * sizeof(unsigned long long) * static_cast<size_t>(n + 1)) release_idle_index(c);
+  c->yix_idle = false;
   if ((rc = reserve(c, c->yix_occ, sizeof(unsigned long long) * (n + 1))) ||
       (rc = reserve(c, c->yix_grid, sizeof(uint32_t) * (static_cast<size_t>(c->catalogue) * (cells + 1) + 1)))) {
     drop();
     return rc;
   }
   // The partition build where its fields fit and its 8 bytes an event of scratch do (the event buffer of
-  // the streaming passes serves as that scratch), else the bucket build with its 4 bytes per (event, cell).
+  // the streaming passes where it is large enough, else a buffer for the build alone), else the bucket build
+  // with its 4 bytes per (event, cell).
   bool parts = ara::yet_parts_fit(c->n_trials, n, c->catalogue, cells, c->num_sms);
-  const size_t ev_before = c->ev_buf.bytes;
+  const size_t parts_bytes = sizeof(unsigned long long) * static_cast<size_t>(n);
+  const bool in_ev_buf = c->ev_buf.bytes >= parts_bytes;
   if (parts) {
-    const bool room = c->ev_buf.bytes >= sizeof(uint2) * static_cast<size_t>(n + 1) || !c->budget ||
-                      c->used - c->ev_buf.bytes + sizeof(uint2) * static_cast<size_t>(n + 1) +
-                              ara::yet_parts_scratch_bytes(n, c->catalogue, cells, c->num_sms) <=
-                          c->budget;
-    parts = room && reserve(c, c->ev_buf, sizeof(uint2) * (n + 1)) == ARA_OK &&
-            reserve(c, c->yix_work, ara::yet_parts_scratch_bytes(n, c->catalogue, cells, c->num_sms)) == ARA_OK;
+    const size_t work_bytes = ara::yet_parts_scratch_bytes(n, c->catalogue, cells, c->num_sms);
+    parts = (!c->budget || c->used + (in_ev_buf ? 0 : parts_bytes) + work_bytes <= c->budget) &&
+            (in_ev_buf || reserve(c, parts_buf, parts_bytes) == ARA_OK) && reserve(c, work, work_bytes) == ARA_OK;
+    if (!parts) drop_scratch();
   }
-  if (!parts && (rc = reserve(c, c->yix_work, ara::yet_bucket_scratch_bytes(c->catalogue, cells)))) {
+  if (!parts && (rc = reserve(c, work, ara::yet_bucket_scratch_bytes(c->catalogue, cells)))) {
     drop();
     return rc;
   }
   const int64_t* off = static_cast<const int64_t*>(c->yet_off.ptr);
   const int32_t* ids = static_cast<const int32_t*>(c->yet_ids.ptr);
   unsigned long long* occ = static_cast<unsigned long long*>(c->yix_occ.ptr);
-  unsigned long long* first = static_cast<unsigned long long*>(c->ev_buf.ptr);
+  unsigned long long* first = static_cast<unsigned long long*>(in_ev_buf ? c->ev_buf.ptr : parts_buf.ptr);
   uint32_t* grid = static_cast<uint32_t*>(c->yix_grid.ptr);
   cudaEvent_t a = nullptr, b = nullptr;
   cudaError_t e = cudaEventCreate(&a);
@@ -1371,29 +1400,29 @@ int ara_build_yet_index(ara_ctx* c) {
   uint32_t max_bucket = 0;
   if (e == cudaSuccess)
     e = parts ? ara::yet_parts_count(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, c->num_sms, first, grid,
-                                     c->yix_work.ptr, c->stream, &launched)
-              : ara::yet_index_count(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, c->yix_work.ptr,
+                                     work.ptr, c->stream, &launched)
+              : ara::yet_index_count(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, work.ptr,
                                      c->stream, &launched);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(&max_bucket,
-                        parts ? c->yix_work.ptr : ara::yet_index_max_bucket(c->yix_work.ptr, c->catalogue, cells),
+                        parts ? work.ptr : ara::yet_index_max_bucket(work.ptr, c->catalogue, cells),
                         sizeof max_bucket, cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   const bool buckets = max_bucket <= kYetBucketSortMax;
   if (e == cudaSuccess && buckets)
     e = parts ? ara::yet_parts_fill(c->n_trials, n, c->catalogue, kYetGridShift, c->num_sms, first, grid, occ,
-                                    c->yix_work.ptr, c->stream, &launched)
-              : ara::yet_index_fill(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, occ, c->yix_work.ptr,
+                                    work.ptr, c->stream, &launched)
+              : ara::yet_index_fill(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, occ, work.ptr,
                                     c->stream, &launched);
   if (e == cudaSuccess && !buckets) {
-    if (c->budget && c->ev_buf.bytes > ev_before) release(c, c->ev_buf);
-    if ((rc = reserve(c, c->yix_work, ara::yet_index_scratch_bytes(n, c->catalogue)))) {
+    drop_scratch();
+    if ((rc = reserve(c, work, ara::yet_index_scratch_bytes(n, c->catalogue)))) {
       if (a) cudaEventDestroy(a);
       if (b) cudaEventDestroy(b);
       drop();
       return rc;
     }
-    e = ara::build_yet_index(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, occ, grid, c->yix_work.ptr,
+    e = ara::build_yet_index(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, occ, grid, work.ptr,
                              c->stream, &launched);
   }
   if (e == cudaSuccess) e = cudaEventRecord(b, c->stream);
@@ -1402,9 +1431,7 @@ int ara_build_yet_index(ara_ctx* c) {
   if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
   if (a) cudaEventDestroy(a);
   if (b) cudaEventDestroy(b);
-  // scratch that a budget counts, or the sort build's 24 bytes an event, is given back
-  if (c->budget || !buckets) release(c, c->yix_work);
-  if (c->budget && c->ev_buf.bytes > ev_before) release(c, c->ev_buf);
+  drop_scratch();
   c->launches += launched;
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -2226,7 +2253,7 @@ void ara_destroy(ara_ctx* c) {
                     &c->pairs,      &c->pairs_hot,      &c->pairs_w,       &c->pairs_ev,       &c->scan_tmp,
                     &c->counters,       &c->ylt_tmp,       &c->diag_tmp,       &c->sel,
                     &c->in_tmp,     &c->out_tmp,        &c->serve_arena,   &c->serve_out,      &c->yix_occ,
-                    &c->yix_grid,   &c->yix_work,       &c->u_event,       &c->idx_acc,
+                    &c->yix_grid,   &c->u_event,       &c->idx_acc,
                     &c->ev_occ,     &c->row_base,       &c->evr_stage,     &c->yet_flags};
   for (DevBuf* b : bufs) release(c, *b);
   for (auto& e : c->ev)

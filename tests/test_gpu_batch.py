@@ -592,3 +592,78 @@ def test_contexts_on_threads_index_unlike_yets(eng):
             assert own.yet_index_info()["method"] == "buckets"
 
     _on_two_threads(build, ((2_000, 1_050), (2_097_152, 1)))
+
+
+def _even_yet(trials, per_trial, C, seed):
+    offsets = np.arange(trials + 1, dtype=np.int64) * per_trial
+    return synth.YET(offsets, np.random.default_rng(seed).integers(0, C, trials * per_trial).astype(np.int32), C)
+
+
+@pytest.mark.parametrize("use", ["a pass", "a tail"])
+def test_yet_index_holds_its_own_memory_only(use):
+    """A build keeps the index's bytes and nothing else; after the next YET's
+    load the first call other than the build gives them back to the device,
+    and a build straight after the load takes them over."""
+    import torch
+
+    from paper_1501_06326_gb300 import ara
+
+    yet, pool = _even_yet(8_000, 1_000, 1 << 20, 3), synth.make_elt_pool(2, 500, 1 << 20, 4)
+    out = np.zeros(50)
+    own = ara.Ara(0)
+
+    def call():
+        if use == "a pass":
+            own.run_layer(pool.elt_ids, (10.0, 1e6, 1e2, 1e8), 1, 0, 50, out)
+        else:
+            own.pml_tvar(out, [2.0])
+
+    try:
+        own.load_pool(pool)
+        free = []
+        for step in ("load", "call", "build", "load", "call", "build", "load", "build", "call"):
+            if step == "load":
+                own.load_yet(yet.offsets, yet.event_ids, yet.catalogue_size)
+            elif step == "build":
+                own.build_yet_index()
+            else:
+                call()
+            free.append(torch.cuda.mem_get_info()[0])
+        slack = 12 << 20  # six buffers' rounding to 2 MB
+        index = own.yet_index_info()["bytes"]
+        assert index >= 8 * yet.n_events
+        assert abs(free[1] - free[2] - index) <= slack
+        assert abs(free[1] - free[4]) <= slack
+        assert abs(free[1] - free[5] - index) <= slack and abs(free[1] - free[8] - index) <= slack
+    finally:
+        own.close()
+
+
+def test_yet_index_leaves_captured_calls_their_buffers():
+    """A layer call captured over a few trials replays with the same bits after
+    an index build, whose scratch is larger than the call's event buffer."""
+    import torch
+
+    from paper_1501_06326_gb300 import ara
+
+    yet, pool = _even_yet(8_000, 1_000, 20_000, 4), synth.make_elt_pool(3, 500, 20_000, 5)
+    stream = torch.cuda.Stream()
+    own = ara.Ara(0, 0, stream.cuda_stream)
+    try:
+        own.load_yet(yet.offsets, yet.event_ids, yet.catalogue_size)
+        own.load_pool(pool)
+        out = torch.zeros(50, dtype=torch.float64, device="cuda")
+        run = lambda: own.run_layer(pool.elt_ids, (10.0, 1e6, 1e2, 1e8), 1, 0, 50, out)  # noqa: E731
+        run()
+        torch.cuda.synchronize()
+        first = out.cpu().numpy()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            run()
+        own.build_yet_index()
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), first) and np.count_nonzero(first) > 0
+    finally:
+        own.close()
