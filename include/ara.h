@@ -327,8 +327,9 @@ ARA_API int ara_set_batch_config(ara_ctx *ctx, int32_t item, int32_t blocks_per_
 /* The event-major index of the loaded YET (Section 2.1's lookup taken from the
  * ELT side): for each catalogue event, its occurrences (trial, event index) in
  * trial order, built on the device: by two stable partitions of the YET's
- * events by id (catalogues of up to 2^22 ids, with 8 bytes per event of
- * scratch); where those do not fit, each occurrence is counted into and placed
+ * events by id (catalogues of up to 2^22 ids, no group of neighbouring ids
+ * with more than a 32nd of the events, 8 bytes per event of scratch); where
+ * those do not fit, each occurrence is counted into and placed
  * in a bucket per (event, 262,144-trial cell), and each bucket sorted; and
  * where a bucket would hold more than 2,048 occurrences, by a stable radix sort
  * of the YET's events by id (the same index each way).  Once built, batched passes (ara_run_layers and the serving loop)

@@ -1370,67 +1370,93 @@ int ara_build_yet_index(ara_ctx* c) {
     drop();
     return rc;
   }
-  // The partition build where its fields fit and its 8 bytes an event of scratch do (the event buffer of
-  // the streaming passes where it is large enough, else a buffer for the build alone), else the bucket build
-  // with its 4 bytes per (event, cell).
-  bool parts = ara::yet_parts_fit(c->n_trials, n, c->catalogue, cells, c->num_sms);
-  const size_t parts_bytes = sizeof(unsigned long long) * static_cast<size_t>(n);
-  const bool in_ev_buf = c->ev_buf.bytes >= parts_bytes;
-  if (parts) {
-    const size_t work_bytes = ara::yet_parts_scratch_bytes(n, c->catalogue, cells, c->num_sms);
-    parts = (!c->budget || c->used + (in_ev_buf ? 0 : parts_bytes) + work_bytes <= c->budget) &&
-            (in_ev_buf || reserve(c, parts_buf, parts_bytes) == ARA_OK) && reserve(c, work, work_bytes) == ARA_OK;
-    if (!parts) drop_scratch();
-  }
-  if (!parts && (rc = reserve(c, work, ara::yet_bucket_scratch_bytes(c->catalogue, cells)))) {
-    drop();
-    return rc;
-  }
   const int64_t* off = static_cast<const int64_t*>(c->yet_off.ptr);
   const int32_t* ids = static_cast<const int32_t*>(c->yet_ids.ptr);
   unsigned long long* occ = static_cast<unsigned long long*>(c->yix_occ.ptr);
-  unsigned long long* first = static_cast<unsigned long long*>(in_ev_buf ? c->ev_buf.ptr : parts_buf.ptr);
   uint32_t* grid = static_cast<uint32_t*>(c->yix_grid.ptr);
-  cudaEvent_t a = nullptr, b = nullptr;
-  cudaError_t e = cudaEventCreate(&a);
-  if (e == cudaSuccess) e = cudaEventCreate(&b);
-  if (e == cudaSuccess) e = cudaEventRecord(a, c->stream);
-  int launched = 0;
-  // partitions or buckets while the largest (event, grid cell) is small; else the radix sort
-  uint32_t max_bucket = 0;
-  if (e == cudaSuccess)
-    e = parts ? ara::yet_parts_count(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, c->num_sms, first, grid,
-                                     work.ptr, c->stream, &launched)
-              : ara::yet_index_count(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, work.ptr,
-                                     c->stream, &launched);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&max_bucket,
-                        parts ? work.ptr : ara::yet_index_max_bucket(work.ptr, c->catalogue, cells),
-                        sizeof max_bucket, cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  const bool buckets = max_bucket <= kYetBucketSortMax;
-  if (e == cudaSuccess && buckets)
-    e = parts ? ara::yet_parts_fill(c->n_trials, n, c->catalogue, kYetGridShift, c->num_sms, first, grid, occ,
-                                    work.ptr, c->stream, &launched)
-              : ara::yet_index_fill(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, occ, work.ptr,
-                                    c->stream, &launched);
-  if (e == cudaSuccess && !buckets) {
-    drop_scratch();
-    if ((rc = reserve(c, work, ara::yet_index_scratch_bytes(n, c->catalogue)))) {
-      if (a) cudaEventDestroy(a);
-      if (b) cudaEventDestroy(b);
-      drop();
-      return rc;
+  // the build's device time: from tm[0] to tm[1] (the partitions' count, where there is one) and from tm[2] to
+  // tm[3], without the allocation of the partitions' scratch
+  struct Times {
+    cudaEvent_t tm[4] = {nullptr, nullptr, nullptr, nullptr};
+    ~Times() {
+      for (cudaEvent_t x : tm)
+        if (x) cudaEventDestroy(x);
     }
-    e = ara::build_yet_index(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, occ, grid, work.ptr,
-                             c->stream, &launched);
+  } times;
+  cudaEvent_t* tm = times.tm;
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreate(&tm[i]);
+  int launched = 0;
+  auto read = [&](const uint32_t* from, uint32_t* to) {
+    const cudaError_t r = cudaMemcpyAsync(to, from, sizeof *to, cudaMemcpyDeviceToHost, c->stream);
+    return r == cudaSuccess ? cudaStreamSynchronize(c->stream) : r;
+  };
+  // scratch of another build in place of what is held
+  auto reserve_work = [&](size_t bytes) {
+    drop_scratch();
+    const int r = reserve(c, work, bytes);
+    if (r) drop();
+    return r;
+  };
+  // The partition build where its fields fit and no bucket of the first partition holds too many of the events,
+  // and where its 8 bytes an event of scratch do (the event buffer of the streaming passes where it is large
+  // enough, else a buffer for the build alone); else the bucket build with its 4 bytes per (event, cell).
+  bool parts = ara::yet_parts_fit(c->n_trials, n, c->catalogue, cells, c->num_sms), counted = false, sorted = false;
+  unsigned long long* first = static_cast<unsigned long long*>(c->ev_buf.ptr);
+  if (parts) {
+    const size_t parts_bytes = sizeof(unsigned long long) * static_cast<size_t>(n);
+    const size_t work_bytes = ara::yet_parts_scratch_bytes(n, c->catalogue, cells, c->num_sms);
+    const bool in_ev_buf = c->ev_buf.bytes >= parts_bytes;
+    uint32_t largest = 0;
+    counted = (!c->budget || c->used + (in_ev_buf ? 0 : parts_bytes) + work_bytes <= c->budget) &&
+              reserve(c, work, work_bytes) == ARA_OK;
+    if (e == cudaSuccess && counted) e = cudaEventRecord(tm[0], c->stream);
+    if (e == cudaSuccess && counted)
+      e = ara::yet_parts_count(ids, n, c->catalogue, cells, c->num_sms, work.ptr, c->stream, &launched);
+    if (e == cudaSuccess && counted) e = cudaEventRecord(tm[1], c->stream);
+    if (e == cudaSuccess && counted) e = read(static_cast<const uint32_t*>(work.ptr), &largest);
+    parts = counted && ara::yet_parts_even(largest, n) && (in_ev_buf || reserve(c, parts_buf, parts_bytes) == ARA_OK);
+    if (!in_ev_buf) first = static_cast<unsigned long long*>(parts_buf.ptr);
+    // a bucket whose (event, cell)s cannot all be small goes to the sort without a count of each (4.2 ms where
+    // 6% of 100M events are alike)
+    sorted = !parts && largest / kYetBucketSortMax >=
+                           static_cast<uint64_t>(cells) * ara::yet_parts_bucket_ids(n, c->catalogue, c->num_sms);
   }
-  if (e == cudaSuccess) e = cudaEventRecord(b, c->stream);
-  if (e == cudaSuccess) e = cudaEventSynchronize(b);
-  float ms = 0.0f;
-  if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
-  if (a) cudaEventDestroy(a);
-  if (b) cudaEventDestroy(b);
+  if (!parts && (rc = reserve_work(sorted ? ara::yet_index_scratch_bytes(n, c->catalogue)
+                                          : ara::yet_bucket_scratch_bytes(c->catalogue, cells))))
+    return rc;
+  if (e == cudaSuccess) e = cudaEventRecord(tm[2], c->stream);
+  if (parts) {
+    if (e == cudaSuccess)
+      e = ara::yet_parts_first(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, c->num_sms, first, grid, work.ptr,
+                               c->stream, &launched);
+    if (e == cudaSuccess)
+      e = ara::yet_parts_fill(c->n_trials, n, c->catalogue, kYetGridShift, c->num_sms, first, grid, occ, work.ptr,
+                              c->stream, &launched);
+  } else {
+    // buckets while the largest (event, grid cell) is small; else the radix sort
+    if (e == cudaSuccess && !sorted) {
+      uint32_t largest = 0;
+      e = ara::yet_index_count(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, work.ptr, c->stream,
+                               &launched);
+      if (e == cudaSuccess) e = read(ara::yet_index_max_bucket(work.ptr, c->catalogue, cells), &largest);
+      sorted = largest > kYetBucketSortMax;
+      if (e == cudaSuccess && !sorted)
+        e = ara::yet_index_fill(off, ids, c->n_trials, c->catalogue, kYetGridShift, grid, occ, work.ptr, c->stream,
+                                &launched);
+      else if (e == cudaSuccess && (rc = reserve_work(ara::yet_index_scratch_bytes(n, c->catalogue))))
+        return rc;
+    }
+    if (e == cudaSuccess && sorted)
+      e = ara::build_yet_index(off, ids, c->n_trials, n, c->catalogue, kYetGridShift, occ, grid, work.ptr, c->stream,
+                               &launched);
+  }
+  if (e == cudaSuccess) e = cudaEventRecord(tm[3], c->stream);
+  if (e == cudaSuccess) e = cudaEventSynchronize(tm[3]);
+  float ms = 0.0f, count_ms = 0.0f;
+  if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, tm[2], tm[3]);
+  if (e == cudaSuccess && counted) e = cudaEventElapsedTime(&count_ms, tm[0], tm[1]);
+  ms += count_ms;
   drop_scratch();
   c->launches += launched;
   if (e != cudaSuccess) {
@@ -1438,7 +1464,7 @@ int ara_build_yet_index(ara_ctx* c) {
     drop();
     return fail(c, ARA_ECUDA, "%s: %s", who, cudaGetErrorString(e));
   }
-  c->yix_sorted = !buckets;
+  c->yix_sorted = sorted;
   c->yix_ready = true;
   c->yix_build_ms = ms;
   c->yix_bytes = static_cast<int64_t>(sizeof(unsigned long long) * (n + 1) +

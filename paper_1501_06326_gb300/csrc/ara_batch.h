@@ -56,15 +56,21 @@ cudaError_t yet_index_fill(const int64_t* off, const int32_t* ids, int64_t n_tri
                            const uint32_t* ev_grid, unsigned long long* occ, void* scratch, cudaStream_t s,
                            int* n_launch);
 // The partition build: two stable partitions by event id through shared
-// memory, the first into `parts` (8 bytes an event).  yet_parts_count makes the
-// first partition, counts each (event, grid cell) and scans the counts into
-// ev_grid; the largest count is left in the first word of `scratch`.
-// yet_parts_fill makes the second partition into occ.  yet_parts_fit: whether a
-// YET's ids, trials and cells fit its fields and shared memory (at most 2^22
-// event ids, 2^31 trials).  `scratch` holds yet_parts_scratch_bytes for both.
+// memory, the first into `parts` (8 bytes an event).  yet_parts_count counts
+// the first partition's buckets, of yet_parts_bucket_ids ids each; the largest
+// one's count is left in the first word of `scratch`, and yet_parts_even says
+// whether it is small enough for one CTA.  yet_parts_first makes the first partition, counts each (event, grid
+// cell) and scans the counts into ev_grid; yet_parts_fill makes the second
+// partition into occ.  yet_parts_fit: whether a YET's ids, trials and cells fit
+// the build's fields and shared memory (at most 2^22 event ids, 2^31 trials).
+// `scratch` holds yet_parts_scratch_bytes for all three.
 bool yet_parts_fit(int64_t n_trials, int64_t n_events, int32_t catalogue, int64_t cells, int num_sms);
 size_t yet_parts_scratch_bytes(int64_t n_events, int32_t catalogue, int64_t cells, int num_sms);
-cudaError_t yet_parts_count(const int64_t* off, const int32_t* ids, int64_t n_trials, int64_t n_events,
+cudaError_t yet_parts_count(const int32_t* ids, int64_t n_events, int32_t catalogue, int64_t cells, int num_sms,
+                            void* scratch, cudaStream_t s, int* n_launch);
+int64_t yet_parts_bucket_ids(int64_t n_events, int32_t catalogue, int num_sms);
+bool yet_parts_even(uint32_t largest, int64_t n_events);
+cudaError_t yet_parts_first(const int64_t* off, const int32_t* ids, int64_t n_trials, int64_t n_events,
                             int32_t catalogue, int grid_shift, int num_sms, unsigned long long* parts,
                             uint32_t* ev_grid, void* scratch, cudaStream_t s, int* n_launch);
 cudaError_t yet_parts_fill(int64_t n_trials, int64_t n_events, int32_t catalogue, int grid_shift, int num_sms,

@@ -667,3 +667,37 @@ def test_yet_index_leaves_captured_calls_their_buffers():
         assert np.array_equal(out.cpu().numpy(), first) and np.count_nonzero(first) > 0
     finally:
         own.close()
+
+
+@pytest.mark.parametrize("shape", ["short-trials", "dense", "dense-long-trials", "uneven"])
+def test_yet_index_of_many_tiles(eng, shape):
+    """YETs whose partitions take several tiles of 16,384 occurrences a CTA: in
+    the first (above 608 tiles; trials from none to thousands of events, so that
+    a tile ends in any of them) and in the second (a catalogue of 300 ids, whose
+    events have far more occurrences than a thread would sort, and which the
+    partitions still index).  A fifth of the events alike: one CTA's
+    bucket, left to the radix sort.  The dense item's bits, over all trials and
+    within a grid cell."""
+    rng = np.random.default_rng(len(shape))
+    lens, C, method = {
+        "short-trials": (np.where(rng.random(400_000) < 0.9, rng.integers(0, 40, 400_000), 0), 1 << 21, "buckets"),
+        "dense": (rng.integers(0, 60, 400_000), 300, "buckets"),
+        "dense-long-trials": (np.concatenate([[0, 3_000_000, 0, 1], rng.integers(0, 20_000, 950)]), 4_000, "buckets"),
+        "uneven": (rng.integers(0, 60, 100_000), 4_000, "radix sort"),
+    }[shape]
+    if shape == "short-trials":
+        lens[::5_000] = 60_000
+    offsets = np.zeros(len(lens) + 1, np.int64)
+    offsets[1:] = np.cumsum(lens)
+    n, N = int(offsets[-1]), len(lens)
+    pool = synth.make_elt_pool(4, min(C // 2, 300), C, 33)
+    ev = rng.integers(0, C, n, dtype=np.int32)
+    if shape == "short-trials":
+        ev[::3] = rng.choice(pool.event_ids, len(ev[::3]))
+    if shape == "uneven":
+        ev[::5] = pool.event_ids[0]
+    yet = synth.YET(offsets, ev, C)
+    layers = [(np.array(ids, np.int32), (10.0, 5e5, 1e2, 5e9), None) for ids in ([0, 1], [1, 2, 3])]
+    for t0, t1 in {(0, N), (N // 3, N - N // 5)}:
+        _assert_same_bits(_run_items(eng, yet, pool, layers, 2, t0, t1))
+    assert eng.yet_index_info()["method"] == method
