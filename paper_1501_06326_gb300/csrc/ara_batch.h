@@ -62,7 +62,8 @@ cudaError_t yet_index_fill(const int64_t* off, const int32_t* ids, int64_t n_tri
 // whether it is small enough for one CTA.  yet_parts_first makes the first partition, counts each (event, grid
 // cell) and scans the counts into ev_grid; yet_parts_fill makes the second
 // partition into occ.  yet_parts_fit: whether a YET's ids, trials and cells fit
-// the build's fields and shared memory (at most 2^22 event ids, 2^31 trials).
+// the build's fields and shared memory (at most 2^22 event ids, 2^31 trials),
+// and its events are enough for it to be the faster one.
 // `scratch` holds yet_parts_scratch_bytes for all three.
 bool yet_parts_fit(int64_t n_trials, int64_t n_events, int32_t catalogue, int64_t cells, int num_sms);
 size_t yet_parts_scratch_bytes(int64_t n_events, int32_t catalogue, int64_t cells, int num_sms);

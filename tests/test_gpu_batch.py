@@ -701,3 +701,34 @@ def test_yet_index_of_many_tiles(eng, shape):
     for t0, t1 in {(0, N), (N // 3, N - N // 5)}:
         _assert_same_bits(_run_items(eng, yet, pool, layers, 2, t0, t1))
     assert eng.yet_index_info()["method"] == method
+
+
+@pytest.mark.parametrize("shape,launches", [("few", 5), ("tile", 7), ("tile-and-one", 7), ("short-trials", 7),
+                                            ("long-trials", 7), ("many-digits", 9)])
+def test_yet_index_partition_edges(eng, shape, launches):
+    """The partitions at the edges of their tiles (16,384 occurrences), of their
+    trial lookup (many empty trials, trials longer than a tile) and of the line
+    below which a YET has too few events for them (16 a catalogue id, which the
+    launches of the build show): the dense item's bits."""
+    rng = np.random.default_rng(len(shape))
+    lens, C = {
+        "few": ([16_000 // 64] * 64, 1_000),
+        "tile": ([16_384 // 64] * 64, 1_000),
+        "tile-and-one": ([16_384 // 64] * 64 + [1], 1_023),
+        "short-trials": (list(rng.integers(0, 3, 30_000)) + [0] * 5_000 + list(rng.integers(0, 2, 20_000)), 1_025),
+        "long-trials": ([3, 40_000, 0, 17_000, 20_011], 2_049),
+        "many-digits": ([1_001] * 600, 16_385),
+    }[shape]
+    offsets = np.zeros(len(lens) + 1, np.int64)
+    offsets[1:] = np.cumsum(lens)
+    n, N = int(offsets[-1]), len(lens)
+    pool = synth.make_elt_pool(5, 400, C, 33)
+    ev = rng.integers(0, C, n, dtype=np.int32)
+    yet = synth.YET(offsets, ev, C)
+    layers = [(np.array(ids, np.int32), (10.0, 5e5, 1e2, 5e7), None) for ids in ([0, 1, 2], [2, 3, 4], [4])]
+    for t0, t1 in {(0, N), (N // 3, N - N // 5), (N // 2, N // 2 + 1)}:
+        _assert_same_bits(_run_items(eng, yet, pool, layers, 2, t0, t1))
+    eng.load_yet(yet.offsets, yet.event_ids, C)
+    eng.timing(reset=True)
+    eng.build_yet_index()
+    assert eng.timing()["kernel_launches"] == launches
