@@ -205,7 +205,7 @@ __device__ bool beta_cf_df(double a, double b, double x, double* num, double* de
   DF u = df_of(a);          // a + 2m
   DF A2{1.0f, 0.0f}, B2{0.0f, 0.0f}, A1{1.0f, 0.0f}, B1{1.0f, 0.0f};
   DF q_prev{1.0f, 0.0f};
-  DF Ap{1.0f, 0.0f}, Bp{1.0f, 0.0f};  // the convergent of the last test
+  double Ap = 1.0, Bp = 1.0;  // the convergent of the last test
   for (int m = 0; m < 20000; ++m) {
     const DF u1 = df_add_f(u, 1.0f), u2 = df_add_f(u, 2.0f);
     // odd term n = 2m + 1: p = -(a + m)(a + b + m) x, q = (a + 2m)(a + 2m + 1)
@@ -235,17 +235,16 @@ __device__ bool beta_cf_df(double a, double b, double x, double* num, double* de
     B1 = df_scale(B1, k);
     B2 = df_scale(B2, k);
     if ((m & 3) == 3) {
-      // |A1/B1 - Ap/Bp| <= 1e-13 |A1/B1|, cross-multiplied (48 bits tell 1e-13; an FP64 division a test,
-      // with its conversions, took a third of the table build)
-      const DF f = df_mul(A1, Bp);
-      const DF d = df_add(f, df_neg(df_mul(Ap, B1)));
-      if (fabsf(d.hi) <= 1e-13f * fabsf(f.hi)) {
-        *num = df_val(B1);
-        *den = df_val(A1);
+      // |A1/B1 - Ap/Bp| <= 1e-13 |A1/B1|, cross-multiplied in FP64 (the quotients' divisions and the conversions
+      // took a third of the table build)
+      const double An = df_val_fast(A1), Bn = df_val_fast(B1), f = An * Bp;
+      if (fabs(fma(-Ap, Bn, f)) <= 1e-13 * fabs(f)) {
+        *num = Bn;
+        *den = An;
         return true;
       }
-      Ap = A1;
-      Bp = B1;
+      Ap = An;
+      Bp = Bn;
     }
   }
   return false;
