@@ -589,8 +589,10 @@ __device__ bool table_segment_ok(float4 nd, float d1, float e1, double tq, doubl
 
 // Coarse tables: a block builds those of 32 records, lane l of every warp the
 // record order[32 block + l] (or that record itself without an order), warp w
-// the nodes j = w, w + 8, .. at t_j = -T1 + j h, then the segments' checks.  The
-// stored float4 is {x_j, w_{j+1} - w_j, h w'_j, h^2 w''_j}.  need[rec] = 1 for
+// the nodes j = w, w + 8, .. at t_j = -T1 + j h, then the segments' checks.  A
+// load of few records takes 8 a block and a thread a node, whose chain of nodes
+// and checks is a quarter as long (1 record 142 us a load against 230, 1,000
+// 382 and 534, 8,000 663 and 667, 16,000 972 and 900).  The stored float4 is {x_j, w_{j+1} - w_j, h w'_j, h^2 w''_j}.  need[rec] = 1 for
 // a Beta record whose coarse table is not exact (a candidate for a fine table).
 // The iteration and fraction lengths follow the shapes and t: with the records
 // in order of a + b a warp's lanes, at the same t, run about equally long,
@@ -601,12 +603,14 @@ __device__ bool table_segment_ok(float4 nd, float d1, float e1, double tq, doubl
 // fraction and new logarithms and exponentials after the last Newton step; of
 // the stress recipe 4.2 ms, 19.8 with the bracketed solver for the roots near
 // 1.  In order of a + b alone 4.0 and 10.2 ms.
-constexpr int kTabRecs = 32;     // records of a block
-constexpr int kTabWarps = 8;
+constexpr int kTabThreads = 256;
 
-__global__ void __launch_bounds__(32 * kTabWarps, 2) k_build_tables(Pair* recs, const BetaShape* shapes, int64_t n,
-                                                                   const int64_t* order, float4* tab,
-                                                                   uint32_t* need) {
+// kTabRecs: records of a block, thread t the record t mod kTabRecs.
+template <int kTabRecs>
+__global__ void __launch_bounds__(kTabThreads, 2) k_build_tables(Pair* recs, const BetaShape* shapes, int64_t n,
+                                                                 const int64_t* order, float4* tab, uint32_t* need) {
+  constexpr int kGroups = kTabThreads / kTabRecs;  // threads of a record
+  static_assert(kTabRecs <= 32 && kGroups <= kTabNodes && kTabNodes == 32, "a bit a record, a lane a node");
   // the nodes' and midpoints' normal values, the same for every record
   __shared__ TabPoint pt[kTabNodes];
   __shared__ double mid_t[kTabNodes], mid_z[kTabNodes];
@@ -616,12 +620,13 @@ __global__ void __launch_bounds__(32 * kTabWarps, 2) k_build_tables(Pair* recs, 
   __shared__ uint32_t s_bad;  // records with a segment that fails its check
   const double h = 2.0 * kTabT1 / (kTabNodes - 1);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * kTabRecs + lane;
+  const int own = threadIdx.x % kTabRecs, group = threadIdx.x / kTabRecs;
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * kTabRecs + own;
   const int64_t rec = i < n ? (order ? order[i] : i) : -1;
+  if (group == 0) s_rec[own] = rec;
   if (warp == 0) {
     const double t = -kTabT1 + h * lane;
     pt[lane] = tab_point(t);
-    s_rec[lane] = rec;
     if (lane == 0) s_bad = 0u;
   } else if (warp == 1) {
     const double t = -kTabT1 + h * lane + 0.5 * h;
@@ -640,35 +645,34 @@ __global__ void __launch_bounds__(32 * kTabWarps, 2) k_build_tables(Pair* recs, 
     lnB = shapes[rec].lnB;
   }
 #pragma unroll 1
-  for (int j = warp; j < kTabNodes; j += kTabWarps) {
+  for (int j = group; j < kTabNodes; j += kGroups) {
     double w = 0.0;
     float4 node = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (beta) node = table_node(pr, a, b, lnB, pt[j], h, &w);
-    s_w[lane][j] = w;
-    s_node[lane][j] = node;
+    s_w[own][j] = w;
+    s_node[own][j] = node;
   }
   __syncthreads();
 #pragma unroll 1
-  for (int j = warp; j < kTabNodes; j += kTabWarps) {
-    float4 node = s_node[lane][j];
+  for (int j = group; j < kTabNodes; j += kGroups) {
+    float4 node = s_node[own][j];
     bool ok = true;
     if (j < kTabNodes - 1) {
-      node.y = static_cast<float>(s_w[lane][j + 1] - s_w[lane][j]);
-      s_node[lane][j].y = node.y;
-      const float4* next = &s_node[lane][j + 1];
+      node.y = static_cast<float>(s_w[own][j + 1] - s_w[own][j]);
+      s_node[own][j].y = node.y;
+      const float4* next = &s_node[own][j + 1];
       if (beta) ok = table_segment_ok(node, next->z, next->w, mid_t[j], mid_z[j], a, b, lnB);
     } else {
       ok = isfinite(node.x) && isfinite(node.z) && isfinite(node.w);
     }
-    const uint32_t bad = __ballot_sync(0xffffffffu, !ok);
-    if (lane == 0 && bad) atomicOr(&s_bad, bad);
+    if (!ok) atomicOr(&s_bad, 1u << own);
   }
   __syncthreads();
 #pragma unroll 1
-  for (int r = warp; r < kTabRecs; r += kTabWarps)
+  for (int r = warp; r < kTabRecs; r += kTabThreads / 32)
     if (s_rec[r] >= 0) tab[s_rec[r] * kTabNodes + lane] = s_node[r][lane];
-  if (warp == 0 && rec >= 0) {
-    const bool all_ok = ((s_bad >> lane) & 1u) == 0u;
+  if (group == 0 && rec >= 0) {
+    const bool all_ok = ((s_bad >> own) & 1u) == 0u;
     if (beta && all_ok) recs[rec].meta = pr.meta | (1u << kMetaExactBit);
     need[rec] = beta && !all_ok ? 1u : 0u;
   }
@@ -758,6 +762,8 @@ __global__ void __launch_bounds__(kTabFineStride, 2) k_build_fine(Pair* recs, co
   }
 }
 
+constexpr int64_t kTabFew = 8000;  // records up to which a block takes 8 and not 32
+
 size_t build_tables_work_words(int64_t n) { return 2 * static_cast<size_t>(n) + 1 + scan_tmp_words(n); }
 
 uint32_t fine_table_cap(int64_t n) {
@@ -792,9 +798,10 @@ cudaError_t launch_build_tables(Pair* recs, const BetaShape* shapes, int64_t n, 
                                 uint32_t* work, uint32_t* elts, cudaStream_t s, int* n_launch) {
   if (n == 0) return cudaSuccess;
   uint32_t *need = work, *slots = work + n, *tmp = slots + n + 1;
-  const int64_t blocks = (n + kTabRecs - 1) / kTabRecs;
-  k_build_tables<<<static_cast<int>(blocks < 2147483647 ? blocks : 2147483647), 32 * kTabWarps, 0, s>>>(
-      recs, shapes, n, order, tab, need);
+  if (n <= kTabFew)
+    k_build_tables<8><<<static_cast<int>((n + 7) / 8), kTabThreads, 0, s>>>(recs, shapes, n, order, tab, need);
+  else
+    k_build_tables<32><<<static_cast<int>((n + 31) / 32), kTabThreads, 0, s>>>(recs, shapes, n, order, tab, need);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   if ((err = scan_exclusive_u32(need, slots, n, tmp, s, n_launch)) != cudaSuccess) return err;

@@ -604,3 +604,25 @@ def test_table_blocks(eng, n):
     ylt, hits, hh = run_gpu(eng, yet, sub, terms, seed=6)
     assert np.array_equal(hits, ref["hits"]) and np.array_equal(hh, ref["hit_hash"])
     check_ylt(ylt, ref)
+
+
+@pytest.mark.parametrize("n", [7, 8, 9, 8_000, 8_001, 8_033])
+def test_table_blocks_of_few_records(eng, n):
+    """Quantile tables at the edges of the builder's small blocks (8 records)
+    and of the load from which a block takes 32: every record's losses against
+    the oracle, through a layer."""
+    C = 9_000
+    rng = np.random.default_rng(n)
+    pool = synth.make_elt_pool(1, C, C, 78, recipe="stress")
+    pick = np.sort(rng.choice(C, n, replace=False))
+    cut = {f: getattr(pool, f)[pick] for f in ("event_ids", "mean", "sigma", "exposure")}
+    cut["sigma"][rng.random(n) < 0.1] = 0.0  # the mean
+    cut["mean"][rng.random(n) < 0.1] = 0.0  # no loss
+    sub = synth.ELTPool(elt_ids=pool.elt_ids, rec_offsets=np.array([0, n], np.int64), terms=pool.terms, **cut)
+    yet = synth.YET(np.arange(0, 40_001, 40, dtype=np.int64),
+                    rng.choice(sub.event_ids, 40_000).astype(np.int32), C)
+    terms = (0.0, 1e12, 0.0, 1e15)
+    ref = oracle.run_layer(yet, sub, terms, seed=6)
+    ylt, hits, hh = run_gpu(eng, yet, sub, terms, seed=6)
+    assert np.array_equal(hits, ref["hits"]) and np.array_equal(hh, ref["hit_hash"])
+    check_ylt(ylt, ref)
