@@ -655,19 +655,18 @@ static int load_elts_impl(ara_ctx* c, const char* who, int32_t n_elts, const int
   int launched = 0;
   ARA_CUDA(c, ara::launch_prepare_records(d_ev, d_mu, d_sg, d_ex, d_offs, n_elts, longest, d_recs, d_shapes, d_flags,
                                           c->stream, sigma_c ? d_sc : nullptr, sigma_c ? d_w : nullptr, &launched));
-  // (the records in order of their shapes, where there are enough for it to pay and its scratch fits)
+  // the records in order of their shapes, where there are enough for it to pay: its scratch of 32 bytes a record
+  // lies in the fine tables' staging (4 KB a slot, at least a slot for 16 records), which is written after the
+  // coarse tables have read the order
   int64_t* order = nullptr;
-  const size_t sel_before = c->sel.bytes;
-  if (R >= kShapeOrderMin && (!c->budget || c->used + ara::shape_order_bytes(R) <= c->budget) &&
-      reserve(c, c->sel, ara::shape_order_bytes(R)) == ARA_OK)
-    ARA_CUDA(c, ara::launch_shape_order(d_shapes, R, c->sel.ptr, &order, c->stream, &launched));
+  if (R >= kShapeOrderMin && ara::shape_order_bytes(R) <= c->elt_tabf_stage.bytes)
+    ARA_CUDA(c, ara::launch_shape_order(d_shapes, R, d_tabf, &order, c->stream, &launched));
   ARA_CUDA(c, ara::launch_build_tables(d_recs, d_shapes, R, order, d_jobs, static_cast<int>(jobs.size()),
                                        fine_off[n_elts], d_tab, d_tabf, d_work, d_flags, c->stream, &launched));
   c->launches += launched;
   std::vector<uint32_t> hf(4 * static_cast<size_t>(n_elts));
   ARA_CUDA(c, cudaMemcpyAsync(hf.data(), d_flags, sizeof(uint32_t) * hf.size(), cudaMemcpyDeviceToHost, c->stream));
   ARA_CUDA(c, cudaStreamSynchronize(c->stream));
-  if (c->budget && c->sel.bytes > sel_before) release(c, c->sel);  // the ELTs' own buffers may need its room
   for (int32_t i = 0; i < n_elts; ++i) {
     const uint32_t f = hf[4 * i];
     const char* why = nullptr;

@@ -626,3 +626,34 @@ def test_table_blocks_of_few_records(eng, n):
     ylt, hits, hh = run_gpu(eng, yet, sub, terms, seed=6)
     assert np.array_equal(hits, ref["hits"]) and np.array_equal(hh, ref["hit_hash"])
     check_ylt(ylt, ref)
+
+
+def test_elt_load_leaves_captured_calls_their_buffers(eng):
+    """The ranked trials of a YLT, captured before a load of many records (whose
+    order takes scratch of its own), replay with the same results after it."""
+    import torch
+
+    from paper_1501_06326_gb300 import ara
+
+    stream = torch.cuda.Stream()
+    own = ara.Ara(0, 0, stream.cuda_stream)
+    try:
+        ylt = torch.randn(20_000, dtype=torch.float64, device="cuda")
+        vals = torch.zeros(50, dtype=torch.float64, device="cuda")
+        trials = torch.zeros(50, dtype=torch.int64, device="cuda")
+        torch.cuda.synchronize()
+        run = lambda: own.top_m(ylt, 50, 0, vals, trials)  # noqa: E731
+        run()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            run()
+        free = torch.cuda.mem_get_info()[0]
+        own.load_pool(synth.make_elt_pool(10, 20_000, 1_000_000, 5))
+        assert torch.cuda.mem_get_info()[0] < free
+        vals.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        want, order = torch.sort(ylt, descending=True)
+        assert torch.equal(vals, want[:50]) and torch.equal(trials, order[:50])
+    finally:
+        own.close()
