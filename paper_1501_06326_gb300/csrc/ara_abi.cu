@@ -185,6 +185,21 @@ struct ara_ctx {
 
 namespace {
 
+// Whether the context's stream is being captured (queries and frees then wait for another call).
+bool stream_captured(ara_ctx* c) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
+// While it lives, this thread's queries and frees do not end another stream's capture, which is none of theirs.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The index and kernel times of the last layer pass, from its events (which must have completed).
 bool read_stat_times(ara_ctx* c) {
   ara_ctx::Timed& t = c->stat_ev;
@@ -234,13 +249,9 @@ bool timed_begin(ara_ctx* c, int kind, ara_ctx::Timed* t) {
     return true;
   }
   if (c->timed.size() >= kTimedHeld) {
-    // (an event query is not allowed while a stream is captured)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
-      cudaGetLastError();
-      cap = cudaStreamCaptureStatusActive;
-    }
-    while (cap == cudaStreamCaptureStatusNone && c->timed.size() >= kTimedHeld) {
+    const bool captured = stream_captured(c);
+    RelaxedCapture relaxed;
+    while (!captured && c->timed.size() >= kTimedHeld) {
       if (cudaEventQuery(c->timed.front().last()) != cudaSuccess) {
         cudaGetLastError();
         break;
@@ -308,19 +319,9 @@ bool release_idle_index(ara_ctx* c) {
 int bind(ara_ctx* c, bool keep_index = false) {
   if (!c) return ARA_EINVAL;
   ARA_CUDA(c, cudaSetDevice(c->device));
-  if (!keep_index && c->yix_idle) {
-    // (memory cannot be freed while the stream is captured; a capture elsewhere is none of this call's)
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess) {
-      cudaGetLastError();
-      capture = cudaStreamCaptureStatusActive;
-    }
-    if (capture == cudaStreamCaptureStatusNone) {
-      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-      ARA_CUDA(c, cudaThreadExchangeStreamCaptureMode(&mode));
-      release_idle_index(c);
-      ARA_CUDA(c, cudaThreadExchangeStreamCaptureMode(&mode));
-    }
+  if (!keep_index && c->yix_idle && !stream_captured(c)) {
+    RelaxedCapture relaxed;
+    release_idle_index(c);
   }
   return ARA_OK;
 }

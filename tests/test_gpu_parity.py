@@ -657,3 +657,34 @@ def test_elt_load_leaves_captured_calls_their_buffers(eng):
         assert torch.equal(vals, want[:50]) and torch.equal(trials, order[:50])
     finally:
         own.close()
+
+
+def test_calls_beside_another_streams_capture(eng):
+    """Calls on a context's own stream, more of them than it holds timing events
+    for, while another stream is captured in CUDA's strictest mode: the calls
+    and the capture succeed."""
+    import torch
+
+    from paper_1501_06326_gb300 import ara
+
+    own_stream, other = torch.cuda.Stream(), torch.cuda.Stream()
+    own = ara.Ara(0, 0, own_stream.cuda_stream)
+    try:
+        ylt = torch.rand(1_000, dtype=torch.float64, device="cuda")
+        pml, tvar = torch.zeros(1, dtype=torch.float64, device="cuda"), torch.zeros(1, dtype=torch.float64, device="cuda")
+        x = torch.zeros(8, device="cuda")
+        torch.cuda.synchronize()
+        for _ in range(3):  # (the events of a call before any capture)
+            own.pml_tvar(ylt, [10.0], pml, tvar)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=other, capture_error_mode="global"):
+            x += 1.0
+            for _ in range(200):
+                own.pml_tvar(ylt, [10.0], pml, tvar)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.all(x == 1.0) and own.timing()["pml_calls"] == 203
+        assert float(pml[0]) == float(torch.sort(ylt, descending=True)[0][99])
+    finally:
+        own.close()
