@@ -1040,7 +1040,10 @@ static int run_layer_impl(ara_ctx* c, const ara_layer* L, uint64_t seed, int64_t
   // 0.4 records a catalogue event (a hit event of 1.2 pairs on average).  Losses, us, lanes and windows, 25M
   // pairs of 3.0 records an event 555 and 410, 1.5: 502 and 394, 0.5: 428 and 393, 0.33: 407 and 392 (0.3 and
   // tables that fit L1: 329 and 345), 0.2: 250 and 257, 0.075 (75M): 1,005 and 1,114.
-  p.windows = static_cast<double>(pl.ix.n_recs) >= 0.4 * c->catalogue;
+  // With ARA_NEWTON_ONLY every event is deferred, and windows mix events of few and of many pairs in the list,
+  // whose lanes wait for the longest: ms, lanes and windows, 1.0 records an event 6.4 and 7.8, 0.5: 1.65 and 2.06,
+  // 10: 10.3 and 9.7.
+  p.windows = static_cast<double>(pl.ix.n_recs) >= ((L->flags & ARA_NEWTON_ONLY) ? 4.0 : 0.4) * c->catalogue;
   p.tile_trials = pl.tile_trials;
   p.e0 = pl.e0;
   p.ev_buf = pl.g.ev_buf;
