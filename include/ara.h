@@ -485,10 +485,11 @@ ARA_API int ara_merge_top(const double *values, const int64_t *trials, int64_t c
  * cudaFree, which can synchronise the whole device, are not acceptable.  It
  * needs no context (creating one allocates).  The paper has no counterpart.
  *
- * The select state lives in a fixed block of device memory that belongs to
- * the library (ARA_NOALLOC_SCRATCH_BYTES per GPU, held from the library's
- * first use on that GPU until the process exits).  Every call on a GPU
- * reuses that one block: calls that may overlap on the GPU (other streams,
+ * The results for host arrays, and the select state for long YLTs (a short
+ * one's is in shared memory), live in a fixed block of device memory that
+ * belongs to the library (ARA_NOALLOC_SCRATCH_BYTES per GPU, held from the
+ * library's first use on that GPU until the process exits).  Every call on a
+ * GPU reuses that one block: calls that may overlap on the GPU (other streams,
  * other host threads) race and must be serialised by the caller.
  *
  *   ylt          device (or managed) memory, n >= 1 year losses

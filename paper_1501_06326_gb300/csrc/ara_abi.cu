@@ -135,7 +135,8 @@ struct ara_ctx {
   DevBuf ev_occ;     // per-event output: O_k beside each event buffer record (float)
   DevBuf row_base;   //   rows before each tile (exclusive scan of tile_cnt) and its scan scratch
   DevBuf evr_stage;  //   rows and max_occ staged on the device for host arrays
-  DevBuf sel;       // select / sort scratch
+  DevBuf sel;       // sort scratch
+  DevBuf sel_wide;  // scratch of ara_pml_tvar on long YLTs
   DevBuf in_tmp;    // staging of host inputs for pml/sort
   DevBuf out_tmp;   // small device outputs
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // of a pass without timing (the serving loop's)
@@ -176,6 +177,7 @@ struct ara_ctx {
   DevBuf serve_arena;                   // year losses of the admitted requests
   std::map<size_t, size_t> arena_free;  // free blocks of the arena: offset -> bytes
   DevBuf serve_out;                     // device result slots (PML, TVaR)
+  DevBuf serve_sel;                     // scratch of the requests' selects on long YLTs
   cudaStream_t serve_side = nullptr;    // the requests' PML/TVaR and result copies, beside the passes
   cudaEvent_t serve_join = nullptr;     // the passes' stream up to a point, for the side stream to wait on
   double* serve_host = nullptr;         // pinned host result slots
@@ -325,6 +327,9 @@ int bind(ara_ctx* c, bool keep_index = false) {
   }
   return ARA_OK;
 }
+
+// Bytes of scratch for the selects of a YLT of n year losses: for a launch's most jobs, or under a budget for one.
+size_t select_scratch(const ara_ctx* c, int64_t n) { return ara::select_scratch_bytes(n, c->budget ? 0 : 1 << 20); }
 
 // Make b hold at least `bytes` (contents are not preserved).
 int reserve(ara_ctx* c, DevBuf& b, size_t bytes) {
@@ -1653,6 +1658,7 @@ std::vector<std::pair<DevBuf*, size_t>> serve_workspace(ara_ctx* c) {
       {&c->idx_acc, sizeof(unsigned long long) * (ARA_MAX_BATCH_LAYERS * static_cast<size_t>(kServeChunk) +
                                                   idx_queue_words(0, kServeChunk, ARA_MAX_BATCH_LAYERS))},
       {&c->serve_out, 2 * sizeof(double) * ARA_SERVE_MAX_RP * kServeSlots},
+      {&c->serve_sel, select_scratch(c, c->n_trials)},
   };
   if (any_corr) w.push_back({&c->pairs_w, sizeof(float2) * (n_recs + 1)});
   return w;
@@ -1860,7 +1866,8 @@ int serve_launch_round(ara_ctx* c, const char* who, int32_t* n_failed) {
       if (e == cudaSuccess) e = cudaStreamWaitEvent(c->serve_side, c->serve_join, 0);
       int launched = 0;
       if (e == cudaSuccess)
-        e = ara::pml_tvar_batch(specs.data(), static_cast<int>(specs.size()), c->serve_side, &launched);
+        e = ara::pml_tvar_batch(specs.data(), static_cast<int>(specs.size()), c->serve_sel.ptr, c->serve_sel.bytes,
+                                c->serve_side, &launched);
       c->launches += launched;
       for (size_t k = 0; k < done.size() && e == cudaSuccess; ++k) {
         const ServeReq& q = c->serve_reqs[done[k]];
@@ -2041,12 +2048,19 @@ int ara_pml_tvar(ara_ctx* c, const double* ylt, int64_t n, const double* rps, in
   }
   double* d_pml = pml_dev ? pml_out : c->h_out;
   double* d_tvar = tvar_dev ? tvar_out : c->h_out + n_rp;
+  const ara::SelectSpec spec{d_ylt, n, h_rps.data(), n_rp, d_pml, d_tvar};
+  // the scratch of a long YLT's select (the call does without where it cannot be had); it never grows, so that
+  // captured calls keep theirs
+  if (const size_t bytes = select_scratch(c, n); c->sel_wide.bytes < bytes && ara::select_takes_scratch(spec)) {
+    const std::string err = c->err;
+    RelaxedCapture relaxed;
+    if (reserve(c, c->sel_wide, bytes)) c->err = err;
+  }
   ara_ctx::Timed timed;
   if (!timed_begin(c, 2, &timed)) return fail(c, ARA_ECUDA, "ara_pml_tvar: cannot create timing events");
   int launched = 0;
   ARA_CUDA(c, cudaEventRecord(timed.e[0], c->stream));
-  const ara::SelectSpec spec{d_ylt, n, h_rps.data(), n_rp, d_pml, d_tvar};
-  ARA_CUDA(c, ara::pml_tvar_batch(&spec, 1, c->stream, &launched));
+  ARA_CUDA(c, ara::pml_tvar_batch(&spec, 1, c->sel_wide.ptr, c->sel_wide.bytes, c->stream, &launched));
   ARA_CUDA(c, cudaEventRecord(timed.e[1], c->stream));
   timed_end(c, timed);
   c->launches += launched;
@@ -2280,7 +2294,7 @@ void ara_destroy(ara_ctx* c) {
                     &c->elt_flags,  &c->ev_buf,         &c->tile_cnt,      &c->def_acc,        &c->yet_off,
                     &c->yet_ids,    &c->marks,          &c->word_base,     &c->rankdir,        &c->slot_start,
                     &c->pairs,      &c->pairs_hot,      &c->pairs_w,       &c->pairs_ev,       &c->scan_tmp,
-                    &c->counters,       &c->ylt_tmp,       &c->diag_tmp,       &c->sel,
+                    &c->counters,       &c->ylt_tmp,       &c->diag_tmp,       &c->sel,            &c->sel_wide,       &c->serve_sel,
                     &c->in_tmp,     &c->out_tmp,        &c->serve_arena,   &c->serve_out,      &c->yix_occ,
                     &c->yix_grid,   &c->u_event,       &c->idx_acc,
                     &c->ev_occ,     &c->row_base,       &c->evr_stage,     &c->yet_flags};

@@ -18,11 +18,6 @@ cudaError_t sort_pairs_ascending(unsigned long long* keys, int64_t* vals, int64_
                                  cudaStream_t s, int* n_launch);
 
 // --------------------------------------------------------------- PML/TVaR
-// PML/TVaR of several YLTs: a launch for up to 32 jobs (a YLT and a group of up
-// to four return periods) of one length class, without scratch; a job gives
-// the same bits in any batch.  rps: host arrays, read during the call;
-// pml/tvar: device arrays of n_rp.  n >= 1 and 1 <= n_rp, else
-// cudaErrorInvalidValue.
 struct SelectSpec {
   const double* ylt;
   int64_t n;
@@ -31,7 +26,19 @@ struct SelectSpec {
   double* pml;
   double* tvar;
 };
-cudaError_t pml_tvar_batch(const SelectSpec* specs, int n_specs, cudaStream_t s, int* n_launch);
+// PML/TVaR of several YLTs: a launch (seven for long YLTs) for up to 32 jobs (a
+// YLT and a group of up to four return periods) of one length class; a job
+// gives the same bits in any batch.  rps: host arrays, read during the call;
+// pml/tvar: device arrays of n_rp.  n >= 1 and 1 <= n_rp, else
+// cudaErrorInvalidValue.  `scratch`: device memory for long YLTs.
+// select_scratch_bytes(n, n_rp) takes all periods of one together (0 where n
+// needs none whatever the periods), select_scratch_bytes(n, 0) (12.5 KB) a job at a time in more
+// launches, with the same bits; with less, a long YLT is passed over by one
+// cluster, and its TVaR can differ in the last bit.
+bool select_takes_scratch(const SelectSpec& spec);
+size_t select_scratch_bytes(int64_t n, int n_rp);
+cudaError_t pml_tvar_batch(const SelectSpec* specs, int n_specs, void* scratch, size_t scratch_bytes, cudaStream_t s,
+                           int* n_launch);
 
 // --------------------------------------------------------------- event-major YET index
 // occ[i] = (trial << 32) | event index, grouped by event id and in trial order

@@ -11,6 +11,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <utility>
@@ -209,6 +210,48 @@ __device__ __noinline__ void sel_pick(SelShared& sm, int g, int bits) {
   __syncthreads();
 }
 
+// Per period the sum of this thread's values above its key kth.  A warp
+// collects the values above the lowest of the keys in its ring of 64 and adds 32
+// at a time, as an FP64 add costs a whole warp's time however few lanes need it.
+template <int kStride>
+__device__ __forceinline__ void sel_sums(const SelJob& j, int first, const unsigned long long (&kth)[kSelGroup],
+                                         unsigned long long* ring, double (&sum)[kSelGroup]) {
+  const unsigned int lane = threadIdx.x & 31u;
+  unsigned long long lowest = ~0ull;
+#pragma unroll
+  for (int r = 0; r < kSelGroup; ++r) {
+    sum[r] = 0.0;
+    lowest = kth[r] < lowest ? kth[r] : lowest;
+  }
+  const unsigned int lowest_hi = static_cast<unsigned int>(lowest >> 32);
+  unsigned int held = 0u;
+  auto add = [&](unsigned long long key, bool valid) {
+    const double v = value_of(key);
+#pragma unroll
+    for (int r = 0; r < kSelGroup; ++r)
+      if (valid && key > kth[r]) sum[r] += v;
+  };
+  sel_values<kStride>(j, first, [&](double v, bool valid) {
+    bool above = valid && key_hi(v) >= lowest_hi;
+    if (__ballot_sync(0xffffffffu, above) == 0u) return;
+    const unsigned long long key = key_of(v);
+    above = above && key > lowest;
+    const unsigned int mm = __ballot_sync(0xffffffffu, above);
+    if (above) ring[held + __popc(mm & ((1u << lane) - 1u))] = key;
+    held += __popc(mm);
+    __syncwarp();
+    if (held >= 32u) {
+      add(ring[lane], true);
+      held -= 32u;
+      const unsigned long long rest = ring[32 + lane];
+      __syncwarp();
+      ring[lane] = rest;
+      __syncwarp();
+    }
+  });
+  add(lane < held ? ring[lane] : 0ull, lane < held);
+}
+
 template <int kCtas>
 __global__ void __launch_bounds__(kSelThreads, 1) k_select(const __grid_constant__ SelBatch b) {
   extern __shared__ __align__(16) unsigned char sel_smem[];
@@ -327,44 +370,13 @@ __global__ void __launch_bounds__(kSelThreads, 1) k_select(const __grid_constant
     if (rank == 0 && static_cast<int>(t) < j.g) j.pml[t] = value_of(sm.prefix[t]);
     return;  // (no CTA reads another's shared memory any more)
   }
-  // sums of the values above each period's key.  A warp collects the values above the lowest of the keys
-  // and adds 32 at a time, as an FP64 add costs a whole warp's time however few lanes need it
+  // sums of the values above each period's key
   double sum[kSelGroup];
-  unsigned long long kth[kSelGroup], lowest = ~0ull;
+  unsigned long long kth[kSelGroup];
 #pragma unroll
-  for (int r = 0; r < kSelGroup; ++r) {
-    sum[r] = 0.0;
-    kth[r] = r < j.g ? sm.prefix[r] : ~0ull;
-    lowest = kth[r] < lowest ? kth[r] : lowest;
-  }
+  for (int r = 0; r < kSelGroup; ++r) kth[r] = r < j.g ? sm.prefix[r] : ~0ull;
   __syncthreads();  // few shares ring's memory
-  const unsigned int lowest_hi = static_cast<unsigned int>(lowest >> 32);
-  unsigned int held = 0u;
-  auto add = [&](unsigned long long key, bool valid) {
-    const double v = value_of(key);
-#pragma unroll
-    for (int r = 0; r < kSelGroup; ++r)
-      if (valid && key > kth[r]) sum[r] += v;
-  };
-  sel_values<kStride>(j, first, [&](double v, bool valid) {
-    bool above = valid && key_hi(v) >= lowest_hi;
-    if (__ballot_sync(0xffffffffu, above) == 0u) return;
-    const unsigned long long key = key_of(v);
-    above = above && key > lowest;
-    const unsigned int mm = __ballot_sync(0xffffffffu, above);
-    if (above) sm.ring[warp][held + __popc(mm & ((1u << lane) - 1u))] = key;
-    held += __popc(mm);
-    __syncwarp();
-    if (held >= 32u) {
-      add(sm.ring[warp][lane], true);
-      held -= 32u;
-      const unsigned long long rest = sm.ring[warp][32 + lane];
-      __syncwarp();
-      sm.ring[warp][lane] = rest;
-      __syncwarp();
-    }
-  });
-  add(lane < held ? sm.ring[warp][lane] : 0ull, lane < held);
+  sel_sums<kStride>(j, first, kth, sm.ring[warp], sum);
 #pragma unroll
   for (int r = 0; r < kSelGroup; ++r) {
 #pragma unroll
@@ -392,10 +404,230 @@ __global__ void __launch_bounds__(kSelThreads, 1) k_select(const __grid_constant
   if (kCtas > 1) cluster.sync();  // the CTAs' sums stay until they are read
 }
 
-// CTAs of a YLT's cluster: by its length alone, so that a job gives the same
-// bits in any batch.  One CTA holds a YLT of up to 8 values a thread; a few
-// shorten the passes of a middle one more than their cluster barriers cost.
-int sel_ctas(int64_t n) { return n <= 8 * kSelThreads ? 1 : n <= 64 * kSelThreads ? 4 : 16; }
+// The wide select, for YLTs longer than kSelWide: all SMs pass over the YLT, in
+// a launch for each digit and one for the sums.  A launch first picks the digit
+// before it from its counts (every CTA the same), then counts its own in shared
+// memory and adds the counts to the job's scratch.  Six digits of 11 bits (the
+// last of 9); eight of 8 where the scratch must be small, with the same results.
+// Up to about 1M values it is bound by the launches' latency (11 us each, 78 in
+// all), a long YLT by reading it seven times (64M values, 512 MB: 5.2 TB/s).
+constexpr int kWideCtas = 152;  // one an SM
+constexpr int kWideBits = 11, kWideBitsSmall = 8;
+
+template <int kBits>
+struct WideScratch {
+  static constexpr int kBins = 1 << kBits, kDigits = (64 + kBits - 1) / kBits;
+  // counts of digit L in hist[of(L)]: the launch of digit L reads those of digit L - 1, adds its own and clears those
+  // of digit L + 1; the last digit's are in hist[0], so that the sums' parts, [CTA][period], take the other two
+  unsigned int hist[3][kSelGroup][kBins];
+  __device__ static int of(int digit) { return (digit + 3 - (kDigits - 1) % 3) % 3; }
+  __device__ double* parts() { return reinterpret_cast<double*>(&hist[1][0][0]); }
+  unsigned long long prefix[2][kSelGroup], want[2][kSelGroup];  // after digit L: [L & 1]
+  unsigned int done, pad;  // CTAs whose sums are there
+  static_assert(2 * sizeof(unsigned int) * kSelGroup * kBins >= sizeof(double) * kWideCtas * kSelGroup, "parts fit");
+};
+
+struct WideBatch {
+  SelJob job[kSelBatchMax];
+  void* scratch;  // one a job
+};
+
+template <int kBits>
+struct WideShared {
+  unsigned int hist[kSelGroup][1 << kBits];
+  unsigned int warp_sum[kSelWarps];
+  unsigned long long prefix[kSelGroup], want[kSelGroup];
+};
+
+// Digit L is the key's bits [wide_shift(L), wide_shift(L) + its width).
+template <int kBits>
+__device__ __forceinline__ int wide_shift(int digit) {
+  const int low = 64 - kBits * (digit + 1);
+  return low > 0 ? low : 0;
+}
+
+// Picks each period's digit L from its counts (all threads, the r-th quarter period r; ends with a barrier).
+template <int kBits>
+__device__ __forceinline__ void wide_pick(const SelJob& j, WideScratch<kBits>& w, WideShared<kBits>& sm, int digit) {
+  constexpr int kBins = 1 << kBits, kOwn = kBins / 256;  // bins of a thread
+  const unsigned int t = threadIdx.x, lane = t & 31u, r = t >> 8, u = t & 255u;
+  const bool live = static_cast<int>(r) < j.g;
+  unsigned long long mine = 0ull, want = 0ull;
+  unsigned int c[kOwn], sum = 0u;
+  if (live) {
+    unsigned int slot = r;  // periods of the same prefix share the first one's counts
+    want = j.m[r];
+    if (digit > 0) {
+      const unsigned long long* pre = w.prefix[(digit - 1) & 1];
+      mine = pre[r];
+      want = w.want[(digit - 1) & 1][r];
+      for (unsigned int q = r; q-- > 0u;)
+        if (pre[q] == mine) slot = q;
+    } else {
+      slot = 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < kOwn; ++q) {
+      c[q] = w.hist[w.of(digit)][slot][kBins - 1 - (kOwn * u + q)];  // from the top
+      sum += c[q];
+    }
+  }
+  unsigned int incl = sum;
+#pragma unroll
+  for (int dd = 1; dd < 32; dd <<= 1) {
+    const unsigned int o = __shfl_up_sync(0xffffffffu, incl, dd);
+    if (lane >= static_cast<unsigned int>(dd)) incl += o;
+  }
+  if (lane == 31u) sm.warp_sum[t >> 5] = incl;
+  __syncthreads();
+  unsigned long long above = incl - sum;
+#pragma unroll
+  for (unsigned int q = 0; q < 7; ++q)
+    if (q < ((t >> 5) & 7u)) above += sm.warp_sum[r * 8 + q];
+  if (live && above < want && want <= above + sum) {
+    const int width = digit == 0 ? kBits : wide_shift<kBits>(digit - 1) - wide_shift<kBits>(digit);
+#pragma unroll
+    for (int q = 0; q < kOwn; ++q) {
+      if (above < want && want <= above + c[q]) {
+        const unsigned long long pre = (mine << width) | (kBins - 1 - (kOwn * u + q)), left = want - above;
+        sm.prefix[r] = pre;
+        sm.want[r] = left;
+        if (blockIdx.x == 0) {
+          w.prefix[digit & 1][r] = pre;
+          w.want[digit & 1][r] = left;
+        }
+      }
+      above += c[q];
+    }
+  }
+  __syncthreads();
+}
+
+template <int kBits>
+__global__ void __launch_bounds__(kSelThreads, 1) k_wide_digit(const __grid_constant__ WideBatch b, int digit) {
+  __shared__ WideShared<kBits> sm;
+  const SelJob& j = b.job[blockIdx.y];
+  WideScratch<kBits>& w = static_cast<WideScratch<kBits>*>(b.scratch)[blockIdx.y];
+  constexpr int kWords = kSelGroup << kBits;
+  const unsigned int t = threadIdx.x;
+  for (int i = t; i < kWords; i += kSelThreads) (&sm.hist[0][0])[i] = 0u;
+  if (digit > 0) wide_pick<kBits>(j, w, sm, digit - 1);
+  if (blockIdx.x == 0)
+    for (int i = t; i < kWords; i += kSelThreads) (&w.hist[w.of(digit + 1)][0][0])[i] = 0u;
+  __syncthreads();
+  // the prefixes counted here: of periods with the same one the first's
+  unsigned long long own[kSelGroup];
+#pragma unroll
+  for (int k = 0; k < kSelGroup; ++k) {
+    own[k] = k >= j.g ? ~0ull : digit == 0 ? 0ull : sm.prefix[k];
+#pragma unroll
+    for (int q = 0; q < k; ++q)
+      if (own[q] == own[k]) own[k] = ~0ull;
+  }
+  const int first = static_cast<int>(blockIdx.x * kSelThreads + t), shift = wide_shift<kBits>(digit);
+  constexpr int kStride = kWideCtas * kSelThreads;
+  if (shift >= 32) {  // the digit and those before it are in the key's upper half
+    unsigned int own32[kSelGroup];
+#pragma unroll
+    for (int k = 0; k < kSelGroup; ++k) own32[k] = own[k] == ~0ull ? ~0u : static_cast<unsigned int>(own[k]);
+    const int sh = shift - 32;
+    sel_values<kStride>(j, first, [&](double v, bool valid) {
+      const unsigned int h = key_hi(v) >> sh, top = !valid ? ~0u - 1u : digit == 0 ? 0u : h >> kBits;
+#pragma unroll
+      for (int k = 0; k < kSelGroup; ++k)
+        if (top == own32[k]) atomicAdd(&sm.hist[k][h & ((1u << kBits) - 1u)], 1u);
+    });
+  } else {
+    const int width = wide_shift<kBits>(digit - 1) - shift;
+    const unsigned int mask = (1u << width) - 1u;
+    sel_values<kStride>(j, first, [&](double v, bool valid) {
+      const unsigned long long key = key_of(v) >> shift, top = valid ? key >> width : ~0ull - 1ull;
+#pragma unroll
+      for (int k = 0; k < kSelGroup; ++k)
+        if (top == own[k]) atomicAdd(&sm.hist[k][static_cast<unsigned int>(key) & mask], 1u);
+    });
+  }
+  __syncthreads();
+  for (int i = t; i < kWords; i += kSelThreads) {
+    const unsigned int c = (&sm.hist[0][0])[i];
+    if (c) atomicAdd(&(&w.hist[w.of(digit)][0][0])[i], c);
+  }
+}
+
+template <int kBits>
+__global__ void __launch_bounds__(kSelThreads, 1) k_wide_sums(const __grid_constant__ WideBatch b) {
+  __shared__ WideShared<kBits> sm;
+  __shared__ double part[kSelWarps][kSelGroup];
+  __shared__ bool last;
+  __shared__ unsigned long long ring[kSelWarps][64];
+  const SelJob& j = b.job[blockIdx.y];
+  WideScratch<kBits>& w = static_cast<WideScratch<kBits>*>(b.scratch)[blockIdx.y];
+  const unsigned int t = threadIdx.x, lane = t & 31u, warp = t >> 5;
+  wide_pick<kBits>(j, w, sm, WideScratch<kBits>::kDigits - 1);
+  if (blockIdx.x == 0 && static_cast<int>(t) < j.g) {
+    if (j.ties) j.ties[t] = sm.want[t];
+    j.pml[t] = value_of(sm.prefix[t]);
+  }
+  if (!j.tvar) return;
+  double sum[kSelGroup];
+  unsigned long long kth[kSelGroup];
+#pragma unroll
+  for (int r = 0; r < kSelGroup; ++r) kth[r] = r < j.g ? sm.prefix[r] : ~0ull;
+  sel_sums<kWideCtas * kSelThreads>(j, static_cast<int>(blockIdx.x * kSelThreads + t), kth, ring[warp], sum);
+#pragma unroll
+  for (int r = 0; r < kSelGroup; ++r) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) sum[r] += __shfl_down_sync(0xffffffffu, sum[r], d);
+    if (lane == 0) part[warp][r] = sum[r];
+  }
+  __syncthreads();
+  double* parts = w.parts();
+  if (t < static_cast<unsigned int>(kSelGroup)) {
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < kSelWarps; ++q) s += part[q][t];
+    parts[blockIdx.x * kSelGroup + t] = s;
+    __threadfence();
+  }
+  __syncthreads();
+  if (t == 0) last = atomicAdd(&w.done, 1u) == static_cast<unsigned int>(kWideCtas - 1);
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (static_cast<int>(t) < j.g) {  // the last CTA adds the parts in order
+    double s = 0.0;
+#pragma unroll 8
+    for (int c = 0; c < kWideCtas; ++c) s += __ldcg(&parts[c * kSelGroup + t]);
+    const double v = value_of(sm.prefix[t]);
+    j.tvar[t] = (s + static_cast<double>(sm.want[t]) * v) / static_cast<double>(j.m[t]);
+  }
+}
+
+template <int kBits>
+cudaError_t launch_wide_of(const WideBatch& b, int n_jobs, bool sums, cudaStream_t s, int* n_launch) {
+  using Scratch = WideScratch<kBits>;
+  cudaError_t err = cudaMemsetAsync(b.scratch, 0, sizeof(Scratch) * n_jobs, s);
+  if (err != cudaSuccess) return err;
+  const dim3 grid(kWideCtas, n_jobs);
+  for (int digit = 0; digit < Scratch::kDigits; ++digit) {
+    k_wide_digit<kBits><<<grid, kSelThreads, 0, s>>>(b, digit);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  }
+  k_wide_sums<kBits><<<sums ? grid : dim3(1, n_jobs), kSelThreads, 0, s>>>(b);
+  if (n_launch) *n_launch += Scratch::kDigits + 1;
+  return cudaGetLastError();
+}
+
+// The widest digits whose scratch fits `bytes` for a job (0: none).
+int wide_bits(size_t bytes) {
+  return bytes >= sizeof(WideScratch<kWideBits>) ? kWideBits
+         : bytes >= sizeof(WideScratch<kWideBitsSmall>) ? kWideBitsSmall
+                                                        : 0;
+}
+cudaError_t launch_wide(const WideBatch& b, int bits, int n_jobs, bool sums, cudaStream_t s, int* n_launch) {
+  return bits == kWideBits ? launch_wide_of<kWideBits>(b, n_jobs, sums, s, n_launch)
+                           : launch_wide_of<kWideBitsSmall>(b, n_jobs, sums, s, n_launch);
+}
 
 // m = ceil(n / rp), within [1, n]
 unsigned long long sel_rank(int64_t n, double rp) {
@@ -406,26 +638,35 @@ unsigned long long sel_rank(int64_t n, double rp) {
 }
 
 template <int kCtas>
-cudaError_t launch_select_of(const SelBatch& b, int n_jobs, cudaStream_t s) {
-  cudaError_t err;
-  if ((err = cudaFuncSetAttribute(k_select<kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(SelShared))) !=
-          cudaSuccess ||
-      (kCtas > 8 && (err = cudaFuncSetAttribute(k_select<kCtas>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) !=
-                        cudaSuccess))
-    return err;
+struct SelLaunch {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kCtas, n_jobs);
-  cfg.blockDim = dim3(kSelThreads);
-  cfg.dynamicSmemBytes = sizeof(SelShared);
-  cfg.stream = s;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = kCtas;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_select<kCtas>, b);
+  SelLaunch(int n_jobs, cudaStream_t s) {
+    cfg.gridDim = dim3(kCtas, n_jobs);
+    cfg.blockDim = dim3(kSelThreads);
+    cfg.dynamicSmemBytes = sizeof(SelShared);
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kCtas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  SelLaunch(const SelLaunch&) = delete;
+  static cudaError_t attributes() {
+    const cudaError_t err =
+        cudaFuncSetAttribute(k_select<kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(SelShared));
+    return err != cudaSuccess || kCtas <= 8
+               ? err
+               : cudaFuncSetAttribute(k_select<kCtas>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
+};
+template <int kCtas>
+cudaError_t launch_select_of(const SelBatch& b, int n_jobs, cudaStream_t s) {
+  const SelLaunch<kCtas> l(n_jobs, s);
+  const cudaError_t err = l.attributes();
+  return err != cudaSuccess ? err : cudaLaunchKernelEx(&l.cfg, k_select<kCtas>, b);
 }
 cudaError_t launch_select(const SelBatch& b, int n_jobs, int ctas, cudaStream_t s) {
   return ctas == 1 ? launch_select_of<1>(b, n_jobs, s)
@@ -433,36 +674,112 @@ cudaError_t launch_select(const SelBatch& b, int n_jobs, int ctas, cudaStream_t 
                      : launch_select_of<16>(b, n_jobs, s);
 }
 
+// CTAs of a YLT's cluster.  One CTA holds a YLT of up to 8 values a thread; a
+// few shorten the passes of a middle one more than their cluster barriers cost.
+int sel_ctas(int64_t n) { return n <= 8 * kSelThreads ? 1 : n <= 64 * kSelThreads ? 4 : 16; }
+
+// Whether the current device places a cluster of 16 CTAs (not a portable size:
+// a GPC with 16 SMs free for it), asked once a device.
+bool sel_places_16() {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices];  // 0: not asked, 1: yes, 2: no
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return false;
+  if (known[dev].load() == 0) {
+    SelLaunch<16> l(1, nullptr);
+    int clusters = 0;
+    const bool ok = l.attributes() == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, k_select<16>, &l.cfg) == cudaSuccess && clusters > 0;
+    if (!ok) cudaGetLastError();
+    known[dev].store(ok ? 1 : 2);
+  }
+  return known[dev].load() == 1;
+}
+
+// Whether a job takes the wide select: by its YLT's length and its largest
+// rank (for k_top_collect's, without sums, 0), so that it gives the same bits in
+// any batch.  Above kSelWide the cluster's 16 SMs take longer than all SMs'
+// launches, above half of it where a quarter of the values are summed.  Device
+// us by cluster and wide, two periods of 100 and 250: 300,000 trials 46 and 79, 1M
+// 65 and 80, 2M (4 passes over it) 110 and 88, 16M 860 and 236, 64M 3,420 and
+// 686; of 1.05 and 2: 500,000 96 and 83, 1M 163 and 88, 16M 1,870 and 367.  (Five launches with candidates in
+// device memory, before the clusters: 1M 95 and 120, 16M 1,000 and 930.)
+constexpr int64_t kSelWide = 1 << 20;
+bool sel_wide(int64_t n, unsigned long long largest) {
+  return n > kSelWide || (n > kSelWide / 2 && largest > static_cast<unsigned long long>(n / 4)) ||
+         (sel_ctas(n) == 16 && !sel_places_16());
+}
+bool sel_may_be_wide(int64_t n) { return sel_wide(n, static_cast<unsigned long long>(n)); }
+
 }  // namespace
 
-cudaError_t pml_tvar_batch(const SelectSpec* specs, int n_specs, cudaStream_t s, int* n_launch) {
+size_t select_scratch_bytes(int64_t n, int n_rp) {
+  const int groups = (n_rp + kSelGroup - 1) / kSelGroup;
+  if (!sel_may_be_wide(n)) return 0;
+  return groups < 1 ? sizeof(WideScratch<kWideBitsSmall>)
+                    : sizeof(WideScratch<kWideBits>) * static_cast<size_t>(groups < kSelBatchMax ? groups : kSelBatchMax);
+}
+
+// A job's periods and ranks, and the largest of these.
+static unsigned long long sel_group(const SelectSpec& q, int r0, SelJob* j) {
+  j->g = (q.n_rp - r0 < kSelGroup) ? (q.n_rp - r0) : kSelGroup;
+  unsigned long long largest = 0ull;
+  for (int r = 0; r < kSelGroup; ++r) {
+    j->m[r] = r < j->g ? sel_rank(q.n, q.rps[r0 + r]) : 1ull;
+    largest = j->m[r] > largest ? j->m[r] : largest;
+  }
+  return largest;
+}
+
+bool select_takes_scratch(const SelectSpec& q) {
+  SelJob j;
+  for (int r0 = 0; r0 < q.n_rp; r0 += kSelGroup)
+    if (sel_wide(q.n, sel_group(q, r0, &j))) return true;
+  return false;
+}
+
+cudaError_t pml_tvar_batch(const SelectSpec* specs, int n_specs, void* scratch, size_t scratch_bytes, cudaStream_t s,
+                           int* n_launch) {
   for (int i = 0; i < n_specs; ++i)
     if (specs[i].n < 1 || specs[i].n_rp < 1) return cudaErrorInvalidValue;
-  // one launch per cluster size and kSelBatchMax jobs
-  for (int ctas : {1, 4, 16}) {
-    SelBatch b;
+  // one launch (or one of each of the wide select's) per class of lengths and batch of jobs
+  WideBatch b;
+  b.scratch = scratch;
+  const int bits = wide_bits(scratch_bytes);
+  const size_t room = bits == kWideBits ? scratch_bytes / sizeof(WideScratch<kWideBits>) : bits ? 1 : 0;
+  for (int ctas : {1, 4, 16, kWideCtas}) {
+    const bool wide = ctas == kWideCtas;
+    const int most = static_cast<int>(wide && room < kSelBatchMax ? room : kSelBatchMax);
     int n_jobs = 0;
     auto flush = [&]() -> cudaError_t {
       if (n_jobs == 0) return cudaSuccess;
-      const cudaError_t e = launch_select(b, n_jobs, ctas, s);
-      if (n_launch) *n_launch += 1;
+      cudaError_t e;
+      if (wide) {
+        e = launch_wide(b, bits, n_jobs, true, s, n_launch);
+      } else {
+        SelBatch narrow;
+        for (int k = 0; k < n_jobs; ++k) narrow.job[k] = b.job[k];
+        e = launch_select(narrow, n_jobs, ctas, s);
+        if (n_launch) *n_launch += 1;
+      }
       n_jobs = 0;
       return e;
     };
     cudaError_t err;
     for (int i = 0; i < n_specs; ++i) {
       const SelectSpec& q = specs[i];
-      if (sel_ctas(q.n) != ctas) continue;
       for (int r0 = 0; r0 < q.n_rp; r0 += kSelGroup) {
-        if (n_jobs == kSelBatchMax && (err = flush()) != cudaSuccess) return err;
-        SelJob& j = b.job[n_jobs++];
+        SelJob j;
+        if ((sel_wide(q.n, sel_group(q, r0, &j)) && (room > 0 || !sel_places_16())) != wide || (!wide && sel_ctas(q.n) != ctas))
+          continue;
+        if (most < 1) return cudaErrorInvalidValue;
+        if (n_jobs == most && (err = flush()) != cudaSuccess) return err;
         j.ylt = q.ylt;
         j.n = q.n;
         j.pml = q.pml + r0;
         j.tvar = q.tvar + r0;
         j.ties = nullptr;
-        j.g = (q.n_rp - r0 < kSelGroup) ? (q.n_rp - r0) : kSelGroup;
-        for (int r = 0; r < kSelGroup; ++r) j.m[r] = r < j.g ? sel_rank(q.n, q.rps[r0 + r]) : 1ull;
+        b.job[n_jobs++] = j;
       }
     }
     if ((err = flush()) != cudaSuccess) return err;
@@ -942,16 +1259,19 @@ cudaError_t top_gather_device(const double* ylt, const int64_t* order, int64_t m
   return cudaGetLastError();
 }
 
-size_t top_scratch_bytes(int64_t m) { return radix_scratch_bytes(m) + 2 * sizeof(unsigned int) * kTopSegments + 512; }
+// scratch: the m-th value, the segments' counts, the wide select's, the sort's
+constexpr size_t kTopCountsBytes = (2 * sizeof(unsigned int) * kTopSegments + 255) & ~size_t(255);
+constexpr size_t kTopWideBytes = (sizeof(WideScratch<kWideBits>) + 255) & ~size_t(255);
+
+size_t top_scratch_bytes(int64_t m) { return radix_scratch_bytes(m) + 256 + kTopCountsBytes + kTopWideBytes; }
 
 cudaError_t top_order_device(const double* ylt, int64_t n, int64_t m, int64_t* order, void* scratch, cudaStream_t s,
                              int* n_launch) {
   unsigned char* base = static_cast<unsigned char*>(scratch);
   TopKth* kth = reinterpret_cast<TopKth*>(base);
   unsigned int* counts = reinterpret_cast<unsigned int*>(base + 256);
-  const RxScratch x = radix_scratch(base + 256 + ((2 * sizeof(unsigned int) * kTopSegments + 255) & ~size_t(255)), m);
-  SelBatch b;
-  SelJob& j = b.job[0];
+  const RxScratch x = radix_scratch(base + 256 + kTopCountsBytes + kTopWideBytes, m);
+  SelJob j;
   j.ylt = ylt;
   j.n = n;
   j.pml = &kth->value;
@@ -959,12 +1279,23 @@ cudaError_t top_order_device(const double* ylt, int64_t n, int64_t m, int64_t* o
   j.ties = &kth->ties;
   j.g = 1;
   for (int r = 0; r < kSelGroup; ++r) j.m[r] = r == 0 ? static_cast<unsigned long long>(m) : 1ull;
-  cudaError_t err = launch_select(b, 1, sel_ctas(n), s);
+  cudaError_t err;
+  if (sel_wide(n, 0)) {
+    WideBatch b;
+    b.job[0] = j;
+    b.scratch = base + 256 + kTopCountsBytes;
+    err = launch_wide(b, kWideBits, 1, false, s, n_launch);
+  } else {
+    SelBatch b;
+    b.job[0] = j;
+    err = launch_select(b, 1, sel_ctas(n), s);
+    if (n_launch) *n_launch += 1;
+  }
   if (err != cudaSuccess) return err;
   k_top_count<<<kTopSegments, kTopThreads, 0, s>>>(ylt, n, kth, counts);
   k_top_collect<<<kTopSegments, kTopThreads, 0, s>>>(ylt, n, kth, counts, x.keys[1], x.vals[1]);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  if (n_launch) *n_launch += 3;
+  if (n_launch) *n_launch += 2;
   return radix_order<false>(nullptr, x, m, order, s, n_launch);
 }
 
@@ -973,8 +1304,8 @@ cudaError_t top_order_device(const double* ylt, int64_t n, int64_t m, int64_t* o
 // =============================================================== allocation-free PML / TVaR
 //
 // A fixed block of device memory, owned by the library, holds the device
-// outputs of ara_pml_tvar_noalloc (the select's state is in shared memory).  In host code the
-// name of a __device__ array is only a host-side stand-in; the kernels get
+// outputs of ara_pml_tvar_noalloc for host arrays and the wide select's scratch
+// (the other selects' state is in shared memory).  In host code the name of a __device__ array is only a host-side stand-in; the kernels get
 // the block's device address, looked up once per device.
 namespace {
 
@@ -983,8 +1314,9 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[ARA_NOALLOC_SCR
 constexpr int kNoallocMaxDevices = 64;
 void* g_noalloc_addr[kNoallocMaxDevices] = {};  // device address of the block, per device
 
-static_assert(ARA_NOALLOC_SCRATCH_BYTES >= 2 * ARA_NOALLOC_MAX_RP * sizeof(double),
-              "fixed block too small for the outputs");
+constexpr size_t kNoallocOutBytes = 2 * ARA_NOALLOC_MAX_RP * sizeof(double);
+static_assert(ARA_NOALLOC_SCRATCH_BYTES >= kNoallocOutBytes + sizeof(ara::WideScratch<ara::kWideBitsSmall>) && kNoallocOutBytes % 16 == 0,
+              "fixed block too small for the outputs and a job's scratch");
 
 }  // namespace
 
@@ -1014,7 +1346,7 @@ extern "C" ARA_API int ara_pml_tvar_noalloc(const double* ylt, int64_t n, const 
     g_noalloc_addr[dev] = addr;
   }
   unsigned char* block = static_cast<unsigned char*>(g_noalloc_addr[dev]);
-  double* d_out = reinterpret_cast<double*>(block);                      // 2 * ARA_NOALLOC_MAX_RP doubles
+  double* d_out = reinterpret_cast<double*>(block);  // 2 * ARA_NOALLOC_MAX_RP doubles, then a wide select's scratch
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   // 0: host memory, 1: device (or managed) memory of this GPU, -1: another GPU's memory
   auto kind_of = [dev](const void* p) {
@@ -1033,7 +1365,9 @@ extern "C" ARA_API int ara_pml_tvar_noalloc(const double* ylt, int64_t n, const 
   double* d_pml = pml_dev ? pml_out : d_out;
   double* d_tvar = tvar_dev ? tvar_out : d_out + ARA_NOALLOC_MAX_RP;
   const ara::SelectSpec spec{ylt, n, return_periods, n_rp, d_pml, d_tvar};
-  if (ara::pml_tvar_batch(&spec, 1, s, nullptr) != cudaSuccess) return ARA_ECUDA;
+  if (ara::pml_tvar_batch(&spec, 1, block + kNoallocOutBytes, ARA_NOALLOC_SCRATCH_BYTES - kNoallocOutBytes, s,
+                          nullptr) != cudaSuccess)
+    return ARA_ECUDA;
   if (!pml_dev && cudaMemcpyAsync(pml_out, d_pml, sizeof(double) * n_rp, cudaMemcpyDeviceToHost, s) != cudaSuccess)
     return ARA_ECUDA;
   if (!tvar_dev && cudaMemcpyAsync(tvar_out, d_tvar, sizeof(double) * n_rp, cudaMemcpyDeviceToHost, s) != cudaSuccess)

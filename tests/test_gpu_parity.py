@@ -688,3 +688,49 @@ def test_calls_beside_another_streams_capture(eng):
         assert float(pml[0]) == float(torch.sort(ylt, descending=True)[0][99])
     finally:
         own.close()
+
+
+@pytest.mark.parametrize("n", [524_288, 524_289, 1_048_576, 1_048_577, 2_345_678])
+@pytest.mark.parametrize("kind", ["spread", "cut", "tied", "signed"])
+def test_long_ylts(eng, n, kind):
+    """PML, TVaR and the top trials on both sides of the lengths from which all
+    SMs pass over the YLT (with a quarter of the values to sum, and in any
+    case): spread values, values cut at both ends, few distinct ones, negative
+    ones and infinities among them.  The allocation-free call and a context
+    with a budget, whose scratch takes narrower digits, give the same bits."""
+    import torch
+
+    from paper_1501_06326_gb300 import ara
+
+    rng = np.random.default_rng(n)
+    y = rng.lognormal(8, 2, n)
+    if kind == "cut":
+        y = np.clip(y - 3_000.0, 0.0, 50_000.0)
+    elif kind == "tied":
+        y = np.minimum(np.floor(y / 1_000.0), 7.0)
+    elif kind == "signed":
+        y = np.where(rng.random(n) < 0.5, -y, y)
+        y[:3] = np.inf, -np.inf, -0.0
+    rps = [np.array([100.0, 250.0]), np.array([1.0, 1.5, 4.0, 10.0, float(n), 1e9])]
+    if kind == "signed":
+        rps[1] = rps[1][1:]  # the mean of all would be inf - inf
+    y_dev = torch.from_numpy(y).cuda()
+    s = np.sort(y)[::-1]
+    small = ara.Ara(0, 64 << 20)
+    try:
+        for rp in rps:
+            pml, tvar = eng.pml_tvar(y_dev, rp)
+            m = np.clip(np.ceil(n / rp), 1, n).astype(np.int64)
+            assert np.array_equal(pml, s[m - 1])
+            assert np.allclose(tvar, [np.sum(s[:k]) / k for k in m], rtol=1e-12, atol=0)
+            p2, t2 = np.zeros(rp.size), np.zeros(rp.size)
+            assert ara.ara_pml_tvar_noalloc(y_dev, n, rp, rp.size, p2, t2) == ara.ARA_OK
+            assert np.array_equal(pml, p2) and np.array_equal(tvar, t2)
+            p3, t3 = small.pml_tvar(y_dev, rp)
+            assert np.array_equal(pml, p3) and np.array_equal(tvar, t3)
+    finally:
+        small.close()
+    order = np.lexsort((np.arange(n), -y))
+    for k in (1, 1_000, n // 8):
+        vals, trials = eng.top_m(y_dev, k)
+        assert np.array_equal(vals, y[order[:k]]) and np.array_equal(trials, order[:k])
