@@ -734,3 +734,38 @@ def test_long_ylts(eng, n, kind):
     for k in (1, 1_000, n // 8):
         vals, trials = eng.top_m(y_dev, k)
         assert np.array_equal(vals, y[order[:k]]) and np.array_equal(trials, order[:k])
+
+
+@pytest.mark.parametrize("catalogue", [1_000, 9_000], ids=["windows", "lanes"])
+@pytest.mark.parametrize("n,per_trial", [(401, 300), (3_649, 75), (21_901, 40)])
+def test_year_losses_over_tiles(eng, n, per_trial, catalogue):
+    """Without a retention a year loss depends on the tile in its last bits: a
+    whole run, runs over pieces (other tile sizes, other first trials) and a
+    context with a budget (tiles of eight) agree to the double-float sums'
+    rounding, four units of 2^-48 for each of a trial's losses; the hits and
+    the batched passes, whose sums are integers, exactly."""
+    from paper_1501_06326_gb300 import ara
+
+    rng = np.random.default_rng(n)
+    offsets = np.zeros(n + 1, np.int64)
+    offsets[1:] = np.cumsum(rng.integers(per_trial // 2, 3 * per_trial // 2, n))
+    pool = synth.make_elt_pool(3, 900, catalogue, 12, recipe="stress")
+    yet = synth.YET(offsets, rng.integers(0, catalogue, int(offsets[-1])).astype(np.int32), catalogue)
+    terms = (0.0, 1e12, 0.0, 1e15)
+    ids = [int(i) for i in pool.elt_ids]
+    ylt, hits, hh = run_gpu(eng, yet, pool, terms, seed=4, t0=0, t1=n)
+    many = np.empty((2, n))
+    eng.run_layers([(ids, terms), (ids[:1], terms)], 4, 0, n, many)
+    tol = 4.0 * 2.0**-48 * (hits + 8)
+    small = ara.Ara(0, 64 << 20)
+    try:
+        for own, t0, t1 in ((eng, n // 3, n), (eng, 5, 40), (small, 0, n), (small, 3, n)):
+            part, h, hash_ = run_gpu(own, yet, pool, terms, seed=4, t0=t0, t1=t1)
+            assert np.all(np.abs(part - ylt[t0:t1]) <= tol[t0:t1] * ylt[t0:t1])
+            assert np.array_equal(h, hits[t0:t1]) and np.array_equal(hash_, hh[t0:t1])
+            sub = np.empty((2, t1 - t0))
+            own.run_layers([(ids, terms), (ids[:1], terms)], 4, t0, t1, sub)
+            assert np.array_equal(sub, many[:, t0:t1])
+    finally:
+        small.close()
+    check_ylt(ylt[:50], oracle.run_layer(yet, pool, terms, seed=4, trials=np.arange(50)))
