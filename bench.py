@@ -73,7 +73,8 @@ def _peaks():
 
 
 NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e, nominal
-LAYER_SOURCES = ("ara_layer.cu", "ara_device_math.cuh", "ara_internal.h")  # what k_gather and k_losses compile from
+# what k_gather and k_losses compile from
+LAYER_SOURCES = ("ara_layer.cu", "ara_device_math.cuh", "ara_internal.h", "ara_window.cuh")
 
 
 def _kernel_source_hash() -> str:

@@ -460,7 +460,8 @@ ARA_API int ara_debug_record_losses(ara_ctx *ctx, int64_t n, const float *mean, 
  * doubles) in descending order, ties by trial index, to values_out, and their
  * global trial indices (trial_offset + local index) to trials_out (m entries
  * each, host or device memory).  When m > n the last m - n entries are
- * (-INFINITY, -1).  Runs the device radix sort of the YLT.
+ * (-INFINITY, -1).  Runs the device radix sort of the YLT, or, for few of many,
+ * a select and a sort of those.
  * Errors: ARA_EINVAL (n < 1 or >= 2^31, m < 1, trial_offset < 0), ARA_ENOMEM,
  * ARA_ECUDA.
  *
