@@ -485,11 +485,11 @@ int yet_begin(ara_ctx* c, int64_t n_trials, const int64_t* offsets, const int32_
   // The index belongs to the YET being replaced.  Its buffers are held for the next build (to free and
   // allocate 8 bytes an event costs 2.7 ms at 400M events, in a renewal of 9.4) until the next call shows
   // whether there is one; not under a budget, nor where the device then has less than a quarter free, nor
-  // from before the replaced YET.
+  // from before the replaced YET, nor small ones (to ask for the free memory takes as long).
   release_idle_index(c);
   c->yix_idle = c->yix_occ.ptr || c->yix_grid.ptr;
   c->yix_ready = false;
-  if (c->budget) release_idle_index(c);
+  if (c->budget || c->yix_occ.bytes < (size_t{32} << 20)) release_idle_index(c);
   if (!c->copy_stream) {
     ARA_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
     ARA_CUDA(c, cudaEventCreateWithFlags(&c->yet_ready, cudaEventDisableTiming));
@@ -1396,7 +1396,7 @@ int ara_build_yet_index(ara_ctx* c) {
   } times;
   cudaEvent_t* tm = times.tm;
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreate(&tm[i]);
+  for (int i = 2; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreate(&tm[i]);
   int launched = 0;
   auto read = [&](const uint32_t* from, uint32_t* to) {
     const cudaError_t r = cudaMemcpyAsync(to, from, sizeof *to, cudaMemcpyDeviceToHost, c->stream);
@@ -1421,6 +1421,7 @@ int ara_build_yet_index(ara_ctx* c) {
     uint32_t largest = 0;
     counted = (!c->budget || c->used + (in_ev_buf ? 0 : parts_bytes) + work_bytes <= c->budget) &&
               reserve(c, work, work_bytes) == ARA_OK;
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreate(&tm[i]);
     if (e == cudaSuccess && counted) e = cudaEventRecord(tm[0], c->stream);
     if (e == cudaSuccess && counted)
       e = ara::yet_parts_count(ids, n, c->catalogue, cells, c->num_sms, work.ptr, c->stream, &launched);
