@@ -341,12 +341,14 @@ ARA_API int ara_set_batch_config(ara_ctx *ctx, int32_t item, int32_t blocks_per_
  * 262,144 trials (the serving chunk), so that a pass's slices of trials find
  * their occurrences without a search.  It takes 8 bytes per YET event and
  * 4 * (ceil(n_trials / 262144) + 1) per catalogue id, and lasts until the next
- * YET load.  That load frees its buffers, or, without a budget and where a
- * quarter of the device's memory is free, leaves them for the new YET's build,
- * and the next call on the context other than the build, an ELT load or
- * ara_finish_yet frees them.  The partition and bucket builds need 4 bytes per
- * (catalogue id, cell) of scratch besides, the radix sort about 24 bytes per event.  Errors: ARA_ENOTLOADED; ARA_EINVAL (served requests queued or
- * running, or 2^32 or more events); ARA_ENOMEM; ARA_ECUDA.
+ * YET load.  That load frees its buffers, or, without a budget and where they
+ * are small or a quarter of the device's memory is free, leaves them for the
+ * new YET's build, and the next call on the context other than the build, an
+ * ELT load or ara_finish_yet frees them.  The partition and bucket builds need 4 bytes per
+ * (catalogue id, cell) and up to 10 MB of scratch besides, which without a
+ * budget stay with the index; the radix sort needs about 24 bytes per event.
+ * Errors: ARA_ENOTLOADED; ARA_EINVAL (served requests queued or running, or
+ * 2^32 or more events); ARA_ENOMEM; ARA_ECUDA.
  * ara_yet_index_info reports whether the index is built, its bytes, the
  * device time of its build and how it was built (0 partitions or buckets, 1 radix sort, -1
  * not built); any pointer may be NULL. */

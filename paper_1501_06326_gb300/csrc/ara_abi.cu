@@ -118,7 +118,7 @@ struct ara_ctx {
   DevBuf marks, word_base, rankdir, slot_start, pairs, pairs_hot, pairs_w, pairs_ev, scan_tmp;
   DevBuf ev_buf, tile_cnt;  // hit-event records of the layer kernels
   // event-major index of the YET (ara_build_yet_index) and the indexed passes' buffers
-  DevBuf yix_occ, yix_grid;
+  DevBuf yix_occ, yix_grid, yix_work;  // (work: a build's counts)
   bool yix_ready = false;
   bool yix_idle = false;   // its buffers are held without an index
   bool yix_sorted = false;  // built by the radix sort (a bucket was too large)
@@ -313,6 +313,7 @@ bool release_idle_index(ara_ctx* c) {
   c->yix_idle = false;
   release(c, c->yix_occ);
   release(c, c->yix_grid);
+  release(c, c->yix_work);
   return true;
 }
 
@@ -484,12 +485,13 @@ int yet_begin(ara_ctx* c, int64_t n_trials, const int64_t* offsets, const int32_
   c->yet_loaded = false;
   // The index belongs to the YET being replaced.  Its buffers are held for the next build (to free and
   // allocate 8 bytes an event costs 2.7 ms at 400M events, in a renewal of 9.4) until the next call shows
-  // whether there is one; not under a budget, nor where the device then has less than a quarter free, nor
-  // from before the replaced YET, nor small ones (to ask for the free memory takes as long).
+  // whether there is one; not under a budget, nor where 256 MB or more would be held and the device then has
+  // less than a quarter free (asked below; it takes 20 us), nor from before the replaced YET, nor very small ones
+  // (which the driver cuts from a block).
   release_idle_index(c);
   c->yix_idle = c->yix_occ.ptr || c->yix_grid.ptr;
   c->yix_ready = false;
-  if (c->budget || c->yix_occ.bytes < (size_t{32} << 20)) release_idle_index(c);
+  if (c->budget || c->yix_occ.bytes < (size_t{1} << 20)) release_idle_index(c);
   if (!c->copy_stream) {
     ARA_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
     ARA_CUDA(c, cudaEventCreateWithFlags(&c->yet_ready, cudaEventDisableTiming));
@@ -507,7 +509,7 @@ int yet_begin(ara_ctx* c, int64_t n_trials, const int64_t* offsets, const int32_
   if ((rc = reserve(c, c->yet_off, sizeof(int64_t) * (n_trials + 1)))) return rc;
   // ids: padded by 8 entries so that 32-byte loads near the end stay inside the buffer
   if ((rc = reserve(c, c->yet_ids, sizeof(int32_t) * (n_events + 8)))) return rc;
-  if (c->yix_idle) {
+  if (c->yix_idle && c->yix_occ.bytes >= (size_t{256} << 20)) {
     size_t room = 0, total = 0;
     ARA_CUDA(c, cudaMemGetInfo(&room, &total));
     if (room < total / 4) release_idle_index(c);
@@ -1363,7 +1365,11 @@ int ara_build_yet_index(ara_ctx* c) {
     return fail(c, ARA_EINVAL, "%s: the YET holds 2^32 or more events", who);
   const int64_t n = c->n_events;
   const int64_t cells = ara::yet_grid_cells(c->n_trials, kYetGridShift);
-  DevBuf work, parts_buf;  // scratch
+  // scratch: the counts, which without a budget stay with the index and go with it (to allocate and free 10 MB
+  // takes 200 us), and the first partition, in the event buffer where that is large enough, else in a buffer of
+  // the build alone
+  DevBuf& work = c->yix_work;
+  DevBuf parts_buf;
   auto drop_scratch = [&]() {
     release(c, work);
     release(c, parts_buf);
@@ -1404,14 +1410,13 @@ int ara_build_yet_index(ara_ctx* c) {
   };
   // scratch of another build in place of what is held
   auto reserve_work = [&](size_t bytes) {
-    drop_scratch();
+    if (work.bytes < bytes) drop_scratch();
     const int r = reserve(c, work, bytes);
     if (r) drop();
     return r;
   };
   // The partition build where its fields fit and no bucket of the first partition holds too many of the events,
-  // and where its 8 bytes an event of scratch do (the event buffer of the streaming passes where it is large
-  // enough, else a buffer for the build alone); else the bucket build with its 4 bytes per (event, cell).
+  // and where its 8 bytes an event of scratch do; else the bucket build with its 4 bytes per (event, cell).
   bool parts = ara::yet_parts_fit(c->n_trials, n, c->catalogue, cells, c->num_sms), counted = false, sorted = false;
   unsigned long long* first = static_cast<unsigned long long*>(c->ev_buf.ptr);
   if (parts) {
@@ -1469,7 +1474,8 @@ int ara_build_yet_index(ara_ctx* c) {
   if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, tm[2], tm[3]);
   if (e == cudaSuccess && counted) e = cudaEventElapsedTime(&count_ms, tm[0], tm[1]);
   ms += count_ms;
-  drop_scratch();
+  release(c, parts_buf);
+  if (c->budget || sorted) release(c, work);
   c->launches += launched;
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -1480,7 +1486,8 @@ int ara_build_yet_index(ara_ctx* c) {
   c->yix_ready = true;
   c->yix_build_ms = ms;
   c->yix_bytes = static_cast<int64_t>(sizeof(unsigned long long) * (n + 1) +
-                                      sizeof(uint32_t) * (static_cast<size_t>(c->catalogue) * (cells + 1) + 1));
+                                      sizeof(uint32_t) * (static_cast<size_t>(c->catalogue) * (cells + 1) + 1) +
+                                      work.bytes);
   c->serve_ready = false;  // the serving arena is sized again around the index
   return ARA_OK;
 }
@@ -2300,7 +2307,7 @@ void ara_destroy(ara_ctx* c) {
                     &c->pairs,      &c->pairs_hot,      &c->pairs_w,       &c->pairs_ev,       &c->scan_tmp,
                     &c->counters,       &c->ylt_tmp,       &c->diag_tmp,       &c->sel,            &c->sel_wide,       &c->serve_sel,
                     &c->in_tmp,     &c->out_tmp,        &c->serve_arena,   &c->serve_out,      &c->yix_occ,
-                    &c->yix_grid,   &c->u_event,       &c->idx_acc,
+                    &c->yix_grid,   &c->yix_work,       &c->u_event,       &c->idx_acc,
                     &c->ev_occ,     &c->row_base,       &c->evr_stage,     &c->yet_flags};
   for (DevBuf* b : bufs) release(c, *b);
   for (auto& e : c->ev)
