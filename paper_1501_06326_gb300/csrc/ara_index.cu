@@ -152,8 +152,8 @@ __global__ void k_sort_cells(const uint32_t* __restrict__ ev_grid, int64_t n_buc
 // (low digit << 53 | trial << 22 | event index), into a buffer of 8 bytes an
 // event; the second partitions each of those buckets by the low digit and
 // unpacks.  Both keep the (trial, event index) order, so no sort follows.
-// What bounds it is memory: 4 B an event for the first count, 4 + 8 for the
-// first partition, 8 for the second count, 8 + 8 for the second partition.
+// It moves 4 B an event for the first count, 4 + 8 for the first partition, 8
+// for the second count, 8 + 8 for the second partition.
 // Stores go out in runs of one digit (about 8 occurrences, 64 bytes, of a tile
 // of 16,384 at 2,048 digits), where the bucket build's atomic slot claims store
 // 8 bytes at a time; tiles follow one another in a segment, so the next run of
@@ -162,7 +162,7 @@ __global__ void k_sort_cells(const uint32_t* __restrict__ ev_grid, int64_t n_buc
 // memory and its latency at 16 warps an SM: issue 31%.  One CTA of 512 threads
 // an SM with the next tile's items loaded while a tile goes out; without that
 // 3.6 ms, and as two CTAs of 256 threads with tiles of 8,192 (runs half as long)
-// 3.5 ms.  The build: 6.5 ms at 400,000 trials x 1,000 events, against 14.8 ms
+// 3.5 ms.  The build: 6.4 ms at 400,000 trials x 1,000 events, against 14.9 ms
 // by buckets.
 
 constexpr int kPartThreads = 512;

@@ -592,17 +592,20 @@ __device__ bool table_segment_ok(float4 nd, float d1, float e1, double tq, doubl
 // the nodes j = w, w + 8, .. at t_j = -T1 + j h, then the segments' checks.  A
 // load of few records takes 8 a block and a thread a node, whose chain of nodes
 // and checks is a quarter as long (1 record 142 us a load against 230, 1,000
-// 382 and 534, 8,000 663 and 667, 16,000 972 and 900).  The stored float4 is {x_j, w_{j+1} - w_j, h w'_j, h^2 w''_j}.  need[rec] = 1 for
-// a Beta record whose coarse table is not exact (a candidate for a fine table).
+// 382 and 534, 8,000 663 and 667, 16,000 972 and 900).  The stored float4 is
+// {x_j, w_{j+1} - w_j, h w'_j, h^2 w''_j}.  need[rec] = 1 for a Beta record whose
+// coarse table is not exact (a candidate for a fine table).
 // The iteration and fraction lengths follow the shapes and t: with the records
 // in order of a + b a warp's lanes, at the same t, run about equally long,
 // where a warp per record with a lane per node ran 13 of its 32 lanes (30 now).
-// Bound by the FP64 pipe (76% active: logs, exps and divisions around the
-// double-float fraction).  150,000 records of the plain recipe: 3.6 ms, a warp
-// per record 10.7, and 15.1 with an FP64 division for each test of the
-// fraction and new logarithms and exponentials after the last Newton step; of
-// the stress recipe 4.2 ms, 19.8 with the bracketed solver for the roots near
-// 1.  In order of a + b alone 4.0 and 10.2 ms.
+// Bound by the FP64 pipe (77% active: logs, exps and divisions around the
+// double-float fraction).  150,000 records of the plain recipe: 3.9 ms (3.6 with
+// the fraction's stop test in double-float too), a warp per record 10.7, and
+// 15.1 with an FP64 division for each test of the fraction and new logarithms
+// and exponentials after the last Newton step; of the stress recipe 4.5 ms (4.2),
+// 19.8 with the bracketed solver for the roots near 1.  Against those new
+// logarithms a node's FP64 root agrees to about 1e-15, and its FP32 value was
+// another in one of 100 million nodes compared.
 constexpr int kTabThreads = 256;
 
 // kTabRecs: records of a block, thread t the record t mod kTabRecs.
