@@ -392,7 +392,6 @@ cudaMemcpyKind kind_to_device(const void* src) {
   return is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
 }
 
-
 }  // namespace
 
 extern "C" {
@@ -2102,7 +2101,7 @@ int ara_top_m(ara_ctx* c, const double* ylt, int64_t n, int64_t m, int64_t trial
   const int64_t m_valid = std::min(m, n);
   const bool collect = n >= (int64_t(1) << 19) && m_valid <= n / 8;
   // scratch: the sort's, then the order, then staged outputs for host arrays
-  const size_t sort_bytes = ((collect ? ara::top_scratch_bytes(m_valid) : ara::sort_scratch_bytes(n)) + 255) & ~size_t(255);
+  const size_t sort_bytes = ((collect ? ara::top_scratch_bytes(n, m_valid) : ara::sort_scratch_bytes(n)) + 255) & ~size_t(255);
   const size_t order_bytes = (sizeof(int64_t) * static_cast<size_t>(collect ? m_valid : n) + 255) & ~size_t(255);
   const size_t stage_bytes = (vals_dev && trials_dev) ? 0 : 2 * sizeof(int64_t) * static_cast<size_t>(m);
   if ((rc = reserve(c, c->sel, sort_bytes + order_bytes + stage_bytes))) return rc;

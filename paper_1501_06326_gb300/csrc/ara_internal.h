@@ -285,8 +285,8 @@ constexpr int kEventRowsThreads = 256;
 // Scratch size in bytes for n year losses.
 size_t sort_scratch_bytes(int64_t n);
 // The first m of sort_desc_device's order, m <= n < 2^32, without ordering the
-// rest.  Scratch top_scratch_bytes(m).
-size_t top_scratch_bytes(int64_t m);
+// rest.  Scratch top_scratch_bytes(n, m).
+size_t top_scratch_bytes(int64_t n, int64_t m);
 cudaError_t top_order_device(const double* ylt, int64_t n, int64_t m, int64_t* order, void* scratch, cudaStream_t s,
                              int* n_launch);
 // vals/trials[i] = ylt[order[i]], trial_offset + order[i] for i < m_valid;

@@ -1263,14 +1263,18 @@ cudaError_t top_gather_device(const double* ylt, const int64_t* order, int64_t m
 constexpr size_t kTopCountsBytes = (2 * sizeof(unsigned int) * kTopSegments + 255) & ~size_t(255);
 constexpr size_t kTopWideBytes = (sizeof(WideScratch<kWideBits>) + 255) & ~size_t(255);
 
-size_t top_scratch_bytes(int64_t m) { return radix_scratch_bytes(m) + 256 + kTopCountsBytes + kTopWideBytes; }
+size_t top_wide_bytes(int64_t n) { return sel_wide(n, 0) ? kTopWideBytes : 0; }
+
+size_t top_scratch_bytes(int64_t n, int64_t m) {
+  return radix_scratch_bytes(m) + 256 + kTopCountsBytes + top_wide_bytes(n);
+}
 
 cudaError_t top_order_device(const double* ylt, int64_t n, int64_t m, int64_t* order, void* scratch, cudaStream_t s,
                              int* n_launch) {
   unsigned char* base = static_cast<unsigned char*>(scratch);
   TopKth* kth = reinterpret_cast<TopKth*>(base);
   unsigned int* counts = reinterpret_cast<unsigned int*>(base + 256);
-  const RxScratch x = radix_scratch(base + 256 + kTopCountsBytes + kTopWideBytes, m);
+  const RxScratch x = radix_scratch(base + 256 + kTopCountsBytes + top_wide_bytes(n), m);
   SelJob j;
   j.ylt = ylt;
   j.n = n;
