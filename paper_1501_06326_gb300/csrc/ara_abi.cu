@@ -31,8 +31,8 @@ constexpr int64_t kShapeOrderMin = 4096;
 // occurrences stream through it (16 layers: 2^19 trials; measured on batched-16, 6.2 ms a pass against
 // 8.1 ms in one slice and 6.6 ms at 2^18).
 constexpr int kYetGridShift = 18;
-// The index is built by buckets per (event, grid cell) while no bucket holds more occurrences than this
-// (each bucket is sorted by one thread), else by the radix sort.
+// Where the index is built by buckets per (event, grid cell), it is while no bucket holds more occurrences than
+// this (each bucket is sorted by one thread), else by the radix sort.
 constexpr uint32_t kYetBucketSortMax = 2048;
 constexpr int64_t kIdxSliceBytes = int64_t{64} << 20;
 int idx_slice_shift(int n_layers) {
@@ -250,7 +250,7 @@ bool timed_begin(ara_ctx* c, int kind, ara_ctx::Timed* t) {
     for (int i = 0; i < t->n(); ++i) t->e[i] = c->ev[i];
     return true;
   }
-  if (c->timed.size() >= kTimedHeld) {
+  if (c->timed.size() >= kTimedHeld + 8) {  // (eight at a time)
     const bool captured = stream_captured(c);
     RelaxedCapture relaxed;
     while (!captured && c->timed.size() >= kTimedHeld) {
